@@ -3,6 +3,7 @@
 // second-Born Dyson iteration (Sec. 2.3). Every numerical step is a kernel of
 // this library; the host only sequences launches and reads scalars.
 #include "common.cuh"
+#include "crt.cuh"
 #include "tc_sys.cuh"
 
 #include <math.h>
@@ -52,6 +53,20 @@ bool ensure(fedvr_ctx *ctx, DevBuf &buf, size_t bytes, const char *name) {
     ctx->failed = true;
     return false;
   }
+  buf.bytes = bytes;
+  return true;
+}
+
+bool ensure_optional(fedvr_ctx *ctx, DevBuf &buf, size_t bytes) {
+  if (buf.bytes >= bytes) return true;
+  void *p = nullptr;
+  if (cudaMalloc(&p, bytes) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  drop_graph(ctx);  // the captured iteration holds the old address
+  if (buf.ptr) cudaFree(buf.ptr);
+  buf.ptr = p;
   buf.bytes = bytes;
   return true;
 }
@@ -131,6 +146,60 @@ int ensure_c1f(fedvr_ctx *ctx, int n, int M) {
   return FEDVR_OK;
 }
 
+// First convolution of the FP64 path: by residues on the tensor cores
+// (crt_conv.cu) where its workspace can be had, with the FP64 kernel behind it
+// for inputs that are not finite; else the FP64 kernel alone. conv_f64_prepare
+// allocates and is called outside graph capture; conv_f64_source forms the
+// residues of the source stack A (once for several applications to other G).
+int conv_f64_prepare(fedvr_ctx *ctx, int n, int M, int np, bool ext, CrtConv *plan) {
+  plan->bytes = 0;
+  CrtConv c;
+  if (crt_conv_plan(n, M, np, ext, ctx->num_sms, &c) && ensure_optional(ctx, ctx->w_crt, c.bytes)) {
+    *plan = c;
+    return FEDVR_OK;
+  }
+  return ensure_c1f(ctx, n, M);
+}
+int conv_f64_source(fedvr_ctx *ctx, const CrtConv &c, const ConvCoef *coef, const double *dHF,
+                    const double *A, cudaStream_t s, int *launches) {
+  if (!c.bytes) return FEDVR_OK;
+  FEDVR_CK(ctx, crt_conv_source(c, ctx->w_crt.ptr, A, dHF, coef, s));
+  *launches += 2;
+  return FEDVR_OK;
+}
+int conv_f64_apply(fedvr_ctx *ctx, const CrtConv &c, int n, int M, const ConvCoef *coef,
+                   const double *dHF, const double *A, const double *G, double *I1, cudaStream_t s,
+                   int *launches) {
+  if (!c.bytes) {
+    FEDVR_CK(ctx, conv1_fp64(n, M, coef, dHF, A, G, I1, s, P<double>(ctx->w_c1f)));
+    *launches += conv1_fp64_splits(n, M) > 1 ? 2 : 1;
+    return FEDVR_OK;
+  }
+  FEDVR_CK(ctx, crt_conv_apply(c, ctx->w_crt.ptr, G, coef, I1, ctx->num_sms, s));
+  FEDVR_CK(ctx, conv1_fp64(n, M, coef, dHF, A, G, I1, s, nullptr, P<int>(ctx->w_crt)));
+  *launches += 6;
+  return FEDVR_OK;
+}
+// The whole first convolution (trapezoid or, with coef4, the fourth-order table).
+int conv_f64(fedvr_ctx *ctx, const CrtConv &c, int n, int M, const ConvCoef *coef,
+             const ConvCoef4 *coef4, const double *dHF, const double *A, const double *G, double *I1,
+             cudaStream_t s, int *launches) {
+  if (!coef4) {
+    if (int r = conv_f64_source(ctx, c, coef, dHF, A, s, launches)) return r;
+    return conv_f64_apply(ctx, c, n, M, coef, dHF, A, G, I1, s, launches);
+  }
+  if (!c.bytes) {
+    FEDVR_CK(ctx, conv1_fp64_q4(n, M, coef4, dHF, A, G, I1, s, P<double>(ctx->w_c1f)));
+    *launches += conv1_fp64_splits(n, M) > 1 ? 2 : 1;
+    return FEDVR_OK;
+  }
+  FEDVR_CK(ctx, crt_conv_source4(c, ctx->w_crt.ptr, A, dHF, coef4, s));
+  FEDVR_CK(ctx, crt_conv_apply4(c, ctx->w_crt.ptr, G, coef4, I1, ctx->num_sms, s));
+  FEDVR_CK(ctx, conv1_fp64_q4(n, M, coef4, dHF, A, G, I1, s, nullptr, P<int>(ctx->w_crt)));
+  *launches += 8;
+  return FEDVR_OK;
+}
+
 // GW screened interaction of g and Sigma^GW = spin g o w: the damped fixed-point
 // iteration w <- (1 - a) w + a (V Q V - spin V (Q * w)) from w (V Q V when
 // !w_valid) until max|w_new - w| < tol, with Q * w the periodic convolution of
@@ -144,12 +213,16 @@ int gw_solve(fedvr_ctx *ctx, int n, int M, const double *V, const double *G, dou
   cudaStream_t s = ctx->stream;
   const size_t stack = (size_t)M * n * n;
   const long nn = (long)n * n;
+  int launches = 0;
+  CrtConv plan;
+  if (int r = conv_f64_prepare(ctx, n, M, 2, false, &plan)) return r;
   FEDVR_CK(ctx, gw_bubble(n, M, V, G, Q, T1, VQV, s));
+  if (int r = conv_f64_source(ctx, plan, coef, dummy, Q, s, &launches)) return r;
   if (!w_valid) FEDVR_CK(ctx, launch_copy(stack, VQV, w, s));
   double r = 0.0;
   int it = 0;
   for (it = 1; it <= max_iter; ++it) {
-    FEDVR_CK(ctx, conv1_fp64(n, M, coef, dummy, Q, w, C, s, P<double>(ctx->w_c1f)));
+    if (int r = conv_f64_apply(ctx, plan, n, M, coef, dummy, Q, w, C, s, &launches)) return r;
     FEDVR_CK(ctx, launch_copy(stack, VQV, Nw, s));
     FEDVR_CK(ctx, dgemm(false, false, n, n, n, -ctx->spin, V, n, 0, C, n, nn, nullptr, 0, 1.0, Nw,
                         n, nn, M, s));
@@ -225,7 +298,8 @@ int gw_workspace(fedvr_ctx *ctx, int n, int M) {
   ENSURE(ctx, g_res, 16);
   ENSURE(ctx, w_t1, dsz(stack));
   ENSURE(ctx, w_t2, dsz(stack));
-  return ensure_c1f(ctx, n, M);
+  CrtConv plan;
+  return conv_f64_prepare(ctx, n, M, 2, false, &plan);
 }
 
 // Tables of the fourth-order variant for the mesh in w_tau (M points).
@@ -591,19 +665,13 @@ int phase_mid(fedvr_ctx *ctx, cudaStream_t s, int *launches) {
 
 // (3) FP64 first convolution (the split path launches its tensor-core kernel instead).
 int phase_conv1_fp64(fedvr_ctx *ctx, cudaStream_t s, int *launches) {
-  const int extra = conv1_fp64_splits(ctx->n, ctx->M) > 1 ? 1 : 0;  // the split sum
-  if (ctx->quad_order == 4) {
-    FEDVR_CK(ctx, conv1_fp64_q4(ctx->n, ctx->M, P<ConvCoef4>(ctx->w_q4coef), P<double>(ctx->w_dHF),
-                                P<double>(ctx->w_S), P<double>(ctx->w_G), P<double>(ctx->w_I1), s,
-                                P<double>(ctx->w_c1f)));
-    *launches += 1 + extra;
-    return FEDVR_OK;
-  }
-  FEDVR_CK(ctx, conv1_fp64(ctx->n, ctx->M, P<ConvCoef>(ctx->w_coef), P<double>(ctx->w_dHF),
-                           P<double>(ctx->w_S), P<double>(ctx->w_G), P<double>(ctx->w_I1), s,
-                           P<double>(ctx->w_c1f)));
-  *launches += 1 + extra;
-  return FEDVR_OK;
+  const bool q4 = ctx->quad_order == 4;
+  CrtConv plan{};  // the workspace of either path was allocated by fedvr_2b_prepare
+  if (ctx->c1_crt && !crt_conv_plan(ctx->n, ctx->M, q4 ? 4 : 2, true, ctx->num_sms, &plan))
+    return fail(ctx, FEDVR_ERR_STATE, "residue workspace of another run");
+  return conv_f64(ctx, plan, ctx->n, ctx->M, P<ConvCoef>(ctx->w_coef),
+                  q4 ? P<ConvCoef4>(ctx->w_q4coef) : nullptr, P<double>(ctx->w_dHF),
+                  P<double>(ctx->w_S), P<double>(ctx->w_G), P<double>(ctx->w_I1), s, launches);
 }
 
 
@@ -789,7 +857,7 @@ void fedvr_destroy(fedvr_ctx *ctx) {
                     &ctx->k_S, &ctx->k_T1, &ctx->k_R, &ctx->k_aux, &ctx->k_out,
                     &ctx->k_part, &ctx->k_sh, &ctx->k_aop, &ctx->k_o, &ctx->k_flag, &ctx->k_x,
                     &ctx->g_w, &ctx->g_vqv, &ctx->g_c, &ctx->g_new, &ctx->g_coef, &ctx->g_res,
-                    &ctx->m_t, &ctx->m_src, &ctx->m_y, &ctx->w_c1f};
+                    &ctx->m_t, &ctx->m_src, &ctx->m_y, &ctx->w_c1f, &ctx->w_crt};
   drop_graph(ctx);
   if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
   for (DevBuf *b : bufs) release(*b);
@@ -1088,7 +1156,9 @@ int fedvr_2b_prepare(fedvr_ctx *ctx, double beta, int u, int p, int precision) {
   ENSURE(ctx, w_part, dsz(4 * (size_t)M + 3 * (size_t)n));  // launch_energy's partials
   ENSURE(ctx, w_red, dsz(8));
   if (!is_split(precision)) {
-    if (int r = ensure_c1f(ctx, n, M)) return r;
+    CrtConv plan;
+    if (int r = conv_f64_prepare(ctx, n, M, ctx->quad_order == 4 ? 4 : 2, true, &plan)) return r;
+    ctx->c1_crt = plan.bytes > 0;
   }
   if (is_split(precision)) {
     float *ws, *S32;
@@ -2004,18 +2074,16 @@ int fedvr_conv_sigma_g(fedvr_ctx *ctx, int n, double beta, int u, int p, const d
     if (int r = sync(ctx)) return r;
     return flag_status(ctx, h_err, err);
   }
-  if (ctx->quad_order == 4) {
-    if (int r = check_quad(ctx, precision, M)) return r;
+  const bool q4 = ctx->quad_order == 4;
+  if (q4) {
     if (int r = build_quad4(ctx, M, beta)) return r;
-    if (int r = ensure_c1f(ctx, n, M)) return r;
-    FEDVR_CK(ctx, conv1_fp64_q4(n, M, P<ConvCoef4>(ctx->w_q4coef), dHF, Sigma, G, I1, ctx->stream,
-                                P<double>(ctx->w_c1f)));
-    return FEDVR_OK;
   }
-  if (int r = ensure_c1f(ctx, n, M)) return r;
-  FEDVR_CK(ctx, conv1_fp64(n, M, P<ConvCoef>(ctx->w_coef), dHF, Sigma, G, I1, ctx->stream,
-                           P<double>(ctx->w_c1f)));
-  return FEDVR_OK;
+  CrtConv plan;
+  int launches = 0;
+  if (int r = conv_f64_prepare(ctx, n, M, q4 ? 4 : 2, true, &plan)) return r;
+  return conv_f64(ctx, plan, n, M, P<ConvCoef>(ctx->w_coef),
+                  q4 ? P<ConvCoef4>(ctx->w_q4coef) : nullptr, dHF, Sigma, G, I1, ctx->stream,
+                  &launches);
 }
 
 int fedvr_conv_g0(fedvr_ctx *ctx, int n, double beta, int u, int p, const double *eps,

@@ -104,6 +104,9 @@ struct fedvr_ctx {
   fedvr::DevBuf m_t, m_src, m_y;
   // partial stacks of the FP64 first convolution's mesh-range splits (small launches)
   fedvr::DevBuf w_c1f;
+  // residue workspace of the FP64 first convolution (crt_conv.cu)
+  fedvr::DevBuf w_crt;
+  bool c1_crt = false;  // the prepared run's first convolution runs by residues
 };
 
 namespace fedvr {
@@ -113,6 +116,8 @@ int fail(fedvr_ctx *ctx, int code, const char *fmt, ...);
 // workspace (split-TF32 or FP64 per the prepared precision); synchronous.
 int sigma_of_current_g(fedvr_ctx *ctx);
 int cuda_fail(fedvr_ctx *ctx, cudaError_t e, const char *what, const char *file, int line);
+// The same for an optional workspace: false (no error recorded) if it cannot be had.
+bool ensure_optional(fedvr_ctx *ctx, DevBuf &buf, size_t bytes);
 // Ensure buf holds at least `bytes`; returns false (and records the error) on failure.
 bool ensure(fedvr_ctx *ctx, DevBuf &buf, size_t bytes, const char *name);
 void release(DevBuf &buf);
@@ -219,6 +224,11 @@ cudaError_t make_tmap_rows16(CUtensorMap *map, const void *base, int n, int M, i
 cudaError_t make_tmap_tail16(CUtensorMap *map, const void *base, int n, int cols, int pitch,
                              int rows);
 
+// 3-D map over FP16 planes [planes][rows][pitch] (pitch a multiple of 64), box
+// 64 halves x box_rows x 1, rows beyond `rows` read as zero.
+cudaError_t make_tmap_planes16(CUtensorMap *map, const void *base, long pitch, int rows, int planes,
+                               int box_rows);
+
 // sigma2_tc.cu (tensor cores, split TF32): the split workspace of a system
 // holds 4 * M*n*ld + n*ld floats (g32, gh, gl, VQ, V32; ld = n rounded up to 32).
 size_t sigma2_tc_smem_bytes(int n);
@@ -238,11 +248,13 @@ cudaError_t launch_sigma_to_f32(int n, int M, const double *S, float *S32, cudaS
 // (conv1_fp64_splits(n, M) - 1) M n n doubles that lets a small launch split
 // the mesh-point range over more CTAs (partial sums added in split order).
 int conv1_fp64_splits(int n, int M);
+// gate (device int, may be NULL): the kernel runs only if *gate != 0.
 cudaError_t conv1_fp64(int n, int M, const ConvCoef *coef, const double *dHF, const double *A,
-                       const double *G, double *I1, cudaStream_t s, double *part = nullptr);
+                       const double *G, double *I1, cudaStream_t s, double *part = nullptr,
+                       const int *gate = nullptr);
 cudaError_t conv1_fp64_q4(int n, int M, const ConvCoef4 *coef, const double *dHF,
                           const double *A, const double *G, double *I1, cudaStream_t s,
-                          double *part = nullptr);
+                          double *part = nullptr, const int *gate = nullptr);
 // W (may be NULL): per-(i, j) weights replacing w_j (fourth-order variant;
 // wm, wp are then its end weights wL, wR).
 cudaError_t launch_conv2_kernel(int n, int M, double beta, const double *tau, const double *w,

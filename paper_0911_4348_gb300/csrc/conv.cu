@@ -72,10 +72,14 @@ __global__ void __launch_bounds__(256) conv1_fp64_kernel(int n, int M, int rows,
                                                          const double *__restrict__ A,
                                                          const double *__restrict__ G,
                                                          double *__restrict__ I1,
-                                                         double *__restrict__ part) {
+                                                         double *__restrict__ part,
+                                                         const int *__restrict__ gate) {
   extern __shared__ double c1s[];
+  if (gate && *gate == 0) return;
   double *Xs = c1s, *Ys = c1s + rows * kC1K;
-  const int i = blockIdx.y, a0 = blockIdx.x * rows;
+  const int tiles = (n + rows - 1) / rows;
+  for (long blk = blockIdx.x; blk < (long)tiles * M * splits; blk += gridDim.x) {
+  const int a0 = (int)(blk % tiles) * rows, i = (int)(blk / tiles % M);
   const int nr = min(rows, n - a0), nout = nr * n;
   const long nn = (long)n * n;
   const int tid = threadIdx.x;
@@ -90,7 +94,7 @@ __global__ void __launch_bounds__(256) conv1_fp64_kernel(int n, int M, int rows,
     yo[q] = o < nout ? o % n : 0;
     nq += o < nout ? 1 : 0;
   }
-  const int sp = blockIdx.z;
+  const int sp = (int)(blk / tiles / M);
   const int j0 = (int)((long)M * sp / splits), j1 = (int)((long)M * (sp + 1) / splits);
   for (int j = j0; j < j1; ++j) {
     const CoefView cv = coef_view(coef[(long)i * M + j], M);
@@ -127,6 +131,7 @@ __global__ void __launch_bounds__(256) conv1_fp64_kernel(int n, int M, int rows,
     const int o = tid + 256 * q;
     out[(long)i * nn + (long)(a0 + o / n) * n + o % n] = acc[q];
   }
+  }
 }
 
 // I1 += the partial stacks of splits 1 .. parts, in split order.
@@ -143,7 +148,8 @@ inline int c1_rows(int n) { return n < 256 * kC1Q / n ? n : 256 * kC1Q / n; }
 
 template <typename Coef>
 cudaError_t launch_conv1_fp64(int n, int M, const Coef *coef, const double *dHF, const double *A,
-                              const double *G, double *I1, double *part, cudaStream_t s) {
+                              const double *G, double *I1, double *part, cudaStream_t s,
+                              const int *gate) {
   const int rows = c1_rows(n);
   if (rows < 1) return cudaErrorInvalidValue;
   const size_t sm = (size_t)(rows * kC1K + kC1K * n) * sizeof(double);
@@ -152,8 +158,10 @@ cudaError_t launch_conv1_fp64(int n, int M, const Coef *coef, const double *dHF,
   if (e != cudaSuccess) return e;
   const int tiles = (n + rows - 1) / rows;
   const int splits = part ? conv1_fp64_splits(n, M) : 1;
-  dim3 grid((unsigned)tiles, (unsigned)M, (unsigned)splits);
-  conv1_fp64_kernel<Coef><<<grid, 256, sm, s>>>(n, M, rows, splits, coef, dHF, A, G, I1, part);
+  const long blocks = (long)tiles * M * splits;
+  const unsigned grid = (unsigned)(gate ? (blocks < 608 ? blocks : 608) : blocks);
+  conv1_fp64_kernel<Coef><<<grid, 256, sm, s>>>(n, M, rows, splits, coef, dHF, A, G, I1, part,
+                                                gate);
   e = cudaGetLastError();
   if (e != cudaSuccess || splits == 1) return e;
   const long count = (long)M * n * n;
@@ -379,15 +387,16 @@ int conv1_fp64_splits(int n, int M) {
 }
 
 cudaError_t conv1_fp64(int n, int M, const ConvCoef *coef, const double *dHF, const double *A,
-                       const double *G, double *I1, cudaStream_t s, double *part) {
-  return launch_conv1_fp64<ConvCoef>(n, M, coef, dHF, A, G, I1, part, s);
+                       const double *G, double *I1, cudaStream_t s, double *part,
+                       const int *gate) {
+  return launch_conv1_fp64<ConvCoef>(n, M, coef, dHF, A, G, I1, part, s, gate);
 }
 
 cudaError_t conv1_fp64_q4(int n, int M, const ConvCoef4 *coef, const double *dHF,
                           const double *A, const double *G, double *I1, cudaStream_t s,
-                          double *part) {
+                          double *part, const int *gate) {
   if (M < 4) return cudaErrorInvalidValue;
-  return launch_conv1_fp64<ConvCoef4>(n, M, coef, dHF, A, G, I1, part, s);
+  return launch_conv1_fp64<ConvCoef4>(n, M, coef, dHF, A, G, I1, part, s, gate);
 }
 
 cudaError_t launch_quad4_tables(int M, double beta, const double *tau, ConvCoef4 *coef,

@@ -68,6 +68,22 @@ cudaError_t make_tmap_rows16(CUtensorMap *map, const void *base, int n, int M, i
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
+cudaError_t make_tmap_planes16(CUtensorMap *map, const void *base, long pitch, int rows, int planes,
+                               int box_rows) {
+  std::call_once(g_encode_once, load_encoder);
+  if (!g_encode) return cudaErrorNotSupported;
+  if (box_rows < 1 || box_rows > 256 || pitch % 64 != 0 || pitch < 64) return cudaErrorInvalidValue;
+  const cuuint64_t dims[3] = {(cuuint64_t)pitch, (cuuint64_t)rows, (cuuint64_t)planes};
+  const cuuint64_t strides[2] = {(cuuint64_t)pitch * 2, (cuuint64_t)rows * (cuuint64_t)pitch * 2};
+  const cuuint32_t box[3] = {64, (cuuint32_t)box_rows, 1};
+  const cuuint32_t estr[3] = {1, 1, 1};
+  CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<void *>(base), dims,
+                        strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                        CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
 cudaError_t make_tmap_tail16(CUtensorMap *map, const void *base, int n, int cols, int pitch,
                              int rows) {
   std::call_once(g_encode_once, load_encoder);
