@@ -180,7 +180,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   } else if (warp == 12) {
     // ---- TMA: g_j rows 0..Np-1, 32 columns per chunk, hi and lo ----
-    if (lane == 0) {
+    if (tc::elect_one()) {
       uint32_t cc = 0;
       for (long w = blockIdx.x; w < items && !*abort_flag; w += gridDim.x) {
         while (cur + 1 < n_sys && w >= prefix[cur + 1]) ++cur;
@@ -214,7 +214,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   } else if (warp == 13) {
     // ---- MMA issue: one accumulator block per JB mesh points ----
-    if (lane == 0) {
+    if (tc::elect_one()) {
       uint32_t cc = 0, tcount = 0;
       for (long w = blockIdx.x; w < items && !*abort_flag; w += gridDim.x) {
         while (cur + 1 < n_sys && w >= prefix[cur + 1]) ++cur;
@@ -326,7 +326,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   __syncthreads();
   if (*abort_flag) {
-    if (warp == 13 && lane == 0) {
+    if (warp == 13 && (issued || lane == 0)) {
       if (issued) tc::mma_commit(drain);
       atomicExch(err, 1);
       if (issued) tc::mbar_wait(drain, 0, kWaitNs);
@@ -643,7 +643,7 @@ __global__ void __launch_bounds__(kThreadsH, 1)
     }
   } else if (warp == 20) {
     // ---- TMA: g_j FP16 split rows 0..Np-1, 64 columns per chunk, hi and lo ----
-    if (lane == 0) {
+    if (tc::elect_one()) {
       uint32_t cc = 0;
       for (long w = blockIdx.x; w < items && !*abort_flag; w += gridDim.x) {
         while (cur + 1 < n_sys && w >= prefix[cur + 1]) ++cur;
@@ -693,7 +693,7 @@ __global__ void __launch_bounds__(kThreadsH, 1)
     }
   } else if (warp == 21) {
     // ---- MMA issue (kind::f16, K = 16 per instruction) ----
-    if (lane == 0) {
+    if (tc::elect_one()) {
       uint32_t cc = 0, tcount = 0;
       for (long w = blockIdx.x; w < items && !*abort_flag; w += gridDim.x) {
         while (cur + 1 < n_sys && w >= prefix[cur + 1]) ++cur;
@@ -814,7 +814,7 @@ __global__ void __launch_bounds__(kThreadsH, 1)
 
   __syncthreads();
   if (*abort_flag) {
-    if (warp == 21 && lane == 0) {
+    if (warp == 21 && (issued || lane == 0)) {
       if (issued) tc::mma_commit(drain);
       atomicExch(err, 1);
       if (issued) tc::mbar_wait(drain, 0, kWaitNs);

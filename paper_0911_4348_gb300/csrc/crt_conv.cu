@@ -509,7 +509,7 @@ __global__ void __launch_bounds__(kThreads, 1) crt_conv_kernel(const __grid_cons
     }
   } else if (warp == kTmaWarp) {
     // ---- TMA: Np rows x 64 columns of this modulus' plane of g ----
-    if (lane == 0) {
+    if (tc::elect_one()) {
       int s = 0;
       uint32_t ph = 1;
       for (long w = blockIdx.x; w < p.items && !*abort_flag; w += gridDim.x) {
@@ -531,7 +531,7 @@ __global__ void __launch_bounds__(kThreads, 1) crt_conv_kernel(const __grid_cons
     }
   } else if (warp == kMmaWarp) {
     // ---- MMA issue ----
-    if (lane == 0) {
+    if (tc::elect_one()) {
       const uint32_t idesc = tc::idesc_f16(128, p.Np);
       int s = 0;
       uint32_t ph = 0;
@@ -642,7 +642,7 @@ __global__ void __launch_bounds__(kThreads, 1) crt_conv_kernel(const __grid_cons
 
   __syncthreads();
   if (*abort_flag) {
-    if (warp == kMmaWarp && lane == 0) {
+    if (warp == kMmaWarp && (issued || lane == 0)) {
       if (issued) tc::mma_commit(drain);
       atomicExch(p.flag, 2);  // the FP64 kernel that follows recomputes the result
       if (issued) tc::mbar_wait(drain, 0, kWaitNs);

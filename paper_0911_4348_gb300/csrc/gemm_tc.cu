@@ -279,7 +279,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tf32x3_kernel(GemmArgs p) {
     }
   } else if (warp == 12) {
     // ---- MMA issue (kind::tf32, K = 8 per instruction) ----
-    if (lane == 0) {
+    if (tc::elect_one()) {
       const uint32_t idesc = tc::idesc_tf32(128, Nt);
       for (int kc = 0; kc < KC; ++kc) {
         const int s = kc & 1;
@@ -342,7 +342,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tf32x3_kernel(GemmArgs p) {
   __syncthreads();
   if (*abort_flag) {
     // let MMAs still in flight finish (bounded) before the TMEM goes away
-    if (warp == 12 && lane == 0) {
+    if (warp == 12 && (issued || lane == 0)) {
       if (issued) tc::mma_commit(drain);
       atomicExch(p.err, 1);
       if (issued) tc::mbar_wait(drain, 0, kWaitNs);

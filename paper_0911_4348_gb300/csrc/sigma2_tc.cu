@@ -257,7 +257,7 @@ __global__ void __launch_bounds__(XRoles<F16>::kThreads, 1)
     }
   } else if (warp == R::kTma) {
     // ---- TMA: gb = G[M-1-j] rows 0..Np-1, one chunk of columns per stage, hi and lo ----
-    if (lane == 0) {
+    if (tc::elect_one()) {
       uint32_t cc = 0;
       for (long w = blockIdx.x; w < items && !*abort_flag; w += gridDim.x) {
         while (cur + 1 < n_sys && w >= prefix[cur + 1]) ++cur;
@@ -289,7 +289,7 @@ __global__ void __launch_bounds__(XRoles<F16>::kThreads, 1)
     }
   } else if (warp == R::kMma) {
     // ---- MMA issue: one accumulator per tile ----
-    if (lane == 0) {
+    if (tc::elect_one()) {
       uint32_t cc = 0, tcount = 0;
       for (long w = blockIdx.x; w < items && !*abort_flag; w += gridDim.x, ++tcount) {
         while (cur + 1 < n_sys && w >= prefix[cur + 1]) ++cur;
@@ -471,7 +471,7 @@ __global__ void __launch_bounds__(XRoles<F16>::kThreads, 1)
   __syncthreads();
   if (*abort_flag) {
     // let MMAs still in flight finish (bounded) before the TMEM goes away
-    if (warp == R::kMma && lane == 0) {
+    if (warp == R::kMma && (issued || lane == 0)) {
       if (issued) tc::mma_commit(drain);
       atomicExch(err, 1);
       if (issued) tc::mbar_wait(drain, 0, kWaitNs);
