@@ -200,6 +200,22 @@ int conv_f64(fedvr_ctx *ctx, const CrtConv &c, int n, int M, const ConvCoef *coe
   return FEDVR_OK;
 }
 
+// Second-Born self-energy of the FP64 path: the exchange by residues where its
+// workspace can be had (sigma_f64_prepare, outside capture).
+int sigma_f64_prepare(fedvr_ctx *ctx, int n, int M, CrtSigma *plan) {
+  plan->bytes = 0;
+  CrtSigma c;
+  if (crt_sigma_plan(n, M, &c) && ensure_optional(ctx, ctx->w_crtx, c.bytes)) *plan = c;
+  return FEDVR_OK;
+}
+int sigma_f64(fedvr_ctx *ctx, const CrtSigma &c, int n, int M, double spin, const double *V,
+              const double *G, double *Sigma, cudaStream_t s, int *launches) {
+  FEDVR_CK(ctx, sigma2_fp64(n, M, spin, V, G, Sigma, P<double>(ctx->w_t1), P<double>(ctx->w_t2),
+                            P<double>(ctx->w_t3), s, &c, ctx->w_crtx.ptr, ctx->num_sms));
+  *launches += c.bytes ? 7 + 5 * ((c.nm + c.group - 1) / c.group) : 4;
+  return FEDVR_OK;
+}
+
 // GW screened interaction of g and Sigma^GW = spin g o w: the damped fixed-point
 // iteration w <- (1 - a) w + a (V Q V - spin V (Q * w)) from w (V Q V when
 // !w_valid) until max|w_new - w| < tol, with Q * w the periodic convolution of
@@ -629,9 +645,10 @@ int phase_sigma_pre(fedvr_ctx *ctx, bool warm, cudaStream_t s, int *launches, in
     ctx->gw_last_inner = it;
     *launches += 2 + 2 * it;
   } else {
-    FEDVR_CK(ctx, sigma2_fp64(n, M, ctx->spin, V, G, S, P<double>(ctx->w_t1), P<double>(ctx->w_t2),
-                              P<double>(ctx->w_t3), s));
-    *launches += 4;
+    CrtSigma plan{};  // its workspace was allocated by fedvr_2b_prepare
+    if (ctx->x_crt && !crt_sigma_plan(n, M, &plan))
+      return fail(ctx, FEDVR_ERR_STATE, "residue workspace of another run");
+    if (int r = sigma_f64(ctx, plan, n, M, ctx->spin, V, G, S, s, launches)) return r;
   }
   return FEDVR_OK;
 }
@@ -857,7 +874,7 @@ void fedvr_destroy(fedvr_ctx *ctx) {
                     &ctx->k_S, &ctx->k_T1, &ctx->k_R, &ctx->k_aux, &ctx->k_out,
                     &ctx->k_part, &ctx->k_sh, &ctx->k_aop, &ctx->k_o, &ctx->k_flag, &ctx->k_x,
                     &ctx->g_w, &ctx->g_vqv, &ctx->g_c, &ctx->g_new, &ctx->g_coef, &ctx->g_res,
-                    &ctx->m_t, &ctx->m_src, &ctx->m_y, &ctx->w_c1f, &ctx->w_crt};
+                    &ctx->m_t, &ctx->m_src, &ctx->m_y, &ctx->w_c1f, &ctx->w_crt, &ctx->w_crtx};
   drop_graph(ctx);
   if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
   for (DevBuf *b : bufs) release(*b);
@@ -1159,6 +1176,11 @@ int fedvr_2b_prepare(fedvr_ctx *ctx, double beta, int u, int p, int precision) {
     CrtConv plan;
     if (int r = conv_f64_prepare(ctx, n, M, ctx->quad_order == 4 ? 4 : 2, true, &plan)) return r;
     ctx->c1_crt = plan.bytes > 0;
+    CrtSigma xplan{};
+    if (ctx->self_energy == 0) {
+      if (int r = sigma_f64_prepare(ctx, n, M, &xplan)) return r;
+    }
+    ctx->x_crt = xplan.bytes > 0;
   }
   if (is_split(precision)) {
     float *ws, *S32;
@@ -2013,9 +2035,10 @@ int fedvr_sigma2(fedvr_ctx *ctx, int n, int M, double spin, const double *V, con
   ENSURE(ctx, w_t1, dsz(stack));
   ENSURE(ctx, w_t2, dsz(stack));
   ENSURE(ctx, w_t3, dsz(stack));
-  FEDVR_CK(ctx, sigma2_fp64(n, M, spin, V, G, Sigma, P<double>(ctx->w_t1), P<double>(ctx->w_t2),
-                            P<double>(ctx->w_t3), ctx->stream));
-  return FEDVR_OK;
+  CrtSigma plan;
+  int launches = 0;
+  if (int r = sigma_f64_prepare(ctx, n, M, &plan)) return r;
+  return sigma_f64(ctx, plan, n, M, spin, V, G, Sigma, ctx->stream, &launches);
 }
 
 int fedvr_conv_sigma_g(fedvr_ctx *ctx, int n, double beta, int u, int p, const double *dHF,

@@ -107,6 +107,9 @@ struct fedvr_ctx {
   // residue workspace of the FP64 first convolution (crt_conv.cu)
   fedvr::DevBuf w_crt;
   bool c1_crt = false;  // the prepared run's first convolution runs by residues
+  // and of the FP64 exchange (crt_sigma.cu)
+  fedvr::DevBuf w_crtx;
+  bool x_crt = false;
 };
 
 namespace fedvr {
@@ -192,8 +195,12 @@ cudaError_t launch_phi_table(int n, int M, double beta, const double *eps, const
                              double mu_host, const double *tau, double *phi, cudaStream_t s);
 
 // sigma2.cu (FP64 path)
+// crt (may be NULL): the exchange by residues on the tensor cores with its
+// workspace ws (crt_sigma.cu), the FP64 kernel behind it.
+struct CrtSigma;
 cudaError_t sigma2_fp64(int n, int M, double spin, const double *V, const double *G,
-                        double *Sigma, double *Q, double *T1, double *W, cudaStream_t s);
+                        double *Sigma, double *Q, double *T1, double *W, cudaStream_t s,
+                        const CrtSigma *crt = nullptr, void *ws = nullptr, int num_sms = 0);
 // GW pieces: the bubble Q_j = g_j o g_{M-1-j} and V Q_j V; Sigma = spin g o w.
 cudaError_t gw_bubble(int n, int M, const double *V, const double *G, double *Q, double *T1,
                       double *VQV, cudaStream_t s);

@@ -39,7 +39,6 @@ struct CrtMods {
   int nm;
   float p[kCrtMax], ip[kCrtMax];
   float mul[kCrtMax], sub[kCrtMax];  // residue of x * mul (mul: 1 or the CRT inverse)
-  float fold[kCrtMax];               // the CRT inverse
   uint32_t r21[kCrtMax], r42[kCrtMax], mg[kCrtMax];
 };
 // Of the moduli m0 .. m0 + count - 1 of nm (count < 0: all). inverse: mul =
@@ -100,5 +99,22 @@ cudaError_t crt_conv_apply(const CrtConv &c, void *ws, const double *G, const Co
                            double *I1, int num_sms, cudaStream_t s);
 cudaError_t crt_conv_apply4(const CrtConv &c, void *ws, const double *G, const ConvCoef4 *coef,
                             double *I1, int num_sms, cudaStream_t s);
+
+// Second-Born self-energy by residues (crt_sigma.cu): plan and workspace.
+struct CrtSigma {
+  CrtK k;
+  int nm, q, CT, Np, NCB;   // moduli, entry bits, column tiles, their width, chunks per mesh point
+  int nr, ph;               // rows and pitch (16-bit values) of a plain operand matrix
+  int group;                // moduli whose operand planes are held at one time
+  int nA, nB;               // stages of A, buffers of gb
+  long T;                   // 128-row tiles per mesh point
+  size_t o_exp, o_g, o_gt, o_B, o_V, o_Vn, o_R, bytes;
+  size_t smem;
+};
+bool crt_sigma_plan(int n, int M, CrtSigma *out);
+// Sigma = spin g o W - X[g] with the exchange X by residues, W = V Q V given; the
+// first int of ws as for crt_conv_apply.
+cudaError_t crt_sigma_apply(const CrtSigma &c, void *ws, double spin, const double *V, const double *G,
+                            const double *W, double *Sigma, int num_sms, cudaStream_t s);
 
 }  // namespace fedvr

@@ -56,9 +56,7 @@ CrtMods crt_mods(int nm, bool inverse, int m0, int count) {
   c.nm = count < 0 ? nm : count;
   for (int m = 0; m < c.nm; ++m) {
     const int p = kCrtMod[m0 + m];
-    const int inv = inv_mod(prod_mod(nm, m0 + m, p), p);
-    const int mul = inverse ? inv : 1;
-    c.fold[m] = (float)inv;
+    const int mul = inverse ? inv_mod(prod_mod(nm, m0 + m, p), p) : 1;
     c.p[m] = (float)p;
     c.ip[m] = 1.0f / (float)p;
     c.mul[m] = (float)mul;
@@ -714,9 +712,9 @@ cudaError_t apply_t(const CrtConv &c, void *wsv, const double *G, const Coef *co
   int *E = reinterpret_cast<int *>(ws + c.o_E);
   const int n = c.k.n, M = c.k.M;
   crt_exp_stack_kernel<<<M, 256, 0, s>>>((long)n * n, G, eg, flag);
-  crt_g_kernel<false><<<dim3(M + 3, (n + 31) / 32, (c.k.nc + 63) / 64), 256, 0, s>>>(
+  crt_g_kernel<<<dim3(M + 3, (n + 31) / 32, (c.k.nc + 63) / 64), 256, 0, s>>>(
       crt_mods(c.nm, true), c.k, c.q, G, eg, reinterpret_cast<uint32_t *>(ws + c.o_B),
-      nullptr);
+      nullptr, 0, 0);
   crt_coef_kernel<Coef, NP><<<M + 1, 256, 0, s>>>(crt_mods(c.nm, false), M, c.Mp,
                                                   (uint32_t)(n * c.k.nc), coef, es, eg, E,
                                                   reinterpret_cast<CrtEntry<NP> *>(ws + c.o_C));

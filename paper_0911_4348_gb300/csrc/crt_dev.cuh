@@ -145,17 +145,27 @@ __device__ __forceinline__ void put_source(const CrtMods &mods, const CrtK &kk, 
   }
 }
 
+// Two small integers as one word of FP16 or bfloat16 values.
+template <bool BF16>
+__device__ __forceinline__ uint32_t pack16(float r0, float r1) {
+  if constexpr (BF16) {
+    return __byte_perm(__float_as_uint(r0), __float_as_uint(r1), 0x7632);
+  } else {
+    const __half2 h = __floats2half2_rn(r0, r1);
+    return *reinterpret_cast<const uint32_t *>(&h);
+  }
+}
+
 // Residue planes of g as FP16 rows over the flattened contraction index:
-// out[m][b][x(j, c)] = g_j[c][b] (times mods.mul). With bytes, also the plain
-// residues of the transposed matrices, bytes[m][j][b][nc]. A 64 (c) x 32 (b) tile
-// of one mesh point per CTA, transposed through shared memory. CTAs j >= M
+// out[m][b][x(j, c)] = g_j[c][b] (times mods.mul). With nat, also as plain
+// bfloat16 rows nat[m][j][b][c] ([nr] rows of ph values). A 64 (c) x 32 (b) tile of
+// one mesh point per CTA, transposed through shared memory. CTAs j >= M
 // write the zeros that pad the last chunk of each rest.
-template <bool BYTES>
 static __global__ void __launch_bounds__(256) crt_g_kernel(CrtMods mods, CrtK k, int qb,
                                                     const double *__restrict__ G,
                                                     const int *__restrict__ expo,
                                                     uint32_t *__restrict__ out,
-                                                    uint16_t *__restrict__ bytes) {
+                                                    uint32_t *__restrict__ nat, int nr, int ph) {
   __shared__ long long sh[64][33];
   const int j = blockIdx.x, b0 = blockIdx.y * 32, c0 = blockIdx.z * 64;
   const int n = k.n, e = j < k.M ? expo[j] : kCrtZero;
@@ -182,16 +192,10 @@ static __global__ void __launch_bounds__(256) crt_g_kernel(CrtMods mods, CrtK k,
     split21(sh[2 * lane + 1][bb], a0[1], a1[1], a2[1]);
     const long o = ((long)(b0 + bb) * k.KP + crt_x(k, j, c)) / 2;
     for (int m = 0; m < mods.nm; ++m) {
-      float r0 = residue(a0[0], a1[0], a2[0], mods, m), r1 = residue(a0[1], a1[1], a2[1], mods, m);
-      if constexpr (BYTES) {
-        if (j < k.M)
-          bytes[((((long)m * k.M + j) * n + b0 + bb) * k.nc + c) / 2] = (uint16_t)(
-              (__float_as_uint(r0 + kRound) & 0xffu) | ((__float_as_uint(r1 + kRound) & 0xffu) << 8));
-        r0 = modf_bal(r0 * mods.fold[m], mods.p[m], mods.ip[m]);
-        r1 = modf_bal(r1 * mods.fold[m], mods.p[m], mods.ip[m]);
-      }
-      const __half2 h = __floats2half2_rn(r0, r1);
-      out[(long)m * plane + o] = *reinterpret_cast<const uint32_t *>(&h);
+      const float x0 = residue(a0[0], a1[0], a2[0], mods, m), x1 = residue(a0[1], a1[1], a2[1], mods, m);
+      out[(long)m * plane + o] = pack16<false>(x0, x1);
+      if (nat && j < k.M)
+        nat[((((long)m * k.M + j) * nr + b0 + bb) * ph + c) / 2] = pack16<true>(x0, x1);
     }
   }
 }

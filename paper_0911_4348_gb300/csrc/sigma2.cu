@@ -8,6 +8,7 @@
 // element (the paper's count). X is symmetric for symmetric g, gb, so only
 // rows a >= b are formed and the result is mirrored.
 #include "common.cuh"
+#include "crt.cuh"
 
 #include <mutex>
 
@@ -37,11 +38,15 @@ __global__ void __launch_bounds__(256) exchange_fp64_kernel(int n, int M, int ro
                                                             const double *__restrict__ V,
                                                             const double *__restrict__ G,
                                                             const double *__restrict__ W,
-                                                            double *__restrict__ Sigma) {
+                                                            double *__restrict__ Sigma,
+                                                            const int *__restrict__ gate) {
   extern __shared__ double xsm[];
+  if (gate && *gate == 0) return;
   double *Xs = xsm, *Ys = Xs + rows * kXL, *Vs = Ys + kXL * n, *Ps = Vs + rows * n;
-  const int j = blockIdx.z, b = blockIdx.y, a0 = b + blockIdx.x * rows;
-  if (a0 >= n) return;  // past the last row of this column
+  const int tiles = (n + rows - 1) / rows;
+  for (long blk = blockIdx.x; blk < (long)tiles * n * M; blk += gridDim.x) {
+  const int b = (int)(blk / tiles % n), j = (int)(blk / tiles / n), a0 = b + (int)(blk % tiles) * rows;
+  if (a0 >= n) continue;  // past the last row of this column
   const int nr = min(rows, n - a0), nout = nr * n, tid = threadIdx.x;
   const long nn = (long)n * n;
   const double *g = G + (long)j * nn;
@@ -98,6 +103,8 @@ __global__ void __launch_bounds__(256) exchange_fp64_kernel(int n, int M, int ro
     Sigma[(long)j * nn + ab] = v;
     Sigma[(long)j * nn + (long)b * n + a] = v;
   }
+  __syncthreads();  // Ps and the staged operands are rewritten by the next block
+  }
 }
 
 // Sigma^GW = spin g o w (elementwise over the stack).
@@ -130,7 +137,8 @@ cudaError_t launch_gw_sigma(long count, double spin, const double *G, const doub
 }
 
 cudaError_t sigma2_fp64(int n, int M, double spin, const double *V, const double *G,
-                        double *Sigma, double *Q, double *T1, double *W, cudaStream_t s) {
+                        double *Sigma, double *Q, double *T1, double *W, cudaStream_t s,
+                        const CrtSigma *crt, void *ws, int num_sms) {
   long nn = (long)n * n;
   long tot = (long)M * nn;
   polarisation_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(n, M, G, Q);
@@ -147,8 +155,15 @@ cudaError_t sigma2_fp64(int n, int M, double spin, const double *V, const double
   e = cudaFuncSetAttribute(exchange_fp64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)sm);
   if (e != cudaSuccess) return e;
-  dim3 grid((unsigned)((n + rows - 1) / rows), (unsigned)n, (unsigned)M);
-  exchange_fp64_kernel<<<grid, 256, sm, s>>>(n, M, rows, spin, V, G, W, Sigma);
+  const int *gate = nullptr;
+  if (crt && crt->bytes) {
+    e = crt_sigma_apply(*crt, ws, spin, V, G, W, Sigma, num_sms, s);
+    if (e != cudaSuccess) return e;
+    gate = reinterpret_cast<const int *>(ws);
+  }
+  const long blocks = (long)((n + rows - 1) / rows) * n * M;
+  exchange_fp64_kernel<<<(unsigned)(gate && blocks > 608 ? 608 : blocks), 256, sm, s>>>(
+      n, M, rows, spin, V, G, W, Sigma, gate);
   return cudaGetLastError();
 }
 

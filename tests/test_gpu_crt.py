@@ -95,3 +95,42 @@ def test_first_convolution_not_finite_and_zero(ctx):
     ctx.conv_sigma_g(40.0, u, p, _dev(dHF), _dev(A), _dev(0.0 * G), I1)
     torch.cuda.synchronize()
     assert not I1.cpu().numpy().any()
+
+
+def _sigma_case(n, M, seed):
+    rng = W.system_rng(95, seed)
+    mag = 10.0 ** rng.uniform(-4, 1, size=(M, 1, 1))
+    G = mag * W.random_symmetric_stack(rng, M, n)
+    return G, W.random_symmetric(rng, n)
+
+
+# n up to 64, 65 .. and above 256 (two column tiles), every remainder of the
+# 64-wide slices, one and two buffers of gb, a single tile row and partial tiles
+@pytest.mark.parametrize("n,M", [(16, 700), (17, 500), (33, 40), (39, 20), (48, 9), (63, 4), (64, 4),
+                                 (65, 3), (97, 2), (130, 3), (199, 2), (240, 2), (255, 2), (256, 2),
+                                 (257, 2), (299, 2)])
+def test_second_born(ctx, n, M):
+    G, V = _sigma_case(n, M, n)
+    S = torch.empty((M, n, n), dtype=torch.float64, device="cuda")
+    ctx.sigma2(_dev(V), _dev(G), S, 1.5)
+    torch.cuda.synchronize()
+    got = S.cpu().numpy()
+    js = range(M) if n < 100 and M < 50 else [0, M // 2, M - 1]
+    for j in js:  # against each mesh point's own largest entry
+        want = O.sigma2_tau(G[j], G[M - 1 - j], V, 1.5)
+        assert np.max(np.abs(got[j] - want)) < TOL * np.max(np.abs(want)), j
+    assert np.array_equal(got, got.transpose(0, 2, 1))
+
+
+def test_second_born_not_finite(ctx):
+    n, M = 65, 3
+    G, V = _sigma_case(n, M, 1)
+    G[1, 2, 3] = G[1, 3, 2] = np.nan
+    S = torch.empty((M, n, n), dtype=torch.float64, device="cuda")
+    ctx.sigma2(_dev(V), _dev(G), S)
+    torch.cuda.synchronize()
+    got = S.cpu().numpy()
+    assert np.isnan(got[1]).all()  # every sum of that mesh point meets the entry
+    for j in (0, 2):
+        want = O.sigma2_tau(G[j], G[M - 1 - j], V, 2.0)
+        assert np.max(np.abs(got[j] - want)) < TOL * np.max(np.abs(want))
