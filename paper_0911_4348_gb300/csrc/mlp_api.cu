@@ -18,7 +18,7 @@ struct fedvr_mlp {
   int adam_t = 0;
   long rows = 0, cap = 0;  // training rows held / capacity
   unsigned long long seed = 0;
-  fedvr::DevBuf W, m, v, g, Wbf, act, Y, dbuf, part, X, T, idx, bX, bT, sdev, F, S1;
+  fedvr::DevBuf W, m, v, g, Wbf, act, Y, dbuf, part, X, T, idx, bX, bT, sdev, F, S1, slices;
 };
 
 namespace {
@@ -101,6 +101,7 @@ int ensure_rows(fedvr_mlp *m, int rows) {
   MENSURE(m, Y, (size_t)rows * L.dout * sizeof(float));
   MENSURE(m, dbuf, (size_t)2 * rows * wide * sizeof(float));
   MENSURE(m, part, 256 * sizeof(double));
+  MENSURE(m, slices, fedvr::mlp_slice_floats(m->L) * sizeof(float));
   return FEDVR_OK;
 }
 
@@ -170,7 +171,7 @@ void fedvr_mlp_destroy(fedvr_mlp *m) {
   if (!m) return;
   cudaStreamSynchronize(m->stream);
   DevBuf *bufs[] = {&m->W, &m->m, &m->v, &m->g, &m->Wbf, &m->act, &m->Y, &m->dbuf, &m->part,
-                    &m->X, &m->T, &m->idx, &m->bX, &m->bT, &m->sdev, &m->F, &m->S1};
+                    &m->X, &m->T, &m->idx, &m->bX, &m->bT, &m->sdev, &m->F, &m->S1, &m->slices};
   for (DevBuf *b : bufs) fedvr::release(*b);
   delete m;
 }
@@ -227,7 +228,8 @@ int fedvr_mlp_loss_grad(fedvr_mlp *m, const float *X, const float *T, int rows, 
   if (m->failed) return FEDVR_ERR_STATE;
   if (int r = ensure_rows(m, rows)) return r;
   MCK(m, fedvr::mlp_loss_grad(m->L, P<float>(m->W), rows, X, T, P<float>(m->act), P<float>(m->Y),
-                              P<float>(m->dbuf), P<float>(m->g), P<double>(m->part), m->stream));
+                              P<float>(m->dbuf), P<float>(m->g), P<double>(m->part),
+                              P<float>(m->slices), m->stream));
   int st;
   const double l = read_loss(m, &st);
   if (st) return st;
@@ -339,7 +341,8 @@ int fedvr_mlp_train(fedvr_mlp *m, int epochs, int batch, double lr, double *fina
       MCK(m, fedvr::mlp_gather(rows, L.dout, ix, P<float>(m->T), P<float>(m->bT), m->stream));
       MCK(m, fedvr::mlp_loss_grad(L, P<float>(m->W), rows, P<float>(m->bX), P<float>(m->bT),
                                   P<float>(m->act), P<float>(m->Y), P<float>(m->dbuf),
-                                  P<float>(m->g), P<double>(m->part), m->stream));
+                                  P<float>(m->g), P<double>(m->part),
+                              P<float>(m->slices), m->stream));
       MCK(m, fedvr::mlp_adam(L.nparam, (float)lr, ++m->adam_t, P<float>(m->g), P<float>(m->m),
                              P<float>(m->v), P<float>(m->W), m->stream));
       if (e == epochs - 1) {
