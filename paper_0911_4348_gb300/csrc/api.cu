@@ -261,6 +261,14 @@ int gw_solve(fedvr_ctx *ctx, int n, int M, const double *V, const double *G, dou
   return FEDVR_OK;
 }
 
+// Whether the ladder's convolution runs by residues: as a first convolution of
+// n^2 x n^2 matrices it takes 2 M^2 n^6 multiply-adds' worth of FP16 products
+// instead of 4 M^2 n^5 on the FP64 pipe, and seven launches. Measured ms per
+// application, FP64 / residues: n = 5, M = 33: 0.057 / 0.092; n = 7, M = 33: 0.126 /
+// 0.146; n = 7, M = 65: 0.361 / 0.272; n = 11, M = 65: 2.12 / 0.76; n = 15, M = 129:
+// 34.5 / 8.9; n = 24, M = 17: 6.2 / 3.6.
+bool tm_crt(int n, int M) { return 2.0 * M * M * pow((double)n, 6.0) >= 5e8; }
+
 // T-matrix ladder of g and Sigma^T: the damped fixed-point iteration
 // t <- (1 - a) t + a (V^ K V^ - V^ (K * t)) from t (the source V^ K V^ when
 // !t_valid) until max|t_new - t| < tol, with K * t the periodic convolution of
@@ -271,12 +279,22 @@ int tm_solve(fedvr_ctx *ctx, int n, int M, const double *V, const double *G, dou
              unsigned long long *res_d, double mixing, double tol, int max_iter, int *iters) {
   cudaStream_t s = ctx->stream;
   const size_t pstack = (size_t)M * n * n * n * n;
+  // the ladder's convolution K * t by residues (pair space as matrices of n^2)
+  // where its workspace can be had: K's residues once, Y holding K meanwhile
+  CrtConv plan;
+  const bool crt = tm_crt(n, M) && crt_conv_plan(n * n, M, 2, false, ctx->num_sms, &plan) &&
+                   ensure_optional(ctx, ctx->w_crt, plan.bytes);
+  if (crt) {
+    FEDVR_CK(ctx, tm_pairs(n, M, G, Y, s));
+    FEDVR_CK(ctx, crt_conv_source(plan, ctx->w_crt.ptr, Y, nullptr, coef, s));
+  }
   FEDVR_CK(ctx, tm_source(n, M, V, G, src, s));
   if (!t_valid) FEDVR_CK(ctx, launch_copy(pstack, src, t, s));
   double r = 0.0;
   int it = 0;
   for (it = 1; it <= max_iter; ++it) {
-    FEDVR_CK(ctx, tm_ladder(n, M, coef, G, t, Y, s));
+    if (crt) FEDVR_CK(ctx, crt_conv_apply(plan, ctx->w_crt.ptr, t, coef, Y, ctx->num_sms, s, true));
+    FEDVR_CK(ctx, tm_ladder(n, M, coef, G, t, Y, s, crt ? P<int>(ctx->w_crt) : nullptr));
     FEDVR_CK(ctx, cudaMemsetAsync(res_d, 0, sizeof(unsigned long long), s));
     FEDVR_CK(ctx, tm_update(n, M, V, src, Y, t, mixing, res_d, s));
     unsigned long long bits = 0;

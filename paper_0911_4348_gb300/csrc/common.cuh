@@ -212,8 +212,11 @@ cudaError_t launch_gw_sigma(long count, double spin, const double *G, const doub
 // t <- (1 - m) t + m (S - V^ Y) with *res = max|t_new - t| (double bits), and
 // Sigma^T = sum_kl [spin t(ak; bl) - t(ak; lb)] g_{M-1-j}(l, k).
 cudaError_t tm_source(int n, int M, const double *V, const double *G, double *S, cudaStream_t s);
+// gate (device int, may be NULL): tm_ladder runs only if *gate != 0. tm_pairs:
+// K_j = g_j (x) g_j, M matrices of n^2 x n^2.
 cudaError_t tm_ladder(int n, int M, const ConvCoef *coef, const double *G, const double *T,
-                      double *Y, cudaStream_t s);
+                      double *Y, cudaStream_t s, const int *gate = nullptr);
+cudaError_t tm_pairs(int n, int M, const double *G, double *K, cudaStream_t s);
 cudaError_t tm_update(int n, int M, const double *V, const double *S, const double *Y, double *T,
                       double mixing, unsigned long long *res, cudaStream_t s);
 cudaError_t tm_sigma(int n, int M, double spin, const double *G, const double *T, double *Sigma,

@@ -94,9 +94,10 @@ cudaError_t crt_conv_source(const CrtConv &c, void *ws, const double *A, const d
                             const ConvCoef *coef, cudaStream_t s);
 cudaError_t crt_conv_source4(const CrtConv &c, void *ws, const double *A, const double *dHF,
                              const ConvCoef4 *coef, cudaStream_t s);
-// I1 = table applied to (A, G).
+// I1 = table applied to (A, G); transposed: the matrices of G and I1 are stored
+// transposed.
 cudaError_t crt_conv_apply(const CrtConv &c, void *ws, const double *G, const ConvCoef *coef,
-                           double *I1, int num_sms, cudaStream_t s);
+                           double *I1, int num_sms, cudaStream_t s, bool transposed = false);
 cudaError_t crt_conv_apply4(const CrtConv &c, void *ws, const double *G, const ConvCoef4 *coef,
                             double *I1, int num_sms, cudaStream_t s);
 

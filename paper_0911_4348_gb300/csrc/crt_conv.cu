@@ -651,14 +651,15 @@ __global__ void __launch_bounds__(kThreads, 1) crt_conv_kernel(const __grid_cons
   if (warp == 0) tc::tmem_dealloc(tmem, 512);
 }
 
-// I1[row][col] from the residue planes R[S][nm][rows][ncR]; row = (i, a).
+// I1[row][col] from the residue planes R[S][nm][rows][ncR]; row = (i, a); tr: every
+// matrix is written transposed.
 template <int W>
 __global__ void __launch_bounds__(256) crt_rebuild_kernel(const __grid_constant__ CrtWords<W> t, int n,
                                                           long rows, int ncR, int S,
                                                           const int8_t *__restrict__ R,
                                                           const int *__restrict__ E,
                                                           const int *__restrict__ flag, int qb,
-                                                          double *__restrict__ out) {
+                                                          bool tr, double *__restrict__ out) {
   if (*flag) return;
   const long plane = rows * ncR;
   const long total = rows * n;
@@ -680,7 +681,8 @@ __global__ void __launch_bounds__(256) crt_rebuild_kernel(const __grid_constant_
     const int q = (int)rintf(f);
 #pragma unroll
     for (int i = 0; i < W; ++i) acc[i] -= (long long)q * (long long)t.P[i];
-    out[x] = crt_value<W>(acc, E[row / n] - kCrtQC - 2 * qb);
+    const long o = tr ? (row / n) * n * n + (long)col * n + row % n : x;
+    out[o] = crt_value<W>(acc, E[row / n] - kCrtQC - 2 * qb);
   }
 }
 
@@ -705,16 +707,20 @@ cudaError_t source_t(const CrtConv &c, void *wsv, const double *A, const double 
 
 template <typename Coef, int NP>
 cudaError_t apply_t(const CrtConv &c, void *wsv, const double *G, const Coef *coef, double *I1,
-                    int num_sms, cudaStream_t s) {
+                    int num_sms, cudaStream_t s, bool tr) {
   uint8_t *ws = reinterpret_cast<uint8_t *>(wsv);
   int *flag = reinterpret_cast<int *>(ws);
   int *es = reinterpret_cast<int *>(ws + c.o_exps), *eg = reinterpret_cast<int *>(ws + c.o_expg);
   int *E = reinterpret_cast<int *>(ws + c.o_E);
   const int n = c.k.n, M = c.k.M;
   crt_exp_stack_kernel<<<M, 256, 0, s>>>((long)n * n, G, eg, flag);
-  crt_g_kernel<<<dim3(M + 3, (n + 31) / 32, (c.k.nc + 63) / 64), 256, 0, s>>>(
-      crt_mods(c.nm, true), c.k, c.q, G, eg, reinterpret_cast<uint32_t *>(ws + c.o_B),
-      nullptr, 0, 0);
+  const dim3 gg(M + 3, (n + 31) / 32, (c.k.nc + 63) / 64);
+  if (tr)
+    crt_g_kernel<true><<<gg, 256, 0, s>>>(crt_mods(c.nm, true), c.k, c.q, G, eg,
+                                          reinterpret_cast<uint32_t *>(ws + c.o_B), nullptr, 0, 0);
+  else
+    crt_g_kernel<false><<<gg, 256, 0, s>>>(crt_mods(c.nm, true), c.k, c.q, G, eg,
+                                           reinterpret_cast<uint32_t *>(ws + c.o_B), nullptr, 0, 0);
   crt_coef_kernel<Coef, NP><<<M + 1, 256, 0, s>>>(crt_mods(c.nm, false), M, c.Mp,
                                                   (uint32_t)(n * c.k.nc), coef, es, eg, E,
                                                   reinterpret_cast<CrtEntry<NP> *>(ws + c.o_C));
@@ -755,7 +761,7 @@ cudaError_t apply_t(const CrtConv &c, void *wsv, const double *G, const Coef *co
   const long total = (long)M * n * n;
   crt_rebuild_kernel<7><<<(unsigned)std::min<long>((total + 255) / 256, 152 * 16), 256, 0, s>>>(
       crt_words<7>(c.nm), n, (long)M * n, c.ncR, c.S, reinterpret_cast<const int8_t *>(ws + c.o_R), E,
-      flag, c.q, I1);
+      flag, c.q, tr, I1);
   return cudaGetLastError();
 }
 
@@ -826,12 +832,12 @@ cudaError_t crt_conv_source4(const CrtConv &c, void *ws, const double *A, const 
   return source_t<ConvCoef4>(c, ws, A, dHF, coef, s);
 }
 cudaError_t crt_conv_apply(const CrtConv &c, void *ws, const double *G, const ConvCoef *coef,
-                           double *I1, int num_sms, cudaStream_t s) {
-  return apply_t<ConvCoef, 2>(c, ws, G, coef, I1, num_sms, s);
+                           double *I1, int num_sms, cudaStream_t s, bool transposed) {
+  return apply_t<ConvCoef, 2>(c, ws, G, coef, I1, num_sms, s, transposed);
 }
 cudaError_t crt_conv_apply4(const CrtConv &c, void *ws, const double *G, const ConvCoef4 *coef,
                             double *I1, int num_sms, cudaStream_t s) {
-  return apply_t<ConvCoef4, 4>(c, ws, G, coef, I1, num_sms, s);
+  return apply_t<ConvCoef4, 4>(c, ws, G, coef, I1, num_sms, s, false);
 }
 
 }  // namespace fedvr

@@ -160,7 +160,9 @@ __device__ __forceinline__ uint32_t pack16(float r0, float r1) {
 // out[m][b][x(j, c)] = g_j[c][b] (times mods.mul). With nat, also as plain
 // bfloat16 rows nat[m][j][b][c] ([nr] rows of ph values). A 64 (c) x 32 (b) tile of
 // one mesh point per CTA, transposed through shared memory. CTAs j >= M
-// write the zeros that pad the last chunk of each rest.
+// write the zeros that pad the last chunk of each rest. TR: the matrices are given
+// transposed (G[j][b][c]).
+template <bool TR>
 static __global__ void __launch_bounds__(256) crt_g_kernel(CrtMods mods, CrtK k, int qb,
                                                     const double *__restrict__ G,
                                                     const int *__restrict__ expo,
@@ -171,10 +173,10 @@ static __global__ void __launch_bounds__(256) crt_g_kernel(CrtMods mods, CrtK k,
   const int n = k.n, e = j < k.M ? expo[j] : kCrtZero;
   const double *g = G + (long)j * n * n;
   for (int q = threadIdx.x; q < 64 * 32; q += 256) {
-    const int c = q >> 5, b = q & 31;
+    const int c = TR ? q & 63 : q >> 5, b = TR ? q >> 6 : q & 31;
     long long x = 0;
     if (e != kCrtZero && c0 + c < n && b0 + b < n)
-      x = quantise(g[(long)(c0 + c) * n + b0 + b], qb - e);
+      x = quantise(TR ? g[(long)(b0 + b) * n + c0 + c] : g[(long)(c0 + c) * n + b0 + b], qb - e);
     sh[c][b] = x;
   }
   __syncthreads();

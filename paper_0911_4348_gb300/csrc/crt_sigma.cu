@@ -584,7 +584,7 @@ cudaError_t crt_sigma_apply(const CrtSigma &c, void *wsv, double spin, const dou
                                               reinterpret_cast<uint2 *>(ws + c.o_V));
     crt_rows_kernel<true><<<gx, 256, 0, s>>>(crt_mods(c.nm, true, m0, cnt), c.k, c.nr, c.ph, c.q, mat, V,
                                              eV, reinterpret_cast<uint2 *>(ws + c.o_Vn));
-    crt_g_kernel<<<dim3(M + 3, (n + 31) / 32, (c.k.nc + 63) / 64), 256, 0, s>>>(
+    crt_g_kernel<false><<<dim3(M + 3, (n + 31) / 32, (c.k.nc + 63) / 64), 256, 0, s>>>(
         mods, c.k, c.q, G, eg, reinterpret_cast<uint32_t *>(ws + c.o_B),
         reinterpret_cast<uint32_t *>(ws + c.o_gt), c.nr, c.ph);
     e = cudaGetLastError();

@@ -50,10 +50,12 @@ __global__ void tm_source_kernel(int n, long count, const double *__restrict__ V
 // application at 0.95 of the pipe.
 __global__ void tm_ladder_kernel(int n, int M, const ConvCoef *__restrict__ coef,
                                  const double *__restrict__ G, const double *__restrict__ T,
-                                 double *__restrict__ Y) {
+                                 double *__restrict__ Y, const int *__restrict__ gate) {
   __shared__ double X[1024], gr[1024], tmp[1024];
+  if (gate && *gate == 0) return;
   const int n2 = n * n;
-  const int i = (int)(blockIdx.x / n2), bl = (int)(blockIdx.x % n2);
+  for (long blk = blockIdx.x; blk < (long)M * n2; blk += gridDim.x) {
+  const int i = (int)(blk / n2), bl = (int)(blk % n2);
   const int tid = threadIdx.x, a = tid / n, k = tid % n;
   double acc = 0.0, lo = 0.0, hi = 0.0;  // sums of rows kc and kc + 1
   bool ulo = false, uhi = false;         // whether they hold anything (the same for the block)
@@ -101,6 +103,21 @@ __global__ void tm_ladder_kernel(int n, int M, const ConvCoef *__restrict__ coef
   if (uhi) sandwich(kc + 1, hi);
   if (ulo) sandwich(kc, lo);
   Y[((long)i * n2 + bl) * n2 + tid] = acc;
+  }
+}
+
+// K_j = g_j (x) g_j as M matrices of n^2 rows (a, k) and columns (a', k'), for the
+// ladder's convolution by residues (the first convolution's kernel at n^2).
+__global__ void tm_pair_kernel(int n, long count, const double *__restrict__ G,
+                               double *__restrict__ K) {
+  const long n2 = (long)n * n, n4 = n2 * n2;
+  for (long x = (long)blockIdx.x * blockDim.x + threadIdx.x; x < count;
+       x += (long)gridDim.x * blockDim.x) {
+    const long j = x / n4;
+    const int r = (int)(x % n4), ak = r / (int)n2, cq = r % (int)n2;
+    const double *g = G + j * n2;
+    K[x] = g[(ak / n) * n + cq / n] * g[(ak % n) * n + cq % n];
+  }
 }
 
 // t_new = S - V_ak Y; *res = max |t_new - t| (bit pattern of a non-negative
@@ -161,9 +178,17 @@ cudaError_t tm_source(int n, int M, const double *V, const double *G, double *S,
 }
 
 cudaError_t tm_ladder(int n, int M, const ConvCoef *coef, const double *G, const double *T,
-                      double *Y, cudaStream_t s) {
+                      double *Y, cudaStream_t s, const int *gate) {
   if (n < 1 || n > 32) return cudaErrorInvalidValue;
-  tm_ladder_kernel<<<(unsigned)((long)M * n * n), n * n, 0, s>>>(n, M, coef, G, T, Y);
+  const long blocks = (long)M * n * n;
+  tm_ladder_kernel<<<(unsigned)(gate && blocks > 608 ? 608 : blocks), n * n, 0, s>>>(n, M, coef, G, T, Y,
+                                                                                    gate);
+  return cudaGetLastError();
+}
+
+cudaError_t tm_pairs(int n, int M, const double *G, double *K, cudaStream_t s) {
+  const long count = (long)M * n * n * n * n;
+  tm_pair_kernel<<<blocks_for(count), 256, 0, s>>>(n, count, G, K);
   return cudaGetLastError();
 }
 

@@ -134,3 +134,31 @@ def test_second_born_not_finite(ctx):
     for j in (0, 2):
         want = O.sigma2_tau(G[j], G[M - 1 - j], V, 2.0)
         assert np.max(np.abs(got[j] - want)) < TOL * np.max(np.abs(want))
+
+
+def test_ladder_from_an_unsymmetric_start(ctx):
+    # the ladder's convolution as a residue product of n^2 x n^2 matrices (n = 7,
+    # M = 65), from a random t without the pair symmetries: rows, columns and the
+    # transposed storage have to match the oracle's
+    from paper_0911_4348_gb300 import FedvrError
+    rng = W.system_rng(93, 7)
+    n, u, p, beta = 7, 4, 8, 12.0
+    h = W.random_symmetric(rng, n)
+    V = 0.2 * np.abs(W.random_symmetric(rng, n))
+    e, C = np.linalg.eigh(h)
+    mesh = O.power_mesh(beta, u, p)
+    G = O.g0_mesh(e, C, 0.5 * (e[2] + e[3]), mesh["tau"], beta)
+    M = G.shape[0]
+    t0 = 0.01 * rng.uniform(-1, 1, (M, n, n, n, n))  # t0[j][a][k][b][l]
+    want = O.sigma_tmatrix(G, V, 2.0, mesh, O.bose_lag_table(mesh["tau"], beta), t0=t0, tol=1e-4)
+    t = _dev(t0.transpose(0, 3, 4, 1, 2))
+    S = torch.empty((M, n, n), dtype=torch.float64, device="cuda")
+    it = ctx.sigma_tmatrix(beta, u, p, _dev(V), _dev(G), S, t=t, t_valid=True, t_tol=1e-4)
+    torch.cuda.synchronize()
+    assert it == want["iters"]
+    assert maxrel(S.cpu().numpy(), want["Sigma"]) < TOL
+    assert maxrel(t.cpu().numpy().transpose(0, 3, 4, 1, 2), want["t"]) < TOL
+    G[3, 1, 1] = np.nan
+    with pytest.raises(FedvrError) as err:
+        ctx.sigma_tmatrix(beta, u, p, _dev(V), _dev(G), S)
+    assert err.value.code == -6
