@@ -386,10 +386,10 @@ int eig(fedvr_ctx *ctx, double *A, const double *Vinit, double *eps, double *C) 
     FEDVR_CK(ctx, launch_identity(n, V, ctx->stream));
   }
   cudaError_t err = cudaSuccess;
-  int sweeps = jacobi_eig(n, A, P<double>(ctx->b_A2), V, P<double>(ctx->b_J),
-                          P<double>(ctx->b_scal), 1e-14, 60, ctx->stream, &err);
-  if (err != cudaSuccess) return cuda_fail(ctx, err, "jacobi_eig", __FILE__, __LINE__);
-  if (sweeps < 0) return fail(ctx, FEDVR_ERR_NOCONV, "Jacobi did not converge in 60 sweeps");
+  int sweeps = sym_eig(n, &A, &V, P<double>(ctx->b_eig), P<double>(ctx->b_scal), 1e-14, 60,
+                       ctx->stream, &err);
+  if (err != cudaSuccess) return cuda_fail(ctx, err, "sym_eig", __FILE__, __LINE__);
+  if (sweeps < 0) return fail(ctx, FEDVR_ERR_NOCONV, "the eigensolver did not converge in 60 sweeps");
   FEDVR_CK(ctx, launch_sort_eig(n, A, V, eps, C, ctx->stream));
   return FEDVR_OK;
 }
@@ -881,8 +881,8 @@ void fedvr_destroy(fedvr_ctx *ctx) {
   DevBuf *bufs[] = {&ctx->b_xi, &ctx->b_om, &ctx->b_edges, &ctx->b_nodes, &ctx->b_weights,
                     &ctx->b_elem, &ctx->b_local, &ctx->b_tt, &ctx->b_T, &ctx->b_v, &ctx->b_V,
                     &ctx->b_h, &ctx->b_eps, &ctx->b_C, &ctx->b_rho, &ctx->b_rho_new,
-                    &ctx->b_rho_mix, &ctx->b_F, &ctx->b_Sigma0, &ctx->b_f, &ctx->b_A, &ctx->b_A2,
-                    &ctx->b_J, &ctx->b_scal, &ctx->b_hf_tmp, &ctx->b_sigma_init, &ctx->w_tau,
+                    &ctx->b_rho_mix, &ctx->b_F, &ctx->b_Sigma0, &ctx->b_f, &ctx->b_A,
+                    &ctx->b_eig, &ctx->b_scal, &ctx->b_hf_tmp, &ctx->b_sigma_init, &ctx->w_tau,
                     &ctx->w_w, &ctx->w_wm, &ctx->w_wp, &ctx->w_coef, &ctx->w_K, &ctx->w_phi,
                     &ctx->w_G0, &ctx->w_G, &ctx->w_S, &ctx->w_I1, &ctx->w_I2, &ctx->w_t1,
                     &ctx->w_t2, &ctx->w_t3, &ctx->w_dHF, &ctx->w_part, &ctx->w_red, &ctx->w_tc,
@@ -1045,8 +1045,7 @@ int solve_hf(fedvr_ctx *ctx, double beta, double tol, int max_iter, double *E_hf
   ENSURE(ctx, b_Sigma0, dsz(nn));
   ENSURE(ctx, b_f, dsz(n));
   ENSURE(ctx, b_A, dsz(nn));
-  ENSURE(ctx, b_A2, dsz(nn));
-  ENSURE(ctx, b_J, dsz(4 * (n / 2 + 2)));
+  ENSURE(ctx, b_eig, dsz(4 * nn));
   ENSURE(ctx, b_hf_tmp, dsz(nn > 512 ? nn : 512));
   double *eps = P<double>(ctx->b_eps), *C = P<double>(ctx->b_C), *rho = P<double>(ctx->b_rho);
   double *rho_new = P<double>(ctx->b_rho_new), *rho_mix = P<double>(ctx->b_rho_mix);
@@ -1063,12 +1062,11 @@ int solve_hf(fedvr_ctx *ctx, double beta, double tol, int max_iter, double *E_hf
   bool conv = false;
   for (it = 1; it <= max_iter; ++it) {
     FEDVR_CK(ctx, launch_hf_selfenergy(n, spin, rho, V, h, nullptr, F, s));
-    // A = C^T F C in the previous eigenbasis, Jacobi from there (warm start)
+    // A = C^T F C in the previous eigenbasis, diagonalised from there (warm start)
     double *t = rho_mix;
     FEDVR_CK(ctx, dgemm(false, false, n, n, n, 1.0, F, n, 0, C, n, 0, nullptr, 0, 0.0, t, n, 0, 1, s));
     FEDVR_CK(ctx, dgemm(true, false, n, n, n, 1.0, C, n, 0, t, n, 0, nullptr, 0, 0.0, A, n, 0, 1, s));
-    FEDVR_CK(ctx, launch_copy(nn, C, rho_new, s));  // starting basis (rho_new is free here)
-    if (int r = eig(ctx, A, rho_new, eps, C)) return r;
+    if (int r = eig(ctx, A, C, eps, C)) return r;
     FEDVR_CK(ctx, launch_mu_fermi(n, nocc, beta, eps, mu_dev, f, s));
     FEDVR_CK(ctx, dgemm(false, true, n, n, n, 1.0, C, n, 0, C, n, 0, f, 0, 0.0, rho_new, n, 0, 1, s));
     unsigned long long *bits = reinterpret_cast<unsigned long long *>(scal + 5);
@@ -1089,7 +1087,7 @@ int solve_hf(fedvr_ctx *ctx, double beta, double tol, int max_iter, double *E_hf
   if (!conv) return fail(ctx, FEDVR_ERR_NOCONV, "HF not converged after %d iterations", max_iter);
   // Sigma0 = F - h; E_hf on rho0 = C f C^T
   FEDVR_CK(ctx, launch_axpby(nn, 1.0, F, -1.0, h, P<double>(ctx->b_Sigma0), s));
-  FEDVR_CK(ctx, launch_energy_hf(n, spin, h, V, rho_new, scal + 6, s));
+  FEDVR_CK(ctx, launch_energy_hf(n, spin, h, V, rho_new, P<double>(ctx->b_eig), scal + 6, s));
   double out[3];
   FEDVR_CK(ctx, cudaMemcpyAsync(out, scal + 4, 3 * sizeof(double), cudaMemcpyDeviceToHost, s));
   if (int r = sync(ctx)) return r;

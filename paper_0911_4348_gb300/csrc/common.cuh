@@ -89,8 +89,8 @@ struct fedvr_ctx {
   // named device buffers
   fedvr::DevBuf b_xi, b_om, b_edges, b_nodes, b_weights, b_elem, b_local, b_tt;
   fedvr::DevBuf b_T, b_v, b_V, b_h;
-  fedvr::DevBuf b_eps, b_C, b_rho, b_rho_new, b_rho_mix, b_F, b_Sigma0, b_f, b_A, b_A2,
-      b_J, b_scal, b_hf_tmp;
+  fedvr::DevBuf b_eps, b_C, b_rho, b_rho_new, b_rho_mix, b_F, b_Sigma0, b_f, b_A,
+      b_eig, b_scal, b_hf_tmp;
   fedvr::DevBuf b_sigma_init;
   // solve_2b / stage workspace
   fedvr::DevBuf w_tau, w_w, w_wm, w_wp, w_coef, w_K, w_phi, w_G0, w_G, w_S, w_I1, w_I2,
@@ -171,12 +171,13 @@ cudaError_t launch_quad4_tables(int M, double beta, const double *tau, ConvCoef4
 cudaError_t dgemm(bool ta, bool tb, int M, int N, int K, double alpha, const double *A,
                   long lda, long sA, const double *B, long ldb, long sB, const double *sk,
                   long sS, double beta, double *C, long ldc, long sC, int batch, cudaStream_t s);
-// Symmetric eigen-decomposition by cyclic-by-rounds Jacobi on the device.
-// A (n x n, overwritten), V (n x n, in: starting basis or identity, out:
-// eigenvectors as columns, unsorted), scratch A2 (n x n), J (rotation scratch,
-// >= 2*(n+1) doubles), scal (>= 4 doubles). Returns sweeps used or <0.
-int jacobi_eig(int n, double *A, double *A2, double *V, double *J, double *scal, double tol,
-               int max_sweeps, cudaStream_t s, cudaError_t *err);
+// Symmetric eigen-decomposition on the device: cyclic-by-rounds Jacobi sweeps,
+// Newton steps once the rotations left are small. *A (n x n, overwritten), *V
+// (in: starting basis or identity, out: eigenvectors as columns, unsorted), work
+// (4 n^2 doubles), scal (>= 4 doubles). On return *A and *V name the buffers,
+// theirs or work's, that hold the result. Returns the passes used or <0.
+int sym_eig(int n, double **A, double **V, double *work, double *scal, double tol, int max_sweeps,
+            cudaStream_t s, cudaError_t *err);
 // Sort eigenpairs ascending: eps_out[r] = diag(A)[idx], C_out[:, r] = V[:, idx].
 cudaError_t launch_sort_eig(int n, const double *A, const double *V, double *eps_out,
                             double *C_out, cudaStream_t s);
@@ -293,7 +294,7 @@ cudaError_t launch_update(int n, int M, double mixing, const double *G0, const d
 cudaError_t launch_axpby(size_t count, double a, const double *x, double b, const double *y,
                          double *out, cudaStream_t s);
 cudaError_t launch_energy_hf(int n, double spin, const double *h, const double *V,
-                             const double *rho, double *out, cudaStream_t s);
+                             const double *rho, double *rows, double *out, cudaStream_t s);
 cudaError_t launch_energy(int n, int M, double spin, const double *h, const double *V,
                           const double *G, const double *A, const double *w, double *part,
                           double *out, cudaStream_t s);

@@ -165,35 +165,16 @@ __global__ void energy_rows_kernel(int n, int M, double spin, const double *__re
 
 // out[0] = E0 = sigma Tr[h rho] + (sigma/2) Tr[Sigma^HF[rho] rho]
 //              - (sigma/2) sum_j w_j part[j];  out[1] = N = sigma Tr rho;  rho = G[M-1].
-// With rows (from energy_rows_kernel) the one-body sums are taken over its row
-// partials in a fixed order; without, directly (single-matrix use by the HF loop).
-__global__ void energy_final_kernel(int n, int M, double spin, const double *__restrict__ h,
-                                    const double *__restrict__ V, const double *__restrict__ G,
-                                    const double *__restrict__ w, const double *__restrict__ part,
+// The one-body sums are taken over energy_rows_kernel's row partials in a fixed
+// order; part may be NULL (a single matrix, no correlation term).
+__global__ void energy_final_kernel(int n, int M, double spin, const double *__restrict__ w,
+                                    const double *__restrict__ part,
                                     const double *__restrict__ rows, double *out) {
-  long nn = (long)n * n;
-  const double *rho = G + (long)(M - 1) * nn;
   double e1 = 0.0, e2 = 0.0, tr = 0.0, ec = 0.0;
-  if (rows) {
-    for (int a = threadIdx.x; a < n; a += blockDim.x) {
-      e1 += rows[a];
-      e2 += rows[n + a];
-      tr += rows[2 * n + a];
-    }
-  } else {
-    for (long e = threadIdx.x; e < nn; e += blockDim.x) {
-      int a = (int)(e / n), b = (int)(e % n);
-      double r = rho[e];
-      e1 += h[e] * r;
-      double shf = -V[e] * r;
-      if (a == b) {
-        double hart = 0.0;
-        for (int k = 0; k < n; ++k) hart += V[(long)a * n + k] * rho[(long)k * n + k];
-        shf += spin * hart;
-        tr += r;
-      }
-      e2 += shf * r;
-    }
+  for (int a = threadIdx.x; a < n; a += blockDim.x) {
+    e1 += rows[a];
+    e2 += rows[n + a];
+    tr += rows[2 * n + a];
   }
   if (part)
     for (int j = threadIdx.x; j < M; j += blockDim.x) {
@@ -243,9 +224,10 @@ cudaError_t launch_axpby(size_t count, double a, const double *x, double b, cons
 }
 
 cudaError_t launch_energy_hf(int n, double spin, const double *h, const double *V,
-                             const double *rho, double *out, cudaStream_t s) {
-  // a one-point "stack" whose only member is rho, with no correlation term
-  energy_final_kernel<<<1, 256, 0, s>>>(n, 1, spin, h, V, rho, nullptr, nullptr, nullptr, out);
+                             const double *rho, double *rows, double *out, cudaStream_t s) {
+  // rows: 3 n doubles of scratch; a one-point "stack" whose only member is rho, with no correlation term
+  energy_rows_kernel<<<n, 256, 0, s>>>(n, 1, spin, h, V, rho, rows);
+  energy_final_kernel<<<1, 256, 0, s>>>(n, 1, spin, nullptr, nullptr, rows, out);
   return cudaGetLastError();
 }
 
@@ -265,7 +247,7 @@ cudaError_t launch_energy(int n, int M, double spin, const double *h, const doub
                           double *out, cudaStream_t s) {
   energy_part_kernel<<<M * kE, 256, 0, s>>>(n, M, G, A, part);
   energy_rows_kernel<<<n, 256, 0, s>>>(n, M, spin, h, V, G, part + (long)kE * M);
-  energy_final_kernel<<<1, 256, 0, s>>>(n, M, spin, h, V, G, w, part, part + (long)kE * M, out);
+  energy_final_kernel<<<1, 256, 0, s>>>(n, M, spin, w, part, part + (long)kE * M, out);
   return cudaGetLastError();
 }
 
