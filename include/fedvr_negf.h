@@ -152,7 +152,7 @@ int fedvr_get_operators(const fedvr_ctx *ctx, double *T, double *v, double *V, d
 
 /* Self-consistent HF at inverse temperature beta: F = h + Sigma^HF[rho],
  * Sigma^HF = sigma diag(V diag rho) - V o rho (sigma = 2), diagonalisation on
- * the GPU (Jacobi sweeps, then Newton steps), chemical potential from the Fermi normalisation
+ * the GPU (Jacobi), chemical potential from the Fermi normalisation
  * sum_a f(eps_a - mu) = n_elec/2 solved in its balanced holes = particles form,
  * rho' = C diag f C^T, linear mixing 0.5, stop when max|rho' - rho| < tol.
  * Outputs (host, may be NULL): E_hf = 2 Tr[h rho] + Tr[Sigma^HF rho] (no E_nn)

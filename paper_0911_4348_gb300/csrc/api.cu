@@ -386,10 +386,14 @@ int eig(fedvr_ctx *ctx, double *A, const double *Vinit, double *eps, double *C) 
     FEDVR_CK(ctx, launch_identity(n, V, ctx->stream));
   }
   cudaError_t err = cudaSuccess;
-  int sweeps = sym_eig(n, &A, &V, P<double>(ctx->b_eig), P<double>(ctx->b_scal), 1e-14, 60,
+  int sweeps = sym_eig(n, &A, P<double>(ctx->b_eig), V, P<double>(ctx->b_scal), 1e-14, 60,
                        ctx->stream, &err);
   if (err != cudaSuccess) return cuda_fail(ctx, err, "sym_eig", __FILE__, __LINE__);
-  if (sweeps < 0) return fail(ctx, FEDVR_ERR_NOCONV, "the eigensolver did not converge in 60 sweeps");
+  if (sweeps == -3) {
+    ctx->failed = true;
+    return fail(ctx, FEDVR_ERR_TIMEOUT, "a Jacobi sweep's bounded wait gave up");
+  }
+  if (sweeps < 0) return fail(ctx, FEDVR_ERR_NOCONV, "Jacobi did not converge in 60 sweeps");
   FEDVR_CK(ctx, launch_sort_eig(n, A, V, eps, C, ctx->stream));
   return FEDVR_OK;
 }
@@ -1045,7 +1049,7 @@ int solve_hf(fedvr_ctx *ctx, double beta, double tol, int max_iter, double *E_hf
   ENSURE(ctx, b_Sigma0, dsz(nn));
   ENSURE(ctx, b_f, dsz(n));
   ENSURE(ctx, b_A, dsz(nn));
-  ENSURE(ctx, b_eig, dsz(4 * nn));
+  ENSURE(ctx, b_eig, dsz(nn + 3 * (size_t)n));
   ENSURE(ctx, b_hf_tmp, dsz(nn > 512 ? nn : 512));
   double *eps = P<double>(ctx->b_eps), *C = P<double>(ctx->b_C), *rho = P<double>(ctx->b_rho);
   double *rho_new = P<double>(ctx->b_rho_new), *rho_mix = P<double>(ctx->b_rho_mix);
@@ -1062,7 +1066,7 @@ int solve_hf(fedvr_ctx *ctx, double beta, double tol, int max_iter, double *E_hf
   bool conv = false;
   for (it = 1; it <= max_iter; ++it) {
     FEDVR_CK(ctx, launch_hf_selfenergy(n, spin, rho, V, h, nullptr, F, s));
-    // A = C^T F C in the previous eigenbasis, diagonalised from there (warm start)
+    // A = C^T F C in the previous eigenbasis, Jacobi from there (warm start)
     double *t = rho_mix;
     FEDVR_CK(ctx, dgemm(false, false, n, n, n, 1.0, F, n, 0, C, n, 0, nullptr, 0, 0.0, t, n, 0, 1, s));
     FEDVR_CK(ctx, dgemm(true, false, n, n, n, 1.0, C, n, 0, t, n, 0, nullptr, 0, 0.0, A, n, 0, 1, s));

@@ -171,12 +171,13 @@ cudaError_t launch_quad4_tables(int M, double beta, const double *tau, ConvCoef4
 cudaError_t dgemm(bool ta, bool tb, int M, int N, int K, double alpha, const double *A,
                   long lda, long sA, const double *B, long ldb, long sB, const double *sk,
                   long sS, double beta, double *C, long ldc, long sC, int batch, cudaStream_t s);
-// Symmetric eigen-decomposition on the device: cyclic-by-rounds Jacobi sweeps,
-// Newton steps once the rotations left are small. *A (n x n, overwritten), *V
-// (in: starting basis or identity, out: eigenvectors as columns, unsorted), work
-// (4 n^2 doubles), scal (>= 4 doubles). On return *A and *V name the buffers,
-// theirs or work's, that hold the result. Returns the passes used or <0.
-int sym_eig(int n, double **A, double **V, double *work, double *scal, double tol, int max_sweeps,
+// Symmetric eigen-decomposition by cyclic-by-rounds Jacobi on the device, one
+// launch per sweep. *A (n x n, overwritten; on return the one of *A and A2 that
+// holds the diagonal form), A2 (n x n scratch), V (n x n, in: starting basis or
+// identity, out: eigenvectors as columns, unsorted), scal (>= 4 doubles). Returns
+// the sweeps used, -1 on a CUDA error, -2 without convergence, -3 if a bounded
+// wait of the sweep gave up.
+int sym_eig(int n, double **A, double *A2, double *V, double *scal, double tol, int max_sweeps,
             cudaStream_t s, cudaError_t *err);
 // Sort eigenpairs ascending: eps_out[r] = diag(A)[idx], C_out[:, r] = V[:, idx].
 cudaError_t launch_sort_eig(int n, const double *A, const double *V, double *eps_out,

@@ -8,21 +8,31 @@ namespace fedvr {
 namespace {
 
 // out = add + sigma diag(V diag rho) - V o rho - sub   (add/sub may be NULL)
-// One block per row a; the Hartree sum of the row's diagonal entry is taken by
-// the whole block (one thread alone was a chain of n additions).
+// One block per row a. The Hartree sum of its diagonal entry is one thread's chain
+// of additions in k order, from shared memory (from global memory, behind the
+// strided diagonal of rho, the chain took 27 us at n = 199, now 12).
+constexpr int kHartChunk = 1024;
 __global__ void __launch_bounds__(128)
     hf_selfenergy_kernel(int n, double spin, const double *__restrict__ rho,
                          const double *__restrict__ V, const double *__restrict__ addm,
                          const double *__restrict__ subm, double *__restrict__ out) {
-  __shared__ double part[4];
+  __shared__ double va[kHartChunk], rd[kHartChunk];
   const int a = blockIdx.x;
   const long row = (long)a * n;
   double hart = 0.0;
-  for (int k = threadIdx.x; k < n; k += 128) hart += V[row + k] * rho[(long)k * n + k];
-  for (int o = 16; o > 0; o >>= 1) hart += __shfl_xor_sync(0xffffffffu, hart, o);
-  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = hart;
-  __syncthreads();
-  hart = (part[0] + part[1]) + (part[2] + part[3]);
+  for (int k0 = 0; k0 < n; k0 += kHartChunk) {
+    const int kn = min(kHartChunk, n - k0);
+    for (int k = threadIdx.x; k < kn; k += 128) {
+      va[k] = V[row + k0 + k];
+      rd[k] = rho[(long)(k0 + k) * (n + 1)];
+    }
+    __syncthreads();
+    if (threadIdx.x == a % 128) {
+#pragma unroll 8
+      for (int k = 0; k < kn; ++k) hart += va[k] * rd[k];
+    }
+    __syncthreads();
+  }
   for (int b = threadIdx.x; b < n; b += 128) {
     double v = -V[row + b] * rho[row + b];
     if (a == b) v += spin * hart;
@@ -32,17 +42,52 @@ __global__ void __launch_bounds__(128)
   }
 }
 
+__device__ __forceinline__ double softplus(double z) { return fmax(z, 0.0) + log1p(exp(-fabs(z))); }
+
+// log-sum-exp of -softplus(beta * x_a) over a in [lo, hi), x_a = sgn*(mu - eps_a),
+// by the 256 threads t of one of the block's two groups (named barrier 1 + grp);
+// z0 the smallest beta x_a. Levels whose term is below exp(-79) of the first are
+// passed over: they change no bit of the sum. sh: 16 doubles of the group.
+__device__ double lse_exact(const double *eps, int lo, int hi, double mu, double beta, double sgn,
+                            double z0, int t, int grp, double *sh) {
+  if (lo >= hi) return -INFINITY;
+  const double most = fmax(z0, 0.0) + 80.0;
+  const auto meet = [&] { asm volatile("bar.sync %0, 256;" ::"r"(1 + grp) : "memory"); };
+  const auto value = [&](int a) {  // -softplus, or -inf for a level passed over
+    const double z = a < hi ? beta * (sgn * (mu - eps[a])) : INFINITY;
+    return z > most ? -INFINITY : -softplus(z);
+  };
+  const double v0 = value(lo + t);
+  double m = v0;
+  for (int a = lo + t + 256; a < hi; a += 256) m = fmax(m, value(a));
+  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((t & 31) == 0) sh[t >> 5] = m;
+  meet();
+  m = sh[0];
+  for (int w = 1; w < 8; ++w) m = fmax(m, sh[w]);
+  double s = 0.0;
+  for (int a = lo + t; a < hi; a += 256) {
+    const double v = a == lo + t ? v0 : value(a);
+    if (v > -INFINITY || v != v) s += exp(v - m);
+  }
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if ((t & 31) == 0) sh[8 + (t >> 5)] = s;
+  meet();
+  s = sh[8];
+  for (int w = 1; w < 8; ++w) s += sh[8 + w];
+  return m + log(s);
+}
+
 // log of sum_a f(z_a), f(z) = 1 / (exp(z) + 1), over the levels first, first +
 // step, ... (count of them), z_a = beta sgn (mu - eps_a) ascending along them;
-// *slope = the mean of 1 - f with the weights f. One warp. The sum is relative to
-// its first and largest term; the rest stops where it is below exp(-50) of that.
-__device__ double lse_group(const double *eps, int first, int step, int count, double mu,
+// *slope = the mean of 1 - f with the weights f. One warp.
+__device__ double lse_slope(const double *eps, int first, int step, int count, double mu,
                             double beta, double sgn, double *slope) {
   const int lane = threadIdx.x & 31;
   *slope = 0.0;
   if (count <= 0) return -INFINITY;
   const double z0 = beta * (sgn * (mu - eps[first]));
-  const double sp0 = fmax(z0, 0.0) + log1p(exp(-fabs(z0)));
+  const double sp0 = softplus(z0);
   double s = 0.0, ds = 0.0;
   for (int i0 = 0; i0 < count; i0 += 32) {
     const int i = i0 + lane;
@@ -64,41 +109,66 @@ __device__ double lse_group(const double *eps, int first, int step, int count, d
   return log(s) - sp0;
 }
 
-// mu from the Fermi normalisation in balanced form: D(mu) = log sum_{a<nocc}
-// f(mu - eps_a) - log sum_{a>=nocc} f(eps_a - mu) = 0, a decreasing function,
-// nearly a line of slope -2 beta in the gap. Newton steps inside a bracket that
-// starts as [eps_0 - 1, eps_{n-1} + 1], from the middle of the gap; its midpoint where a step would leave it
-// or the last one did not halve |D|. It ends where the step is below the
-// rounding of the levels next to mu, or the bracket has no point inside.
-// Bound by the latency of a chain of exponentials on one SM: warp 0 sums the
-// holes, warp 1 the particles, only levels that count. Bisection to the last bit
-// with all levels in every step: 1260 us at n = 199.
-// Then f_a = 1/(exp(beta (eps_a - mu)) + 1) in overflow-free form. eps ascending.
-__global__ void __launch_bounds__(64)
+// mu from the Fermi normalisation in balanced form: sum_{a<nocc} f(mu - eps_a)
+// = sum_{a>=nocc} f(eps_a - mu), compared as log-sum-exps; bisection on
+// [eps_0 - 1, eps_{n-1} + 1] until the midpoint stops moving. Then
+// f_a = 1/(exp(beta (eps_a - mu)) + 1) in overflow-free form. eps ascending.
+// Bound by the latency of a chain of exponentials on one SM. A Newton iteration
+// from the middle of the gap (warp 0 the holes, warp 1 the particles, only levels
+// that count) finds the zero first; a midpoint further from it than the
+// comparison's rounding reaches then needs no evaluation, which leaves about 7 of
+// 55: 1260 us before, 213 now (n = 199), and the same mu to the last bit.
+__global__ void __launch_bounds__(512)
     mu_fermi_kernel(int n, int nocc, double beta, const double *eps, double *mu_out, double *f) {
-  __shared__ double val[2], der[2];
+  __shared__ double sh[2][16], val[2], der[2];
   double lo = eps[0] - 1.0, hi = eps[n - 1] + 1.0;
-  double mu = 0.5 * (eps[nocc > 0 ? nocc - 1 : 0] + eps[nocc < n ? nocc : n - 1]), last = INFINITY;
-  const double scale = fmax(fabs(eps[nocc > 0 ? nocc - 1 : 0]), fabs(eps[nocc < n ? nocc : n - 1]));
-  for (int it = 0; it < 400 && lo < mu && mu < hi; ++it) {
-    double slope;
-    const double v = threadIdx.x < 32 ? lse_group(eps, nocc - 1, -1, nocc, mu, beta, 1.0, &slope)
-                                      : lse_group(eps, nocc, 1, n - nocc, mu, beta, -1.0, &slope);
-    __syncthreads();  // the last round's values have been read
-    if ((threadIdx.x & 31) == 0) {
-      val[threadIdx.x >> 5] = v;
-      der[threadIdx.x >> 5] = slope;
+  const double below = eps[nocc > 0 ? nocc - 1 : 0], above = eps[nocc < n ? nocc : n - 1];
+  double zero = 0.5 * (below + above), margin = INFINITY;
+  if (nocc > 0 && nocc < n) {
+    for (int it = 0; it < 40; ++it) {
+      if (threadIdx.x < 64) {
+        double slope;
+        const double v = threadIdx.x < 32
+                             ? lse_slope(eps, nocc - 1, -1, nocc, zero, beta, 1.0, &slope)
+                             : lse_slope(eps, nocc, 1, n - nocc, zero, beta, -1.0, &slope);
+        if ((threadIdx.x & 31) == 0) {
+          val[threadIdx.x >> 5] = v;
+          der[threadIdx.x >> 5] = slope;
+        }
+      }
+      __syncthreads();
+      const double h = val[0], p = val[1], d = der[0] + der[1];
+      __syncthreads();  // read before the next iteration's
+      const double step = (h - p) / (beta * d);
+      const double noise = 2e-14 * (1.0 + fabs(h) + fabs(p)) / (beta * d);
+      if (!(d > 1e-3) || !(fabs(step) < INFINITY)) break;
+      zero += step;
+      if (fabs(step) <= 0.25 * noise) {
+        margin = noise + 1e-15 * fabs(zero);
+        break;
+      }
     }
-    __syncthreads();
-    const double D = val[0] - val[1];
-    if (D > 0.0) lo = mu; else hi = mu;
-    const double step = D / (beta * (der[0] + der[1]));
-    if (fabs(step) <= 1.1e-16 * fmax(scale, fabs(mu))) break;
-    const double next = mu + step;
-    const bool newton = lo < next && next < hi && fabs(D) <= 0.5 * last;
-    last = newton ? fabs(D) : INFINITY;
-    mu = newton ? next : 0.5 * (lo + hi);
   }
+  for (int it = 0; it < 400; ++it) {
+    const double mid = 0.5 * (lo + hi);
+    if (!(lo < mid && mid < hi)) break;
+    bool up;
+    if (fabs(mid - zero) > margin) {
+      up = mid < zero;
+    } else {
+      const int grp = threadIdx.x / 256, t = threadIdx.x % 256;  // the holes, the particles
+      const double v =
+          grp == 0 ? lse_exact(eps, 0, nocc, mid, beta, 1.0, beta * (mid - below), t, 0, sh[0])
+                   : lse_exact(eps, nocc, n, mid, beta, -1.0, beta * (above - mid), t, 1, sh[1]);
+      if (t == 0) val[grp] = v;
+      __syncthreads();
+      const double holes = val[0], parts = val[1];
+      __syncthreads();  // read before the next midpoint's
+      up = holes - parts > 0.0;
+    }
+    if (up) lo = mid; else hi = mid;
+  }
+  double mu = 0.5 * (lo + hi);
   if (threadIdx.x == 0) *mu_out = mu;
   for (int a = threadIdx.x; a < n; a += blockDim.x) {
     double y = beta * (eps[a] - mu);
@@ -135,7 +205,7 @@ cudaError_t launch_hf_selfenergy(int n, double spin, const double *rho, const do
 
 cudaError_t launch_mu_fermi(int n, int nocc, double beta, const double *eps, double *mu_out,
                             double *f, cudaStream_t s) {
-  mu_fermi_kernel<<<1, 64, 0, s>>>(n, nocc, beta, eps, mu_out, f);
+  mu_fermi_kernel<<<1, 512, 0, s>>>(n, nocc, beta, eps, mu_out, f);
   return cudaGetLastError();
 }
 

@@ -5,12 +5,15 @@
 
 #include <math.h>
 
+#include <string.h>
+
+#include <algorithm>
 #include <utility>
 
 namespace fedvr {
 namespace {
 
-// C = alpha * op(A) diag(sk) op(B) + beta * C + diag * I, one BM x BN tile per
+// C = alpha * op(A) diag(sk) op(B) + beta * C, one BM x BN tile per
 // block of TX x TX threads, each owning rows ty + TX i and columns tx + TX j.
 // Bound by the FP64 pipe (two FMA per SM and cycle): what counts is how evenly
 // the tiles fall on the SMs, and that the next operand tile is in flight (in
@@ -21,7 +24,7 @@ __global__ void __launch_bounds__(TX *TX)
     dgemm_kernel(int M, int N, int K, double alpha, const double *__restrict__ A, long lda,
                  long sA, const double *__restrict__ B, long ldb, long sB,
                  const double *__restrict__ sk, long sS, double beta, double *__restrict__ C,
-                 long ldc, long sC, double diag) {
+                 long ldc, long sC) {
   constexpr int NT = TX * TX, RI = BM / TX, RJ = BN / TX;
   constexpr int EA = BM * BK / NT, EB = BN * BK / NT;
   const long bz = blockIdx.z;
@@ -97,9 +100,7 @@ __global__ void __launch_bounds__(TX *TX)
       int gn = n0 + tx + TX * j;
       if (gn >= N) continue;
       double *c = C + (long)gm * ldc + gn;
-      double v = (beta == 0.0) ? alpha * acc[i][j] : alpha * acc[i][j] + beta * *c;
-      if (gm == gn) v += diag;
-      *c = v;
+      *c = (beta == 0.0) ? alpha * acc[i][j] : alpha * acc[i][j] + beta * *c;
     }
   }
 }
@@ -116,7 +117,6 @@ struct GemmArgs {
   double beta;
   double *C;
   long ldc, sC;
-  double diag;
   int batch;
 };
 
@@ -125,7 +125,7 @@ void dgemm_run(bool ta, bool tb, const GemmArgs &g, cudaStream_t s) {
   const dim3 grid((g.N + BN - 1) / BN, (g.M + BM - 1) / BM, g.batch);
   auto run = [&](auto kernel) {
     kernel<<<grid, TX * TX, 0, s>>>(g.M, g.N, g.K, g.alpha, g.A, g.lda, g.sA, g.B, g.ldb, g.sB, g.sk,
-                                    g.sS, g.beta, g.C, g.ldc, g.sC, g.diag);
+                                    g.sS, g.beta, g.C, g.ldc, g.sC);
   };
   if (ta) tb ? run(dgemm_kernel<true, true, BM, BN, BK, TX>) : run(dgemm_kernel<true, false, BM, BN, BK, TX>);
   else tb ? run(dgemm_kernel<false, true, BM, BN, BK, TX>) : run(dgemm_kernel<false, false, BM, BN, BK, TX>);
@@ -157,124 +157,154 @@ cudaError_t dgemm_any(bool ta, bool tb, const GemmArgs &g, cudaStream_t s) {
 // Round-robin schedule on m = n rounded up to even: position 0 fixed, others
 // rotate; pair k joins positions k and m-1-k.
 __device__ __forceinline__ int rr_member(int pos, int r, int m) {
-  return pos == 0 ? 0 : 1 + (pos - 1 + r) % (m - 1);
+  if (pos == 0) return 0;
+  const int x = pos - 1 + r;  // < 2 (m - 1)
+  return 1 + (x < m - 1 ? x : x - (m - 1));
 }
 
-// One round: every block works out the rotations of its own 16 row pairs and 16
-// column pairs (or of its 16 column pairs, for a tile of V) and applies them to
-// its 16 x 16 tile of pair blocks. One launch per round instead of a launch for
-// the rotations and one that applies them: the round is a chain of latencies,
-// not of work. The entries of the tile are fetched before the rotations.
+// One sweep per launch: the rounds are a chain of latencies (fetch, a divide,
+// square root, divide, square root and divide for the rotation, the update, and
+// making it visible), not of work. Each block of the resident grid works out the
+// rotations of its 8 row pairs and 16 column pairs (or 16 column pairs, for a tile
+// of V), applies them to its 8 x 16 pair blocks of A (32 x 16 of V: the same 64
+// FP64 warp instructions, which the SM's slow FP64 pipe takes 1000 cycles for),
+// whose entries were fetched before the rotations, and meets the others at one
+// barrier per round. At n = 199 two launches per round took 7.1 us, this takes
+// 4.4.
 __device__ __forceinline__ void rr_pair(int k, int r, int m, int *p, int *q) {
   const int a = rr_member(k, r, m), b = rr_member(m - 1 - k, r, m);
   *p = min(a, b);
   *q = max(a, b);
 }
 
-__global__ void __launch_bounds__(256)
-    jacobi_round_kernel(int n, int m, int r, int tiles, const double *__restrict__ Ain,
-                        double *__restrict__ Aout, double *__restrict__ V) {
-  __shared__ double cs[32], sn[32];
-  const int npair = m / 2, tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  const int bx = blockIdx.x % tiles, by = blockIdx.x / tiles;
-  const bool isV = by >= tiles;  // the tiles of V follow those of A
-  const int k2 = bx * 16 + tx, k1 = by * 16 + ty;
-  const int row = (by - tiles) * 16 + ty;
-  int p2 = 0, q2 = n, p1 = 0, q1 = n;
-  const bool in = k2 < npair && (isV ? row < n : k1 < npair);
-  double xpp = 0.0, xpq = 0.0, xqp = 0.0, xqq = 0.0;
-  if (in) {
-    rr_pair(k2, r, m, &p2, &q2);
-    if (isV) {
-      xpp = V[(long)row * n + p2];
-      if (q2 < n) xpq = V[(long)row * n + q2];
-    } else {
-      rr_pair(k1, r, m, &p1, &q1);
-      xpp = Ain[(long)p1 * n + p2];
-      if (q2 < n) xpq = Ain[(long)p1 * n + q2];
-      if (q1 < n) xqp = Ain[(long)q1 * n + p2];
-      if (q1 < n && q2 < n) xqq = Ain[(long)q1 * n + q2];
-    }
-  }
-  if (threadIdx.x < 32) {  // rotations: lanes 0..15 the column pairs, 16..31 the row pairs
-    const int k = threadIdx.x < 16 ? bx * 16 + threadIdx.x : by * 16 + threadIdx.x - 16;
-    int p = 0, q = n;
-    if (k < npair) rr_pair(k, r, m, &p, &q);
-    double c = 1.0, s = 0.0;
-    if (q < n) {
-      double apq = Ain[(long)p * n + q];
-      double app = Ain[(long)p * n + p], aqq = Ain[(long)q * n + q];
-      double mag = fabs(apq);
-      if (mag > 0.0) {
-        double tau = (aqq - app) / (2.0 * apq);
-        double t;
-        if (fabs(tau) > 1e150) t = 0.5 / tau;
-        else t = (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
-        c = 1.0 / sqrt(1.0 + t * t);
-        s = t * c;
+// All blocks of the grid meet: thread 0 adds itself to the counter and waits for
+// `target` arrivals. False if the wait gave up (the caller then leaves: flag set).
+__device__ __forceinline__ bool sweep_barrier(unsigned *counter, unsigned target) {
+  __shared__ int ok;
+  __syncthreads();  // this block's stores are done
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(counter, 1u);
+    int good = 0;
+    for (long spin = 0; spin < (1L << 23); ++spin) {
+      unsigned seen;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(counter) : "memory");
+      if (seen >= target) {
+        good = 1;
+        break;
       }
     }
-    cs[threadIdx.x] = c;
-    sn[threadIdx.x] = s;
+    ok = good;
   }
   __syncthreads();
-  if (!in) return;
-  const double c2 = cs[tx], s2 = sn[tx];
-  if (isV) {
-    if (q2 >= n) return;
-    V[(long)row * n + p2] = c2 * xpp - s2 * xpq;
-    V[(long)row * n + q2] = s2 * xpp + c2 * xpq;
-    return;
-  }
-  const double c1 = cs[16 + ty], s1 = sn[16 + ty];
-  const bool hq1 = q1 < n, hq2 = q2 < n;
-  // rows: J1^T X
-  double ypp = c1 * xpp - s1 * xqp, ypq = c1 * xpq - s1 * xqq;
-  double yqp = s1 * xpp + c1 * xqp, yqq = s1 * xpq + c1 * xqq;
-  // cols: (J1^T X) J2
-  Aout[(long)p1 * n + p2] = c2 * ypp - s2 * ypq;
-  if (hq2) Aout[(long)p1 * n + q2] = s2 * ypp + c2 * ypq;
-  if (hq1) Aout[(long)q1 * n + p2] = c2 * yqp - s2 * yqq;
-  if (hq1 && hq2) Aout[(long)q1 * n + q2] = s2 * yqp + c2 * yqq;
+  return ok != 0;
 }
 
-// The generator of a simultaneous small rotation of all pairs: X_pq =
-// A_pq / (A_qq - A_pp) from the upper triangle, X antisymmetric exactly. One
-// block per row (the divisions want every SM); stats[0] = max |A_pq| without NaN, stats[1] = max row sum of |X|
-// as bits (an Inf or NaN stays the largest).
-__global__ void __launch_bounds__(64)
-    newton_generator_kernel(int n, const double *__restrict__ A, double *__restrict__ X,
-                            unsigned long long *stats) {
-  __shared__ double part;
-  const int row = blockIdx.x, lane = threadIdx.x & 31;
-  const double d = A[(long)row * n + row];
-  double sum = 0.0, off = 0.0;
-  for (int j = threadIdx.x; j < n; j += 64) {
-    double x = 0.0;
-    if (j != row) {
-      const double e = row < j ? A[(long)row * n + j] : A[(long)j * n + row];
-      if (e != 0.0) x = e / (A[(long)j * n + j] - d);
-      off = fmax(off, fabs(e));
-      sum += fabs(x);
+// a b - c d and a b + c d with the first product fused into the sum
+__device__ __forceinline__ double mul_sub(double a, double b, double c, double d) {
+  return fma(a, b, -__dmul_rn(c, d));
+}
+__device__ __forceinline__ double mul_add(double a, double b, double c, double d) {
+  return fma(a, b, __dmul_rn(c, d));
+}
+
+// sync[0]: arrivals; sync[1]: set when a wait gave up (the sweep is then void).
+// Cooperative launch: every block is resident. A is read and written past L1.
+constexpr int kJr = 8, kJc = 16, kJv = 32;  // row pairs and column pairs of a tile, rows of V
+__global__ void __launch_bounds__(kJr *kJc)
+    jacobi_sweep_kernel(int n, int m, int all, double *A, double *A2, double *V,
+                        unsigned long long *maxoff, unsigned *sync) {
+  __shared__ double cs[kJc + kJr], sn[kJc + kJr];
+  const int npair = m / 2, tx = threadIdx.x % kJc, ty = threadIdx.x / kJc;
+  const int tc = (npair + kJc - 1) / kJc, ta = tc * ((npair + kJr - 1) / kJr);
+  double *Ain = A, *Aout = A2;
+  for (int r = 0; r < m - 1; ++r) {
+    for (int tile = blockIdx.x; tile < all; tile += gridDim.x) {
+      const bool isV = tile >= ta;  // the tiles of V follow those of A
+      const int bx = (isV ? tile - ta : tile) % tc, by = (isV ? tile - ta : tile) / tc;
+      const int k2 = bx * kJc + tx, k1 = by * kJr + ty;
+      int p2 = 0, q2 = n, p1 = 0, q1 = n;
+      const bool in = k2 < npair && (isV || k1 < npair);
+      double x[kJv / kJr][2];  // V: rows by kJv + ty + kJr y; A: x[0], x[1] the 2 x 2 block
+#pragma unroll
+      for (int y = 0; y < kJv / kJr; ++y) x[y][0] = x[y][1] = 0.0;
+      if (in) {
+        rr_pair(k2, r, m, &p2, &q2);
+        if (isV) {
+#pragma unroll
+          for (int y = 0; y < kJv / kJr; ++y) {
+            const int row = by * kJv + ty + kJr * y;
+            if (row < n) {
+              x[y][0] = __ldcg(V + (long)row * n + p2);
+              if (q2 < n) x[y][1] = __ldcg(V + (long)row * n + q2);
+            }
+          }
+        } else {
+          rr_pair(k1, r, m, &p1, &q1);
+          x[0][0] = __ldcg(Ain + (long)p1 * n + p2);
+          if (q2 < n) x[0][1] = __ldcg(Ain + (long)p1 * n + q2);
+          if (q1 < n) x[1][0] = __ldcg(Ain + (long)q1 * n + p2);
+          if (q1 < n && q2 < n) x[1][1] = __ldcg(Ain + (long)q1 * n + q2);
+        }
+      }
+      if (threadIdx.x < (isV ? kJc : kJc + kJr)) {  // rotations: the column pairs', then the row pairs'
+        const int k = threadIdx.x < kJc ? bx * kJc + threadIdx.x : by * kJr + threadIdx.x - kJc;
+        int p = 0, q = n;
+        if (k < npair) rr_pair(k, r, m, &p, &q);
+        double c = 1.0, s = 0.0;
+        if (q < n) {
+          const double apq = __ldcg(Ain + (long)p * n + q);
+          const double app = __ldcg(Ain + (long)p * n + p), aqq = __ldcg(Ain + (long)q * n + q);
+          const double mag = fabs(apq);
+          if (mag > 0.0) {
+            if (tile < tc && threadIdx.x < kJc)
+              atomicMax(maxoff, (unsigned long long)__double_as_longlong(mag));
+            double tau = (aqq - app) / (2.0 * apq);
+            double t;
+            if (fabs(tau) > 1e150) t = 0.5 / tau;
+            else t = (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
+            c = 1.0 / sqrt(1.0 + t * t);
+            s = t * c;
+          }
+        }
+        cs[threadIdx.x] = c;
+        sn[threadIdx.x] = s;
+      }
+      __syncthreads();
+      if (in) {
+        const double c2 = cs[tx], s2 = sn[tx];
+        if (isV) {
+#pragma unroll
+          for (int y = 0; y < kJv / kJr; ++y) {
+            const int row = by * kJv + ty + kJr * y;
+            if (row < n && q2 < n) {
+              __stcg(V + (long)row * n + p2, mul_sub(c2, x[y][0], s2, x[y][1]));
+              __stcg(V + (long)row * n + q2, mul_add(s2, x[y][0], c2, x[y][1]));
+            }
+          }
+        } else {
+          const double c1 = cs[kJc + ty], s1 = sn[kJc + ty];
+          const bool hq1 = q1 < n, hq2 = q2 < n;
+          // rows: J1^T X
+          const double ypp = mul_sub(c1, x[0][0], s1, x[1][0]), ypq = mul_sub(c1, x[0][1], s1, x[1][1]);
+          const double yqp = mul_add(s1, x[0][0], c1, x[1][0]), yqq = mul_add(s1, x[0][1], c1, x[1][1]);
+          // cols: (J1^T X) J2
+          __stcg(Aout + (long)p1 * n + p2, mul_sub(c2, ypp, s2, ypq));
+          if (hq2) __stcg(Aout + (long)p1 * n + q2, mul_add(s2, ypp, c2, ypq));
+          if (hq1) __stcg(Aout + (long)q1 * n + p2, mul_sub(c2, yqp, s2, yqq));
+          if (hq1 && hq2) __stcg(Aout + (long)q1 * n + q2, mul_add(s2, yqp, c2, yqq));
+        }
+      }
+      if (all > gridDim.x) __syncthreads();  // cs, sn are read before the next tile's
     }
-    X[(long)row * n + j] = x;
+    if (!sweep_barrier(sync, (unsigned)(r + 1) * gridDim.x)) {
+      if (threadIdx.x == 0) atomicExch(sync + 1, 1u);
+      return;
+    }
+    double *t = Ain;
+    Ain = Aout;
+    Aout = t;
   }
-  for (int o = 16; o > 0; o >>= 1) {
-    sum += __shfl_xor_sync(0xffffffffu, sum, o);
-    off = fmax(off, __shfl_xor_sync(0xffffffffu, off, o));
-  }
-  if (threadIdx.x == 32) part = sum;
-  __syncthreads();
-  if (lane == 0) atomicMax(stats, (unsigned long long)__double_as_longlong(off));
-  if (threadIdx.x == 0)
-    atomicMax(stats + 1, (unsigned long long)__double_as_longlong(fabs(sum + part)));
-}
-
-// Q = I + scale X
-__global__ void newton_start_kernel(int n, const double *__restrict__ X, double scale,
-                                    double *__restrict__ Q) {
-  const long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx < (long)n * n) Q[idx] = (idx / n == idx % n) ? 1.0 : scale * X[idx];
 }
 
 __global__ void max_abs_kernel(size_t count, const double *a, unsigned long long *out) {
@@ -335,89 +365,54 @@ cudaError_t dgemm(bool ta, bool tb, int M, int N, int K, double alpha, const dou
                   long sS, double beta, double *C, long ldc, long sC, int batch, cudaStream_t s) {
   if (M <= 0 || N <= 0 || batch <= 0) return cudaSuccess;
   return dgemm_any(ta, tb, GemmArgs{M, N, K, alpha, A, lda, sA, B, ldb, sB, sk, sS, beta, C, ldc, sC,
-                                    0.0, batch}, s);
+                                    batch}, s);
 }
 
-// Each pass is either a Jacobi sweep (n - 1 rounds of rotations, each waiting
-// for the last) or, once the off-diagonal part E is small against the gaps, one
-// Newton step: with D = diag A and [D, X] = -E, Q = exp(X) takes A = D + E to
-//   A' = D + [E, X] / 2 + O(E X^2),   max |E'| <= 1.5 |X| max |E|,
-// |X| the largest row sum: as quadratic as a sweep, but four to ten matrix
-// products (of the FP64 pipe's rate) instead of n - 1 dependent launches. X is
-// antisymmetric and exp(X) is summed until its next term is below 1e-18, so Q is
-// orthogonal to rounding. |X| <= 1/4 takes the step: there every pass gains at
-// least a factor 2.7, and a pass that gained less than 2 (gaps at the rounding's
-// level) hands back to the sweep. Clusters closer than their coupling keep
-// |X| large and stay with the sweeps.
-// A Hartree-Fock solve at n = 199 (57 warm-started eigenproblems): 152 sweeps of
-// 1.4 ms before, now 9 sweeps of 1.0 ms and 114 steps of 0.04 to 0.2 ms.
-int sym_eig(int n, double **Aio, double **Vio, double *work, double *scal, double tol, int max_sweeps,
+int sym_eig(int n, double **Aio, double *A2, double *V, double *scal, double tol, int max_sweeps,
             cudaStream_t s, cudaError_t *err) {
-  // scal[0]: max |A_ij| at start; scal[1], scal[2]: max |A_pq| before the pass, |X|
+  // scal[0]: max |A_ij| at start; scal[1]: max pre-rotation |A_pq| within a sweep;
+  // scal[2]: the sweep's barrier and its error flag
   unsigned long long *bits = reinterpret_cast<unsigned long long *>(scal);
+  unsigned *sync = reinterpret_cast<unsigned *>(scal + 2);
   *err = cudaMemsetAsync(scal, 0, 3 * sizeof(double), s);
   if (*err != cudaSuccess) return -1;
   const size_t nn = (size_t)n * n;
-  const int m = n + (n & 1), npair = m / 2, tiles = (npair + 15) / 16;
-  const unsigned ground = (unsigned)(tiles * (tiles + (n + 15) / 16));
-  double *A2 = work, *X = work + nn, *Q = work + 2 * nn, *T = work + 3 * nn, *A = *Aio, *V = *Vio;
+  double *A = *Aio;
   max_abs_kernel<<<64, 256, 0, s>>>(nn, A, bits);
-  auto product = [&](bool ta, double alpha, const double *L, const double *R, double diag, double *out) {
-    if (*err != cudaSuccess) return;
-    *err = dgemm_any(ta, false, GemmArgs{n, n, n, alpha, L, n, 0, R, n, 0, nullptr, 0, 0.0, out, n, 0,
-                                         diag, 1}, s);
-  };
-  double host[3], last = 0.0;
+  int dev = 0, sms = 0, per = 0;
+  *err = cudaGetDevice(&dev);
+  if (*err == cudaSuccess) *err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (*err == cudaSuccess)
+    *err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, jacobi_sweep_kernel,
+                                                         kJr * kJc, 0);
+  if (*err != cudaSuccess) return -1;
+  int m = n + (n & 1), npair = m / 2;
+  int all = (npair + kJc - 1) / kJc * ((npair + kJr - 1) / kJr + (n + kJv - 1) / kJv);
+  const int grid = std::max(1, std::min(all, sms * std::min(per, 4)));
+  double host[3];
   int sweep = 0;
   for (sweep = 1; sweep <= max_sweeps; ++sweep) {
     if (sweep > 1) {
-      *err = cudaMemsetAsync(bits + 1, 0, 2 * sizeof(unsigned long long), s);
+      *err = cudaMemsetAsync(scal + 1, 0, 2 * sizeof(double), s);
       if (*err != cudaSuccess) return -1;
     }
-    newton_generator_kernel<<<n, 64, 0, s>>>(n, A, X, bits + 1);
-    *err = cudaGetLastError();
-    if (*err != cudaSuccess) return -1;
+    if (n > 1) {
+      unsigned long long *off = bits + 1;
+      void *args[] = {&n, &m, &all, &A, &A2, &V, &off, &sync};
+      *err = cudaLaunchCooperativeKernel(jacobi_sweep_kernel, dim3(grid), dim3(kJr * kJc), args, 0, s);
+      if (*err != cudaSuccess) return -1;
+      std::swap(A, A2);  // m - 1 rounds, an odd number
+    }
     *err = cudaMemcpyAsync(host, scal, 3 * sizeof(double), cudaMemcpyDeviceToHost, s);
     if (*err == cudaSuccess) *err = cudaStreamSynchronize(s);
     if (*err != cudaSuccess) return -1;
-    const double anorm = host[0], off = host[1], xn = host[2];
-    if (n == 1 || anorm == 0.0) return 0;
-    const bool enough = off <= tol * anorm;  // this pass is the last
-    if (xn <= 0.25 && off <= (last > 0.0 ? 0.5 * last : off)) {
-      int terms = 1;
-      for (double t = xn; (t *= xn / (terms + 1)) > 1e-18;) ++terms;
-      const unsigned ge = (unsigned)((nn + 255) / 256);
-      newton_start_kernel<<<ge, 256, 0, s>>>(n, X, 1.0 / terms, Q);
-      *err = cudaGetLastError();
-      for (int j = terms - 1; j >= 1; --j) {
-        product(false, 1.0 / j, X, Q, 1.0, T);
-        std::swap(Q, T);
-      }
-      product(false, 1.0, V, Q, 0.0, T);
-      if (*err != cudaSuccess) return -1;
-      // what the step leaves is below rounding: D stands
-      if (1.5 * off * xn <= 1e-18 * anorm) {
-        std::swap(V, T);
-        break;
-      }
-      product(false, 1.0, A, Q, 0.0, A2);
-      product(true, 1.0, Q, A2, 0.0, A);
-      if (*err != cudaSuccess) return -1;
-      std::swap(V, T);
-      last = off;
-    } else {
-      for (int r = 0; r < m - 1; ++r) {
-        jacobi_round_kernel<<<ground, 256, 0, s>>>(n, m, r, tiles, A, A2, V);
-        std::swap(A, A2);
-      }
-      *err = cudaGetLastError();
-      if (*err != cudaSuccess) return -1;
-      last = 0.0;
-    }
-    if (enough) break;
+    unsigned state[2];
+    memcpy(state, host + 2, sizeof(state));
+    if (state[1]) return -3;
+    if (n == 1 || host[0] == 0.0) break;
+    if (host[1] <= tol * host[0]) break;
   }
   *Aio = A;
-  *Vio = V;
   return sweep > max_sweeps ? -2 : sweep;
 }
 
