@@ -25,6 +25,8 @@
 // partial stack; a fixed-order sum then adds the partials into I1, so results
 // do not depend on the schedule. S > 1 only pays when there are too few row
 // tiles to fill the GPU (small systems) or to balance the last wave.
+#include <algorithm>
+
 #include "common.cuh"
 #include "tc.cuh"
 #include "tc_sys.cuh"
@@ -877,31 +879,25 @@ __global__ void split_f16_kernel(int n, long rows, int ld16, const double *__res
   if (__any_sync(0xffffffffu, bad) && lane == 0 && flag) atomicOr(flag, 2);
 }
 
-// scale->maxC = max over (i, j) of |c1| + |c2|; scale->maxS = 0 (one block).
+// scale->maxC = max over (i, j) of |c1| + |c2|, scale->maxV the largest |V32| entry
+// exactly (V32 = (float)V); *scale is zero before. Non-negative floats order like
+// their bits. (One block over M^2 coefficients took 592 us at M = 1025.)
 __global__ void scale_init_kernel(long mm, const int4 *__restrict__ coef32, long nn,
                                   const double *__restrict__ V, TcScale *scale) {
-  __shared__ float sh[2][256];
   float m = 0.f, v = 0.f;
-  for (long x = threadIdx.x; x < mm; x += blockDim.x) {
+  const long step = (long)gridDim.x * blockDim.x, first = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  for (long x = first; x < mm; x += step) {
     const int4 c = coef32[x];
     m = fmaxf(m, fabsf(__int_as_float(c.z)) + fabsf(__int_as_float(c.w)));
   }
-  for (long x = threadIdx.x; x < nn; x += blockDim.x) v = fmaxf(v, (float)fabs(V[x]));
-  sh[0][threadIdx.x] = m;
-  sh[1][threadIdx.x] = v;
-  __syncthreads();
-  for (int st = 128; st > 0; st >>= 1) {
-    if (threadIdx.x < st) {
-      sh[0][threadIdx.x] = fmaxf(sh[0][threadIdx.x], sh[0][threadIdx.x + st]);
-      sh[1][threadIdx.x] = fmaxf(sh[1][threadIdx.x], sh[1][threadIdx.x + st]);
-    }
-    __syncthreads();
+  for (long x = first; x < nn; x += step) v = fmaxf(v, (float)fabs(V[x]));
+  for (int o = 16; o > 0; o >>= 1) {
+    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
   }
-  if (threadIdx.x == 0) {
-    scale->maxC = sh[0][0];
-    scale->maxV = sh[1][0];  // the largest |V32| entry exactly: V32 = (float)V
-    scale->maxS = 0u;
-    scale->pad = 0u;
+  if ((threadIdx.x & 31) == 0) {
+    atomicMax(reinterpret_cast<unsigned *>(&scale->maxC), __float_as_uint(m));
+    atomicMax(reinterpret_cast<unsigned *>(&scale->maxV), __float_as_uint(v));
   }
 }
 
@@ -972,7 +968,11 @@ cudaError_t launch_split_f16(int n, int M, const double *G, void *h16, cudaStrea
 
 cudaError_t launch_scale_init(int M, const int4 *coef32, int n, const double *V, TcScale *scale,
                               cudaStream_t s) {
-  scale_init_kernel<<<1, 256, 0, s>>>((long)M * M, coef32, (long)n * n, V, scale);
+  cudaError_t e = cudaMemsetAsync(scale, 0, sizeof(TcScale), s);
+  if (e != cudaSuccess) return e;
+  const long most = std::max((long)M * M, (long)n * n);
+  const unsigned blocks = (unsigned)std::min(304L, (most + 255) / 256);
+  scale_init_kernel<<<blocks, 256, 0, s>>>((long)M * M, coef32, (long)n * n, V, scale);
   return cudaGetLastError();
 }
 
