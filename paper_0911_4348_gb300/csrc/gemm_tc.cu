@@ -26,16 +26,19 @@
 // largest group among its rows (a block-triangular B: the rows of group g need
 // k < (g + 1) k_tri); a tile whose slice lies beyond that writes zeros.
 //
-// Producers take one row of A and 16 consecutive k per thread; in MC mode the 32
+// Producers take one row of A and eight consecutive k per thread; in MC mode the 32
 // lanes of a warp hold 32 consecutive rows, so every load instruction is
-// coalesced along the rows.
+// coalesced along the rows. FP32 values are fetched one chunk ahead.
 //
 // One CTA per 128 x Nt output tile (Nt <= 256, a multiple of 16): warps 0-3
-// drain TMEM, warps 4-11 load, convert, split and store both operands of a
-// 32-wide k chunk into the K-major 128-byte-swizzled stage layout, warp 12
+// drain TMEM, warps 4-19 load, convert, split and store both operands of a
+// 32-wide k chunk into the K-major 128-byte-swizzled stage layout, warp 20
 // issues the MMAs. Two stages handed over with mbarriers (full: one arrival per
 // producer warp; empty: MMA commit); every wait is bounded and a timeout sets
-// the error flag.
+// the error flag. Bound by the producers' instructions and their latency (the
+// tensor pipe is 15 percent busy): a product of the real-time
+// rows (n = 39, K to 6300, 16 slices) took 46 us on average with eight producer
+// warps that fetched as they went, now 40.
 #include <type_traits>
 
 #include "common.cuh"
@@ -46,7 +49,9 @@ namespace fedvr {
 namespace {
 
 constexpr uint64_t kWaitNs = 2000000000ull;
-constexpr int kWarps = 13;  // 0-3 epilogue, 4-11 producers, 12 MMA
+constexpr int kProd = 16;           // producer warps
+constexpr int kWarps = 4 + kProd + 1;  // 0-3 epilogue, then the producers, then MMA
+constexpr int kPT = kProd * 32;
 constexpr int kThreads = kWarps * 32;
 constexpr uint32_t kTileA = 128 * 128;  // one 128-row x 32-value FP32 operand copy
 
@@ -76,7 +81,7 @@ __device__ __forceinline__ void put1(uint8_t *t, uint32_t lo_off, int r, int k, 
 
 // Four consecutive k values from row offset off of an FP32 operand (zeros
 // beyond kend or for a dead row); 16-byte load when all four lie before kend.
-__device__ __forceinline__ float4 ld4(const float *X, long off, int k, int kend, bool live) {
+__device__ __forceinline__ float4 ld4(const float *X, int off, int k, int kend, bool live) {
   float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
   if (!live) return v;
   if (k + 4 <= kend) return *reinterpret_cast<const float4 *>(X + off + k);
@@ -125,8 +130,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tf32x3_kernel(GemmArgs p) {
     tc::tmem_relinquish();
   }
   if (tid == 0) {
-    tc::mbar_init(&full[0], 8);  // one arrival per producer warp
-    tc::mbar_init(&full[1], 8);
+    tc::mbar_init(&full[0], kProd);  // one arrival per producer warp
+    tc::mbar_init(&full[1], kProd);
     tc::mbar_init(&empty[0], 1);
     tc::mbar_init(&empty[1], 1);
     tc::mbar_init(accf, 1);
@@ -140,39 +145,50 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tf32x3_kernel(GemmArgs p) {
   const uint32_t tmem = *tmem_slot;
   bool issued = false;
 
-  if (warp >= 4 && warp < 12) {
+  if (warp >= 4 && warp < 4 + kProd) {
     bool vec_done = false;
     if constexpr (!A_MC && !B_MC && std::is_same<TA, float>::value &&
                   std::is_same<TB, float>::value) {
       if (p.vec) {
         // ---- producers, FP32 operands along k: a 32-value chunk row is 8 float4, eight
-        // lanes cover one 128-byte row segment (A: 4 float4 per thread, B: up to 8) ----
+        // lanes cover one 128-byte row segment (A: 2 float4 per thread, B: up to 4) ----
         vec_done = true;
         const int pt = tid - 128;
         const float *A = reinterpret_cast<const float *>(p.A) + (long)z * p.a_sz;
         const float *B = reinterpret_cast<const float *>(p.B) + (long)z * p.b_sz;
-        long aoff4[4], boff4[8];
-        bool alive4[4], blive4[8];
+        constexpr int QA = 1024 / kPT, QB = 2048 / kPT;
+        int aoff4[QA], boff4[QB];
+        bool alive4[QA], blive4[QB];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int r = row0 + ((pt + 256 * q) >> 3);
+        for (int q = 0; q < QA; ++q) {
+          const int r = row0 + ((pt + kPT * q) >> 3);
           alive4[q] = r < p.R;
-          aoff4[q] = alive4[q] ? (long)(r / p.G) * p.a_sg + (long)(r % p.G) * p.a_sw : 0;
+          aoff4[q] = alive4[q] ? (r / p.G) * p.a_sg + (r % p.G) * p.a_sw : 0;
         }
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          const int c = (pt + 256 * q) >> 3;
+        for (int q = 0; q < QB; ++q) {
+          const int c = (pt + kPT * q) >> 3;
           blive4[q] = c < Nt && col0 + c < p.N;
-          boff4[q] = blive4[q] ? (long)(col0 + c) * p.b_s : 0;
+          boff4[q] = blive4[q] ? (col0 + c) * p.b_s : 0;
         }
         const int c4 = (pt & 7) * 4;
-        for (int kc = 0; kc < KC; ++kc) {
+        float4 an[QA], bn[QB];
+        const auto fetch = [&](int kc) {
           const int k = kbeg + kc * 32 + c4;
-          float4 av[4], bv[8];
 #pragma unroll
-          for (int q = 0; q < 4; ++q) av[q] = ld4(A, aoff4[q], k, kend, alive4[q]);
+          for (int q = 0; q < QA; ++q) an[q] = ld4(A, aoff4[q], k, kend, alive4[q]);
 #pragma unroll
-          for (int q = 0; q < 8; ++q) bv[q] = ld4(B, boff4[q], k, kend, blive4[q]);
+          for (int q = 0; q < QB; ++q)
+            if (kPT * q < Nt * 8) bn[q] = ld4(B, boff4[q], k, kend, blive4[q]);
+        };
+        if (KC > 0) fetch(0);
+        for (int kc = 0; kc < KC; ++kc) {
+          float4 av[QA], bv[QB];
+#pragma unroll
+          for (int q = 0; q < QA; ++q) av[q] = an[q];
+#pragma unroll
+          for (int q = 0; q < QB; ++q) bv[q] = bn[q];
+          if (kc + 1 < KC) fetch(kc + 1);  // in flight while this chunk is split and stored
           const int s = kc & 1;
           const uint32_t use = kc >> 1;
           if (use > 0 && !tc::warp_wait(&empty[s], (use - 1) & 1, kWaitNs)) {
@@ -181,12 +197,12 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tf32x3_kernel(GemmArgs p) {
           }
           uint8_t *st = smem + s * stage_bytes;
 #pragma unroll
-          for (int q = 0; q < 4; ++q)
-            put4(st, kTileA, (pt + 256 * q) >> 3, c4, reinterpret_cast<const float *>(&av[q]));
+          for (int q = 0; q < QA; ++q)
+            put4(st, kTileA, (pt + kPT * q) >> 3, c4, reinterpret_cast<const float *>(&av[q]));
           uint8_t *sb = st + 2 * kTileA;
 #pragma unroll
-          for (int q = 0; q < 8; ++q) {
-            const int c = (pt + 256 * q) >> 3;
+          for (int q = 0; q < QB; ++q) {
+            const int c = (pt + kPT * q) >> 3;
             if (c < Nt) put4(sb, tileB, c, c4, reinterpret_cast<const float *>(&bv[q]));
           }
           tc::fence_smem_to_async();
@@ -200,13 +216,14 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tf32x3_kernel(GemmArgs p) {
       const TA *A = reinterpret_cast<const TA *>(p.A) + (long)z * p.a_sz;
       const TA *A2 = reinterpret_cast<const TA *>(p.A2);
       const TB *B = reinterpret_cast<const TB *>(p.B) + (long)z * p.b_sz;
-      // A: one row and 16 consecutive k per thread. MC: warp w takes rows
-      // (w & 3) * 32 + lane and k half w >> 2, so each load instruction reads 32
-      // consecutive rows at one k (rows are contiguous in MC); KC: row pt / 2, k half
-      // pt & 1 (k is contiguous in KC)
+      // A: one row and KA consecutive k per thread. MC: warp w takes rows
+      // (w & 3) * 32 + lane and k part w >> 2, so each load instruction reads 32
+      // consecutive rows at one k (rows are contiguous in MC); KC: row pt / RT, k part
+      // pt % RT (k is contiguous in KC)
+      constexpr int RT = kPT / 128, KA = 32 / RT;
       const int wp = pt >> 5;
-      const int ra = A_MC ? (wp & 3) * 32 + lane : (pt >> 1);
-      const int kh = A_MC ? (wp >> 2) * 16 : (pt & 1) * 16;
+      const int ra = A_MC ? (wp & 3) * 32 + lane : pt / RT;
+      const int kh = A_MC ? (wp >> 2) * KA : pt % RT * KA;
       int aoff0 = 0, aoff20 = 0;
       bool alive0;
       {
@@ -218,43 +235,45 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tf32x3_kernel(GemmArgs p) {
           if (MUL2) aoff20 = (p.nG - 1 - g) * p.a_sg + w;
         }
       }
-      // B columns of this thread: MC 32 consecutive local columns (one k per lane),
-      // KC one local column
-      const int cb = B_MC ? (pt >> 5) * 32 : pt;
-      for (int kc = 0; kc < KC; ++kc) {
+      // B: MC NB consecutive local columns at one k per lane, KC one local column and NB
+      // consecutive k
+      constexpr int NB = 256 / kProd, CT = 32 / NB;
+      const int cb = B_MC ? wp * NB : pt / CT;
+      const int kb0 = B_MC ? lane : pt % CT * NB;
+      TA an[KA], a2n[MUL2 ? KA : 1];
+      TB bn[NB];
+      const auto fetch = [&](int kc) {
         const int k0 = kbeg + kc * 32;
-        float av[16], bv[32];
-        if (A_MC) {
 #pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            const int k = k0 + kh + i;
-            float x = 0.f;
-            if (alive0 && k < kend) {
-              x = (float)A[aoff0 + k * p.a_sk];
-              if (MUL2) x *= (float)A2[aoff20 + k * p.a_sk];
-            }
-            av[i] = x;
-          }
-        } else {
-          const int kb = k0 + kh;
-#pragma unroll
-          for (int i = 0; i < 16; ++i)
-            av[i] = (alive0 && kb + i < kend) ? (float)A[aoff0 + kb + i] : 0.f;
+        for (int i = 0; i < KA; ++i) {
+          const int k = k0 + kh + i;
+          const bool ok = alive0 && k < kend;
+          an[i] = ok ? A[aoff0 + (A_MC ? k * p.a_sk : k)] : (TA)0;
+          if (MUL2) a2n[MUL2 ? i : 0] = ok ? A2[aoff20 + k * p.a_sk] : (TA)0;
         }
-        if (B_MC) {
-          const int k = k0 + lane;
+        if (cb < Nt) {
 #pragma unroll
-          for (int i = 0; i < 32; ++i) {
-            const int c = col0 + cb + i;
-            bv[i] = (cb + i < Nt && c < p.N && k < kend) ? (float)B[k * p.b_s + c] : 0.f;
+          for (int i = 0; i < NB; ++i) {
+            const int c = B_MC ? cb + i : cb, k = k0 + kb0 + (B_MC ? 0 : i);
+            const bool ok = c < Nt && col0 + c < p.N && k < kend;
+            bn[i] = ok ? B[B_MC ? k * p.b_s + col0 + c : (col0 + c) * p.b_s + k] : (TB)0;
           }
-        } else {
-          const int c = col0 + cb;
-          const bool ok = cb < Nt && c < p.N;
-#pragma unroll
-          for (int i = 0; i < 32; ++i)
-            bv[i] = (ok && k0 + i < kend) ? (float)B[c * p.b_s + k0 + i] : 0.f;
         }
+      };
+      // FP64 operands would spill: fetched and used in the same chunk
+      constexpr bool ahead = sizeof(TA) == 4 && sizeof(TB) == 4;
+      if (ahead && KC > 0) fetch(0);
+      for (int kc = 0; kc < KC; ++kc) {
+        if (!ahead) fetch(kc);
+        float av[KA], bv[NB];
+#pragma unroll
+        for (int i = 0; i < KA; ++i) {
+          av[i] = (float)an[i];
+          if (MUL2) av[i] *= (float)a2n[MUL2 ? i : 0];
+        }
+#pragma unroll
+        for (int i = 0; i < NB; ++i) bv[i] = (float)bn[i];
+        if (ahead && kc + 1 < KC) fetch(kc + 1);  // in flight while this chunk is split and stored
         const int s = kc & 1;
         const uint32_t use = kc >> 1;
         if (use > 0 && !tc::warp_wait(&empty[s], (use - 1) & 1, kWaitNs)) {
@@ -263,21 +282,21 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tf32x3_kernel(GemmArgs p) {
         }
         uint8_t *st = smem + s * stage_bytes;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) put4(st, kTileA, ra, kh + 4 * q, av + 4 * q);
+        for (int q = 0; q < KA / 4; ++q) put4(st, kTileA, ra, kh + 4 * q, av + 4 * q);
         uint8_t *sb = st + 2 * kTileA;
         if (B_MC) {
 #pragma unroll
-          for (int i = 0; i < 32; ++i)
+          for (int i = 0; i < NB; ++i)
             if (cb + i < Nt) put1(sb, tileB, cb + i, lane, bv[i]);
         } else if (cb < Nt) {
 #pragma unroll
-          for (int q = 0; q < 8; ++q) put4(sb, tileB, cb, 4 * q, bv + 4 * q);
+          for (int q = 0; q < NB / 4; ++q) put4(sb, tileB, cb, kb0 + 4 * q, bv + 4 * q);
         }
         tc::fence_smem_to_async();
         tc::warp_arrive(&full[s]);
       }
     }
-  } else if (warp == 12) {
+  } else if (warp == 4 + kProd) {
     // ---- MMA issue (kind::tf32, K = 8 per instruction) ----
     if (tc::elect_one()) {
       const uint32_t idesc = tc::idesc_tf32(128, Nt);
@@ -342,7 +361,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tf32x3_kernel(GemmArgs p) {
   __syncthreads();
   if (*abort_flag) {
     // let MMAs still in flight finish (bounded) before the TMEM goes away
-    if (warp == 12 && (issued || lane == 0)) {
+    if (warp == 4 + kProd && (issued || lane == 0)) {
       if (issued) tc::mma_commit(drain);
       atomicExch(p.err, 1);
       if (issued) tc::mbar_wait(drain, 0, kWaitNs);
