@@ -893,7 +893,7 @@ void fedvr_destroy(fedvr_ctx *ctx) {
                     &ctx->w_K32, &ctx->w_tab, &ctx->w_btab, &ctx->w_c1p,
                     &ctx->w_coef32, &ctx->w_h16, &ctx->w_xrow, &ctx->w_dens,
                     &ctx->w_q4coef, &ctx->w_q4W, &ctx->w_q4w, &ctx->k_L, &ctx->k_G,
-                    &ctx->k_S, &ctx->k_T1, &ctx->k_R, &ctx->k_aux, &ctx->k_out,
+                    &ctx->k_S, &ctx->k_R, &ctx->k_aux, &ctx->k_out,
                     &ctx->k_part, &ctx->k_sh, &ctx->k_aop, &ctx->k_o, &ctx->k_flag, &ctx->k_x,
                     &ctx->g_w, &ctx->g_vqv, &ctx->g_c, &ctx->g_new, &ctx->g_coef, &ctx->g_res,
                     &ctx->m_t, &ctx->m_src, &ctx->m_y, &ctx->w_c1f, &ctx->w_crt, &ctx->w_crtx};
@@ -903,6 +903,9 @@ void fedvr_destroy(fedvr_ctx *ctx) {
   for (int i = 0; i < 7; ++i)
     if (ctx->ev[i]) cudaEventDestroy(ctx->ev[i]);
   for (cudaEvent_t e : ctx->kbe_events) cudaEventDestroy(e);
+  if (ctx->kbe_side) cudaStreamDestroy(ctx->kbe_side);
+  if (ctx->kbe_fork) cudaEventDestroy(ctx->kbe_fork);
+  if (ctx->kbe_join) cudaEventDestroy(ctx->kbe_join);
   delete ctx;
 }
 

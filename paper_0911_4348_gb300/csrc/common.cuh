@@ -85,6 +85,8 @@ struct fedvr_ctx {
   int kbe_T = 0, kbe_n = 0;
   double kbe_stats[8] = {0, 0, 0, 0, 0, 0, 0, 0};
   std::vector<cudaEvent_t> kbe_events;
+  cudaStream_t kbe_side = nullptr;  // -i h_HF F beside the split-mode products (kbe.cu)
+  cudaEvent_t kbe_fork = nullptr, kbe_join = nullptr;
 
   // named device buffers
   fedvr::DevBuf b_xi, b_om, b_edges, b_nodes, b_weights, b_elem, b_local, b_tt;
@@ -97,7 +99,7 @@ struct fedvr_ctx {
       w_t1, w_t2, w_t3, w_dHF, w_part, w_red, w_tc, w_K32, w_tab, w_btab, w_c1p, w_coef32, w_h16,
       w_xrow, w_dens, w_q4coef, w_q4W, w_q4w;
   // real-time propagation: two-time L and Gt, self-energy row, scratch, outputs
-  fedvr::DevBuf k_L, k_G, k_S, k_T1, k_R, k_aux, k_out, k_part, k_sh, k_aop, k_o, k_flag, k_x;
+  fedvr::DevBuf k_L, k_G, k_S, k_R, k_aux, k_out, k_part, k_sh, k_aop, k_o, k_flag, k_x;
   // GW: screened interaction w, V Q V, convolution and update scratch, periodic table, flag
   fedvr::DevBuf g_w, g_vqv, g_c, g_new, g_coef, g_res;
   // T-matrix: the ladder t, its source V^ K V^ and the convolution (pair-space stacks)

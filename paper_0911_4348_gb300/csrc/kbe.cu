@@ -106,26 +106,38 @@ __global__ void rho_real_kernel(int n, long ld, const double *rho, double2 *L) {
 
 // h_HF = h + diag(dv) + Sigma^HF[rho], Sigma^HF = spin diag(V diag rho) - V o rho
 // (Eq. sigmahf with rho = L(t, t)).
-__global__ void hf_kernel(int n, double spin, const double *h, const double *dv, const double *V,
-                          const double2 *L, long off, long ld, double2 *out) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= n * n) return;
-  const int a = idx / n, b = idx % n;
-  const double2 r = L[off + a * ld + b];
-  const double vab = V[idx];
-  double2 s = make_double2(-vab * r.x, -vab * r.y);
-  if (a == b) {
-    double2 H = make_double2(0.0, 0.0);
-    for (int c = 0; c < n; ++c) {
-      const double2 rc = L[off + (long)c * ld + c];
-      H.x = fma(V[a * n + c], rc.x, H.x);
-      H.y = fma(V[a * n + c], rc.y, H.y);
-    }
-    s.x = spin * H.x + s.x;
-    s.y = spin * H.y + s.y;
+// One block per row a; its Hartree sum is shared by the block.
+__global__ void __launch_bounds__(64)
+    hf_kernel(int n, double spin, const double *h, const double *dv, const double *V,
+              const double2 *L, long off, long ld, double2 *out) {
+  __shared__ double2 part[2];
+  const int a = blockIdx.x;
+  double2 H = make_double2(0.0, 0.0);
+  for (int c = threadIdx.x; c < n; c += 64) {
+    const double2 rc = L[off + (long)c * ld + c];
+    H.x = fma(V[a * n + c], rc.x, H.x);
+    H.y = fma(V[a * n + c], rc.y, H.y);
   }
-  const double hd = h[idx] + ((a == b && dv) ? dv[a] : 0.0);
-  out[idx] = make_double2(hd + s.x, s.y);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    H.x += __shfl_xor_sync(0xffffffffu, H.x, o);
+    H.y += __shfl_xor_sync(0xffffffffu, H.y, o);
+  }
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = H;
+  __syncthreads();
+  for (int b = threadIdx.x; b < n; b += 64) {
+    const double2 r = L[off + a * ld + b];
+    const double vab = V[a * n + b];
+    double2 s = make_double2(-vab * r.x, -vab * r.y);
+    double hd = h[a * n + b];
+    if (a == b) {
+      const double2 sum = addz(part[0], part[1]);
+      s.x = spin * sum.x + s.x;
+      s.y = spin * sum.y + s.y;
+      if (dv) hd += dv[a];
+    }
+    out[a * n + b] = make_double2(hd + s.x, s.y);
+  }
 }
 
 // Second-Born self-energy of row i, entry e = 2k + w (w = 0: s^< from
@@ -133,49 +145,75 @@ __global__ void hf_kernel(int n, double spin, const double *h, const double *dv,
 // the reversed line gb = -H^H:
 //   S = spin g o (V Q V) - X,  Q_kl = g_kl gb_lk = -g_kl conj(H_kl),
 //   X_ab = sum_kl V_ak V_bl g_al gb_lk g_kb.
-// First V Q into T1 [e][n][n].
-__global__ void vq_kernel(int n, int i, long ld, const double2 *L, const double2 *G,
-                          const double *V, double2 *T1) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= n * n) return;
+// The direct term, one block per kDirRows rows and entry: Q, the block's rows of
+// V Q and V live in shared memory, in FP64 or (split mode, whose exchange
+// carries FP32) in FP32. Writes S. Two launches with V Q through global memory
+// and Q rebuilt by every row took 67 (FP32) and 51 us (FP64) on average at n =
+// 39; Q is now formed once per 16 rows.
+constexpr int kDirRows = 16;
+template <class R> struct Pair;
+template <> struct Pair<float> { using type = float2; };
+template <> struct Pair<double> { using type = double2; };
+template <class R> size_t direct_smem(int n) {
+  return ((size_t)n * n + (size_t)kDirRows * n) * 2 * sizeof(R) + (size_t)n * n * sizeof(R);
+}
+template <class R>
+__global__ void __launch_bounds__(256)
+    direct_kernel(int n, int i, long ld, const double2 *L, const double2 *G, const double *V,
+                  double spin, int Tcap, double2 *S) {
+  using R2 = typename Pair<R>::type;
+  extern __shared__ double2 ds[];
+  R2 *q = reinterpret_cast<R2 *>(ds), *t1 = q + n * n;
+  R *v = reinterpret_cast<R *>(t1 + kDirRows * n);
   const int e = blockIdx.y, kt = e >> 1, w = e & 1;
-  const int a = idx / n, l = idx % n;
+  const int a0 = blockIdx.x * kDirRows, nout = min(kDirRows, n - a0) * n;
   const long off = blk(i, kt, n, ld);
   const double2 *g = (w ? G : L) + off, *H = (w ? L : G) + off;
-  double2 acc = make_double2(0.0, 0.0);
-  for (int k = 0; k < n; ++k) {
-    const double2 q = cmul(g[k * ld + l], conjz(H[k * ld + l]));  // -Q_kl
-    const double v = V[a * n + k];
-    acc.x = fma(-v, q.x, acc.x);
-    acc.y = fma(-v, q.y, acc.y);
+  for (int x = threadIdx.x; x < n * n; x += 256) {
+    const int k = x / n, l = x % n;
+    const double2 gg = g[k * ld + l], hh = H[k * ld + l];
+    const R gr = (R)gg.x, gi = (R)gg.y, hr = (R)hh.x, hi = (R)hh.y;
+    R2 y;  // g conj(H) = -Q_kl
+    y.x = gr * hr + gi * hi;
+    y.y = gi * hr - gr * hi;
+    q[x] = y;
+    v[x] = (R)V[x];
   }
-  T1[(long)e * n * n + idx] = acc;
-}
-
-// Direct term S_e = spin g o (T1 V), written to the row's S[w][k].
-__global__ void direct_kernel(int n, int i, long ld, const double2 *L, const double2 *G,
-                              const double *V, const double2 *T1, double spin, int Tcap,
-                              double2 *S) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= n * n) return;
-  const int e = blockIdx.y, kt = e >> 1, w = e & 1;
-  const int a = idx / n, b = idx % n;
-  const double2 *t1 = T1 + (long)e * n * n + (long)a * n;
-  double2 W = make_double2(0.0, 0.0);
-  for (int l = 0; l < n; ++l) {
-    const double v = V[l * n + b];
-    W.x = fma(t1[l].x, v, W.x);
-    W.y = fma(t1[l].y, v, W.y);
+  __syncthreads();
+  for (int x = threadIdx.x; x < nout; x += 256) {
+    const int r = x / n, l = x % n;
+    const R *va = v + (a0 + r) * n;
+    R2 acc;
+    acc.x = acc.y = R(0);
+    for (int k = 0; k < n; ++k) {
+      acc.x = fma(-va[k], q[k * n + l].x, acc.x);
+      acc.y = fma(-va[k], q[k * n + l].y, acc.y);
+    }
+    t1[x] = acc;
   }
-  const double2 g = (w ? G : L)[blk(i, kt, n, ld) + a * ld + b];
-  S[((long)w * Tcap + kt) * n * n + idx] = cmul(scalez(spin, g), W);
+  __syncthreads();
+  for (int x = threadIdx.x; x < nout; x += 256) {
+    const int r = x / n, b = x % n, a = a0 + r;
+    R2 W;
+    W.x = W.y = R(0);
+    for (int l = 0; l < n; ++l) {
+      W.x = fma(t1[r * n + l].x, v[l * n + b], W.x);
+      W.y = fma(t1[r * n + l].y, v[l * n + b], W.y);
+    }
+    S[((long)w * Tcap + kt) * n * n + a * n + b] =
+        cmul(scalez(spin, g[a * ld + b]), make_double2(W.x, W.y));
+  }
 }
 
 // Exchange term (n > 16), one CTA per (column b, entry e): with g and
 // Hb_lk = V_bl gb_lk in shared memory, the (a, k) pairs of a chunk of rows
-// are spread over the threads (four per thread), each computing
+// are spread over the threads (XP per thread), each computing
 // P_ak = sum_l g_al Hb_lk and v_ak = V_ak P_ak g_kb into shared memory; then
-// one thread per row adds X_ab = sum_k v_ak in k order and S_ab -= X_ab.
+// one thread per row adds X_ab = sum_k v_ak in k order and S_ab -= X_ab. Bound by
+// the FP64 pipe (4 n^4 DFMA per entry), so no pair is padded but in a thread's
+// last: XP is what the fewest chunks of equal rows take. Four pairs in chunks of
+// 1024 / n rows (2048 for the 1521 pairs of n = 39) took 623 us on average over a
+// propagation to T = 25, now 554.
 // Small n (<= 16): one warp per row a, lanes over k, warp-shuffle sum over k
 // (fewer FP64 instructions in the k-sum than the pair layout below).
 __global__ void __launch_bounds__(256) exchange_rows_kernel(int n, int i, long ld,
@@ -213,14 +251,25 @@ __global__ void __launch_bounds__(256) exchange_rows_kernel(int n, int i, long l
   }
 }
 
-constexpr int kXPairs = 4;  // (a, k) pairs per thread and chunk
-inline int xchg_rows(int n) { return n < 256 * kXPairs / n ? n : 256 * kXPairs / n; }
+struct XchgPlan {
+  int rows, pairs;  // rows of a chunk, pairs per thread
+};
+inline XchgPlan xchg_plan(int n) {
+  const int most = n <= 72 ? 2048 : 1024;  // pairs of a chunk (shared memory)
+  const int chunks = (n * n + most - 1) / most;
+  int rows = (n + chunks - 1) / chunks;
+  if (rows * n > most) rows = most / n;
+  return {rows, (rows * n + 255) / 256};
+}
+inline size_t xchg_smem(int n) {
+  return (size_t)(2 * n * n + xchg_plan(n).rows * n) * sizeof(double2);
+}
 
-__global__ void __launch_bounds__(256) exchange_kernel(int n, int i, long ld, const double2 *L,
-                                                       const double2 *G, const double *V,
-                                                       int Tcap, double2 *S) {
+template <int XP>
+__global__ void __launch_bounds__(256)
+    exchange_kernel(int n, int rows, int i, long ld, const double2 *L, const double2 *G,
+                    const double *V, int Tcap, double2 *S) {
   extern __shared__ double2 xs[];
-  const int rows = n < 256 * kXPairs / n ? n : 256 * kXPairs / n;
   double2 *gs = xs, *hb = xs + n * n, *vs = xs + 2 * n * n;
   const int b = blockIdx.x, e = blockIdx.y, kt = e >> 1, w = e & 1;
   const long off = blk(i, kt, n, ld);
@@ -237,25 +286,33 @@ __global__ void __launch_bounds__(256) exchange_kernel(int n, int i, long ld, co
   double2 *Sout = S + ((long)w * Tcap + kt) * n * n;
   for (int a0 = 0; a0 < n; a0 += rows) {
     const int nr = min(rows, n - a0), np = nr * n;
-    int pa[kXPairs], pk[kXPairs];
-    double2 P[kXPairs];
+    const bool last = threadIdx.x + 256 * (XP - 1) < np;
+    int pa[XP], pk[XP];
+    double2 P[XP];
 #pragma unroll
-    for (int q = 0; q < kXPairs; ++q) {
+    for (int q = 0; q < XP; ++q) {
       const int pp = threadIdx.x + 256 * q;
-      pa[q] = pp < np ? a0 + pp / n : a0;
+      pa[q] = (pp < np ? a0 + pp / n : a0) * n;
       pk[q] = pp < np ? pp % n : 0;
       P[q] = make_double2(0.0, 0.0);
     }
-    for (int l = 0; l < n; ++l) {
+    if (last) {
+      for (int l = 0; l < n; ++l) {
 #pragma unroll
-      for (int q = 0; q < kXPairs; ++q) cmla(P[q], gs[pa[q] * n + l], hb[l * n + pk[q]]);
+        for (int q = 0; q < XP; ++q) cmla(P[q], gs[pa[q] + l], hb[l * n + pk[q]]);
+      }
+    } else {
+      for (int l = 0; l < n; ++l) {
+#pragma unroll
+        for (int q = 0; q < XP - 1; ++q) cmla(P[q], gs[pa[q] + l], hb[l * n + pk[q]]);
+      }
     }
 #pragma unroll
-    for (int q = 0; q < kXPairs; ++q) {
+    for (int q = 0; q < XP; ++q) {
       const int pp = threadIdx.x + 256 * q;
       if (pp < np) {
         double2 v = make_double2(0.0, 0.0);
-        cmla(v, scalez(V[pa[q] * n + pk[q]], P[q]), gs[pk[q] * n + b]);
+        cmla(v, scalez(V[pa[q] + pk[q]], P[q]), gs[pk[q] * n + b]);
         vs[pp] = v;
       }
     }
@@ -271,131 +328,179 @@ __global__ void __launch_bounds__(256) exchange_kernel(int n, int i, long ld, co
   }
 }
 
-// Split mode's direct term and exchange k-sum in FP32 (their inputs carry the
-// split products' precision): T1 = V Q as float2, then S = spin g o (T1 V).
-__global__ void vq32_kernel(int n, int i, long ld, const double2 *L, const double2 *G,
-                            const double *V, float2 *T1) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= n * n) return;
-  const int e = blockIdx.y, kt = e >> 1, w = e & 1;
-  const int a = idx / n, l = idx % n;
-  const long off = blk(i, kt, n, ld);
-  const double2 *g = (w ? G : L) + off, *H = (w ? L : G) + off;
-  float2 acc = make_float2(0.f, 0.f);
-  for (int k = 0; k < n; ++k) {
-    const double2 gg = g[k * ld + l], hh = H[k * ld + l];
-    const float gr = (float)gg.x, gi = (float)gg.y, hr = (float)hh.x, hi = (float)hh.y;
-    const float qr = gr * hr + gi * hi, qi = gi * hr - gr * hi;  // g conj(H) = -Q_kl
-    const float v = (float)V[a * n + k];
-    acc.x = fmaf(-v, qr, acc.x);
-    acc.y = fmaf(-v, qi, acc.y);
-  }
-  T1[(long)e * n * n + idx] = acc;
+using XchgKernel = void (*)(int, int, int, long, const double2 *, const double2 *, const double *,
+                            int, double2 *);
+inline XchgKernel xchg_kernel(int n) {
+  static constexpr XchgKernel k[8] = {exchange_kernel<1>, exchange_kernel<2>, exchange_kernel<3>,
+                                      exchange_kernel<4>, exchange_kernel<5>, exchange_kernel<6>,
+                                      exchange_kernel<7>, exchange_kernel<8>};
+  return k[xchg_plan(n).pairs - 1];
 }
-__global__ void direct32_kernel(int n, int i, long ld, const double2 *L, const double2 *G,
-                                const double *V, const float2 *T1, double spin, int Tcap,
-                                double2 *S) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= n * n) return;
-  const int e = blockIdx.y, kt = e >> 1, w = e & 1;
-  const int a = idx / n, b = idx % n;
-  const float2 *t1 = T1 + (long)e * n * n + (long)a * n;
-  float2 W = make_float2(0.f, 0.f);
-  for (int l = 0; l < n; ++l) {
-    const float v = (float)V[l * n + b];
-    W.x = fmaf(t1[l].x, v, W.x);
-    W.y = fmaf(t1[l].y, v, W.y);
-  }
-  const double2 g = (w ? G : L)[blk(i, kt, n, ld) + a * ld + b];
-  S[((long)w * Tcap + kt) * n * n + idx] = cmul(scalez(spin, g), make_double2(W.x, W.y));
+
+// x as a pair of floats (48 bits), and the product of two pairs rounded to FP32.
+// The FP64 pipe does neither the product nor its rounding fast.
+__device__ __forceinline__ float2 two_floats(double x) {
+  const float hi = (float)x;
+  return make_float2(hi, (float)(x - (double)hi));
+}
+__device__ __forceinline__ float mul_pairs(float2 a, float2 b) {
+  const float p = a.x * b.x;
+  float e = fmaf(a.x, b.x, -p);
+  e = fmaf(a.x, b.y, e);
+  e = fmaf(a.y, b.x, e);
+  return p + e;
 }
 
 // Operands of the batched exchange product of row i, entry e = 2k + w:
 // Ap_e[(p, a)][(q, l)] the real form of g (rows re/im of the output, columns
 // re/im parts of the contraction), Bp_e[(b, k)][(q, l)] = part q of
-// V_bl gb_lk = -V_bl conj(H_kl).
-__global__ void xop_kernel(int n, int i, long ld, const double2 *L, const double2 *G,
-                           const double *V, int xld, float *Ap, float *Bp) {
+// V_bl gb_lk = -V_bl conj(H_kl). One block per kXopB values of b and entry, H in
+// shared memory as pairs of floats. Bound by writing Bp (2 n^3 floats per
+// entry): two FP64 products and conversions per value took 41 us on average
+// at n = 39, T = 81, now 22.
+constexpr int kXopB = 8;
+size_t xop_smem(int n) { return ((size_t)2 * n * n + (size_t)kXopB * n) * sizeof(float2); }
+__global__ void __launch_bounds__(256)
+    xop_kernel(int n, int i, long ld, const double2 *L, const double2 *G, const double *V, int xld,
+               float *Ap, float *Bp) {
+  extern __shared__ double2 xo[];
+  float2 *hx = reinterpret_cast<float2 *>(xo), *hy = hx + n * n, *vs = hy + n * n;
   const int e = blockIdx.y, kt = e >> 1, w = e & 1;
+  const int b0 = blockIdx.x * kXopB, nb = min(kXopB, n - b0);
   const long off = blk(i, kt, n, ld), n2 = (long)n * n;
   const double2 *g = (w ? G : L) + off, *H = (w ? L : G) + off;
-  float *A = Ap + (long)e * 2 * n * xld, *B = Bp + (long)e * n2 * xld;
-  for (long q = (long)blockIdx.x * blockDim.x + threadIdx.x; q < n2 * n; q += (long)gridDim.x * blockDim.x) {
-    const int b = (int)(q / n2), k = (int)((q / n) % n), l = (int)(q % n);
+  float *A = Ap + (long)e * 2 * n * xld, *B = Bp + ((long)e * n2 + (long)b0 * n) * xld;
+  for (int x = threadIdx.x; x < n2; x += 256) {
+    const int k = x / n, l = x % n;
     const double2 h = H[k * ld + l];
-    const double v = V[b * n + l];
-    float *row = B + ((long)b * n + k) * xld;
-    row[l] = (float)(-v * h.x);
-    row[n + l] = (float)(v * h.y);
-    if (q < n2) {  // Ap from g: element (a, l) = (k, l) here
-      const int a = (int)(q / n), ll = (int)(q % n);
-      const double2 x = g[a * ld + ll];
-      A[(long)a * xld + ll] = (float)x.x;
-      A[(long)a * xld + n + ll] = (float)(-x.y);
-      A[(long)(n + a) * xld + ll] = (float)x.y;
-      A[(long)(n + a) * xld + n + ll] = (float)x.x;
+    hx[x] = two_floats(-h.x);
+    hy[x] = two_floats(h.y);
+    if (b0 == 0) {  // Ap from g: element (a, l) = (k, l) here
+      const double2 y = g[k * ld + l];
+      A[(long)k * xld + l] = (float)y.x;
+      A[(long)k * xld + n + l] = (float)(-y.y);
+      A[(long)(n + k) * xld + l] = (float)y.y;
+      A[(long)(n + k) * xld + n + l] = (float)y.x;
     }
+  }
+  for (int x = threadIdx.x; x < nb * n; x += 256) vs[x] = two_floats(V[b0 * n + x]);
+  __syncthreads();
+  int k = threadIdx.x / n, l = threadIdx.x % n;
+  for (int x = threadIdx.x; x < n2; x += 256) {  // x = k n + l
+    const float2 p = hx[x], q = hy[x];
+    float *out = B + (long)k * xld + l;
+    for (int b = 0; b < nb; ++b, out += (long)n * xld) {
+      const float2 v = vs[b * n + l];
+      out[0] = mul_pairs(v, p);
+      out[n] = mul_pairs(v, q);
+    }
+    k += 256 / n;
+    l += 256 % n;
+    if (l >= n) l -= n, ++k;
   }
 }
 
 // k-sum of the exchange from the product (FP32, like the product): S_e[a][b] -=
-// sum_k V_ak P_ak g_kb with P_ak = P_e[(b, k)][(0, a)] + i P_e[(b, k)][(1, a)];
-// thread per (a, b).
-__global__ void xsum_kernel(int n, int i, long ld, const double2 *L, const double2 *G,
-                            const double *V, const float *P, int Tcap, double2 *S) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= n * n) return;
-  const int e = blockIdx.y, kt = e >> 1, w = e & 1, a = idx % n, b = idx / n;
+// sum_k V_ak P_ak g_kb with P_ak = P_e[(b, k)][(0, a)] + i P_e[(b, k)][(1, a)].
+// One block per kXsumB columns b and entry; V^T and the columns of g in shared
+// memory in FP32. Bound by reading P (2 n^3 floats per entry): with V and g
+// converted again by every thread 39 us on average at n = 39, T = 81, now
+// 18.
+constexpr int kXsumB = 6, kXsumK = 10;
+size_t xsum_smem(int n) { return ((size_t)n * n + (size_t)2 * kXsumB * n) * sizeof(float); }
+__global__ void __launch_bounds__(256)
+    xsum_kernel(int n, int i, long ld, const double2 *L, const double2 *G, const double *V,
+                const float *P, int Tcap, double2 *S) {
+  extern __shared__ double2 xq[];
+  float2 *gs = reinterpret_cast<float2 *>(xq);
+  float *vt = reinterpret_cast<float *>(gs + kXsumB * n);
+  const int e = blockIdx.y, kt = e >> 1, w = e & 1;
+  const int b0 = blockIdx.x * kXsumB, nb = min(kXsumB, n - b0);
   const long off = blk(i, kt, n, ld), n2 = (long)n * n;
   const double2 *g = (w ? G : L) + off;
-  const float *Pe = P + (long)e * 2 * n2 * n;
-  float xr = 0.f, xi = 0.f;
-  for (int k = 0; k < n; ++k) {
-    const float *pr = Pe + ((long)b * n + k) * 2 * n;
-    const double2 gk = g[k * ld + b];
-    const float v = (float)V[a * n + k], pre = v * pr[a], pim = v * pr[n + a];
-    const float gr = (float)gk.x, gi = (float)gk.y;
-    xr = fmaf(pre, gr, xr);
-    xr = fmaf(-pim, gi, xr);
-    xi = fmaf(pre, gi, xi);
-    xi = fmaf(pim, gr, xi);
+  const float *Pe = P + ((long)e * n2 + (long)b0 * n) * 2 * n;
+  for (int x = threadIdx.x; x < n2; x += 256) vt[x % n * n + x / n] = (float)V[x];
+  for (int x = threadIdx.x; x < nb * n; x += 256) {
+    const double2 y = g[x / nb * ld + b0 + x % nb];
+    gs[x % nb * n + x / nb] = make_float2((float)y.x, (float)y.y);
   }
+  __syncthreads();
   double2 *Se = S + ((long)w * Tcap + kt) * n2;
-  Se[a * n + b] = subz(Se[a * n + b], make_double2(xr, xi));
+  for (int x = threadIdx.x; x < nb * n; x += 256) {
+    const int bb = x / n, a = x % n;
+    const float *p = Pe + (long)bb * n * 2 * n + a;
+    float xr = 0.f, xi = 0.f;
+    float pr[kXsumK], pi[kXsumK], nr[kXsumK], ni[kXsumK];  // this block of k and the next
+    const auto fetch = [&](int k0) {
+#pragma unroll
+      for (int y = 0; y < kXsumK; ++y) {
+        const bool ok = k0 + y < n;
+        nr[y] = ok ? p[(long)(k0 + y) * 2 * n] : 0.f;
+        ni[y] = ok ? p[(long)(k0 + y) * 2 * n + n] : 0.f;
+      }
+    };
+    fetch(0);
+    for (int k0 = 0; k0 < n; k0 += kXsumK) {
+#pragma unroll
+      for (int y = 0; y < kXsumK; ++y) pr[y] = nr[y], pi[y] = ni[y];
+      if (k0 + kXsumK < n) fetch(k0 + kXsumK);
+#pragma unroll
+      for (int y = 0; y < kXsumK; ++y) {
+        if (k0 + y >= n) break;
+        const float2 gk = gs[bb * n + k0 + y];
+        const float v = vt[(k0 + y) * n + a], pre = v * pr[y], pim = v * pi[y];
+        xr = fmaf(pre, gk.x, xr);
+        xr = fmaf(-pim, gk.y, xr);
+        xi = fmaf(pre, gk.y, xi);
+        xi = fmaf(pim, gk.x, xi);
+      }
+    }
+    double2 *out = Se + a * n + b0 + bb;
+    *out = subz(*out, make_double2(xr, xi));
+  }
 }
 
 struct CollArgs {
-  int n, i, j0, Tcap;
+  int n, i, Tcap;
   long ld;
   double dt;
   const double2 *L, *G, *S, *hHF;
   double2 *RL, *RG;
-  int mode;    // 0: rhs of L and Gt for columns j0 .. j0 + ncols - 1; 1: K_L(i, j0) only
   int corr;    // 0: no collision integrals (time-dependent HF)
   int ncols;   // output column blocks j
-  int splits;  // CTAs sharing one column's contraction (partial sums in part)
   int rows;    // output rows a per CTA (rows * n <= 256 * kCollQ)
+  int quota;   // units of work per CTA, at most: column j has ceil(units_j / quota) splits
+  int splits;  // the most splits of a column
   double2 *part;  // [splits][ncols][2][n n] partial sums (splits > 1)
 };
 
 constexpr int kCollQ = 8;   // outputs per thread
 constexpr int kCollKC = 16; // contraction index b per staged slice
 
-// Collision integrals (and with mode 0 the -i h_HF F term) for one time row i.
+// Work units of column j (slices of 16 contraction values).
+__host__ __device__ __forceinline__ int coll_units(int n, int i, int j, int corr) {
+  const int blocks = 1 + (corr && i > 0 ? i + 1 : 0) + (corr && j > 0 ? j + 1 : 0);
+  return blocks * ((n + kCollKC - 1) / kCollKC);
+}
+
+// Collision integrals and the -i h_HF F term for one time row i.
 // CTA (column j, split, row tile): its rows x n outputs of block j are spread
 // over the 256 threads (output o = tid + 256 q, q < kCollQ), so no output is
 // padded. The terms of column j,
-//   kind 0: -i h_HF(i) x [L(i, j), Gt(i, j)]                       (mode 0)
+//   kind 0: -i h_HF(i) x [L(i, j), Gt(i, j)]
 //   kind 1: w^i_s (s^> - s^<)(i, s) x [L(s, j), Gt(s, j)],  s = 0..i
 //   kind 2: [w^j_s s^<(i, s), w^j_s s^>(i, s)] x (L - Gt)(s, j), s = 0..j
-// times the 16-wide slices of b form a list of units; split k of S takes
-// units [U k / S, U (k+1) / S) (an empty range writes zeros). Each unit stages its left factors X [rows][16]
-// and right factors Y [16][n] in shared memory.
+// times the 16-wide slices of b form a list of units; split k of the column's S
+// takes units [U k / S, U (k+1) / S). Each unit stages its left factors X
+// [rows][16] and right factors Y [16][n] in shared memory. Bound by the FP64 pipe:
+// 8 DFMA per output, slice value and pair (L, Gt).
 __global__ void __launch_bounds__(256, 2) collision_kernel(CollArgs p) {
   extern __shared__ double2 cs[];
   const int n = p.n, i = p.i, rows = p.rows;
   double2 *X0 = cs, *X1 = X0 + rows * kCollKC, *Y0 = X1 + rows * kCollKC, *Y1 = Y0 + kCollKC * n;
-  const int split = blockIdx.x % p.splits, jj = blockIdx.x / p.splits, j = p.j0 + jj;
+  const int split = blockIdx.x % p.splits, j = blockIdx.x / p.splits;
+  const int units = coll_units(n, i, j, p.corr), nsplit = (units + p.quota - 1) / p.quota;
+  if (split >= nsplit) return;
   const long ld = p.ld, nn = (long)n * n;
   const int a0 = blockIdx.y * rows, nr = min(rows, n - a0), nout = nr * n;
   const int tid = threadIdx.x;
@@ -411,14 +516,11 @@ __global__ void __launch_bounds__(256, 2) collision_kernel(CollArgs p) {
     yo[q] = (o < nout) ? o % n : 0;
     nq += (o < nout) ? 1 : 0;
   }
-  const int n0 = p.mode == 0 ? 1 : 0;
-  const int n1 = (p.corr && i > 0) ? i + 1 : 0;
-  const int n2 = (p.corr && j > 0) ? j + 1 : 0;
+  const int n0 = 1, n1 = (p.corr && i > 0) ? i + 1 : 0;
   const int nch = (n + kCollKC - 1) / kCollKC;
-  const long units = (long)(n0 + n1 + n2) * nch;
-  const long u0 = units * split / p.splits, u1 = units * (split + 1) / p.splits;
-  for (long u = u0; u < u1; ++u) {
-    const int t = (int)(u / nch), bc = (int)(u % nch) * kCollKC;
+  const int u0 = (int)((long)units * split / nsplit), u1 = (int)((long)units * (split + 1) / nsplit);
+  for (int u = u0; u < u1; ++u) {
+    const int t = u / nch, bc = u % nch * kCollKC;
     const int kind = t < n0 ? 0 : (t < n0 + n1 ? 1 : 2);
     const int s = kind == 0 ? i : (kind == 1 ? t - n0 : t - n0 - n1);
     const double w = kind == 1 ? trap_w(s, i, p.dt) : (kind == 2 ? trap_w(s, j, p.dt) : 0.0);
@@ -486,37 +588,28 @@ __global__ void __launch_bounds__(256, 2) collision_kernel(CollArgs p) {
     const int o = tid + 256 * q, a = a0 + o / n, c = o % n;
     const long e = (long)a * n + c;
     if (p.splits > 1) {
-      double2 *P = p.part + ((long)(split * p.ncols + jj) * 2) * nn;
+      double2 *P = p.part + ((long)(split * p.ncols + j) * 2) * nn;
       P[e] = accL[q];
       P[nn + e] = accG[q];
-    } else if (p.mode == 0) {
+    } else {
       p.RL[(long)j * nn + e] = accL[q];
       p.RG[(long)j * nn + e] = accG[q];
-    } else {
-      p.RL[e] = accL[q];
     }
   }
 }
 
 // Sum of the splits' partial results in split order (deterministic).
-__global__ void coll_reduce_kernel(int n, int j0, int ncols, int splits, int mode,
-                                   const double2 *part, double2 *RL, double2 *RG) {
-  const long nn = (long)n * n;
+__global__ void coll_reduce_kernel(CollArgs p) {
+  const long nn = (long)p.n * p.n;
   const long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= nn) return;
-  const int jj = blockIdx.y;
-  double2 sl = make_double2(0.0, 0.0), sg = sl;
-  for (int k = 0; k < splits; ++k) {
-    const double2 *P = part + ((long)(k * ncols + jj) * 2) * nn;
-    sl = addz(sl, P[e]);
-    sg = addz(sg, P[nn + e]);
-  }
-  if (mode == 0) {
-    RL[(long)(j0 + jj) * nn + e] = sl;
-    RG[(long)(j0 + jj) * nn + e] = sg;
-  } else {
-    RL[e] = sl;
-  }
+  const int j = blockIdx.y, z = blockIdx.z;
+  const int nsplit = (coll_units(p.n, p.i, j, p.corr) + p.quota - 1) / p.quota;
+  double2 sum = make_double2(0.0, 0.0);
+#pragma unroll 4
+  for (int k = 0; k < nsplit; ++k)
+    sum = addz(sum, p.part[((long)(k * p.ncols + j) * 2 + z) * nn + e]);
+  (z ? p.RG : p.RL)[(long)j * nn + e] = sum;
 }
 
 // Predictor (R1 == nullptr) or corrector of time row N+1 and its mirror column.
@@ -586,36 +679,78 @@ __global__ void advance_kernel(int n, int N, long ld, double2 *L, double2 *G, co
 }
 
 // E(t) = spin Tr[h(t) rho] + spin/2 Tr[Sigma^HF rho] + spin/2 Re Tr[i K_L(t, t)]
-// and N(t) = spin Tr rho; one CTA, fixed-order reduction.
-__global__ void observe_kernel(int n, double spin, const double *h, const double *dv,
-                               const double *V, const double2 *L, long off, long ld,
-                               const double2 *K, double *E_out, double *N_out) {
+// and N(t) = spin Tr rho. Only the trace of K_L(t, t) is needed, so it is taken
+// entry by entry instead of from the matrix product (n times the work):
+//   Tr K_L(t, t) = sum_s w_s sum_ab s^>_ab(t, s) L_ba(s, t) - s^<_ab(t, s) Gt_ba(s, t).
+// Blocks a < n: the one-body terms of row a into part[3 a ..]; block n + s: the
+// term of time s into part[3 n + s]. observe_sum_kernel adds them in a fixed order.
+__global__ void __launch_bounds__(128)
+    observe_kernel(int n, int t, double spin, double dt, const double *h, const double *dv,
+                   const double *V, const double2 *L, const double2 *G, long ld, const double2 *S,
+                   int Tcap, double *part) {
+  __shared__ double red[4][4];
+  const int tid = threadIdx.x;
+  double v0 = 0.0, v1 = 0.0, v2 = 0.0;
+  if (blockIdx.x < n) {
+    const int a = blockIdx.x;
+    const double2 *rho = L + blk(t, t, n, ld);
+    const double2 raa = rho[a * ld + a];
+    for (int b = tid; b < n; b += 128) {
+      const double2 rab = rho[a * ld + b], rba = rho[b * ld + a], rbb = rho[b * ld + b];
+      const double v = V[a * n + b];
+      v0 += h[a * n + b] * rba.x;                      // Re h_ab rho_ba (h real)
+      v1 -= v * cmul(rab, rba).x;                      // exchange: -V_ab rho_ab rho_ba
+      v1 += spin * cmul(scalez(v, rbb), raa).x;        // Hartree
+    }
+    if (tid == 0) {
+      if (dv) v0 += dv[a] * raa.x;
+      v2 = raa.x;
+    }
+  } else {
+    const int s = blockIdx.x - n;
+    const long nn = (long)n * n, off = blk(t, s, n, ld);
+    for (int x = tid; x < nn; x += 128) {
+      const int a = x / n, b = x % n;
+      const double2 sl = S[(long)s * nn + x], sg = S[((long)Tcap + s) * nn + x];
+      // F(s, t)_ba = conj(F(t, s)_ab), stored as such for s < t
+      const long at = s < t ? off + a * ld + b : off + b * ld + a;
+      double2 l = L[at], g = G[at];
+      if (s < t) l = conjz(l), g = conjz(g);
+      v0 += cmul(sg, l).y - cmul(sl, g).y;
+    }
+    v0 *= -trap_w(s, t, dt);                           // Re(i K) = -Im K
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    v0 += __shfl_xor_sync(0xffffffffu, v0, o);
+    v1 += __shfl_xor_sync(0xffffffffu, v1, o);
+    v2 += __shfl_xor_sync(0xffffffffu, v2, o);
+  }
+  if ((tid & 31) == 0) {
+    red[0][tid >> 5] = v0;
+    red[1][tid >> 5] = v1;
+    red[2][tid >> 5] = v2;
+  }
+  __syncthreads();
+  if (tid < 3) {
+    const double sum = (red[tid][0] + red[tid][1]) + (red[tid][2] + red[tid][3]);
+    if (blockIdx.x < n) part[3 * blockIdx.x + tid] = sum;
+    else if (tid == 0) part[2 * n + blockIdx.x] = sum;
+  }
+}
+__global__ void observe_sum_kernel(int n, int times, double spin, const double *part,
+                                   double *E_out, double *N_out) {
   __shared__ double red[4][256];
   const int tid = threadIdx.x;
-  double e1 = 0.0, e2 = 0.0, ek = 0.0, nn_ = 0.0;
-  for (int idx = tid; idx < n * n; idx += 256) {
-    const int a = idx / n, b = idx % n;
-    const double2 rab = L[off + a * ld + b], rba = L[off + b * ld + a];
-    e1 += h[idx] * rba.x;                         // Re h_ab rho_ba (h real)
-    e2 -= V[idx] * cmul(rab, rba).x;              // exchange: -V_ab rho_ab rho_ba
-    if (a == b) {
-      const double2 raa = rab;
-      double2 H = make_double2(0.0, 0.0);
-      for (int c = 0; c < n; ++c) {
-        const double2 rc = L[off + (long)c * ld + c];
-        H.x = fma(V[a * n + c], rc.x, H.x);
-        H.y = fma(V[a * n + c], rc.y, H.y);
-      }
-      e2 += spin * cmul(H, raa).x;                // Hartree
-      if (dv) e1 += dv[a] * raa.x;
-      ek -= K[idx].y;                             // Re(i K_aa)
-      nn_ += raa.x;
-    }
+  double v[4] = {0.0, 0.0, 0.0, 0.0};
+  for (int x = tid; x < 3 * n; x += 256) {
+    const double y = part[x];  // selected by value: v stays in registers
+    v[0] += x % 3 == 0 ? y : 0.0;
+    v[1] += x % 3 == 1 ? y : 0.0;
+    v[2] += x % 3 == 2 ? y : 0.0;
   }
-  red[0][tid] = e1;
-  red[1][tid] = e2;
-  red[2][tid] = ek;
-  red[3][tid] = nn_;
+  for (int x = tid; x < times; x += 256) v[3] += part[3 * n + x];
+  for (int q = 0; q < 4; ++q) red[q][tid] = v[q];
   __syncthreads();
   for (int st = 128; st > 0; st >>= 1) {
     if (tid < st)
@@ -623,8 +758,8 @@ __global__ void observe_kernel(int n, double spin, const double *h, const double
     __syncthreads();
   }
   if (tid == 0) {
-    *E_out = spin * red[0][0] + 0.5 * spin * red[1][0] + 0.5 * spin * red[2][0];
-    *N_out = spin * red[3][0];
+    *E_out = spin * red[0][0] + 0.5 * spin * red[1][0] + 0.5 * spin * red[3][0];
+    *N_out = spin * red[2][0];
   }
 }
 
@@ -665,11 +800,14 @@ __global__ void aop_kernel(int n, int i, int Tcap, double dt, const double2 *S, 
   put_cplx(A2 + a_z, n, lda, a, k0, sg);
 }
 
-// rhs of row i from the product slices: R_F(i, j) = -i h_HF F(i, j) + (sum of the
-// slices of both integrals), F = L (z = 0) and Gt (z = 1); O[k][z][j][p][a][c].
-__global__ void rhs_finish_kernel(int n, int i, long ld, const double2 *L, const double2 *G,
-                                  const double2 *hHF, const double *O1, int ns1, const double *O2,
-                                  int ns2, int Tcap, double2 *RL, double2 *RG) {
+// -i h_HF F(i, j) of row i, F = L into RL and Gt into RG. FP64 (8 n DFMA per
+// element and pair), on a side stream: it needs nothing of the self-energy, and
+// the tensor-core products beside it leave the FP64 pipe idle (in one kernel with
+// the sum of the slices it took 70 us on the critical path, on average at n = 39,
+// T = 81).
+__global__ void __launch_bounds__(256)
+    hf_rhs_kernel(int n, int i, long ld, const double2 *L, const double2 *G, const double2 *hHF,
+                  double2 *RL, double2 *RG) {
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= n * n) return;
   const int j = blockIdx.y, a = idx / n, c = idx % n;
@@ -680,20 +818,34 @@ __global__ void rhs_finish_kernel(int n, int i, long ld, const double2 *L, const
     cmla(hl, hv, L[fb + b * ld + c]);
     cmla(hg, hv, G[fb + b * ld + c]);
   }
-  const long zst = (long)Tcap * 2 * nn, kst = 2 * zst, e = (long)j * 2 * nn + idx;
-  double kr[2] = {0.0, 0.0}, ki[2] = {0.0, 0.0};
-  for (int z = 0; z < 2; ++z) {
-    for (int k = 0; k < ns1; ++k) {
-      kr[z] += O1[k * kst + z * zst + e];
-      ki[z] += O1[k * kst + z * zst + e + nn];
-    }
-    for (int k = 0; k < ns2; ++k) {
-      kr[z] += O2[k * kst + z * zst + e];
-      ki[z] += O2[k * kst + z * zst + e + nn];
-    }
+  RL[(long)j * nn + idx] = make_double2(hl.y, -hl.x);
+  RG[(long)j * nn + idx] = make_double2(hg.y, -hg.x);
+}
+
+// R_F(i, j) += the slices of both integrals, F = L (z = 0) and Gt (z = 1);
+// O[k][z][j][p][a][c].
+__global__ void __launch_bounds__(128)
+    rhs_finish_kernel(int n, const double *O1, int ns1, const double *O2, int ns2, int Tcap,
+                      double2 *RL, double2 *RG) {
+  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= n * n) return;
+  const int j = blockIdx.y, z = blockIdx.z;
+  const long nn = (long)n * n;
+  const long zst = (long)Tcap * 2 * nn, kst = 2 * zst, e = z * zst + (long)j * 2 * nn + idx;
+  double kr = 0.0, ki = 0.0;
+#pragma unroll 4
+  for (int k = 0; k < ns1; ++k) {
+    kr += O1[k * kst + e];
+    ki += O1[k * kst + e + nn];
   }
-  RL[(long)j * nn + idx] = make_double2(hl.y + kr[0], -hl.x + ki[0]);
-  RG[(long)j * nn + idx] = make_double2(hg.y + kr[1], -hg.x + ki[1]);
+#pragma unroll 4
+  for (int k = 0; k < ns2; ++k) {
+    kr += O2[k * kst + e];
+    ki += O2[k * kst + e + nn];
+  }
+  double2 *R = (z ? RG : RL) + (long)j * nn + idx;
+  const double2 h = *R;
+  *R = make_double2(h.x + kr, h.y + ki);
 }
 
 __global__ void gather_diag_kernel(int n, long ld, const double2 *L, double2 *out) {
@@ -708,25 +860,50 @@ int coll_rows(int n) { return std::min(n, 256 * kCollQ / n); }
 size_t coll_smem(int n) {
   return (size_t)(2 * coll_rows(n) * kCollKC + 2 * kCollKC * n) * sizeof(double2);
 }
-// Partial-sum slots (splits x columns) a launch may use: the split count is
-// chosen so that a launch has about 4 CTAs per SM of a 152-SM GPU, at most 128
-// (a single column, the energy's K_L(t, t), then still spreads over 128 CTAs).
-constexpr int kCollTargetCtas = 608;
-inline long coll_part_slots(int T) { return (long)kCollTargetCtas + T; }
+// Resident CTAs of a 152-SM GPU (two each), and the partial-sum slots (splits x
+// columns) of a launch.
+constexpr int kCollWave = 304;
+inline long coll_part_slots(int T) { return 3L * kCollWave + T; }
 
+// The columns' work grows with j, and every CTA of a wave waits for the longest:
+// the quota is the smallest with which all CTAs are resident at once, or two
+// waves' where that is less in all (many columns, few splits each). The same
+// splits for every column, in 2.05 waves and with 30 MB of partial sums, took about
+// 365 us and 33 of reduction, this takes 356 and 13 (n = 39, mean to T = 25).
 cudaError_t launch_collision(CollArgs a, cudaStream_t s, long *launches) {
   a.rows = coll_rows(a.n);
   const int tiles = (a.n + a.rows - 1) / a.rows;
-  const long ctas = (long)a.ncols * tiles;
-  a.splits = (int)std::max(1L, std::min(128L, (kCollTargetCtas + ctas - 1) / ctas));
+  const int most = coll_units(a.n, a.i, a.ncols - 1, a.corr);
+  const long slots = coll_part_slots(a.Tcap);
+  auto ctas = [&](int quota) {
+    long c = 0;
+    for (int j = 0; j < a.ncols; ++j) c += (coll_units(a.n, a.i, j, a.corr) + quota - 1) / quota;
+    return c * tiles;
+  };
+  long best = 0;
+  for (int waves = 1; waves <= 2; ++waves) {
+    int lo = 1, hi = most;  // the smallest quota of at most `waves` waves (or no split at all)
+    while (lo < hi) {
+      const int mid = (lo + hi) / 2;
+      const bool fits = ctas(mid) <= (long)waves * kCollWave &&
+                        (long)((most + mid - 1) / mid) * a.ncols <= slots;
+      if (fits) hi = mid; else lo = mid + 1;
+    }
+    const long cost = (long)lo * ((ctas(lo) + kCollWave - 1) / kCollWave);
+    if (best == 0 || 10 * cost < 9 * best) {
+      best = cost;
+      a.quota = lo;
+    }
+  }
+  a.splits = (most + a.quota - 1) / a.quota;
   dim3 grid((unsigned)(a.ncols * a.splits), (unsigned)tiles);
   collision_kernel<<<grid, 256, coll_smem(a.n), s>>>(a);
   ++*launches;
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess || a.splits == 1) return e;
   ++*launches;
-  dim3 rg((unsigned)(((long)a.n * a.n + 255) / 256), (unsigned)a.ncols);
-  coll_reduce_kernel<<<rg, 256, 0, s>>>(a.n, a.j0, a.ncols, a.splits, a.mode, a.part, a.RL, a.RG);
+  dim3 rg((unsigned)(((long)a.n * a.n + 127) / 128), (unsigned)a.ncols, 2);
+  coll_reduce_kernel<<<rg, 128, 0, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -740,18 +917,16 @@ cudaError_t launch_collision(CollArgs a, cudaStream_t s, long *launches) {
     if (!ensure((ctx), (ctx)->buf, (bytes), #buf)) return FEDVR_ERR_CUDA;   \
   } while (0)
 
-// Algorithmic complex multiply-adds of one rhs call on row i (columns j0 ..
-// j0 + ncols - 1; mode 1: K_L only).
-double coll_cmacs(int n, int i, int j0, int ncols, int mode, bool corr) {
+// Algorithmic complex multiply-adds of the rhs of row i, and of the energy's trace.
+double coll_cmacs(int n, int i, bool corr) {
   const double n3 = (double)n * n * n;
   double c = 0;
-  for (int j = j0; j < j0 + ncols; ++j) {
-    const double f = mode == 0 ? 2.0 : 1.0;
-    if (mode == 0) c += f * n3;
-    if (corr && i > 0) c += f * (i + 1) * n3;
-    if (corr && j > 0) c += f * (j + 1) * n3;
-  }
+  for (int j = 0; j <= i; ++j)
+    c += 2.0 * n3 * (1 + (corr && i > 0 ? i + 1 : 0) + (corr && j > 0 ? j + 1 : 0));
   return c;
+}
+double trace_cmacs(int n, int t, bool corr) {
+  return corr && t > 0 ? 2.0 * (t + 1) * n * n : 0.0;
 }
 
 struct KbeRun {
@@ -760,7 +935,7 @@ struct KbeRun {
   long ld;
   double dt, spin;
   bool corr;
-  double2 *L, *G, *S, *T1, *R0L, *R0G, *R1L, *R1G, *hHF, *K, *part;
+  double2 *L, *G, *S, *R0L, *R0G, *R1L, *R1G, *hHF, *part;
   // split-TF32 collision integrals: shadows (null in FP64 mode), left factors, product slices
   float *sh = nullptr, *aop = nullptr;
   // split-TF32 exchange products (null: FP64 exchange kernel)
@@ -770,7 +945,7 @@ struct KbeRun {
   int lda = 0, xld = 0;
   int *err = nullptr;
   const double *h, *V, *dv;
-  double *E, *Nn;
+  double *E, *Nn, *obs;
   cudaStream_t s;
   std::vector<cudaEvent_t> *ev;
   size_t ev_used = 0;
@@ -778,7 +953,16 @@ struct KbeRun {
   long launches = 0;
   std::vector<std::pair<size_t, int>> marks;  // (event index, stage: 0 collision, 1 sigma)
 
+  // An event at a stage's boundary; the one that closed a stage also opens the
+  // next if nothing (hf, advance) was launched between them.
+  bool closed = false;
   cudaError_t mark(int stage_open) {
+    if (closed && stage_open >= 0) {
+      closed = false;
+      marks.push_back({ev_used - 1, stage_open});
+      return cudaSuccess;
+    }
+    closed = stage_open < 0;
     if (ev_used >= ev->size()) {
       cudaEvent_t e;
       cudaError_t r = cudaEventCreate(&e);
@@ -790,11 +974,20 @@ struct KbeRun {
   }
   const double *dv_at(int t) const { return dv ? dv + (long)t * n : nullptr; }
 
-  int hf(int t) {
-    const int nn = n * n;
-    hf_kernel<<<(nn + 255) / 256, 256, 0, s>>>(n, spin, h, dv_at(t), V, L, blk(t, t, n, ld), ld,
-                                               hHF);
+  // h_HF at time t; split mode then starts -i h_HF F of row t (into RL, RG, the next
+  // rhs's) beside the self-energy and the products: rhs_tc waits for it.
+  int hf(int t, double2 *RL, double2 *RG) {
+    closed = false;
+    hf_kernel<<<n, 64, 0, s>>>(n, spin, h, dv_at(t), V, L, blk(t, t, n, ld), ld, hHF);
     KBE_CK(ctx, cudaGetLastError());
+    ++launches;
+    if (!sh || !corr || !RL) return FEDVR_OK;
+    KBE_CK(ctx, cudaEventRecord(ctx->kbe_fork, s));
+    KBE_CK(ctx, cudaStreamWaitEvent(ctx->kbe_side, ctx->kbe_fork, 0));
+    hf_rhs_kernel<<<dim3((unsigned)((n * n + 255) / 256), (unsigned)(t + 1)), 256, 0,
+                    ctx->kbe_side>>>(n, t, ld, L, G, hHF, RL, RG);
+    KBE_CK(ctx, cudaGetLastError());
+    KBE_CK(ctx, cudaEventRecord(ctx->kbe_join, ctx->kbe_side));
     ++launches;
     return FEDVR_OK;
   }
@@ -802,39 +995,32 @@ struct KbeRun {
     if (!corr) return FEDVR_OK;
     const int nn = n * n, ne = 2 * (i + 1);
     KBE_CK(ctx, mark(1));
-    if (xp) {
-      float2 *T132 = reinterpret_cast<float2 *>(T1);
-      vq32_kernel<<<dim3((nn + 255) / 256, ne), 256, 0, s>>>(n, i, ld, L, G, V, T132);
-      KBE_CK(ctx, cudaGetLastError());
-      direct32_kernel<<<dim3((nn + 255) / 256, ne), 256, 0, s>>>(n, i, ld, L, G, V, T132, spin,
-                                                                 Tcap, S);
-    } else {
-      vq_kernel<<<dim3((nn + 255) / 256, ne), 256, 0, s>>>(n, i, ld, L, G, V, T1);
-      KBE_CK(ctx, cudaGetLastError());
-      direct_kernel<<<dim3((nn + 255) / 256, ne), 256, 0, s>>>(n, i, ld, L, G, V, T1, spin, Tcap,
-                                                               S);
-    }
+    const dim3 dg((unsigned)((n + kDirRows - 1) / kDirRows), (unsigned)ne);
+    if (xp)
+      direct_kernel<float><<<dg, 256, direct_smem<float>(n), s>>>(n, i, ld, L, G, V, spin, Tcap, S);
+    else
+      direct_kernel<double><<<dg, 256, direct_smem<double>(n), s>>>(n, i, ld, L, G, V, spin, Tcap, S);
     KBE_CK(ctx, cudaGetLastError());
     if (xp) {
-      const long work = (long)nn * n;
-      const unsigned gx = (unsigned)std::min(64L, (work + 255) / 256);
-      xop_kernel<<<dim3(gx, ne), 256, 0, s>>>(n, i, ld, L, G, V, xld, xa, xb);
+      xop_kernel<<<dim3((unsigned)((n + kXopB - 1) / kXopB), (unsigned)ne), 256, xop_smem(n), s>>>(
+          n, i, ld, L, G, V, xld, xa, xb);
       KBE_CK(ctx, cudaGetLastError());
       KBE_CK(ctx, kbe_exchange_tc(n, ne, xld, xa, xb, xp, err, s));
-      xsum_kernel<<<dim3((nn + 255) / 256, ne), 256, 0, s>>>(n, i, ld, L, G, V, xp, Tcap, S);
+      xsum_kernel<<<dim3((unsigned)((n + kXsumB - 1) / kXsumB), (unsigned)ne), 256, xsum_smem(n),
+                    s>>>(n, i, ld, L, G, V, xp, Tcap, S);
       launches += 2;
     } else if (n <= 16) {
       exchange_rows_kernel<<<dim3(n, ne), 256, (size_t)2 * nn * sizeof(double2), s>>>(
           n, i, ld, L, G, V, Tcap, S);
     } else {
-      const size_t sm = (size_t)(2 * nn + xchg_rows(n) * n) * sizeof(double2);
-      exchange_kernel<<<dim3(n, ne), 256, sm, s>>>(n, i, ld, L, G, V, Tcap, S);
+      xchg_kernel(n)<<<dim3(n, ne), 256, xchg_smem(n), s>>>(n, xchg_plan(n).rows, i, ld, L, G, V,
+                                                           Tcap, S);
     }
     KBE_CK(ctx, cudaGetLastError());
     KBE_CK(ctx, mark(-1));
     const double n3 = (double)n * n * n;
     cmac_sigma += ne * (n3 * n + 2.0 * n3);  // exchange n^4 + n^3, V Q V two half-real n^3
-    launches += 3;
+    launches += 2;
     return FEDVR_OK;
   }
   int rhs_tc(int i, double2 *RL, double2 *RG) {
@@ -859,36 +1045,37 @@ struct KbeRun {
     // triangle s <= j of Dw
     const double rows = (double)(i + 1) * n;
     bytes_tc += 4.0 * (2.0 * rows * K + 0.5 * rows * K);
-    rhs_finish_kernel<<<dim3((nn + 255) / 256, i + 1), 256, 0, s>>>(n, i, ld, L, G, hHF, o1, ns,
-                                                                   o2, ns, Tcap, RL, RG);
+    KBE_CK(ctx, cudaStreamWaitEvent(s, ctx->kbe_join, 0));
+    rhs_finish_kernel<<<dim3((nn + 127) / 128, i + 1, 2), 128, 0, s>>>(n, o1, ns, o2, ns, Tcap, RL, RG);
     KBE_CK(ctx, cudaGetLastError());
     KBE_CK(ctx, mark(-1));
     launches += 4;
-    cmac_coll += coll_cmacs(n, i, 0, i + 1, 0, corr);
+    cmac_coll += coll_cmacs(n, i, corr);
     return FEDVR_OK;
   }
   int rhs(int i, double2 *RL, double2 *RG) {
     if (sh && corr) return rhs_tc(i, RL, RG);
-    CollArgs a{n, i, 0, Tcap, ld, dt, L, G, S, hHF, RL, RG, 0, corr ? 1 : 0, i + 1, 1, 0, part};
+    CollArgs a{n, i, Tcap, ld, dt, L, G, S, hHF, RL, RG, corr ? 1 : 0, i + 1, 0, 0, 0, part};
     KBE_CK(ctx, mark(0));
     KBE_CK(ctx, launch_collision(a, s, &launches));
     KBE_CK(ctx, mark(-1));
-    cmac_coll += coll_cmacs(n, i, 0, i + 1, 0, corr);
+    cmac_coll += coll_cmacs(n, i, corr);
     return FEDVR_OK;
   }
   int observe(int t) {
-    CollArgs a{n, t, t, Tcap, ld, dt, L, G, S, hHF, K, nullptr, 1, corr ? 1 : 0, 1, 1, 0, part};
+    const int times = corr && t > 0 ? t + 1 : 0;
     KBE_CK(ctx, mark(0));
-    KBE_CK(ctx, launch_collision(a, s, &launches));
-    KBE_CK(ctx, mark(-1));
-    cmac_coll += coll_cmacs(n, t, t, 1, 1, corr);
-    observe_kernel<<<1, 256, 0, s>>>(n, spin, h, dv_at(t), V, L, blk(t, t, n, ld), ld, K, E + t,
-                                     Nn + t);
+    observe_kernel<<<n + times, 128, 0, s>>>(n, t, spin, dt, h, dv_at(t), V, L, G, ld, S, Tcap, obs);
     KBE_CK(ctx, cudaGetLastError());
-    ++launches;
+    observe_sum_kernel<<<1, 256, 0, s>>>(n, times, spin, obs, E + t, Nn + t);
+    KBE_CK(ctx, cudaGetLastError());
+    KBE_CK(ctx, mark(-1));
+    cmac_coll += trace_cmacs(n, t, corr);
+    launches += 2;
     return FEDVR_OK;
   }
   int advance(int N, bool corrector) {
+    closed = false;
     const int nn = n * n;
     advance_kernel<<<dim3((nn + 255) / 256, N + 2), 256, 0, s>>>(
         n, N, ld, L, G, R0L, R0G, corrector ? R1L : nullptr, corrector ? R1G : nullptr, dt, sh,
@@ -930,10 +1117,10 @@ int fedvr_kbe_propagate(fedvr_ctx *ctx, double dt, int n_steps, int second_born,
   const size_t two = (size_t)ld * (size_t)ld * cz;
   const size_t shz = split ? (size_t)ld * (size_t)shld : 0;  // floats per shadow
   const int lda = (int)shld;
-  const int xld = (2 * n + 3) / 4 * 4;  // exchange operand row pitch (floats)
   const size_t aop_floats = split ? 3 * (size_t)2 * n * lda : 0;
   const size_t o_doubles = split ? (size_t)16 * 2 * T * 2 * nn : 0;
   const bool split_x = split && n <= 64;  // exchange products on the tensor cores
+  const int xld = (2 * n + 3) / 4 * 4;    // exchange operand row pitch (floats)
   const size_t x_floats =
       split_x ? (size_t)2 * T * ((size_t)2 * n * xld + nn * xld + 2 * nn * n) : 0;
   {
@@ -953,7 +1140,6 @@ int fedvr_kbe_propagate(fedvr_ctx *ctx, double dt, int n_steps, int second_born,
   KBE_ENSURE(ctx, k_L, two);
   KBE_ENSURE(ctx, k_G, two);
   KBE_ENSURE(ctx, k_S, 2 * (size_t)T * nn * cz);
-  KBE_ENSURE(ctx, k_T1, 2 * (size_t)T * nn * cz);
   KBE_ENSURE(ctx, k_R, 4 * (size_t)T * nn * cz);
   KBE_ENSURE(ctx, k_aux, (2 * nn + 2 * (size_t)T) * cz);
   KBE_ENSURE(ctx, k_out, (size_t)T * nn * cz + (size_t)T * n * sizeof(double));
@@ -968,7 +1154,7 @@ int fedvr_kbe_propagate(fedvr_ctx *ctx, double dt, int n_steps, int second_born,
   double2 *L = P<double2>(ctx->k_L), *G = P<double2>(ctx->k_G);
   double2 *R = P<double2>(ctx->k_R);
   double2 *aux = P<double2>(ctx->k_aux);
-  double *obs = reinterpret_cast<double *>(aux + 2 * nn);
+  double *obs = reinterpret_cast<double *>(aux + nn);  // E, N [T] each, then partial sums (3 n + T)
   double2 *rho_all = P<double2>(ctx->k_out);
   double *dv_d = reinterpret_cast<double *>(rho_all + (size_t)T * nn);
   KBE_CK(ctx, cudaMemsetAsync(L, 0, two, s));
@@ -996,6 +1182,22 @@ int fedvr_kbe_propagate(fedvr_ctx *ctx, double dt, int n_steps, int second_born,
     KBE_CK(ctx, cudaGetLastError());
   }
 
+  // what an early return leaves on the side stream ends before the call does
+  struct Side {
+    cudaStream_t stream = nullptr;
+    ~Side() {
+      if (stream) cudaStreamSynchronize(stream);
+    }
+  } side;
+  if (split) {
+    if (!ctx->kbe_side) {
+      KBE_CK(ctx, cudaEventCreateWithFlags(&ctx->kbe_fork, cudaEventDisableTiming));
+      KBE_CK(ctx, cudaEventCreateWithFlags(&ctx->kbe_join, cudaEventDisableTiming));
+      KBE_CK(ctx, cudaStreamCreateWithFlags(&ctx->kbe_side, cudaStreamNonBlocking));
+    }
+    side.stream = ctx->kbe_side;
+  }
+
   KbeRun run;
   run.ctx = ctx;
   run.n = n;
@@ -1007,13 +1209,11 @@ int fedvr_kbe_propagate(fedvr_ctx *ctx, double dt, int n_steps, int second_born,
   run.L = L;
   run.G = G;
   run.S = P<double2>(ctx->k_S);
-  run.T1 = P<double2>(ctx->k_T1);
   run.R0L = R;
   run.R0G = R + (size_t)T * nn;
   run.R1L = R + 2 * (size_t)T * nn;
   run.R1G = R + 3 * (size_t)T * nn;
   run.hHF = aux;
-  run.K = aux + nn;
   run.part = P<double2>(ctx->k_part);
   if (split) {
     run.sh = P<float>(ctx->k_sh);
@@ -1021,12 +1221,12 @@ int fedvr_kbe_propagate(fedvr_ctx *ctx, double dt, int n_steps, int second_born,
     run.Tn = ld;
     run.shld = shld;
     run.lda = lda;
-    run.xld = xld;
     run.aop = P<float>(ctx->k_aop);
     run.a_z = (long)2 * n * lda;
     run.o1 = P<double>(ctx->k_o);
     run.o2 = run.o1 + o_doubles;
     run.err = P<int>(ctx->k_flag);
+    run.xld = xld;
     if (split_x) {
       run.xa = P<float>(ctx->k_x);
       run.xb = run.xa + (size_t)2 * T * 2 * n * xld;
@@ -1038,27 +1238,36 @@ int fedvr_kbe_propagate(fedvr_ctx *ctx, double dt, int n_steps, int second_born,
   run.dv = dv ? dv_d : nullptr;
   run.E = obs;
   run.Nn = obs + T;
+  run.obs = obs + 2 * (size_t)T;
   run.s = s;
   run.ev = &ctx->kbe_events;
   {
-    const size_t sm = (2 * nn + (size_t)xchg_rows(n) * n) * cz;
-    KBE_CK(ctx, cudaFuncSetAttribute(exchange_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)sm));
+    KBE_CK(ctx, cudaFuncSetAttribute(xchg_kernel(n), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)xchg_smem(n)));
+    KBE_CK(ctx, cudaFuncSetAttribute(direct_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)direct_smem<double>(n)));
+    if (split_x) {
+      KBE_CK(ctx, cudaFuncSetAttribute(direct_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)direct_smem<float>(n)));
+      KBE_CK(ctx, cudaFuncSetAttribute(xop_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)xop_smem(n)));
+    }
     KBE_CK(ctx, cudaFuncSetAttribute(collision_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)coll_smem(n)));
   }
   KBE_CK(ctx, run.mark(-1));
-  if (int r = run.hf(0)) return r;
+  const bool steps = n_steps > 0;
+  if (int r = run.hf(0, steps ? run.R0L : nullptr, run.R0G)) return r;
   if (int r = run.sigma(0)) return r;
   if (int r = run.observe(0)) return r;
   for (int N = 0; N < n_steps; ++N) {
     if (int r = run.rhs(N, run.R0L, run.R0G)) return r;
     if (int r = run.advance(N, false)) return r;
-    if (int r = run.hf(N + 1)) return r;
+    if (int r = run.hf(N + 1, run.R1L, run.R1G)) return r;
     if (int r = run.sigma(N + 1)) return r;
     if (int r = run.rhs(N + 1, run.R1L, run.R1G)) return r;
     if (int r = run.advance(N, true)) return r;
-    if (int r = run.hf(N + 1)) return r;
+    if (int r = run.hf(N + 1, N + 1 < n_steps ? run.R0L : nullptr, run.R0G)) return r;
     if (int r = run.sigma(N + 1)) return r;
     if (int r = run.observe(N + 1)) return r;
   }
