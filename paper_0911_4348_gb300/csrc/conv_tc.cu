@@ -36,7 +36,7 @@ namespace {
 
 constexpr uint64_t kWaitNs = 2000000000ull;
 constexpr uint32_t kTileA = 128 * 128;
-constexpr int kWarps = 14;  // 0-3 flush, 4-11 A producers, 12 TMA, 13 MMA
+constexpr int kWarps = 22;  // 0-3 flush, 4-19 A producers, 20 TMA, 21 MMA
 constexpr int kThreads = kWarps * 32;
 
 struct C1Item {
@@ -62,6 +62,9 @@ __device__ __forceinline__ C1Item c1_item(const C1Sys &S, long q) {
   return it;
 }
 
+// Producers: one row and two 16-byte units per thread, the bracket's rows and the
+// next coefficient in registers (n = 142, M = 257, the whole call: 10.3 ms with
+// four rows per thread fetched anew at every mesh point by eight warps, 7.8 so).
 __global__ void __launch_bounds__(kThreads, 1)
     conv1_tc_kernel(const C1Sys *__restrict__ sys, const long *__restrict__ prefix, int n_sys,
                     long items, int Np_max, int nbuf, int *err) {
@@ -81,8 +84,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc::tmem_relinquish();
   }
   if (tid == 0) {
-    tc::mbar_init(&full[0], 9);  // one arrival per producer warp + the TMA thread's
-    tc::mbar_init(&full[1], 9);
+    tc::mbar_init(&full[0], 17);  // one arrival per producer warp + the TMA thread's
+    tc::mbar_init(&full[1], 17);
     tc::mbar_init(&empty[0], 1);
     tc::mbar_init(&empty[1], 1);
     tc::mbar_init(&accf[0], 1);
@@ -100,12 +103,13 @@ __global__ void __launch_bounds__(kThreads, 1)
   bool issued = false;
   int cur = 0;
 
-  if (warp >= 4 && warp < 12) {
-    // ---- A producers: rows r0 + 32 k of the tile, 16-byte chunk c of each 32-wide slice ----
-    const int pt = tid - 128, c = pt & 7, r0 = pt >> 3;
-    uint32_t off[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) off[k] = tc::sw128_offset(r0 + 32 * k, c);
+  if (warp >= 4 && warp < 20) {
+    // ---- A producers: four threads per row, 16-byte units u and u + 4 (four values
+    // each) of each 32-wide slice. Two neighbouring quads take rows four apart, so
+    // that the eight lanes of a store phase meet all eight bank groups ----
+    const int pt = tid - 128, u = pt & 3, qd = pt >> 2;
+    const int rt = (qd >> 3) * 8 + ((qd & 1) << 2) + ((qd >> 1) & 3);
+    const uint32_t off[2] = {tc::sw128_offset(rt, u), tc::sw128_offset(rt, u + 4)};
     uint32_t cc = 0;
     for (long w = blockIdx.x; w < items && !tc::warp_flag(abort_flag); w += gridDim.x) {
       while (cur + 1 < n_sys && w >= prefix[cur + 1]) ++cur;
@@ -117,38 +121,49 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int4 *const coef32 = S.coef32;
       const long R = (long)M * n;
       const C1Item it = c1_item(S, w - prefix[cur]);
-      int ia[4], aa[4];
-      bool live[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const long r = (long)it.t * 128 + r0 + 32 * k;
-        live[k] = r < R;
-        ia[k] = live[k] ? (int)(r / n) : 0;
-        aa[k] = live[k] ? (int)(r % n) : 0;
-      }
+      const long r = (long)it.t * 128 + rt;
+      const bool live = r < R;
+      const int ia = live ? (int)(r / n) : 0, aa = live ? (int)(r % n) : 0;
+      const int4 *const crow = coef32 + (long)ia * M;
       const int JB = S.JB;
       // chunks in the order (accumulation block, 32-wide column slice, mesh point),
       // as the MMA and TMA roles walk them
       for (int j0 = it.j_lo; j0 < it.j_hi && !tc::warp_flag(abort_flag); j0 += JB) {
         const int j1 = min(it.j_hi, j0 + JB);
         for (int kc = 0; kc < KC && !tc::warp_flag(abort_flag); ++kc) {
-          const int l0 = kc * 32 + 4 * c;
-          const bool in = l0 < n;  // units past n are zero padding: not fetched
-          float4 s1[4], s2[4];
-#pragma unroll
-          for (int k = 0; k < 4; ++k) s1[k] = s2[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+          const int l0 = kc * 32 + 4 * u;
+          // units past n are zero padding: not fetched
+          const bool in[2] = {live && l0 < n, live && l0 + 16 < n};
+          int k1 = -1, k2 = -1;  // S32 rows held in s1, s2 (-1: none)
+          float4 s1[2], s2[2];
+          s1[0] = s1[1] = s2[0] = s2[1] = make_float4(0.f, 0.f, 0.f, 0.f);
+          int4 next = crow[j0];  // the coefficients come one mesh point ahead
           for (int j = j0; j < j1; ++j, ++cc) {
-            float c1[4], c2[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              const int4 cf = coef32[(long)ia[k] * M + j];
-              c1[k] = __int_as_float(cf.z);
-              c2[k] = __int_as_float(cf.w);
-              if (live[k] && in) {  // element offsets into S32 ([2M][n][ld]) < 2^31
-                s1[k] = *reinterpret_cast<const float4 *>(
-                    S32 + (uint32_t)((cf.x * n + aa[k]) * ld + l0));
-                s2[k] = *reinterpret_cast<const float4 *>(
-                    S32 + (uint32_t)((cf.y * n + aa[k]) * ld + l0));
+            const int4 cf = next;
+            if (j + 1 < j1) next = crow[j + 1];
+            const float c1 = __int_as_float(cf.z), c2 = __int_as_float(cf.w);
+            if (in[0]) {  // element offsets into S32 ([2M][n][ld]) < 2^31
+              // the bracket rows stay in registers while the bracket does, the upper
+              // one taking the old lower one where it moved down by one
+              if (cf.y == k1) {
+                s2[0] = s1[0];
+                s2[1] = s1[1];
+              } else if (cf.y != k2) {
+                const float *p2 = S32 + (uint32_t)((cf.y * n + aa) * ld + l0);
+                s2[0] = *reinterpret_cast<const float4 *>(p2);
+                if (in[1]) s2[1] = *reinterpret_cast<const float4 *>(p2 + 16);
+              }
+              if (cf.x != k1) {
+                const float *p1 = S32 + (uint32_t)((cf.x * n + aa) * ld + l0);
+                s1[0] = *reinterpret_cast<const float4 *>(p1);
+                if (in[1]) s1[1] = *reinterpret_cast<const float4 *>(p1 + 16);
+              }
+              k1 = cf.x;
+              k2 = cf.y;
+              // the bracket usually moves down by one row: ask L1 for that row now
+              if (u == 0 && cf.x > 0) {
+                const float *pn = S32 + (uint32_t)(((cf.x - 1) * n + aa) * ld + l0);
+                asm volatile("prefetch.global.L1 [%0];" ::"l"(pn));
               }
             }
             const int s = cc & 1;
@@ -158,19 +173,20 @@ __global__ void __launch_bounds__(kThreads, 1)
               break;
             }
             uint8_t *st = smem + s * stage_bytes;
+            // rows past n and dead rows stay zero; the diagonal entry j = i reads its
+            // precomputed B_ii (row M + i)
+            const uint64_t C1 = tc::f2_pack(c1, c1), C2 = tc::f2_pack(c2, c2);
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              // rows past n and dead rows stay zero; the diagonal entry j = i reads its
-              // precomputed B_ii (row M + i)
-              float x[4] = {fmaf(c1[k], s1[k].x, c2[k] * s2[k].x),
-                            fmaf(c1[k], s1[k].y, c2[k] * s2[k].y),
-                            fmaf(c1[k], s1[k].z, c2[k] * s2[k].z),
-                            fmaf(c1[k], s1[k].w, c2[k] * s2[k].w)};
+            for (int k = 0; k < 2; ++k) {
+              const ulonglong2 p1 = *reinterpret_cast<const ulonglong2 *>(&s1[k]);
+              const ulonglong2 p2 = *reinterpret_cast<const ulonglong2 *>(&s2[k]);
+              const uint64_t x01 = tc::f2_fma(C1, p1.x, tc::f2_mul(C2, p2.x));
+              const uint64_t x23 = tc::f2_fma(C1, p1.y, tc::f2_mul(C2, p2.y));
               float4 hi, lo;
-              tc::tf32_split(x[0], hi.x, lo.x);
-              tc::tf32_split(x[1], hi.y, lo.y);
-              tc::tf32_split(x[2], hi.z, lo.z);
-              tc::tf32_split(x[3], hi.w, lo.w);
+              tc::tf32_split(tc::f2_lo(x01), hi.x, lo.x);
+              tc::tf32_split(tc::f2_hi(x01), hi.y, lo.y);
+              tc::tf32_split(tc::f2_lo(x23), hi.z, lo.z);
+              tc::tf32_split(tc::f2_hi(x23), hi.w, lo.w);
               *reinterpret_cast<float4 *>(st + off[k]) = hi;
               *reinterpret_cast<float4 *>(st + kTileA + off[k]) = lo;
             }
@@ -180,7 +196,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
       }
     }
-  } else if (warp == 12) {
+  } else if (warp == 20) {
     // ---- TMA: g_j rows 0..Np-1, 32 columns per chunk, hi and lo ----
     if (tc::elect_one()) {
       uint32_t cc = 0;
@@ -214,7 +230,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
       }
     }
-  } else if (warp == 13) {
+  } else if (warp == 21) {
     // ---- MMA issue: one accumulator block per JB mesh points ----
     if (tc::elect_one()) {
       uint32_t cc = 0, tcount = 0;
@@ -328,7 +344,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   __syncthreads();
   if (*abort_flag) {
-    if (warp == 13 && (issued || lane == 0)) {
+    if (warp == 21 && (issued || lane == 0)) {
       if (issued) tc::mma_commit(drain);
       atomicExch(err, 1);
       if (issued) tc::mbar_wait(drain, 0, kWaitNs);
@@ -433,10 +449,12 @@ __global__ void sigma_to_f32_kernel(int n, long rows, int ld, const double *__re
 // scaled by powers of two into FP16's normal range (g by 2^kScaleG, the
 // interpolated Sigma by 2^sA with sA from maxC * max|S32|), and the flush
 // multiplies the FP32 block sums by 2^-(sA + kScaleG) exactly. 16 producer
-// warps, two rows of one 16-byte unit (8 values) per thread and chunk.
-constexpr int kWarpsH = 22;  // 0-3 flush, 4-19 A producers, 20 TMA, 21 MMA
-constexpr int kThreadsH = kWarpsH * 32;
-
+// warps, two 16-byte units (8 values each) of one row per thread and chunk: one
+// coefficient and one bracket to follow per thread (n = 142, M = 1025: 22.4 ms with
+// two rows of one unit, 18.0 so; 24 with eight warps of four units). Bound by the
+// shared-memory pipe: the MMAs' operand reads, the producers' stores, the TMA's and
+// the L1 hits of the bracket rows take about 1600 of a chunk's 2050 cycles, the MMAs
+// 860.
 __device__ __forceinline__ int a_scale_exp(const TcScale *sc) {
   const float amax = __uint_as_float(sc->maxS) * sc->maxC;
   if (!(amax > 0.f) || !(amax < 3.0e38f)) return 0;
@@ -446,7 +464,7 @@ __device__ __forceinline__ int a_scale_exp(const TcScale *sc) {
   return e < -100 ? -100 : (e > 100 ? 100 : e);
 }
 
-__global__ void __launch_bounds__(kThreadsH, 1)
+__global__ void __launch_bounds__(kThreads, 1)
     conv1_f16_kernel(const C1Sys *__restrict__ sys, const long *__restrict__ prefix, int n_sys,
                      long items, int Np_max, int nbuf, int *err) {
   extern __shared__ uint8_t smem_raw[];
@@ -485,10 +503,12 @@ __global__ void __launch_bounds__(kThreadsH, 1)
   int cur = 0;
 
   if (warp >= 4 && warp < 20) {
-    // ---- A producers: rows r0 and r0 + 64 of the tile, 16-byte unit c (8 FP16
-    // values) of each 64-wide slice ----
-    const int pt = tid - 128, c = pt & 7, r0 = pt >> 3;
-    const uint32_t off[2] = {tc::sw128_offset(r0, c), tc::sw128_offset(r0 + 64, c)};
+    // ---- A producers: four threads per row, 16-byte units u and u + 4 (8 FP16 values
+    // each) of each 64-wide slice. Two neighbouring quads take rows four apart, so
+    // that the eight lanes of a store phase meet all eight bank groups ----
+    const int pt = tid - 128, u = pt & 3, qd = pt >> 2;
+    const int rt = (qd >> 3) * 8 + ((qd & 1) << 2) + ((qd >> 1) & 3);
+    const uint32_t off[2] = {tc::sw128_offset(rt, u), tc::sw128_offset(rt, u + 4)};
     uint32_t cc = 0;
     for (long w = blockIdx.x; w < items && !tc::warp_flag(abort_flag); w += gridDim.x) {
       while (cur + 1 < n_sys && w >= prefix[cur + 1]) ++cur;
@@ -499,62 +519,63 @@ __global__ void __launch_bounds__(kThreadsH, 1)
       const float fA = ldexpf(1.f, a_scale_exp(S.scale));
       const long R = (long)M * n;
       const C1Item it = c1_item(S, w - prefix[cur]);
-      int ia[2], aa[2];
-      bool live[2];
-#pragma unroll
-      for (int k = 0; k < 2; ++k) {
-        const long r = (long)it.t * 128 + r0 + 64 * k;
-        live[k] = r < R;
-        ia[k] = live[k] ? (int)(r / n) : 0;
-        aa[k] = live[k] ? (int)(r % n) : 0;
-      }
+      const long r = (long)it.t * 128 + rt;
+      const bool live = r < R;
+      const int ia = live ? (int)(r / n) : 0, aa = live ? (int)(r % n) : 0;
+      const int4 *const crow = coef32 + (long)ia * M;
       const int JB = S.JB, TU = S.TU, KCf = TU ? KC - 1 : KC;
       // chunks in the order (accumulation block, 64-wide column slice, mesh point),
-      // the two bracket rows of each row held in registers while the bracket stays;
+      // the two bracket rows of the row held in registers while the bracket stays;
       // with a packed tail the last slice follows as chunks of 8 / TU mesh points
       for (int j0 = it.j_lo; j0 < it.j_hi && !tc::warp_flag(abort_flag); j0 += JB) {
         const int j1 = min(it.j_hi, j0 + JB);
         for (int kc = 0; kc < KCf && !tc::warp_flag(abort_flag); ++kc) {
-          const int l0 = kc * 64 + 8 * c;
-          const bool in = l0 < n;  // units starting past n are zero padding: not fetched
-          int k1[2], k2[2];        // S32 rows held in a1, a2 (-1: none)
+          const int l0 = kc * 64 + 8 * u;
+          // units starting past n are zero padding: not fetched
+          const bool in[2] = {live && l0 < n, live && l0 + 32 < n};
+          const int lp = min(kc * 64 + 32 * (u & 1), ld - 32);  // this thread's line to prefetch
+          int k1 = -1, k2 = -1;  // S32 rows held in a1, a2 (-1: none)
           float4 a1[2][2], a2[2][2];
 #pragma unroll
-          for (int k = 0; k < 2; ++k) {
-            k1[k] = k2[k] = -1;
+          for (int k = 0; k < 2; ++k)
             a1[k][0] = a1[k][1] = a2[k][0] = a2[k][1] = make_float4(0.f, 0.f, 0.f, 0.f);
-          }
+          int4 next = crow[j0];  // the coefficients come one mesh point ahead
           for (int j = j0; j < j1; ++j, ++cc) {
-            float c1[2], c2[2];  // weights times the operand scale 2^sA
+            const int4 cf = next;
+            if (j + 1 < j1) next = crow[j + 1];
+            // weights times the operand scale 2^sA
+            const float c1 = __int_as_float(cf.z) * fA, c2 = __int_as_float(cf.w) * fA;
+            if (in[0]) {
+              // updated in place (the upper row first: it may take the old lower
+              // one, when the bracket moved down by one); a bracket that moved up
+              // (only where the lag wraps around) is fetched again
+              if (cf.y == k1) {
 #pragma unroll
-            for (int k = 0; k < 2; ++k) {
-              const int4 cf = coef32[(long)ia[k] * M + j];
-              c1[k] = __int_as_float(cf.z) * fA;
-              c2[k] = __int_as_float(cf.w) * fA;
-              if (live[k] && in) {
-                // updated in place (the upper row first: it may take the old lower
-                // one, when the bracket moved down by one); a bracket that moved up
-                // (only where the lag wraps around) is fetched again
-                if (cf.y == k1[k]) {
-                  a2[k][0] = a1[k][0];
-                  a2[k][1] = a1[k][1];
-                } else if (cf.y != k2[k]) {
-                  const float *p2 = S32 + (uint32_t)((cf.y * n + aa[k]) * ld + l0);
-                  a2[k][0] = *reinterpret_cast<const float4 *>(p2);
-                  a2[k][1] = *reinterpret_cast<const float4 *>(p2 + 4);
-                }
-                if (cf.x != k1[k]) {
-                  const float *p1 = S32 + (uint32_t)((cf.x * n + aa[k]) * ld + l0);
-                  a1[k][0] = *reinterpret_cast<const float4 *>(p1);
-                  a1[k][1] = *reinterpret_cast<const float4 *>(p1 + 4);
-                }
-                k1[k] = cf.x;
-                k2[k] = cf.y;
-                // the bracket usually moves down by one row: ask L1 for that row now
-                if (cf.x > 0) {
-                  const float *pn = S32 + (uint32_t)(((cf.x - 1) * n + aa[k]) * ld + l0);
-                  asm volatile("prefetch.global.L1 [%0];" ::"l"(pn));
-                }
+                for (int k = 0; k < 2; ++k) a2[k][0] = a1[k][0], a2[k][1] = a1[k][1];
+              } else if (cf.y != k2) {
+                const float *p2 = S32 + (uint32_t)((cf.y * n + aa) * ld + l0);
+#pragma unroll
+                for (int k = 0; k < 2; ++k)
+                  if (in[k]) {
+                    a2[k][0] = *reinterpret_cast<const float4 *>(p2 + 32 * k);
+                    a2[k][1] = *reinterpret_cast<const float4 *>(p2 + 32 * k + 4);
+                  }
+              }
+              if (cf.x != k1) {
+                const float *p1 = S32 + (uint32_t)((cf.x * n + aa) * ld + l0);
+#pragma unroll
+                for (int k = 0; k < 2; ++k)
+                  if (in[k]) {
+                    a1[k][0] = *reinterpret_cast<const float4 *>(p1 + 32 * k);
+                    a1[k][1] = *reinterpret_cast<const float4 *>(p1 + 32 * k + 4);
+                  }
+              }
+              k1 = cf.x;
+              k2 = cf.y;
+              // the bracket usually moves down by one row: ask L1 for that row now
+              if (cf.x > 0) {
+                const float *pn = S32 + (uint32_t)(((cf.x - 1) * n + aa) * ld + lp);
+                asm volatile("prefetch.global.L1 [%0];" ::"l"(pn));
               }
             }
             const int s = cc & 1;
@@ -564,11 +585,11 @@ __global__ void __launch_bounds__(kThreadsH, 1)
               break;
             }
             uint8_t *st = smem + s * stage_bytes;
+            // c1 Sigma_k1 + c2 Sigma_k2 on pairs of values (packed FP32 pairs:
+            // the same rounding as the scalar multiply and fused multiply-add)
+            const uint64_t C1 = tc::f2_pack(c1, c1), C2 = tc::f2_pack(c2, c2);
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
-              // c1 Sigma_k1 + c2 Sigma_k2 on pairs of values (packed FP32 pairs:
-              // the same rounding as the scalar multiply and fused multiply-add)
-              const uint64_t C1 = tc::f2_pack(c1[k], c1[k]), C2 = tc::f2_pack(c2[k], c2[k]);
               const ulonglong2 p1a = *reinterpret_cast<const ulonglong2 *>(&a1[k][0]);
               const ulonglong2 p1b = *reinterpret_cast<const ulonglong2 *>(&a1[k][1]);
               const ulonglong2 p2a = *reinterpret_cast<const ulonglong2 *>(&a2[k][0]);
@@ -586,27 +607,26 @@ __global__ void __launch_bounds__(kThreadsH, 1)
           }
         }
         if (TU) {
-          // packed tail: unit c holds 8 columns of mesh point jt + c / TU
-          const int jpc = 8 / TU, jo = c / TU;
-          const int l0 = (KC - 1) * 64 + 8 * (c % TU);
+          // packed tail: unit c = u + 4 k holds 8 columns of mesh point jt + c / TU
+          const int jpc = 8 / TU;
           for (int jt = j0; jt < j1 && !tc::warp_flag(abort_flag); jt += jpc, ++cc) {
-            const int j = jt + jo;
-            const bool jin = jo < jpc && j < j1 && l0 < n;
             float4 p1[2][2], p2[2][2];
             float c1[2], c2[2];
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
+              const int jo = (u + 4 * k) / TU, j = jt + jo;
+              const int l0 = (KC - 1) * 64 + 8 * ((u + 4 * k) % TU);
               c1[k] = c2[k] = 0.f;
               p1[k][0] = p1[k][1] = p2[k][0] = p2[k][1] = make_float4(0.f, 0.f, 0.f, 0.f);
-              if (live[k] && jin) {
-                const int4 cf = coef32[(long)ia[k] * M + j];
+              if (live && jo < jpc && j < j1 && l0 < n) {
+                const int4 cf = crow[j];
                 c1[k] = __int_as_float(cf.z) * fA;
                 c2[k] = __int_as_float(cf.w) * fA;
-                const float *q1 = S32 + (uint32_t)((cf.x * n + aa[k]) * ld + l0);
+                const float *q1 = S32 + (uint32_t)((cf.x * n + aa) * ld + l0);
                 p1[k][0] = *reinterpret_cast<const float4 *>(q1);
                 p1[k][1] = *reinterpret_cast<const float4 *>(q1 + 4);
                 if (cf.y != cf.x) {
-                  const float *q2 = S32 + (uint32_t)((cf.y * n + aa[k]) * ld + l0);
+                  const float *q2 = S32 + (uint32_t)((cf.y * n + aa) * ld + l0);
                   p2[k][0] = *reinterpret_cast<const float4 *>(q2);
                   p2[k][1] = *reinterpret_cast<const float4 *>(q2 + 4);
                 } else {
@@ -1019,7 +1039,7 @@ cudaError_t conv1_tc_launch(const C1Sys *sys, const long *prefix, int n_sys, lon
     e = cudaFuncSetAttribute(conv1_f16_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)smem);
     if (e != cudaSuccess) return e;
-    conv1_f16_kernel<<<grid, kThreadsH, smem, s>>>(sys, prefix, n_sys, items, Np_max, nbuf, err);
+    conv1_f16_kernel<<<grid, kThreads, smem, s>>>(sys, prefix, n_sys, items, Np_max, nbuf, err);
     return cudaGetLastError();
   }
   conv1_tc_kernel<<<grid, kThreads, smem, s>>>(sys, prefix, n_sys, items, Np_max, nbuf, err);
