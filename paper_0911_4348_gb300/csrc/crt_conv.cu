@@ -613,7 +613,8 @@ __global__ void __launch_bounds__(kThreads, 1) crt_conv_kernel(const __grid_cons
 #pragma unroll
           for (int t = 0; t < 16; ++t) v[t] = modf_bal(v[t], pm, ipm);
           if (!last) {
-            tmem_st16(tb + (uint32_t)b * 16, v);
+            tc::tmem_st16(tb + (uint32_t)b * 16, v);
+            tc::tmem_wait_st();
           } else if (row < (long)p.k.M * p.k.n) {
             uint32_t o[4];
 #pragma unroll

@@ -83,8 +83,14 @@ __global__ void split_kernel(int n, long rows, int ld, const double *__restrict_
 // shared memory (pitch stg floats, stg = 4 mod 32, so that the eight values
 // of a read by a quarter-warp fall into distinct banks and the values of b
 // are broadcasts), double-buffered by tile parity and handed over with the
-// bounded sfull barrier; with stg = 0 (shared memory too small for large n)
-// each lane reads its rows from global memory.
+// bounded sfull barrier. With stg = 0 (no room beside the stages, n > 224) each
+// epilogue warp fetches its 8 rows of V and 4 of g into registers, spread over the
+// lanes, while the tile still multiplies, and deals them out 16 columns at a time
+// through a small buffer of its own. For n > 256 there is one accumulator and the
+// next tile's MMAs wait for this pass: the products V_ak g_kb of all but three
+// chunks are then dealt out ahead too, into the TMEM columns beside it. n = 299, M =
+// 1025: 34.5 ms with each lane reading its rows as it went, mostly from L2; 26.6
+// with five chunks in flight and spilled registers; 21.6 so.
 //
 // FP16 variant: 128-byte operand rows hold 64 FP16 values, so a chunk covers
 // 64 contraction terms and the three products run as kind::f16 at twice the
@@ -101,6 +107,10 @@ struct XRoles {
 
 // Bytes after the stages: barriers (256) and the column-half buffer (2 x 128 floats).
 constexpr uint32_t kXBarBytes = 256, kXPartBytes = 2 * 128 * 4;
+// stg = 0: an epilogue warp's buffer (8 rows of V at pitch 20, 4 rows of g, 16
+// columns), the 16-column chunks in flight, those whose products V g wait in TMEM,
+// and the most there are (n <= 320).
+constexpr int kXDeal = 8 * 20 + 4 * 16, kXAhead = 3, kXTmem = 7, kXChunks = 10;
 
 // Exponent eX of the FP16 A operand g V: max|V| < 2^e, |g| < 16.
 __device__ __forceinline__ int x_scale_exp(const TcScale *sc) {
@@ -125,7 +135,7 @@ __device__ __forceinline__ XTile x_tile(const XSys &S, long q) {
   return x;
 }
 
-template <bool F16>
+template <bool F16, bool DEAL>  // DEAL: stg = 0
 __global__ void __launch_bounds__(XRoles<F16>::kThreads, 1)
     exchange_tc_kernel(const XSys *__restrict__ sys, const long *__restrict__ prefix, int n_sys,
                        long items, int Np_max, int nbuf, int stg, int *err) {
@@ -188,31 +198,28 @@ __global__ void __launch_bounds__(XRoles<F16>::kThreads, 1)
       const float *const V32 = S.V32;  // in a register across the memory-clobbering asm
       const float fX = F16 ? ldexpf(1.f, x_scale_exp(S.scale)) : 1.f;
       const int u = F16 ? 8 * c : 4 * c;  // first column of this thread's unit in a chunk
-      uint32_t og[4], ov[4];  // element offsets of row a of g_j and row b of V
-      bool live[4];
+      // the four rows share a; their b are four apart
+      const int a = xt.a0 + (r0 & 7), b = xt.b0 + (r0 >> 3);
+      const float *const ga = gA + a * ld + u, *const vb = V32 + b * ld + u;
+      bool live[4];  // rows a < b of a diagonal block: computed as zeros
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int r = r0 + 32 * k;
-        const int b = xt.b0 + (r >> 3), a = xt.a0 + (r & 7);
-        live[k] = a < n && b <= a;  // rows a < b of a diagonal block: computed as zeros
-        og[k] = live[k] ? (uint32_t)(a * ld + u) : 0u;
-        ov[k] = live[k] ? (uint32_t)(b * ld + u) : 0u;
-      }
+      for (int k = 0; k < 4; ++k) live[k] = a < n && b + 4 * k <= a;
       for (int kc = 0; kc < KC; ++kc, ++cc) {
         const int l0 = kc * R::kCols;
         const bool in = l0 + u < n;  // units past n are zero padding: not fetched
-        float4 gv[4][F16 ? 2 : 1], vv[4][F16 ? 2 : 1];
+        constexpr int H = F16 ? 2 : 1;
+        float4 gv[H], vv[4][H];
+#pragma unroll
+        for (int h = 0; h < H; ++h)
+          gv[h] = live[0] && in ? *reinterpret_cast<const float4 *>(ga + l0 + 4 * h)
+                                : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
 #pragma unroll
-          for (int h = 0; h < (F16 ? 2 : 1); ++h) {
-            if (live[k] && in) {
-              gv[k][h] = *reinterpret_cast<const float4 *>(gA + og[k] + l0 + 4 * h);
-              vv[k][h] = *reinterpret_cast<const float4 *>(V32 + ov[k] + l0 + 4 * h);
-            } else {
-              gv[k][h] = vv[k][h] = make_float4(0.f, 0.f, 0.f, 0.f);
-            }
-          }
+          for (int h = 0; h < H; ++h)
+            vv[k][h] = live[k] && in
+                           ? *reinterpret_cast<const float4 *>(vb + 4 * k * ld + l0 + 4 * h)
+                           : make_float4(0.f, 0.f, 0.f, 0.f);
         }
         const int s = cc & 1;
         const uint32_t use = cc >> 1;
@@ -228,20 +235,20 @@ __global__ void __launch_bounds__(XRoles<F16>::kThreads, 1)
             // (g_al V_bl) 2^eX on pairs of values (packed FP32 pairs, the rounding
             // of the scalar products)
             const uint64_t FX = tc::f2_pack(fX, fX);
-            const ulonglong2 ga = *reinterpret_cast<const ulonglong2 *>(&gv[k][0]);
-            const ulonglong2 gb = *reinterpret_cast<const ulonglong2 *>(&gv[k][1]);
-            const ulonglong2 va = *reinterpret_cast<const ulonglong2 *>(&vv[k][0]);
-            const ulonglong2 vb = *reinterpret_cast<const ulonglong2 *>(&vv[k][1]);
+            const ulonglong2 g0 = *reinterpret_cast<const ulonglong2 *>(&gv[0]);
+            const ulonglong2 g1 = *reinterpret_cast<const ulonglong2 *>(&gv[H - 1]);
+            const ulonglong2 v0 = *reinterpret_cast<const ulonglong2 *>(&vv[k][0]);
+            const ulonglong2 v1 = *reinterpret_cast<const ulonglong2 *>(&vv[k][H - 1]);
             uint4 hi, lo;
-            tc::f16_split2p(tc::f2_mul(tc::f2_mul(ga.x, va.x), FX), hi.x, lo.x);
-            tc::f16_split2p(tc::f2_mul(tc::f2_mul(ga.y, va.y), FX), hi.y, lo.y);
-            tc::f16_split2p(tc::f2_mul(tc::f2_mul(gb.x, vb.x), FX), hi.z, lo.z);
-            tc::f16_split2p(tc::f2_mul(tc::f2_mul(gb.y, vb.y), FX), hi.w, lo.w);
+            tc::f16_split2p(tc::f2_mul(tc::f2_mul(g0.x, v0.x), FX), hi.x, lo.x);
+            tc::f16_split2p(tc::f2_mul(tc::f2_mul(g0.y, v0.y), FX), hi.y, lo.y);
+            tc::f16_split2p(tc::f2_mul(tc::f2_mul(g1.x, v1.x), FX), hi.z, lo.z);
+            tc::f16_split2p(tc::f2_mul(tc::f2_mul(g1.y, v1.y), FX), hi.w, lo.w);
             *reinterpret_cast<uint4 *>(st + off) = hi;
             *reinterpret_cast<uint4 *>(st + kTileA + off) = lo;
           } else {
-            const float x0 = gv[k][0].x * vv[k][0].x, x1 = gv[k][0].y * vv[k][0].y,
-                        x2 = gv[k][0].z * vv[k][0].z, x3 = gv[k][0].w * vv[k][0].w;
+            const float x0 = gv[0].x * vv[k][0].x, x1 = gv[0].y * vv[k][0].y,
+                        x2 = gv[0].z * vv[k][0].z, x3 = gv[0].w * vv[k][0].w;
             float4 hi, lo;
             tc::tf32_split(x0, hi.x, lo.x);
             tc::tf32_split(x1, hi.y, lo.y);
@@ -374,9 +381,35 @@ __global__ void __launch_bounds__(XRoles<F16>::kThreads, 1)
       const int cb = half ? hc : 0, ce = half ? NC : hc;
       const int buf = tcount & 1;
       const uint32_t tu = tcount >> 1;
-      // row a of V (V_ak = V_ka) and row b of g (g_kb = g_bk): staged or global
-      const float *Va, *gb_row;
-      if (stg > 0) {
+      // row a of V (V_ak = V_ka) and row b of g (g_kb = g_bk): staged or dealt out
+      const float *Va = nullptr, *gb_row = nullptr;
+      const int vrow = xt.a0 + (lane >> 2), grow = xt.b0 + 4 * quarter + (lane >> 3);
+      float4 vd[kXAhead];
+      float2 gd[kXAhead];
+      const auto fetch = [&](int x, int ch) {  // chunk ch into slot x
+        if (ch >= ce) return;
+        vd[x] = vrow < n ? *reinterpret_cast<const float4 *>(S.V32 + (long)vrow * ld + ch * 16 +
+                                                             4 * (lane & 3))
+                         : make_float4(0.f, 0.f, 0.f, 0.f);
+        gd[x] = grow < n ? *reinterpret_cast<const float2 *>(gA + (long)grow * ld + ch * 16 +
+                                                             2 * (lane & 7))
+                         : make_float2(0.f, 0.f);
+      };
+      // DEAL: chunk in slot x to the warp's buffer (deal_v, deal_g: this lane's rows of
+      // it), chunk ch on its way into the slot
+      float *const deal = stage_rows + warp * kXDeal;
+      const float *const deal_v = deal + al * 20, *const deal_g = deal + 160 + (lane >> 3) * 16;
+      const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16);
+      const uint32_t mrow = trow + (uint32_t)(S.g.Np + half * 16 * kXTmem);
+      // chunks of this half whose products wait in TMEM
+      const int nt = nbuf == 1 ? min(kXTmem, ce - cb - kXAhead) : 0;
+      const auto deal_out = [&](int x, int ch) {
+        *reinterpret_cast<float4 *>(deal + (lane >> 2) * 20 + 4 * (lane & 3)) = vd[x];
+        *reinterpret_cast<float2 *>(deal + 160 + (lane >> 3) * 16 + 2 * (lane & 7)) = gd[x];
+        fetch(x, ch);
+        __syncwarp();
+      };
+      if constexpr (!DEAL) {
         float *sb = stage_rows + (size_t)buf * 24 * stg;
         for (int rr = warp; rr < 24; rr += R::kEpi) {  // rows >= n copy as zeros
           const int src_row = rr < 8 ? xt.a0 + rr : xt.b0 + rr - 8;
@@ -395,36 +428,85 @@ __global__ void __launch_bounds__(XRoles<F16>::kThreads, 1)
         Va = sb + al * stg;
         gb_row = sb + (8 + bl) * stg;
       } else {
-        Va = S.V32 + (long)(live ? a : 0) * ld;
-        gb_row = gA + (long)(live ? b : 0) * ld;
+#pragma unroll
+        for (int x = 0; x < kXAhead; ++x) fetch(x, cb + x);
+        if (nbuf == 1) {
+#pragma unroll
+          for (int x = 0; x < kXTmem; ++x) {
+            if (x < nt) {
+              float m[16];
+              deal_out(x % kXAhead, cb + x + kXAhead);
+#pragma unroll
+              for (int t4 = 0; t4 < 4; ++t4) {
+                const float4 v = *reinterpret_cast<const float4 *>(deal_v + 4 * t4);
+                const float4 y = *reinterpret_cast<const float4 *>(deal_g + 4 * t4);
+                m[4 * t4] = v.x * y.x;
+                m[4 * t4 + 1] = v.y * y.y;
+                m[4 * t4 + 2] = v.z * y.z;
+                m[4 * t4 + 3] = v.w * y.w;
+              }
+              __syncwarp();
+              tc::tmem_st16(mrow + (uint32_t)(16 * x), m);
+            }
+          }
+          tc::tmem_wait_st();
+        }
+      }
+      float gab = 0.f, wab = 0.f;  // of the direct term, wanted at the end
+      if (half == 0 && live) {
+        gab = gA[(long)a * ld + b];
+        wab = S.W[((long)xt.j * n + b) * ld + a];
       }
       if (!tc::warp_wait(&accf[buf], tu & 1, kWaitNs)) {
         *abort_flag = 1;
         break;
       }
       tc::fence_after_sync();
-      const uint32_t tbase = tmem + (nbuf == 2 ? (uint32_t)(buf * 256) : 0u);
+      const uint32_t prow_t = trow + (nbuf == 2 ? (uint32_t)(buf * 256) : 0u);
       float acc0 = 0.f, acc1 = 0.f;
-      for (int ch = cb; ch < ce; ++ch) {
-        // the chunk's operands are requested before the TMEM read, so the two
-        // latencies overlap
+      // rows are zero beyond n, so padded columns add nothing
+      const auto fold = [&](const float *vp, const float *gp, int ch) {
+        uint32_t pv[16];
+        tc::tmem_ld16_async(prow_t + (uint32_t)(ch * 16), pv);
+        // the chunk's operands are read beside the TMEM read
         float4 vc[4], gc[4];
 #pragma unroll
         for (int t4 = 0; t4 < 4; ++t4) {
-          vc[t4] = (live || stg > 0) ? *reinterpret_cast<const float4 *>(Va + ch * 16 + 4 * t4)
-                                     : make_float4(0.f, 0.f, 0.f, 0.f);
-          gc[t4] = (live || stg > 0) ? *reinterpret_cast<const float4 *>(gb_row + ch * 16 + 4 * t4)
-                                     : make_float4(0.f, 0.f, 0.f, 0.f);
+          vc[t4] = *reinterpret_cast<const float4 *>(vp + 4 * t4);
+          gc[t4] = *reinterpret_cast<const float4 *>(gp + 4 * t4);
         }
-        float pv[16];
-        tc::tmem_ld16(tbase + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(ch * 16), pv);
-        // rows are zero beyond n, so padded columns add nothing
+        tc::tmem_wait_ld(pv);
 #pragma unroll
         for (int t4 = 0; t4 < 4; ++t4) {
-          acc0 = fmaf(vc[t4].x * gc[t4].x, pv[4 * t4], acc0);
-          acc1 = fmaf(vc[t4].y * gc[t4].y, pv[4 * t4 + 1], acc1);
-          acc0 = fmaf(vc[t4].z * gc[t4].z, pv[4 * t4 + 2], acc0);
-          acc1 = fmaf(vc[t4].w * gc[t4].w, pv[4 * t4 + 3], acc1);
+          acc0 = fmaf(vc[t4].x * gc[t4].x, __uint_as_float(pv[4 * t4]), acc0);
+          acc1 = fmaf(vc[t4].y * gc[t4].y, __uint_as_float(pv[4 * t4 + 1]), acc1);
+          acc0 = fmaf(vc[t4].z * gc[t4].z, __uint_as_float(pv[4 * t4 + 2]), acc0);
+          acc1 = fmaf(vc[t4].w * gc[t4].w, __uint_as_float(pv[4 * t4 + 3]), acc1);
+        }
+      };
+      if constexpr (!DEAL) {
+        for (int ch = cb; ch < ce; ++ch) fold(Va + ch * 16, gb_row + ch * 16, ch);
+      } else {
+#pragma unroll
+        for (int x = 0; x < kXChunks; ++x) {
+          if (cb + x < ce) {
+            if (x < kXTmem && x < nt) {
+              uint32_t pv[16], m[16];
+              tc::tmem_ld16_async(prow_t + (uint32_t)((cb + x) * 16), pv);
+              tc::tmem_ld16_async(mrow + (uint32_t)(16 * x), m);
+              tc::tmem_wait_ld(pv);
+              tc::tmem_wait_ld(m);
+#pragma unroll
+              for (int t = 0; t < 16; t += 2) {
+                acc0 = fmaf(__uint_as_float(m[t]), __uint_as_float(pv[t]), acc0);
+                acc1 = fmaf(__uint_as_float(m[t + 1]), __uint_as_float(pv[t + 1]), acc1);
+              }
+            } else {
+              deal_out(x % kXAhead, cb + x + kXAhead);
+              fold(deal_v, deal_g, cb + x);
+              __syncwarp();
+            }
+          }
         }
       }
       tc::fence_before_sync();
@@ -449,7 +531,7 @@ __global__ void __launch_bounds__(XRoles<F16>::kThreads, 1)
       const float X = xh + pb[prow];
       tc::warp_arrive(&pempty[buf]);
       float sig = 0.f;
-      if (live) sig = S.spin * gA[(long)a * ld + b] * S.W[((long)xt.j * n + b) * ld + a] - X;
+      if (live) sig = S.spin * gab * wab - X;
       if (S.smax) {  // largest |Sigma| entry, for the FP16 operand scale of the convolution
         float mx = fabsf(sig);
         for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
@@ -603,24 +685,21 @@ cudaError_t exchange_tc_launch(const XSys *sys, const long *prefix, int n_sys, l
   const size_t stg = exchange_stage_pitch(ld_max);
   const size_t staged = smem + 2 * 24 * stg * sizeof(float);
   const int pitch = staged <= 232448 ? (int)stg : 0;
-  if (pitch) smem = staged;
+  if (!pitch && Np_max > 32 * kXChunks) return cudaErrorInvalidValue;
+  smem = pitch ? staged : smem + 8 * kXDeal * sizeof(float);
   const int grid = (int)(items < num_sms ? items : num_sms);
   const int nbuf = (Np_max <= 256) ? 2 : 1;
-  cudaError_t e;
-  if (f16) {
-    e = cudaFuncSetAttribute(exchange_tc_kernel<true>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const auto run = [&](auto kernel, int threads) {
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    exchange_tc_kernel<true><<<grid, XRoles<true>::kThreads, smem, s>>>(sys, prefix, n_sys, items,
-                                                                        Np_max, nbuf, pitch, err);
-  } else {
-    e = cudaFuncSetAttribute(exchange_tc_kernel<false>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    exchange_tc_kernel<false><<<grid, XRoles<false>::kThreads, smem, s>>>(
-        sys, prefix, n_sys, items, Np_max, nbuf, pitch, err);
-  }
-  return cudaGetLastError();
+    kernel<<<grid, threads, smem, s>>>(sys, prefix, n_sys, items, Np_max, nbuf, pitch, err);
+    return cudaGetLastError();
+  };
+  if (f16)
+    return pitch ? run(exchange_tc_kernel<true, false>, XRoles<true>::kThreads)
+                 : run(exchange_tc_kernel<true, true>, XRoles<true>::kThreads);
+  return pitch ? run(exchange_tc_kernel<false, false>, XRoles<false>::kThreads)
+               : run(exchange_tc_kernel<false, true>, XRoles<false>::kThreads);
 }
 
 }  // namespace fedvr
