@@ -488,7 +488,8 @@ int fedvr_sigma2_noalloc(int n, int M, double spin, const double *V, const doubl
  * (their length depends on n and M only) and the call cuts the mesh-point
  * range into the split count requested with fedvr_conv1_splits (largest
  * candidate in {1, 2, 3, 4, 6, 8, 12, 16} not above it and not above the
- * number of blocks; no request: 1); results of different split counts
+ * number of blocks; no request: up to 4, by how full the last wave of CTAs is);
+ * results of different split counts
  * differ only in the order of the FP64 additions of the block sums. */
 int fedvr_conv_sigma_g(fedvr_ctx *ctx, int n, double beta, int u, int p, const double *dHF,
                        const double *Sigma, const double *G, double *I1, int precision);

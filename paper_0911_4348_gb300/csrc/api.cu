@@ -2087,7 +2087,7 @@ int fedvr_conv_sigma_g(fedvr_ctx *ctx, int n, double beta, int u, int p, const d
     TcScale *scale = nullptr;
     const bool f16 = precision == FEDVR_SPLIT_F16;
     // work split of the mesh-point range: the request of fedvr_conv1_splits
-    // (largest candidate not above it, whole accumulation blocks), else none
+    // (largest candidate not above it, whole accumulation blocks)
     int S = 1;
     if (ctx->c1_request > 1) {
       const int NB = conv1_blocks(n, M, f16);
@@ -2096,6 +2096,22 @@ int fedvr_conv_sigma_g(fedvr_ctx *ctx, int n, double beta, int u, int p, const d
     }
     const size_t stack = (size_t)M * n * n;
     if (S > 1) ENSURE(ctx, w_c1p, dsz((size_t)(S - 1) * stack));
+    if (ctx->c1_request == 0) {
+      // no request: the split with the least time, a chunk of a tile taking about 1 us
+      // and a partial stack three passes over memory (n = 142, M = 1025: 1138 tiles are
+      // 8 waves of 152 CTAs with a last one half empty, 18.4 ms; two splits 17.05)
+      const long RT = ((long)M * n + 127) / 128;
+      const int KC = f16 ? (n + 63) / 64 : (n + 31) / 32, NB = conv1_blocks(n, M, f16);
+      double best = 0.0;
+      int pick = 1;
+      for (int c : {1, 2, 3, 4}) {
+        if (c > NB) break;
+        const double waves = (double)((RT * c + ctx->num_sms - 1) / ctx->num_sms) / c;
+        const double us = waves * M * KC * 1.0 + (c - 1) * stack * 24.0 / 5e6;
+        if (c == 1 || us < 0.98 * best) best = us, pick = c;
+      }
+      if (pick > 1 && ensure_optional(ctx, ctx->w_c1p, dsz((size_t)(pick - 1) * stack))) S = pick;
+    }
     if (f16) {
       if (int r = f16_workspace(ctx, n, M, &h16, &scale)) return r;
       FEDVR_CK(ctx, launch_scale_init(M, P<int4>(ctx->w_coef32), 0, nullptr, scale, s));
