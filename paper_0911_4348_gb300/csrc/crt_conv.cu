@@ -393,6 +393,10 @@ __global__ void __launch_bounds__(kThreads, 1) crt_conv_kernel(const __grid_cons
       const float pm = p.p[it.m], ipm = p.ip[it.m];
       const uint64_t PM = tc::f2_pack(-pm, -pm), IP = tc::f2_pack(ipm, ipm),
                      RN = tc::f2_pack(kRound, kRound), NRN = tc::f2_pack(-kRound, -kRound);
+      // the bits of the largest multiple of p up to 12582912 = 1.5 2^23: base + x are
+      // the bits of a float congruent to x, which needs no subtraction before the
+      // reduction (1 / p is within 2^-24, so its remainder is within p / 2 + 0.75)
+      const int base = 0x4B400000 - 12582912 % (int)pm;
       // walk of the chunks through the sections: full slices, the 32-wide and
       // the 16-wide rest (sh: log2 of the mesh points per chunk)
       int sh, idx, len, sec;
@@ -472,13 +476,13 @@ __global__ void __launch_bounds__(kThreads, 1) crt_conv_kernel(const __grid_cons
             auto word = [&](const uint4 &v) { return x4 == 0 ? v.x : x4 == 1 ? v.y : x4 == 2 ? v.z : v.w; };
             int acc[4];
 #pragma unroll
-            for (int t = 0; t < 4; ++t) acc[t] = 0x4B400000;  // the bits of 12582912.f
+            for (int t = 0; t < 4; ++t) acc[t] = base;
             combine4(word(wv[q][0]), word(wv[q][1]), e[q].c01, acc);
             if constexpr (NP == 4) combine4(word(wv[q][2]), word(wv[q][3]), e[q].c23, acc);
 #pragma unroll
             for (int t = 0; t < 2; ++t) {
               const uint64_t F = (uint64_t)(uint32_t)acc[2 * t] | ((uint64_t)(uint32_t)acc[2 * t + 1] << 32);
-              const uint64_t r = mod2(f2_add(F, NRN), IP, PM, RN, NRN);
+              const uint64_t r = mod2(F, IP, PM, RN, NRN);
               const __half2 hh = __floats2half2_rn(tc::f2_lo(r), tc::f2_hi(r));
               h[2 * x4 + t] = *reinterpret_cast<const uint32_t *>(&hh);
             }
