@@ -86,7 +86,10 @@ PRECISION_BY_STAGE = {
                  "fp32 eigen-kernel table",
         "update_residual_N_E0": "fp64",
         "basis_mesh_tables_hf": "fp64"},
-    "fp64": {"all": "fp64"},
+    "fp64": {"all": "fp64; for all but small systems the exchange, the first convolution (also "
+                    "GW's) and the T-matrix ladder as exact integer products modulo 23 to 44 "
+                    "numbers below 256 (fp16 residues, exact fp32 sums) of entries rounded to "
+                    "54 to 59 bits, rebuilt and rounded to fp64 once"},
 }
 
 
@@ -906,7 +909,9 @@ def main():
         sm_max = float(peaks.get("sm_max_mhz", 2070.0))
         peak = N_SM * FP64_FLOP_PER_CLK_SM * sm_max * 1e6 / 1e12
         bound, punit, psrc = "alu", "TFLOP/s", ("FP64 pipe: 152 SMs x 2 DFMA/clk x 2 flop x "
-                                               f"{sm_max:.0f} MHz (unit counts and clocks)")
+                                               f"{sm_max:.0f} MHz (unit counts and clocks); the residue "
+                                               "products run on the tensor cores beside it, so "
+                                               "the fraction may exceed 1")
     elif dom == "conv2":  # the second convolution's GEMMs run on the FP32 pipe
         sm_max = float(peaks.get("sm_max_mhz", 2070.0))
         peak = N_SM * 128 * 2 * sm_max * 1e6 / 1e12
@@ -943,9 +948,9 @@ def main():
             "algorithmic_flops_per_launch": dom_flops, "peak_source": psrc,
             "stage_ms": avg}
     if gw:
-        roof["kernel"] = ("GW screened interaction (conv1_fp64_kernel, periodic table)"
+        roof["kernel"] = ("GW screened interaction (crt_conv_kernel, periodic table)"
                           if args.self_energy == "gw" else
-                          "T-matrix ladder (tm_ladder_kernel, periodic table)")
+                          "T-matrix ladder (crt_conv_kernel or tm_ladder_kernel, periodic table)")
         roof["inner_iterations_mean"] = float(np.mean(inner))
 
     out = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world,

@@ -59,11 +59,12 @@ typedef enum {
 
 typedef enum {
   FEDVR_FP64 = 0,        /* every contraction to IEEE double accuracy. The first
-                            convolution (and GW's) and the second-order
-                            exchange run as exact integer sums on the tensor
-                            cores: each operand matrix is rounded to 2^-57 of
-                            its largest entry, the sum of the products is
-                            exact and rounded once; small
+                            convolution (and GW's), the second-order
+                            exchange and the T-matrix ladder run as exact
+                            integer sums on the tensor cores: each operand
+                            matrix is rounded to 54 to 59 bits of its largest
+                            entry (weights: of their row's), the sum of the
+                            products is exact and rounded once; small
                             sizes and inputs that are not finite use double
                             arithmetic throughout. */
   FEDVR_SPLIT_TF32 = 1,  /* Sigma^(2) (exchange and V Q V), I^(1) and, for

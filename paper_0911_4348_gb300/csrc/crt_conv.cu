@@ -16,10 +16,10 @@
 // Measured against 113-bit arithmetic on the HF Green's functions of He (n = 15
 // to 119) and on random stacks, the result is within 1e-16 (2-norm, relative; 2
 // to 6e-16 for the FP64 kernel): it is the exact sum of the rounded integers,
-// rounded to FP64 once. n = 119, M = 257: 190 -> 9.0 ms; n = 199, M = 513:
-// 3574 -> 104 ms. What bounds it (ncu, n = 119): the producers' instructions, 3,700
-// warp instructions per chunk of 256 rows x 64 columns against 512 cycles of MMA
-// (issue slots 56 %, FMA-heavy pipe 60 %, tensor pipe 30 %).
+// rounded to FP64 once. n = 119, M = 257: 190 -> 8.8 ms; n = 199, M = 513:
+// 3574 -> 98 ms. What bounds it (ncu, n = 119): the producers' instructions, some
+// 3,400 warp instructions per chunk of 256 rows x 64 columns against 512 cycles of
+// MMA (issue slots 53 %, tensor pipe 32 %).
 #include <algorithm>
 #include <cmath>
 

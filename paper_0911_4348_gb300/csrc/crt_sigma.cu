@@ -2,7 +2,7 @@
 // (crt.cuh; Sec. 2.3, Eq. sigma2ndb): X_ab = sum_kl V_ak V_bl g_al gb_lk g_kb for
 // every mesh point, g = G[j], gb = G[M-1-j].
 //
-// V and the matrices g_j are rounded to integers of 54 to 57 bits relative to
+// V and the matrices g_j are rounded to integers of 57 to 59 bits relative to
 // their largest entries; X is then an integer below 2^(5 q) n^2, held by its
 // residues modulo 38 to 42 moduli. For each modulus, row (b, a) of P^(b) = g
 // diag(V_b) gb is one FP16 product of small integers: the A operand g_al V_bl is
