@@ -458,8 +458,9 @@ int fedvr_sigma2(fedvr_ctx *ctx, int n, int M, double spin, const double *V,
  * service for callers that cannot let the library allocate device memory --
  * processes whose device memory belongs to another allocator (a framework's
  * caching allocator that reserves the pool), or loops that cannot accept the
- * device synchronisation cudaMalloc/cudaFree imply. It computes exactly what
- * fedvr_sigma2 computes with precision FEDVR_FP64 (same kernels), needs no
+ * device synchronisation cudaMalloc/cudaFree imply. It computes what
+ * fedvr_sigma2 computes with precision FEDVR_FP64 (by the double-arithmetic
+ * kernels, so the two may differ by rounding), needs no
  * context, and calls no cudaMalloc, cudaFree or allocating library routine:
  * its workspace is a fixed 12 MiB device array inside the library, which every
  * GPU that loads the library holds until the process exits.
