@@ -523,7 +523,7 @@ int launch_conv1_single(fedvr_ctx *ctx, int splits, int *err, cudaStream_t s, in
   uint8_t *tab = P<uint8_t>(ctx->w_tab);
   FEDVR_CK(ctx, conv1_tc_launch(reinterpret_cast<const C1Sys *>(tab + kTabC),
                                 reinterpret_cast<const long *>(tab + kTabPC), 1,
-                                conv1_items(n, M, splits), g.Np, err, ctx->num_sms, s,
+                                conv1_items(n, M, splits), g.nsz[0], err, ctx->num_sms, s,
                                 ctx->precision == FEDVR_SPLIT_F16));
   *launches += 1;
   if (splits > 1) {
@@ -1544,7 +1544,7 @@ int fedvr_get_history(const fedvr_ctx *ctx, double *buf, int cap, int *len) {
 struct fedvr_batch {
   std::vector<fedvr_ctx *> ctxs;
   std::vector<unsigned long long> gens;  // each context's prepare generation at creation
-  int Np_max = 16, ld_max = 32;
+  int Np_max = 16, Nt_max = 16, ld_max = 32;
   size_t off_c = 0, off_px = 0, off_pc = 0, off_err = 0, off_red = 0;
   std::vector<long> px, pc;
   std::vector<int> S;  // measured split count of each system's first convolution
@@ -1599,7 +1599,7 @@ int enqueue_batch(fedvr_batch *B, const int *active, const int *warm, double mix
     }
   FEDVR_CK(lead, conv1_tc_launch(reinterpret_cast<const C1Sys *>(bt + B->off_c),
                                  reinterpret_cast<const long *>(bt + B->off_pc), n_sys,
-                                 B->pc[n_sys], B->Np_max, d_err, lead->num_sms, s, f16));
+                                 B->pc[n_sys], B->Nt_max, d_err, lead->num_sms, s, f16));
   *launches += 1;
   for (int k = 0; k < n_sys; ++k)
     if (active[k]) {
@@ -1715,7 +1715,7 @@ int tune_batch_splits(fedvr_batch *B, std::vector<C1Sys> &hc) {
         FEDVR_CK(lead, cudaEventRecord(lead->ev[0], s));
         FEDVR_CK(lead, conv1_tc_launch(reinterpret_cast<const C1Sys *>(bt + B->off_c),
                                        reinterpret_cast<const long *>(bt + B->off_pc), n_sys,
-                                       B->pc[n_sys], B->Np_max, d_err, lead->num_sms, s, f16));
+                                       B->pc[n_sys], B->Nt_max, d_err, lead->num_sms, s, f16));
         for (int k = 0; k < n_sys; ++k) {
           fedvr_ctx *c = B->ctxs[k];
           if (B->S[k] > 1)
@@ -1772,6 +1772,7 @@ int fedvr_batch_create(fedvr_batch **out, fedvr_ctx **ctxs, int n_sys, const dou
     }
     const TcGeom g = tc_geom(ctxs[k]->n, ctxs[k]->M);
     B->Np_max = g.Np > B->Np_max ? g.Np : B->Np_max;
+    B->Nt_max = g.nsz[0] > B->Nt_max ? g.nsz[0] : B->Nt_max;
     B->ld_max = g.ld > B->ld_max ? g.ld : B->ld_max;
   }
   for (int k = 0; k < n_sys; ++k) B->gens.push_back(ctxs[k]->prep_gen);
@@ -2100,7 +2101,7 @@ int fedvr_conv_sigma_g(fedvr_ctx *ctx, int n, double beta, int u, int p, const d
       // no request: the split with the least time, a chunk of a tile taking about 1 us
       // and a partial stack three passes over memory (n = 142, M = 1025: 1138 tiles are
       // 8 waves of 152 CTAs with a last one half empty, 18.4 ms; two splits 17.05)
-      const long RT = ((long)M * n + 127) / 128;
+      const long RT = conv1_items(n, M, 1);
       const int KC = f16 ? (n + 63) / 64 : (n + 31) / 32, NB = conv1_blocks(n, M, f16);
       double best = 0.0;
       int pick = 1;
@@ -2128,7 +2129,7 @@ int fedvr_conv_sigma_g(fedvr_ctx *ctx, int n, double beta, int u, int p, const d
     uint8_t *tab = P<uint8_t>(ctx->w_tab);
     FEDVR_CK(ctx, conv1_tc_launch(reinterpret_cast<const C1Sys *>(tab + kTabC),
                                   reinterpret_cast<const long *>(tab + kTabPC), 1,
-                                  conv1_items(n, M, S), g.Np, err, ctx->num_sms, s, f16));
+                                  conv1_items(n, M, S), g.nsz[0], err, ctx->num_sms, s, f16));
     if (S > 1) FEDVR_CK(ctx, conv1_sum_splits((long)stack, S - 1, P<double>(ctx->w_c1p), I1, s));
     ctx->c1_splits = S;
     int h_err = 0;

@@ -40,12 +40,16 @@ constexpr int kWarps = 22;  // 0-3 flush, 4-19 A producers, 20 TMA, 21 MMA
 constexpr int kThreads = kWarps * 32;
 
 struct C1Item {
-  int t, j_lo, j_hi;
+  int t, nt, j_lo, j_hi;
   double *out;  // I1 or the split's partial stack
 };
 
-// Item q of a system: split s = q / RT (split-major, so that the CTAs running
-// at the same time walk the same mesh points and share g_j in L2), tile t.
+// Item q of a system: split s (split-major, so that the CTAs running at the same
+// time walk the same mesh points and share g_j in L2), N tile nt, row tile t. For n >
+// 256 the two N tiles are items of their own, although each forms the A operand
+// again: with both in one item the stages left the rows of Sigma no L1 and the
+// accumulators one buffer, and a chunk took 5100 cycles at n = 299, M = 1025 (212 ms);
+// 170 as two.
 // The FP32 accumulation blocks are the fixed mesh-point ranges
 // [b JB, (b + 1) JB) of the system (JB depends on n and M only); split s
 // takes the whole blocks [s NB / S, (s + 1) NB / S) of the NB blocks, so the
@@ -53,8 +57,9 @@ struct C1Item {
 // ends (the host keeps S <= NB: no split is empty).
 __device__ __forceinline__ C1Item c1_item(const C1Sys &S, long q) {
   C1Item it;
-  const int s = (int)(q / S.RT);
-  it.t = (int)(q % S.RT);
+  const int s = (int)(q / (S.RT * S.g.NT)), q2 = (int)(q % (S.RT * S.g.NT));
+  it.nt = q2 / (int)S.RT;
+  it.t = q2 % (int)S.RT;
   const int NB = (S.g.M + S.JB - 1) / S.JB;
   it.j_lo = (int)(((long)s * NB) / S.S) * S.JB;
   it.j_hi = min(S.g.M, (int)(((long)(s + 1) * NB) / S.S) * S.JB);
@@ -67,11 +72,11 @@ __device__ __forceinline__ C1Item c1_item(const C1Sys &S, long q) {
 // four rows per thread fetched anew at every mesh point by eight warps, 7.8 so).
 __global__ void __launch_bounds__(kThreads, 1)
     conv1_tc_kernel(const C1Sys *__restrict__ sys, const long *__restrict__ prefix, int n_sys,
-                    long items, int Np_max, int nbuf, int *err) {
+                    long items, int Nt_max, int *err) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                               ~uintptr_t(1023));
-  const uint32_t tileB = (uint32_t)Np_max * 128;
+  const uint32_t tileB = (uint32_t)Nt_max * 128;
   const uint32_t stage_bytes = 2 * kTileA + 2 * tileB;
   uint64_t *bars = reinterpret_cast<uint64_t *>(smem + 2 * stage_bytes);
   uint64_t *full = bars, *empty = bars + 2, *accf = bars + 4, *acce = bars + 6, *drain = bars + 8;
@@ -204,9 +209,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         while (cur + 1 < n_sys && w >= prefix[cur + 1]) ++cur;
         const C1Sys &S = sys[cur];
         const C1Item it = c1_item(S, w - prefix[cur]);
-        const uint32_t bytes = 2u * (uint32_t)S.g.Np * 128u;
-        const int NT = S.g.NT, KC = S.g.KC, n00 = S.g.n0[0], n01 = S.g.n0[1];
-        const CUtensorMap *th0 = &S.th[0], *th1 = &S.th[1], *tl0 = &S.tl[0], *tl1 = &S.tl[1];
+        const uint32_t bytes = 2u * (uint32_t)S.g.nsz[it.nt] * 128u;
+        const int KC = S.g.KC, r = S.g.n0[it.nt];
+        const CUtensorMap *th = &S.th[it.nt], *tl = &S.tl[it.nt];
         const int JB = S.JB;
         for (int j0 = it.j_lo; j0 < it.j_hi && !*abort_flag; j0 += JB) {
           const int j1 = min(it.j_hi, j0 + JB);
@@ -220,11 +225,8 @@ __global__ void __launch_bounds__(kThreads, 1)
               }
               uint8_t *st = smem + s * stage_bytes + 2 * kTileA;
               tc::mbar_arrive_expect_tx(&full[s], bytes);
-              for (int nt = 0; nt < NT; ++nt) {
-                const int r = nt ? n01 : n00;
-                tc::tma_load_3d(st + r * 128, nt ? th1 : th0, kc * 32, r, j, &full[s]);
-                tc::tma_load_3d(st + tileB + r * 128, nt ? tl1 : tl0, kc * 32, r, j, &full[s]);
-              }
+              tc::tma_load_3d(st, th, kc * 32, r, j, &full[s]);
+              tc::tma_load_3d(st + tileB, tl, kc * 32, r, j, &full[s]);
             }
           }
         }
@@ -238,24 +240,18 @@ __global__ void __launch_bounds__(kThreads, 1)
         while (cur + 1 < n_sys && w >= prefix[cur + 1]) ++cur;
         const C1Sys &S = sys[cur];
         const C1Item it = c1_item(S, w - prefix[cur]);
-        const int n = S.g.n, KC = S.g.KC, NT = S.g.NT, JB = S.JB;
-        const uint32_t n00 = (uint32_t)S.g.n0[0], n01 = (uint32_t)S.g.n0[1];
-        const uint32_t id0 = tc::idesc_tf32(128, S.g.nsz[0]), id1 = tc::idesc_tf32(128, S.g.nsz[1]);
+        const int n = S.g.n, KC = S.g.KC, JB = S.JB;
+        const uint32_t idesc = tc::idesc_tf32(128, S.g.nsz[it.nt]);
         for (int j0 = it.j_lo; j0 < it.j_hi && !*abort_flag; j0 += JB, ++tcount) {
           const int j1 = min(it.j_hi, j0 + JB);
           const int buf = tcount & 1;
           const uint32_t tu = tcount >> 1;
-          bool ok = true;
-          if (nbuf == 1 && tcount > 0)
-            ok = tc::mbar_wait(&acce[(tcount - 1) & 1], ((tcount - 1) >> 1) & 1, kWaitNs);
-          else if (nbuf == 2 && tu > 0)
-            ok = tc::mbar_wait(&acce[buf], (tu - 1) & 1, kWaitNs);
-          if (!ok) {
+          if (tu > 0 && !tc::mbar_wait(&acce[buf], (tu - 1) & 1, kWaitNs)) {
             *abort_flag = 1;
             break;
           }
           tc::fence_after_sync();
-          const uint32_t dbase = tmem + (nbuf == 2 ? (uint32_t)(buf * 256) : 0u);
+          const uint32_t dbase = tmem + (uint32_t)(buf * 256);
           for (int kc = 0; kc < KC && !*abort_flag; ++kc) {
             const int ksteps = min(4, (n - kc * 32 + 7) / 8);
             for (int j = j0; j < j1; ++j, ++cc) {
@@ -271,17 +267,11 @@ __global__ void __launch_bounds__(kThreads, 1)
               for (int kk = 0; kk < ksteps; ++kk) {
                 const uint64_t ah = tc::sdesc_k128(sa + kk * 32);
                 const uint64_t al = tc::sdesc_k128(sa + kTileA + kk * 32);
-                for (int nt = 0; nt < NT; ++nt) {
-                  const uint32_t r = nt ? n01 : n00;
-                  const uint32_t boff = 2 * kTileA + r * 128 + kk * 32;
-                  const uint64_t bh = tc::sdesc_k128(sa + boff);
-                  const uint64_t bl = tc::sdesc_k128(sa + boff + tileB);
-                  const uint32_t d = dbase + r;
-                  const uint32_t idesc = nt ? id1 : id0;
-                  tc::mma_tf32(d, ah, bh, idesc, (fresh && kk == 0) ? 0u : 1u);
-                  tc::mma_tf32(d, ah, bl, idesc, 1u);
-                  tc::mma_tf32(d, al, bh, idesc, 1u);
-                }
+                const uint64_t bh = tc::sdesc_k128(sa + 2 * kTileA + kk * 32);
+                const uint64_t bl = tc::sdesc_k128(sa + 2 * kTileA + tileB + kk * 32);
+                tc::mma_tf32(dbase, ah, bh, idesc, (fresh && kk == 0) ? 0u : 1u);
+                tc::mma_tf32(dbase, ah, bl, idesc, 1u);
+                tc::mma_tf32(dbase, al, bh, idesc, 1u);
               }
               tc::mma_commit(&empty[s]);
               issued = true;
@@ -307,6 +297,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const C1Item it = c1_item(S, w - prefix[cur]);
       const long row0 = (long)it.t * 128 + warp * 32;
       double *const out = it.out;
+      const int b0 = S.g.n0[it.nt];  // first column
       for (int j0 = it.j_lo; j0 < it.j_hi; j0 += JB, ++tcount) {
         const int buf = tcount & 1;
         const uint32_t tu = tcount >> 1;
@@ -315,15 +306,15 @@ __global__ void __launch_bounds__(kThreads, 1)
           break;
         }
         tc::fence_after_sync();
-        const uint32_t tbase = tmem + (nbuf == 2 ? (uint32_t)(buf * 256) : 0u);
+        const uint32_t tbase = tmem + (uint32_t)(buf * 256);
         const bool first = j0 == it.j_lo;
-        for (int c0 = 0; c0 < n; c0 += 16) {
+        for (int c0 = 0; c0 < S.g.nsz[it.nt] && b0 + c0 < n; c0 += 16) {
           float v[16];
           tc::tmem_ld16(tbase + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
 #pragma unroll
           for (int t = 0; t < 16; ++t) stg[lane * 17 + t] = v[t];
           __syncwarp();
-          const int b = c0 + cl;
+          const int b = b0 + c0 + cl;
 #pragma unroll 4
           for (int i = 0; i < 16; ++i) {
             const int rr = 2 * i + rh;
@@ -466,11 +457,11 @@ __device__ __forceinline__ int a_scale_exp(const TcScale *sc) {
 
 __global__ void __launch_bounds__(kThreads, 1)
     conv1_f16_kernel(const C1Sys *__restrict__ sys, const long *__restrict__ prefix, int n_sys,
-                     long items, int Np_max, int nbuf, int *err) {
+                     long items, int Nt_max, int *err) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                               ~uintptr_t(1023));
-  const uint32_t tileB = (uint32_t)Np_max * 128;
+  const uint32_t tileB = (uint32_t)Nt_max * 128;
   const uint32_t stage_bytes = 2 * kTileA + 2 * tileB;
   uint64_t *bars = reinterpret_cast<uint64_t *>(smem + 2 * stage_bytes);
   uint64_t *full = bars, *empty = bars + 2, *accf = bars + 4, *acce = bars + 6, *drain = bars + 8;
@@ -671,9 +662,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         while (cur + 1 < n_sys && w >= prefix[cur + 1]) ++cur;
         const C1Sys &S = sys[cur];
         const C1Item it = c1_item(S, w - prefix[cur]);
-        const uint32_t bytes = 2u * (uint32_t)S.g.Np * 128u;
-        const int NT = S.g.NT, KC = (S.g.n + 63) / 64, n00 = S.g.n0[0], n01 = S.g.n0[1];
-        const CUtensorMap *th0 = &S.hh[0], *th1 = &S.hh[1], *tl0 = &S.hl[0], *tl1 = &S.hl[1];
+        const uint32_t bytes = 2u * (uint32_t)S.g.nsz[it.nt] * 128u;
+        const int KC = (S.g.n + 63) / 64, r = S.g.n0[it.nt];
+        const CUtensorMap *th = &S.hh[it.nt], *tl = &S.hl[it.nt];
         const int JB = S.JB, TU = S.TU, KCf = TU ? KC - 1 : KC;
         for (int j0 = it.j_lo; j0 < it.j_hi && !*abort_flag; j0 += JB) {
           const int j1 = min(it.j_hi, j0 + JB);
@@ -687,11 +678,8 @@ __global__ void __launch_bounds__(kThreads, 1)
               }
               uint8_t *st = smem + s * stage_bytes + 2 * kTileA;
               tc::mbar_arrive_expect_tx(&full[s], bytes);
-              for (int nt = 0; nt < NT; ++nt) {
-                const int r = nt ? n01 : n00;
-                tc::tma_load_3d(st + r * 128, nt ? th1 : th0, kc * 64, r, j, &full[s]);
-                tc::tma_load_3d(st + tileB + r * 128, nt ? tl1 : tl0, kc * 64, r, j, &full[s]);
-              }
+              tc::tma_load_3d(st, th, kc * 64, r, j, &full[s]);
+              tc::tma_load_3d(st + tileB, tl, kc * 64, r, j, &full[s]);
             }
           }
           // packed tail: columns jt 8 TU .. + 63 (16-byte aligned; past the end zero-filled)
@@ -704,11 +692,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
             uint8_t *st = smem + s * stage_bytes + 2 * kTileA;
             tc::mbar_arrive_expect_tx(&full[s], bytes);
-            for (int nt = 0; nt < NT; ++nt) {
-              const int r = nt ? n01 : n00;
-              tc::tma_load_2d(st + r * 128, &S.th16[nt], jt * 8 * TU, r, &full[s]);
-              tc::tma_load_2d(st + tileB + r * 128, &S.tl16[nt], jt * 8 * TU, r, &full[s]);
-            }
+            tc::tma_load_2d(st, &S.th16[it.nt], jt * 8 * TU, r, &full[s]);
+            tc::tma_load_2d(st + tileB, &S.tl16[it.nt], jt * 8 * TU, r, &full[s]);
           }
         }
       }
@@ -721,25 +706,19 @@ __global__ void __launch_bounds__(kThreads, 1)
         while (cur + 1 < n_sys && w >= prefix[cur + 1]) ++cur;
         const C1Sys &S = sys[cur];
         const C1Item it = c1_item(S, w - prefix[cur]);
-        const int n = S.g.n, KC = (n + 63) / 64, NT = S.g.NT, JB = S.JB, TU = S.TU;
+        const int n = S.g.n, KC = (n + 63) / 64, JB = S.JB, TU = S.TU;
         const int KCf = TU ? KC - 1 : KC;
-        const uint32_t n00 = (uint32_t)S.g.n0[0], n01 = (uint32_t)S.g.n0[1];
-        const uint32_t id0 = tc::idesc_f16(128, S.g.nsz[0]), id1 = tc::idesc_f16(128, S.g.nsz[1]);
+        const uint32_t idesc = tc::idesc_f16(128, S.g.nsz[it.nt]);
         for (int j0 = it.j_lo; j0 < it.j_hi && !*abort_flag; j0 += JB, ++tcount) {
           const int j1 = min(it.j_hi, j0 + JB);
           const int buf = tcount & 1;
           const uint32_t tu = tcount >> 1;
-          bool ok = true;
-          if (nbuf == 1 && tcount > 0)
-            ok = tc::mbar_wait(&acce[(tcount - 1) & 1], ((tcount - 1) >> 1) & 1, kWaitNs);
-          else if (nbuf == 2 && tu > 0)
-            ok = tc::mbar_wait(&acce[buf], (tu - 1) & 1, kWaitNs);
-          if (!ok) {
+          if (tu > 0 && !tc::mbar_wait(&acce[buf], (tu - 1) & 1, kWaitNs)) {
             *abort_flag = 1;
             break;
           }
           tc::fence_after_sync();
-          const uint32_t dbase = tmem + (nbuf == 2 ? (uint32_t)(buf * 256) : 0u);
+          const uint32_t dbase = tmem + (uint32_t)(buf * 256);
           bool fresh = true;  // the block's first chunk overwrites the accumulator
           // full slices, mesh point by mesh point, then the packed tail's chunks
           const int nch = KCf * (j1 - j0) + (TU ? (j1 - j0 + 8 / TU - 1) / (8 / TU) : 0);
@@ -762,17 +741,11 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int kk = 0; kk < ksteps; ++kk) {
               const uint64_t ah = tc::sdesc_k128(sa + kk * 32);
               const uint64_t al = tc::sdesc_k128(sa + kTileA + kk * 32);
-              for (int nt = 0; nt < NT; ++nt) {
-                const uint32_t r = nt ? n01 : n00;
-                const uint32_t boff = 2 * kTileA + r * 128 + kk * 32;
-                const uint64_t bh = tc::sdesc_k128(sa + boff);
-                const uint64_t bl = tc::sdesc_k128(sa + boff + tileB);
-                const uint32_t d = dbase + r;
-                const uint32_t idesc = nt ? id1 : id0;
-                tc::mma_f16(d, ah, bh, idesc, (fresh && kk == 0) ? 0u : 1u);
-                tc::mma_f16(d, ah, bl, idesc, 1u);
-                tc::mma_f16(d, al, bh, idesc, 1u);
-              }
+              const uint64_t bh = tc::sdesc_k128(sa + 2 * kTileA + kk * 32);
+              const uint64_t bl = tc::sdesc_k128(sa + 2 * kTileA + tileB + kk * 32);
+              tc::mma_f16(dbase, ah, bh, idesc, (fresh && kk == 0) ? 0u : 1u);
+              tc::mma_f16(dbase, ah, bl, idesc, 1u);
+              tc::mma_f16(dbase, al, bh, idesc, 1u);
             }
             fresh = false;
             tc::mma_commit(&empty[s]);
@@ -799,6 +772,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const C1Item it = c1_item(S, w - prefix[cur]);
       const long row0 = (long)it.t * 128 + warp * 32;
       double *const out = it.out;
+      const int b0 = S.g.n0[it.nt];  // first column
       for (int j0 = it.j_lo; j0 < it.j_hi; j0 += JB, ++tcount) {
         const int buf = tcount & 1;
         const uint32_t tu = tcount >> 1;
@@ -807,15 +781,15 @@ __global__ void __launch_bounds__(kThreads, 1)
           break;
         }
         tc::fence_after_sync();
-        const uint32_t tbase = tmem + (nbuf == 2 ? (uint32_t)(buf * 256) : 0u);
+        const uint32_t tbase = tmem + (uint32_t)(buf * 256);
         const bool first = j0 == it.j_lo;
-        for (int c0 = 0; c0 < n; c0 += 16) {
+        for (int c0 = 0; c0 < S.g.nsz[it.nt] && b0 + c0 < n; c0 += 16) {
           float v[16];
           tc::tmem_ld16(tbase + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
 #pragma unroll
           for (int t = 0; t < 16; ++t) stg[lane * 17 + t] = v[t];
           __syncwarp();
-          const int b = c0 + cl;
+          const int b = b0 + c0 + cl;
 #pragma unroll 4
           for (int i = 0; i < 16; ++i) {
             const int rr = 2 * i + rh;
@@ -1026,23 +1000,22 @@ cudaError_t conv1_sum_splits(long count, int nparts, const double *part, double 
 }
 
 cudaError_t conv1_tc_launch(const C1Sys *sys, const long *prefix, int n_sys, long items,
-                            int Np_max, int *err, int num_sms, cudaStream_t s, bool f16) {
+                            int Nt_max, int *err, int num_sms, cudaStream_t s, bool f16) {
   // stages + barriers (256 B) + four 32 x 17 float flush staging tiles
-  const size_t smem = 1024 + 2 * (2 * (size_t)kTileA + 2 * (size_t)Np_max * 128) + 256 +
+  const size_t smem = 1024 + 2 * (2 * (size_t)kTileA + 2 * (size_t)Nt_max * 128) + 256 +
                       4 * 32 * 17 * sizeof(float);
   cudaError_t e = cudaFuncSetAttribute(conv1_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem);
   if (e != cudaSuccess) return e;
   const int grid = (int)(items < num_sms ? items : num_sms);
-  const int nbuf = (Np_max <= 256) ? 2 : 1;
   if (f16) {
     e = cudaFuncSetAttribute(conv1_f16_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)smem);
     if (e != cudaSuccess) return e;
-    conv1_f16_kernel<<<grid, kThreads, smem, s>>>(sys, prefix, n_sys, items, Np_max, nbuf, err);
+    conv1_f16_kernel<<<grid, kThreads, smem, s>>>(sys, prefix, n_sys, items, Nt_max, err);
     return cudaGetLastError();
   }
-  conv1_tc_kernel<<<grid, kThreads, smem, s>>>(sys, prefix, n_sys, items, Np_max, nbuf, err);
+  conv1_tc_kernel<<<grid, kThreads, smem, s>>>(sys, prefix, n_sys, items, Nt_max, err);
   return cudaGetLastError();
 }
 

@@ -183,15 +183,16 @@ cudaError_t kbe_rows_tc(int n, int ncols, int K, int Tn, int sh_ld, const float 
 cudaError_t exchange_tc_launch(const XSys *sys, const long *prefix, int n_sys, long items,
                                int Np_max, int ld_max, int *err, int num_sms, cudaStream_t s,
                                bool f16 = false);
+// Nt_max: the widest N tile of the systems.
 cudaError_t conv1_tc_launch(const C1Sys *sys, const long *prefix, int n_sys, long items,
-                            int Np_max, int *err, int num_sms, cudaStream_t s, bool f16 = false);
+                            int Nt_max, int *err, int num_sms, cudaStream_t s, bool f16 = false);
 
 // Work items per system: exchange (j, tile) pairs over the 16 x 8 blocks of
 // each mesh point; convolution (row tile, split) pairs over the M*n stacked
 // rows.
 inline long exchange_items(int n, int M) { return (long)M * exchange_tiles(n); }
 inline long conv1_items(int n, int M, int splits) {
-  return ((long)M * n + 127) / 128 * (long)splits;
+  return ((long)M * n + 127) / 128 * tc_geom(n, M).NT * (long)splits;
 }
 
 // Mesh points JB per FP32 accumulation block of the first convolution, a
