@@ -400,7 +400,11 @@ __global__ void __launch_bounds__(XRoles<F16>::kThreads, 1)
       float *const deal = stage_rows + warp * kXDeal;
       const float *const deal_v = deal + al * 20, *const deal_g = deal + 160 + (lane >> 3) * 16;
       const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16);
-      const uint32_t mrow = trow + (uint32_t)(S.g.Np + half * 16 * kXTmem);
+      // the products' columns start at the launch's widest accumulator, not at this
+      // system's: a warp of one half may be a tile (and a system) ahead of the other
+      // half's, which reads its own columns of the same lanes. 304 + 112 + 96 = 512
+      // columns at the most: the second half has at most nine chunks
+      const uint32_t mrow = trow + (uint32_t)(Np_max + half * 16 * kXTmem);
       // chunks of this half whose products wait in TMEM
       const int nt = nbuf == 1 ? min(kXTmem, ce - cb - kXAhead) : 0;
       const auto deal_out = [&](int x, int ch) {
