@@ -87,9 +87,10 @@ PRECISION_BY_STAGE = {
         "update_residual_N_E0": "fp64",
         "basis_mesh_tables_hf": "fp64"},
     "fp64": {"all": "fp64; for all but small systems the exchange, the first convolution (also "
-                    "GW's) and the T-matrix ladder as exact integer products modulo 23 to 44 "
+                    "GW's) and the T-matrix ladder as exact integer products modulo 23 to 43 "
                     "numbers below 256 (fp16 residues, exact fp32 sums) of entries rounded to "
-                    "54 to 59 bits, rebuilt and rounded to fp64 once"},
+                    "54 to 59 bits relative to scales of their mesh point, row and column, "
+                    "rebuilt and rounded to fp64 once"},
 }
 
 

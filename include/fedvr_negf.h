@@ -58,15 +58,24 @@ typedef enum {
 } fedvr_status;
 
 typedef enum {
-  FEDVR_FP64 = 0,        /* every contraction to IEEE double accuracy. The first
+  FEDVR_FP64 = 0,        /* IEEE double inputs, sums and results. The first
                             convolution (and GW's), the second-order
                             exchange and the T-matrix ladder run as exact
-                            integer sums on the tensor cores: each operand
-                            matrix is rounded to 54 to 59 bits of its largest
-                            entry (weights: of their row's), the sum of the
-                            products is exact and rounded once; small
-                            sizes and inputs that are not finite use double
-                            arithmetic throughout. */
+                            integer sums on the tensor cores: an operand entry
+                            is rounded to 56 to 59 bits relative to
+                            power-of-two scales of its mesh point, row and
+                            column (weights: 54 bits of their row's largest),
+                            the sum of the products is exact and rounded once.
+                            The largest entries are nearer than from double
+                            arithmetic, and scaling rows, columns or mesh
+                            points changes nothing. The bound of entry (a, b)
+                            is relative to the largest products of row a and
+                            column b, though, not to the entry: entries far
+                            below both (a function that decays away from its
+                            diagonal) carry fewer correct bits than a sum in
+                            double arithmetic. Small sizes, inputs that are not
+                            finite and results that cancel 2^10 below their
+                            products use double arithmetic throughout. */
   FEDVR_SPLIT_TF32 = 1,  /* Sigma^(2) (exchange and V Q V), I^(1) and, for
                             n_b >= 96, the I^(2) products on tensor cores:
                             hi+lo TF32 operands, FP32 accumulation, FP64

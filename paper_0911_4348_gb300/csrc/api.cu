@@ -148,9 +148,10 @@ int ensure_c1f(fedvr_ctx *ctx, int n, int M) {
 
 // First convolution of the FP64 path: by residues on the tensor cores
 // (crt_conv.cu) where its workspace can be had, with the FP64 kernel behind it
-// for inputs that are not finite; else the FP64 kernel alone. conv_f64_prepare
+// for what the residues leave to it; else the FP64 kernel alone. conv_f64_prepare
 // allocates and is called outside graph capture; conv_f64_source forms the
-// residues of the source stack A (once for several applications to other G).
+// scales and residues of the source stack A (once for several applications, of
+// which G is the first: that one is called with fresh).
 int conv_f64_prepare(fedvr_ctx *ctx, int n, int M, int np, bool ext, CrtConv *plan) {
   plan->bytes = 0;
   CrtConv c;
@@ -161,23 +162,23 @@ int conv_f64_prepare(fedvr_ctx *ctx, int n, int M, int np, bool ext, CrtConv *pl
   return ensure_c1f(ctx, n, M);
 }
 int conv_f64_source(fedvr_ctx *ctx, const CrtConv &c, const ConvCoef *coef, const double *dHF,
-                    const double *A, cudaStream_t s, int *launches) {
+                    const double *A, const double *G, cudaStream_t s, int *launches) {
   if (!c.bytes) return FEDVR_OK;
-  FEDVR_CK(ctx, crt_conv_source(c, ctx->w_crt.ptr, A, dHF, coef, s));
-  *launches += 2;
+  FEDVR_CK(ctx, crt_conv_source(c, ctx->w_crt.ptr, A, dHF, G, coef, s));
+  *launches += 5;
   return FEDVR_OK;
 }
 int conv_f64_apply(fedvr_ctx *ctx, const CrtConv &c, int n, int M, const ConvCoef *coef,
                    const double *dHF, const double *A, const double *G, double *I1, cudaStream_t s,
-                   int *launches) {
+                   int *launches, bool fresh) {
   if (!c.bytes) {
     FEDVR_CK(ctx, conv1_fp64(n, M, coef, dHF, A, G, I1, s, P<double>(ctx->w_c1f)));
     *launches += conv1_fp64_splits(n, M) > 1 ? 2 : 1;
     return FEDVR_OK;
   }
-  FEDVR_CK(ctx, crt_conv_apply(c, ctx->w_crt.ptr, G, coef, I1, ctx->num_sms, s));
+  FEDVR_CK(ctx, crt_conv_apply(c, ctx->w_crt.ptr, G, coef, I1, ctx->num_sms, s, fresh));
   FEDVR_CK(ctx, conv1_fp64(n, M, coef, dHF, A, G, I1, s, nullptr, P<int>(ctx->w_crt)));
-  *launches += 6;
+  *launches += fresh ? 5 : 7;
   return FEDVR_OK;
 }
 // The whole first convolution (trapezoid or, with coef4, the fourth-order table).
@@ -185,18 +186,18 @@ int conv_f64(fedvr_ctx *ctx, const CrtConv &c, int n, int M, const ConvCoef *coe
              const ConvCoef4 *coef4, const double *dHF, const double *A, const double *G, double *I1,
              cudaStream_t s, int *launches) {
   if (!coef4) {
-    if (int r = conv_f64_source(ctx, c, coef, dHF, A, s, launches)) return r;
-    return conv_f64_apply(ctx, c, n, M, coef, dHF, A, G, I1, s, launches);
+    if (int r = conv_f64_source(ctx, c, coef, dHF, A, G, s, launches)) return r;
+    return conv_f64_apply(ctx, c, n, M, coef, dHF, A, G, I1, s, launches, true);
   }
   if (!c.bytes) {
     FEDVR_CK(ctx, conv1_fp64_q4(n, M, coef4, dHF, A, G, I1, s, P<double>(ctx->w_c1f)));
     *launches += conv1_fp64_splits(n, M) > 1 ? 2 : 1;
     return FEDVR_OK;
   }
-  FEDVR_CK(ctx, crt_conv_source4(c, ctx->w_crt.ptr, A, dHF, coef4, s));
+  FEDVR_CK(ctx, crt_conv_source4(c, ctx->w_crt.ptr, A, dHF, G, coef4, s));
   FEDVR_CK(ctx, crt_conv_apply4(c, ctx->w_crt.ptr, G, coef4, I1, ctx->num_sms, s));
   FEDVR_CK(ctx, conv1_fp64_q4(n, M, coef4, dHF, A, G, I1, s, nullptr, P<int>(ctx->w_crt)));
-  *launches += 8;
+  *launches += 10;
   return FEDVR_OK;
 }
 
@@ -212,7 +213,7 @@ int sigma_f64(fedvr_ctx *ctx, const CrtSigma &c, int n, int M, double spin, cons
               const double *G, double *Sigma, cudaStream_t s, int *launches) {
   FEDVR_CK(ctx, sigma2_fp64(n, M, spin, V, G, Sigma, P<double>(ctx->w_t1), P<double>(ctx->w_t2),
                             P<double>(ctx->w_t3), s, &c, ctx->w_crtx.ptr, ctx->num_sms));
-  *launches += c.bytes ? 7 + 5 * ((c.nm + c.group - 1) / c.group) : 4;
+  *launches += c.bytes ? 8 + 6 * ((c.nm + c.group - 1) / c.group) : 4;
   return FEDVR_OK;
 }
 
@@ -233,12 +234,12 @@ int gw_solve(fedvr_ctx *ctx, int n, int M, const double *V, const double *G, dou
   CrtConv plan;
   if (int r = conv_f64_prepare(ctx, n, M, 2, false, &plan)) return r;
   FEDVR_CK(ctx, gw_bubble(n, M, V, G, Q, T1, VQV, s));
-  if (int r = conv_f64_source(ctx, plan, coef, dummy, Q, s, &launches)) return r;
   if (!w_valid) FEDVR_CK(ctx, launch_copy(stack, VQV, w, s));
+  if (int r = conv_f64_source(ctx, plan, coef, dummy, Q, w, s, &launches)) return r;
   double r = 0.0;
   int it = 0;
   for (it = 1; it <= max_iter; ++it) {
-    if (int r = conv_f64_apply(ctx, plan, n, M, coef, dummy, Q, w, C, s, &launches)) return r;
+    if (int r = conv_f64_apply(ctx, plan, n, M, coef, dummy, Q, w, C, s, &launches, it == 1)) return r;
     FEDVR_CK(ctx, launch_copy(stack, VQV, Nw, s));
     FEDVR_CK(ctx, dgemm(false, false, n, n, n, -ctx->spin, V, n, 0, C, n, nn, nullptr, 0, 1.0, Nw,
                         n, nn, M, s));
@@ -284,16 +285,17 @@ int tm_solve(fedvr_ctx *ctx, int n, int M, const double *V, const double *G, dou
   CrtConv plan;
   const bool crt = tm_crt(n, M) && crt_conv_plan(n * n, M, 2, false, ctx->num_sms, &plan) &&
                    ensure_optional(ctx, ctx->w_crt, plan.bytes);
-  if (crt) {
-    FEDVR_CK(ctx, tm_pairs(n, M, G, Y, s));
-    FEDVR_CK(ctx, crt_conv_source(plan, ctx->w_crt.ptr, Y, nullptr, coef, s));
-  }
   FEDVR_CK(ctx, tm_source(n, M, V, G, src, s));
   if (!t_valid) FEDVR_CK(ctx, launch_copy(pstack, src, t, s));
+  if (crt) {
+    FEDVR_CK(ctx, tm_pairs(n, M, G, Y, s));
+    FEDVR_CK(ctx, crt_conv_source(plan, ctx->w_crt.ptr, Y, nullptr, t, coef, s, true));
+  }
   double r = 0.0;
   int it = 0;
   for (it = 1; it <= max_iter; ++it) {
-    if (crt) FEDVR_CK(ctx, crt_conv_apply(plan, ctx->w_crt.ptr, t, coef, Y, ctx->num_sms, s, true));
+    if (crt)
+      FEDVR_CK(ctx, crt_conv_apply(plan, ctx->w_crt.ptr, t, coef, Y, ctx->num_sms, s, it == 1, true));
     FEDVR_CK(ctx, tm_ladder(n, M, coef, G, t, Y, s, crt ? P<int>(ctx->w_crt) : nullptr));
     FEDVR_CK(ctx, cudaMemsetAsync(res_d, 0, sizeof(unsigned long long), s));
     FEDVR_CK(ctx, tm_update(n, M, V, src, Y, t, mixing, res_d, s));

@@ -216,7 +216,8 @@ cudaError_t launch_gw_sigma(long count, double spin, const double *G, const doub
 // t <- (1 - m) t + m (S - V^ Y) with *res = max|t_new - t| (double bits), and
 // Sigma^T = sum_kl [spin t(ak; bl) - t(ak; lb)] g_{M-1-j}(l, k).
 cudaError_t tm_source(int n, int M, const double *V, const double *G, double *S, cudaStream_t s);
-// gate (device int, may be NULL): tm_ladder runs only if *gate != 0. tm_pairs:
+// gate (may be NULL): the flag and marks of crt.cuh; tm_ladder computes what they
+// leave to it. tm_pairs:
 // K_j = g_j (x) g_j, M matrices of n^2 x n^2.
 cudaError_t tm_ladder(int n, int M, const ConvCoef *coef, const double *G, const double *T,
                       double *Y, cudaStream_t s, const int *gate = nullptr);
@@ -262,7 +263,7 @@ cudaError_t launch_sigma_to_f32(int n, int M, const double *S, float *S32, cudaS
 // (conv1_fp64_splits(n, M) - 1) M n n doubles that lets a small launch split
 // the mesh-point range over more CTAs (partial sums added in split order).
 int conv1_fp64_splits(int n, int M);
-// gate (device int, may be NULL): the kernel runs only if *gate != 0.
+// gate (may be NULL): the flag and marks of crt.cuh; the kernel computes what they leave to it.
 cudaError_t conv1_fp64(int n, int M, const ConvCoef *coef, const double *dHF, const double *A,
                        const double *G, double *I1, cudaStream_t s, double *part = nullptr,
                        const int *gate = nullptr);

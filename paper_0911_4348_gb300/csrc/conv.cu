@@ -12,6 +12,7 @@
 // eigen-factor at the lag times the same split-trapezoid weights,
 // I1~ = C^T I1, I2 = C I2~.
 #include "common.cuh"
+#include "crt.cuh"
 #include "tc_sys.cuh"
 
 #include <math.h>
@@ -75,11 +76,13 @@ __global__ void __launch_bounds__(256) conv1_fp64_kernel(int n, int M, int rows,
                                                          double *__restrict__ part,
                                                          const int *__restrict__ gate) {
   extern __shared__ double c1s[];
-  if (gate && *gate == 0) return;
+  const int mode = gate ? *gate : 1;
+  if (mode == 0) return;
   double *Xs = c1s, *Ys = c1s + rows * kC1K;
   const int tiles = (n + rows - 1) / rows;
   for (long blk = blockIdx.x; blk < (long)tiles * M * splits; blk += gridDim.x) {
   const int a0 = (int)(blk % tiles) * rows, i = (int)(blk / tiles % M);
+  if (mode == kCrtSome && !gate[kCrtRows + i]) continue;
   const int nr = min(rows, n - a0), nout = nr * n;
   const long nn = (long)n * n;
   const int tid = threadIdx.x;

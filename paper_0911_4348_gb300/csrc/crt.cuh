@@ -1,8 +1,9 @@
 // FP64 products on the tensor cores by residue arithmetic (a residue number
 // system with a Chinese-remainder reconstruction, the idea of Ozaki, Uchino and
 // Imamura's "Ozaki scheme II", here with our own moduli, interpolation in the
-// residues and kernels): every FP64 operand is rounded to an integer relative to the largest entry of
-// its matrix, the integers are reduced modulo nm pairwise coprime moduli p_m <
+// residues and kernels): every FP64 operand is rounded to an integer relative to
+// power-of-two scales of its mesh point, row and column, the integers are reduced
+// modulo nm pairwise coprime moduli p_m <
 // 256, each modulus' product runs as ONE kind::f16 tensor-core product of small
 // integers whose FP32 sums are exact, and the integer result is rebuilt exactly
 // and rounded to FP64 once. GB300's FP64 pipe issues 2 DFMA per clock and SM
@@ -25,14 +26,28 @@ constexpr int kCrtMod[kCrtMax] = {
     197, 193, 191, 181, 179, 173, 167, 163, 157, 151, 149, 139, 137, 131, 113,
     109, 107, 103, 101, 97,  89,  83,  79,  73,  71,  67,  61,  59,  53};
 
-// Integer bits of a quantised matrix entry, relative to the largest entry of
-// its mesh point's matrix (|x| <= 2^q): at least kCrtQ, and up to kCrtQMax where
-// the moduli that kCrtQ needs leave room. 56 bits keep every entry within 2^-3
-// of the largest exactly and the others to 2^-57 of it. kCrtQC: of a quadrature
-// weight, relative to the largest of its row.
+// Integer bits of a quantised matrix entry, relative to the product of its
+// mesh point's, row's and column's scales (|x| <= 2^q): at least kCrtQ, and up to
+// kCrtQMax where the moduli that kCrtQ needs leave room. 56 bits keep every
+// entry within 2^-3 of that exactly and the others to 2^-57 of it. kCrtQC: of a
+// quadrature weight, relative to the largest of its row.
 constexpr int kCrtQ = 56, kCrtQMax = 58;
 constexpr int kCrtQC = 54;
+// A result matrix whose largest integer has this many bits less than the largest
+// product could have is computed in double arithmetic instead. On the Green's
+// functions of He and H3+ (n = 11 to 118, M = 33 to 961) it has from 6 bits less to 7
+// more in the convolution and from 5 less to 1 more in the exchange; with 10 less
+// what the integers drop is still below 2^-44 of the largest entry for a single
+// product and about 2^-53 for the sums that occur.
+constexpr int kCrtGuard = 10;
 constexpr int kCrtZero = -100000;  // exponent of an all-zero matrix
+constexpr int kCrtNone = -1000000; // exponent of a zero entry
+constexpr int kCrtFar = -20000;    // least exponent of a row or column that is used (an empty one)
+// The workspaces begin with integers: [0] the flag (0: the result stands; 1: an
+// input was not finite, 2: a bounded wait gave up, the FP64 kernel computes all; 4:
+// it computes the matrices marked), [kCrtTicket] blocks of the last kernel that
+// are done, [kCrtRows + i] 1 for a marked matrix.
+constexpr int kCrtSome = 4, kCrtTicket = 1, kCrtRows = 64;
 
 // Per-modulus constants of the residue kernels (passed by value).
 struct CrtMods {
@@ -81,23 +96,26 @@ struct CrtConv {
   int q;     // integer bits of a matrix entry
   int Mp;    // pitch of the weight table (zero entries from M on)
   int nm, CT, Np, RT, S, ncR;
-  size_t o_exps, o_expg, o_E, o_S, o_B, o_C, o_R, bytes;
+  size_t o_exps, o_expg, o_E, o_er, o_size, o_sm, o_S, o_B, o_C, o_R, bytes;
 };
 // false: outside what the kernel takes (sizes, 32-bit offsets, workspace limit).
 bool crt_conv_plan(int n, int M, int np, bool ext, int num_sms, CrtConv *out);
-// ws: plan.bytes of device memory; its first int is the fallback flag (non-zero:
-// an input was not finite or a bounded wait gave up; the caller's FP64 kernel
-// then computes the result).
+// ws: plan.bytes of device memory beginning with the flag and the marks (kCrtSome);
+// the caller's FP64 kernel follows and computes what they leave to it.
 // Source stack A (and, with ext, the diagonal operands from dHF and the end
-// weights): residues into ws. Resets the flag.
+// weights): scales and residues into ws. G: the stack it will be applied to first,
+// against which the contraction index is balanced. Resets the flag. transposed: the
+// matrices of G are stored transposed.
 cudaError_t crt_conv_source(const CrtConv &c, void *ws, const double *A, const double *dHF,
-                            const ConvCoef *coef, cudaStream_t s);
+                            const double *G, const ConvCoef *coef, cudaStream_t s,
+                            bool transposed = false);
 cudaError_t crt_conv_source4(const CrtConv &c, void *ws, const double *A, const double *dHF,
-                             const ConvCoef4 *coef, cudaStream_t s);
-// I1 = table applied to (A, G); transposed: the matrices of G and I1 are stored
-// transposed.
+                             const double *G, const ConvCoef4 *coef, cudaStream_t s);
+// I1 = table applied to (A, G); fresh: G is the one the source was given (its scales
+// are in ws); transposed: the matrices of G and I1 are stored transposed.
 cudaError_t crt_conv_apply(const CrtConv &c, void *ws, const double *G, const ConvCoef *coef,
-                           double *I1, int num_sms, cudaStream_t s, bool transposed = false);
+                           double *I1, int num_sms, cudaStream_t s, bool fresh,
+                           bool transposed = false);
 cudaError_t crt_conv_apply4(const CrtConv &c, void *ws, const double *G, const ConvCoef4 *coef,
                             double *I1, int num_sms, cudaStream_t s);
 

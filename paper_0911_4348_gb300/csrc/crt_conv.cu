@@ -3,11 +3,24 @@
 // Eq. deq), the periodic convolutions of GW's screened interaction, and the
 // four-row table of the fourth-order variant.
 //
-// Integers: Sigma_k and g_j are rounded to 56 bits relative to the largest
-// entry of each mesh point's matrix, the weights c_p(i, j) (with the matrices'
-// exponents folded in) to 54 bits relative to the largest weight of row i. The
-// triple product c Sigma g summed over (j, c) is then an integer below
-// 2^(166 + log2(np M n)), held exactly by its residues modulo 23 to 26 moduli.
+// Integers: entry (a, c) of Sigma_k is rounded to 56 bits relative to 2^(e_k + r_a +
+// t_c) and entry (c, b) of g_j relative to 2^(f_j - t_c + s_b), the weights c_p(i, j)
+// (with e_k and f_j folded in) to 54 bits relative to the largest weight of row i.
+// e_k, f_j are the exponents of the mesh points' matrices; r_a and s_b those of
+// their rows and columns over all mesh points, which leave the sum and are
+// applied to the result; t_c balances the columns of Sigma against the rows of g,
+// and cancels. So scaling rows, columns or the contraction index (or single mesh
+// points) by powers of two changes no bit that is kept, as in double arithmetic;
+// with one exponent per matrix such inputs lost their small rows and columns, and
+// a contraction index scaled one way in Sigma and the other in g lost everything.
+// The triple product c Sigma g summed over (j, c) is then an integer below
+// 2^(166 + log2(np M n)), held exactly by its residues modulo 23 to 25 moduli.
+//
+// What this keeps of an entry (a, b) is relative to the largest products of row a and
+// column b at any mesh point, not to the entry: entries far below both (a
+// Green's function that decays away from its diagonal) have fewer correct bits than
+// from the FP64 kernel. A result whose largest integer is 2^10 below the largest
+// product (mark_small) is left to the FP64 kernel.
 // The interpolation is done in the residues: for each modulus the A operand
 // sum_p c_p s_p of small integers is formed by the CUDA cores (dp2a on byte
 // pairs), reduced and written as FP16, the B operand is the residue plane of g,
@@ -163,31 +176,160 @@ __global__ void __launch_bounds__(256) crt_exp_kernel(long nn, int M, const doub
   }
 }
 
+// Largest exponent of each entry over the mesh points, relative to the matrices'
+// own: sm [n n] of the source stack (its ext diagonal operands too), gm [n n] of G as
+// stored. `chunk` matrices per block row, the source's first.
+template <typename Coef>
+__global__ void __launch_bounds__(256)
+    crt_entry_kernel(long nn, int M, int Ks, int chunk, const double *__restrict__ A,
+                     const double *__restrict__ dHF, const Coef *__restrict__ coef,
+                     const int *__restrict__ es, const double *__restrict__ G,
+                     const int *__restrict__ eg, int *__restrict__ sm, int *__restrict__ gm) {
+  const long x = (long)blockIdx.x * 256 + threadIdx.x;
+  if (x >= nn) return;
+  const int sc = (Ks + chunk - 1) / chunk;
+  const bool src = (int)blockIdx.y < sc;
+  const int k0 = (src ? blockIdx.y : blockIdx.y - sc) * chunk, k1 = min(src ? Ks : M, k0 + chunk);
+  const double *X = src ? A : G;
+  const int *ex = src ? es : eg;
+  int m = kCrtNone;
+  auto note = [&](double v, int e) {
+    if (e != kCrtZero && v != 0.0) m = max(m, exponent_of(v) - e);
+  };
+#pragma unroll 8
+  for (int k = k0; k < min(k1, M); ++k) note(X[(long)k * nn + x], ex[k]);
+  if (k1 > M) {
+    const double s0 = A[x], s1 = A[(long)(M - 1) * nn + x], h = dHF[x];
+#pragma unroll 8
+    for (int k = max(k0, M); k < k1; ++k) {
+      const double2 w = diag_weights(coef[(long)(k - M) * M + (k - M)]);
+      note(diag_elem(w.x, w.y, s0, s1, h), ex[k]);
+    }
+  }
+  if (m > kCrtNone) atomicMax((src ? sm : gm) + x, m);
+}
+// Matrices per block row of the passes over the mesh points: many blocks, but few
+// enough atomics.
+inline int entry_chunk(long nn) { return nn < 4096 ? 8 : 32; }
+
+// Exponents r_a of the rows of the source, t_c of the contraction index and s_b of
+// the columns of G from the entries' (at most 0, or "none" far below): t_c moves
+// half the distance between what column c of the source and row c of G leave
+// unused, at most three times. Any t_c is right, since r_a and s_b are the largest of
+// what remains. One CTA.
+constexpr int kEquil = 3;
+template <bool TR>
+__global__ void __launch_bounds__(1024)
+    crt_equil_kernel(int n, const int *__restrict__ sm, const int *__restrict__ gm,
+                     int *__restrict__ er, int *__restrict__ et, int *__restrict__ ec,
+                     int *__restrict__ nt) {
+  extern __shared__ int es_[];
+  int *r = es_, *t = r + n, *s = t + n, *cs = s + n, *rg = cs + n;
+  const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
+  const long nn = (long)n * n;
+  // the largest of f(row, col) over the columns of each row, and over the rows of each column
+  auto rows = [&](const int *m, int *out, auto f) {
+    for (int a = wp; a < n; a += 32) {
+      int v = 2 * kCrtNone;
+      for (int c = lane; c < n; c += 32) v = max(v, f(m[(long)a * n + c], a, c));
+      v = __reduce_max_sync(0xffffffffu, v);
+      if (lane == 0) out[a] = v;
+    }
+  };
+  auto cols = [&](const int *m, int *out, auto f) {
+    for (int c = tid; c < n; c += 1024) out[c] = 2 * kCrtNone;
+    __syncthreads();
+    int a = tid / n, c = tid % n;
+    for (long x = tid; x < nn; x += 1024) {
+      const int v = f(m[x], a, c);
+      if (v > out[c]) atomicMax(out + c, v);
+      a += 1024 / n;
+      c += 1024 % n;
+      if (c >= n) c -= n, ++a;
+    }
+  };
+  for (int c = tid; c < n; c += 1024) t[c] = 0;
+  __syncthreads();
+  for (int it = 0;; ++it) {
+    rows(sm, r, [&](int e, int, int c) { return e - t[c]; });
+    if constexpr (TR) rows(gm, s, [&](int e, int, int c) { return e + t[c]; });
+    else cols(gm, s, [&](int e, int c, int) { return e + t[c]; });
+    __syncthreads();
+    for (int c = tid; c < n; c += 1024) {  // empty rows and columns
+      r[c] = max(r[c], kCrtFar);
+      s[c] = max(s[c], kCrtFar);
+    }
+    __syncthreads();
+    if (it == kEquil) break;
+    cols(sm, cs, [&](int e, int a, int) { return e - r[a]; });
+    if constexpr (TR) cols(gm, rg, [&](int e, int b, int) { return e - s[b]; });
+    else rows(gm, rg, [&](int e, int, int b) { return e - s[b]; });
+    __syncthreads();
+    bool moved = false;
+    for (int c = tid; c < n; c += 1024) {
+      // an empty column of the source meets nothing: its row of G is rounded away. A
+      // row of G that is empty now (a later G may fill it) leaves all to the source
+      const int us = cs[c] - t[c], ug = rg[c] + t[c];  // <= 0
+      const int to = cs[c] < kCrtNone / 2 ? kCrtFar : t[c] + (rg[c] < kCrtNone / 2 ? us : (us - ug) / 2);
+      moved |= to != t[c];
+      t[c] = to;
+    }
+    if (!__syncthreads_or(moved)) break;
+  }
+  for (int c = tid; c < n; c += 1024) {
+    er[c] = r[c];
+    et[c] = t[c];
+    ec[c] = s[c];
+    nt[c] = -t[c];
+  }
+}
+
+// s_b of another G with the same t_c: ec[b] = max over j, c of the exponent of
+// g_j[c][b] relative to its matrix, plus t_c.
+template <bool TR>
+__global__ void __launch_bounds__(256)
+    crt_column_kernel(int n, int M, int chunk, const double *__restrict__ G, const int *__restrict__ eg,
+                      const int *__restrict__ et, int *__restrict__ ec) {
+  const long nn = (long)n * n, x = (long)blockIdx.x * 256 + threadIdx.x;
+  if (x >= nn) return;
+  const int k0 = blockIdx.y * chunk, k1 = min(M, k0 + chunk);
+  int m = kCrtNone;
+#pragma unroll 8
+  for (int k = k0; k < k1; ++k) {
+    const double v = G[(long)k * nn + x];
+    const int e = eg[k];
+    if (e != kCrtZero && v != 0.0) m = max(m, exponent_of(v) - e);
+  }
+  if (m == kCrtNone) return;
+  const int c = (int)(TR ? x % n : x / n), b = (int)(TR ? x / n : x % n);
+  m += et[c];
+  if (m > *reinterpret_cast<volatile int *>(ec + b)) atomicMax(ec + b, m);
+}
+
 // Residues of the source stack as bytes: planes [m][k][n nc] in the order of
 // src_off, four columns per thread.
 template <typename Coef>
 __global__ void __launch_bounds__(256)
     crt_source_kernel(CrtMods mods, CrtK kk, int qb, long plane, const double *__restrict__ A,
-                      const double *__restrict__ dHF, const Coef *__restrict__ coef,
-                      const int *__restrict__ expo, uint32_t *__restrict__ out) {
+                      const double *__restrict__ dHF, const Coef *__restrict__ coef, CrtScale sc,
+                      uint32_t *__restrict__ out) {
   const int k = blockIdx.y, n = kk.n, M = kk.M;
   const int q4 = kk.nc / 4;
   const int t = blockIdx.x * 256 + threadIdx.x;
   if (t >= n * q4) return;
   const int a = t / q4, c0 = (t % q4) * 4;
   const long nn = (long)n * n;
-  const int e = expo[k];
   double2 w = make_double2(0.0, 0.0);
   if (k >= M) w = diag_weights(coef[(long)(k - M) * M + (k - M)]);
   long long x[4];
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     x[q] = 0;
-    if (c0 + q < n && e != kCrtZero) {
+    if (c0 + q < n) {
       const long off = (long)a * n + c0 + q;
       const double v = k < M ? A[(long)k * nn + off]
                              : diag_elem(w.x, w.y, A[off], A[(long)(M - 1) * nn + off], dHF[off]);
-      x[q] = quantise(v, qb - e);
+      x[q] = quantise(v, qb - scale_at(sc, k, a, c0 + q));
     }
   }
   put_source(mods, kk, plane, k, a, c0, x, out);
@@ -234,9 +376,19 @@ __global__ void __launch_bounds__(256) crt_coef_kernel(CrtMods mods, int M, int 
                                                        const Coef *__restrict__ coef,
                                                        const int *__restrict__ es,
                                                        const int *__restrict__ eg, int *__restrict__ E,
+                                                       int *__restrict__ head, int *__restrict__ size,
                                                        CrtEntry<NP> *__restrict__ out) {
   __shared__ int sh[8];
   const int i = blockIdx.x;
+  if (threadIdx.x == 0) {  // the marks of the last apply
+    if (i < M) {
+      head[kCrtRows + i] = 0;
+      size[i] = kCrtNone;
+    } else {
+      head[kCrtTicket] = 0;
+      atomicCAS(head, kCrtSome, 0);
+    }
+  }
   for (int x = threadIdx.x + (i < M ? M : 0); x < Mp; x += 256)
     for (int m = 0; m < mods.nm; ++m) out[((long)m * (M + 1) + i) * Mp + x] = CrtEntry<NP>{};
   if (i == M) return;
@@ -253,7 +405,7 @@ __global__ void __launch_bounds__(256) crt_coef_kernel(CrtMods mods, int M, int 
   __syncthreads();
   for (int w = 0; w < 8; ++w) mx = max(mx, sh[w]);
   const int Ei = mx == kCrtZero ? 0 : mx;
-  if (threadIdx.x == 0) E[i] = Ei;
+  if (threadIdx.x == 0) E[i] = mx;  // kCrtZero: no product that is not zero
   for (int j = threadIdx.x; j < M; j += 256) {
     const EntryView v = entry_view(coef[(long)i * M + j], M, i);
     uint32_t a0[NP], a1[NP], a2[NP];
@@ -663,12 +815,16 @@ __global__ void __launch_bounds__(256) crt_rebuild_kernel(const __grid_constant_
                                                           long rows, int ncR, int S,
                                                           const int8_t *__restrict__ R,
                                                           const int *__restrict__ E,
-                                                          const int *__restrict__ flag, int qb,
-                                                          bool tr, double *__restrict__ out) {
-  if (*flag) return;
+                                                          const int *__restrict__ er,
+                                                          const int *__restrict__ ec, int *head,
+                                                          int *__restrict__ size, int qb, bool tr,
+                                                          double *__restrict__ out) {
+  if (*reinterpret_cast<volatile int *>(head)) return;
   const long plane = rows * ncR;
   const long total = rows * n;
-  for (long x = (long)blockIdx.x * 256 + threadIdx.x; x < total; x += (long)gridDim.x * 256) {
+  const long x0 = total * blockIdx.x / gridDim.x, x1 = total * (blockIdx.x + 1) / gridDim.x;
+  CrtSize big;
+  for (long x = x0 + threadIdx.x; x < x1; x += 256) {
     const long row = x / n;
     const int col = (int)(x - row * n);
     const int8_t *r = R + row * ncR + col;
@@ -686,48 +842,82 @@ __global__ void __launch_bounds__(256) crt_rebuild_kernel(const __grid_constant_
     const int q = (int)rintf(f);
 #pragma unroll
     for (int i = 0; i < W; ++i) acc[i] -= (long long)q * (long long)t.P[i];
-    const long o = tr ? (row / n) * n * n + (long)col * n + row % n : x;
-    out[o] = crt_value<W>(acc, E[row / n] - kCrtQC - 2 * qb);
+    const int i = (int)(row / n), a = (int)(row - (long)i * n);
+    const long o = tr ? (long)i * n * n + (long)col * n + a : x;
+    int e;
+    out[o] = crt_value<W>(acc, E[i] + max(er[a], kCrtFar) + max(ec[col], kCrtFar) - kCrtQC - 2 * qb, &e);
+    big.note(size, i, e);
   }
+  big.finish(size);
+  mark_small(head, size, (int)(rows / n), kCrtQC + 2 * qb - kCrtGuard, [&](int i) { return E[i] != kCrtZero; });
+}
+
+// The workspace's small arrays.
+struct ConvWs {
+  int *head, *es, *eg, *E, *er, *et, *ec, *nt, *size, *sm, *gm;
+};
+ConvWs conv_ws(const CrtConv &c, void *wsv) {
+  uint8_t *ws = reinterpret_cast<uint8_t *>(wsv);
+  auto at = [&](size_t o) { return reinterpret_cast<int *>(ws + o); };
+  const long n = c.k.n;
+  int *er = at(c.o_er), *sm = at(c.o_sm);
+  return {at(0), at(c.o_exps), at(c.o_expg), at(c.o_E), er, er + n, er + 2 * n, er + 3 * n,
+          at(c.o_size), sm, sm + n * n};
 }
 
 template <typename Coef>
-cudaError_t source_t(const CrtConv &c, void *wsv, const double *A, const double *dHF,
-                     const Coef *coef, cudaStream_t s) {
+cudaError_t source_t(const CrtConv &c, void *wsv, const double *A, const double *dHF, const double *G,
+                     const Coef *coef, cudaStream_t s, bool tr) {
   uint8_t *ws = reinterpret_cast<uint8_t *>(wsv);
-  int *flag = reinterpret_cast<int *>(ws);
-  int *es = reinterpret_cast<int *>(ws + c.o_exps);
+  const ConvWs w = conv_ws(c, wsv);
   const int n = c.k.n, M = c.k.M;
-  cudaError_t e = cudaMemsetAsync(flag, 0, sizeof(int), s);
-  if (e != cudaSuccess) return e;
-  crt_exp_kernel<Coef><<<c.KS, 256, 0, s>>>((long)n * n, M, A, dHF, coef, es, flag);
+  const long nn = (long)n * n;
   // matrices beyond 2 M (padding rows of the last diagonal entries) are never
   // weighted; they need no residues
-  dim3 grid((unsigned)((n * (c.k.nc / 4) + 255) / 256), (unsigned)(c.ext ? 2 * M : M));
+  const int Ks = c.ext ? 2 * M : M;
+  cudaError_t e = cudaMemsetAsync(w.head, 0, 2 * sizeof(int), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(w.sm, 0x80, 2 * nn * sizeof(int), s);  // far below kCrtNone
+  if (e != cudaSuccess) return e;
+  crt_exp_kernel<Coef><<<c.KS, 256, 0, s>>>(nn, M, A, dHF, coef, w.es, w.head);
+  crt_exp_stack_kernel<<<M, 256, 0, s>>>(nn, G, w.eg, w.head);
+  const int ch = entry_chunk(nn);
+  const dim3 ge((unsigned)((nn + 255) / 256), (unsigned)((Ks + ch - 1) / ch + (M + ch - 1) / ch));
+  crt_entry_kernel<Coef><<<ge, 256, 0, s>>>(nn, M, Ks, ch, A, dHF, coef, w.es, G, w.eg, w.sm, w.gm);
+  const size_t sm = 5 * (size_t)n * sizeof(int);
+  if (tr) crt_equil_kernel<true><<<1, 1024, sm, s>>>(n, w.sm, w.gm, w.er, w.et, w.ec, w.nt);
+  else crt_equil_kernel<false><<<1, 1024, sm, s>>>(n, w.sm, w.gm, w.er, w.et, w.ec, w.nt);
+  dim3 grid((unsigned)((n * (c.k.nc / 4) + 255) / 256), (unsigned)Ks);
   crt_source_kernel<Coef><<<grid, 256, 0, s>>>(crt_mods(c.nm, false), c.k, c.q,
-                                               (long)c.KS * n * c.k.nc, A, dHF, coef, es,
+                                               (long)c.KS * n * c.k.nc, A, dHF, coef,
+                                               CrtScale{w.es, w.er, w.et, 0, 0},
                                                reinterpret_cast<uint32_t *>(ws + c.o_S));
   return cudaGetLastError();
 }
 
 template <typename Coef, int NP>
 cudaError_t apply_t(const CrtConv &c, void *wsv, const double *G, const Coef *coef, double *I1,
-                    int num_sms, cudaStream_t s, bool tr) {
+                    int num_sms, cudaStream_t s, bool tr, bool fresh) {
   uint8_t *ws = reinterpret_cast<uint8_t *>(wsv);
-  int *flag = reinterpret_cast<int *>(ws);
-  int *es = reinterpret_cast<int *>(ws + c.o_exps), *eg = reinterpret_cast<int *>(ws + c.o_expg);
-  int *E = reinterpret_cast<int *>(ws + c.o_E);
+  const ConvWs w = conv_ws(c, wsv);
   const int n = c.k.n, M = c.k.M;
-  crt_exp_stack_kernel<<<M, 256, 0, s>>>((long)n * n, G, eg, flag);
+  const long nn = (long)n * n;
+  if (!fresh) {
+    cudaError_t e = cudaMemsetAsync(w.ec, 0x80, n * sizeof(int), s);
+    if (e != cudaSuccess) return e;
+    crt_exp_stack_kernel<<<M, 256, 0, s>>>(nn, G, w.eg, w.head);
+    const int ch = entry_chunk(nn);
+    const dim3 ge((unsigned)((nn + 255) / 256), (unsigned)((M + ch - 1) / ch));
+    if (tr) crt_column_kernel<true><<<ge, 256, 0, s>>>(n, M, ch, G, w.eg, w.et, w.ec);
+    else crt_column_kernel<false><<<ge, 256, 0, s>>>(n, M, ch, G, w.eg, w.et, w.ec);
+  }
   const dim3 gg(M + 3, (n + 31) / 32, (c.k.nc + 63) / 64);
-  if (tr)
-    crt_g_kernel<true><<<gg, 256, 0, s>>>(crt_mods(c.nm, true), c.k, c.q, G, eg,
-                                          reinterpret_cast<uint32_t *>(ws + c.o_B), nullptr, 0, 0);
-  else
-    crt_g_kernel<false><<<gg, 256, 0, s>>>(crt_mods(c.nm, true), c.k, c.q, G, eg,
-                                           reinterpret_cast<uint32_t *>(ws + c.o_B), nullptr, 0, 0);
+  const CrtScale sg{w.eg, w.nt, w.ec, 0, 0};
+  uint32_t *const B = reinterpret_cast<uint32_t *>(ws + c.o_B);
+  if (tr) crt_g_kernel<true, false><<<gg, 256, 0, s>>>(crt_mods(c.nm, true), c.k, c.q, G, sg, B, 0, 0);
+  else crt_g_kernel<false, false><<<gg, 256, 0, s>>>(crt_mods(c.nm, true), c.k, c.q, G, sg, B, 0, 0);
   crt_coef_kernel<Coef, NP><<<M + 1, 256, 0, s>>>(crt_mods(c.nm, false), M, c.Mp,
-                                                  (uint32_t)(n * c.k.nc), coef, es, eg, E,
+                                                  (uint32_t)(n * c.k.nc), coef, w.es, w.eg, w.E,
+                                                  w.head, w.size,
                                                   reinterpret_cast<CrtEntry<NP> *>(ws + c.o_C));
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
@@ -755,7 +945,7 @@ cudaError_t apply_t(const CrtConv &c, void *wsv, const double *G, const Coef *co
     a.p[m] = (float)kCrtMod[m];
     a.ip[m] = 1.0f / (float)kCrtMod[m];
   }
-  a.flag = flag;
+  a.flag = w.head;
   const size_t smem = 1024 + (size_t)a.nst * stage + 256;
   e = cudaFuncSetAttribute(crt_conv_kernel<NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -765,8 +955,8 @@ cudaError_t apply_t(const CrtConv &c, void *wsv, const double *G, const Coef *co
   if (e != cudaSuccess) return e;
   const long total = (long)M * n * n;
   crt_rebuild_kernel<7><<<(unsigned)std::min<long>((total + 255) / 256, 152 * 16), 256, 0, s>>>(
-      crt_words<7>(c.nm), n, (long)M * n, c.ncR, c.S, reinterpret_cast<const int8_t *>(ws + c.o_R), E,
-      flag, c.q, tr, I1);
+      crt_words<7>(c.nm), n, (long)M * n, c.ncR, c.S, reinterpret_cast<const int8_t *>(ws + c.o_R), w.E,
+      w.er, w.ec, w.head, w.size, c.q, tr, I1);
   return cudaGetLastError();
 }
 
@@ -809,7 +999,8 @@ bool crt_conv_plan(int n, int M, int np, bool ext, int num_sms, CrtConv *out) {
       c.S = S;
     }
   }
-  size_t o = 256;
+  size_t o = (size_t)(kCrtRows + M) * 4;
+  o = (o + 255) / 256 * 256;
   auto take = [&](size_t bytes) {
     const size_t at = o;
     o += (bytes + 255) / 256 * 256;
@@ -818,6 +1009,9 @@ bool crt_conv_plan(int n, int M, int np, bool ext, int num_sms, CrtConv *out) {
   c.o_exps = take((size_t)c.KS * 4);
   c.o_expg = take((size_t)M * 4);
   c.o_E = take((size_t)M * 4);
+  c.o_er = take(4 * (size_t)n * 4);
+  c.o_size = take((size_t)M * 4);
+  c.o_sm = take(2 * (size_t)n * n * 4);
   c.o_S = take((size_t)c.nm * c.KS * n * c.k.nc);
   c.o_B = take((size_t)c.nm * n * c.k.KP * 2);
   c.o_C = take((size_t)c.nm * (M + 1) * c.Mp * (np == 4 ? 16 : 8));
@@ -829,20 +1023,20 @@ bool crt_conv_plan(int n, int M, int np, bool ext, int num_sms, CrtConv *out) {
 }
 
 cudaError_t crt_conv_source(const CrtConv &c, void *ws, const double *A, const double *dHF,
-                            const ConvCoef *coef, cudaStream_t s) {
-  return source_t<ConvCoef>(c, ws, A, dHF, coef, s);
+                            const double *G, const ConvCoef *coef, cudaStream_t s, bool transposed) {
+  return source_t<ConvCoef>(c, ws, A, dHF, G, coef, s, transposed);
 }
 cudaError_t crt_conv_source4(const CrtConv &c, void *ws, const double *A, const double *dHF,
-                             const ConvCoef4 *coef, cudaStream_t s) {
-  return source_t<ConvCoef4>(c, ws, A, dHF, coef, s);
+                             const double *G, const ConvCoef4 *coef, cudaStream_t s) {
+  return source_t<ConvCoef4>(c, ws, A, dHF, G, coef, s, false);
 }
 cudaError_t crt_conv_apply(const CrtConv &c, void *ws, const double *G, const ConvCoef *coef,
-                           double *I1, int num_sms, cudaStream_t s, bool transposed) {
-  return apply_t<ConvCoef, 2>(c, ws, G, coef, I1, num_sms, s, transposed);
+                           double *I1, int num_sms, cudaStream_t s, bool fresh, bool transposed) {
+  return apply_t<ConvCoef, 2>(c, ws, G, coef, I1, num_sms, s, transposed, fresh);
 }
 cudaError_t crt_conv_apply4(const CrtConv &c, void *ws, const double *G, const ConvCoef4 *coef,
                             double *I1, int num_sms, cudaStream_t s) {
-  return apply_t<ConvCoef4, 4>(c, ws, G, coef, I1, num_sms, s, false);
+  return apply_t<ConvCoef4, 4>(c, ws, G, coef, I1, num_sms, s, false, true);
 }
 
 }  // namespace fedvr

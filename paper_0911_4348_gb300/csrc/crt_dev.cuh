@@ -38,11 +38,29 @@ __device__ __forceinline__ void split21(long long x, uint32_t &a0, uint32_t &a1,
 __device__ __forceinline__ double pow2d(int e) {  // 2^e for -1022 <= e <= 1023
   return __longlong_as_double((long long)(e + 1023) << 52);
 }
-// x 2^s to the nearest integer (|result| <= 2^60 by the caller's choice of s;
-// the scale is applied in two factors so that neither leaves the range)
+// x 2^s to the nearest integer (|result| <= 2^60 by the caller's choice of s).
+// The scale is applied in two factors so that neither leaves the range; beyond
+// +-1200 it only meets zeros and values that round to zero.
 __device__ __forceinline__ long long quantise(double x, int s) {
+  s = max(-1200, min(1200, s));
   const int h = s / 2;
   return __double2ll_rn(x * pow2d(h) * pow2d(s - h));
+}
+// e with 2^(e - 1) <= |x| < 2^e for a finite x that is not zero, kCrtNone for zero.
+__device__ __forceinline__ int exponent_of(double x) {
+  const int f = (__double2hiint(x) >> 20) & 0x7ff;
+  return f ? f - 1022 : x != 0.0 ? ilogb(x) + 1 : kCrtNone;
+}
+
+// Exponent subtracted from entry (r, c) of matrix j before it is rounded:
+// base[j] + row[j srow + r] + col[j scol + c]. base may be NULL (zero).
+struct CrtScale {
+  const int *base, *row, *col;
+  long srow, scol;
+};
+__device__ __forceinline__ int scale_at(const CrtScale &s, int j, int r, int c) {
+  return (s.base ? s.base[j] : 0) + max(s.row[j * s.srow + r], kCrtFar) +
+         max(s.col[j * s.scol + c], kCrtFar);
 }
 
 // v mod p on a packed pair of exact integers.
@@ -141,35 +159,36 @@ __device__ __forceinline__ uint32_t pack16(float r0, float r1) {
   }
 }
 
-// Residue planes of g as FP16 rows over the flattened contraction index:
-// out[m][b][x(j, c)] = g_j[c][b] (times mods.mul). With nat, also as plain
-// bfloat16 rows nat[m][j][b][c] ([nr] rows of ph values). A 64 (c) x 32 (b) tile of
+// Residue planes of g over the contraction index, entry (c, b) rounded relative to
+// scale_at(sc, j, c, b). NAT false: FP16 rows over the flattened contraction index,
+// out[m][b][x(j, c)] = g_j[c][b] (times mods.mul). NAT true: plain bfloat16 rows
+// out[m][j][b][c] ([nr] rows of ph values). A 64 (c) x 32 (b) tile of
 // one mesh point per CTA, transposed through shared memory. CTAs j >= M
 // write the zeros that pad the last chunk of each rest. TR: the matrices are given
 // transposed (G[j][b][c]).
-template <bool TR>
+template <bool TR, bool NAT>
 static __global__ void __launch_bounds__(256) crt_g_kernel(CrtMods mods, CrtK k, int qb,
-                                                    const double *__restrict__ G,
-                                                    const int *__restrict__ expo,
-                                                    uint32_t *__restrict__ out,
-                                                    uint32_t *__restrict__ nat, int nr, int ph) {
+                                                    const double *__restrict__ G, CrtScale sc,
+                                                    uint32_t *__restrict__ out, int nr, int ph) {
   __shared__ long long sh[64][33];
   const int j = blockIdx.x, b0 = blockIdx.y * 32, c0 = blockIdx.z * 64;
-  const int n = k.n, e = j < k.M ? expo[j] : kCrtZero;
+  const int n = k.n;
   const double *g = G + (long)j * n * n;
   for (int q = threadIdx.x; q < 64 * 32; q += 256) {
     const int c = TR ? q & 63 : q >> 5, b = TR ? q >> 6 : q & 31;
     long long x = 0;
-    if (e != kCrtZero && c0 + c < n && b0 + b < n)
-      x = quantise(TR ? g[(long)(b0 + b) * n + c0 + c] : g[(long)(c0 + c) * n + b0 + b], qb - e);
+    if (j < k.M && c0 + c < n && b0 + b < n)
+      x = quantise(TR ? g[(long)(b0 + b) * n + c0 + c] : g[(long)(c0 + c) * n + b0 + b],
+                   qb - scale_at(sc, j, c0 + c, b0 + b));
     sh[c][b] = x;
   }
   __syncthreads();
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-  const long plane = (long)n * k.KP / 2;  // half2 words per modulus
+  const long plane = (long)n * k.KP / 2;  // half2 words per modulus (NAT false)
   const int c = c0 + 2 * lane;
   if (c >= k.nc) return;
   if (j >= k.M) {  // the mesh points that pad the last chunk of a rest: zeros
+    if (NAT) return;
     const int r = c - 64 * k.full;
     if (r < 0 || j >= (k.n2 && r < 32 ? 2 * k.n2 : 4 * k.n1)) return;
   }
@@ -177,12 +196,11 @@ static __global__ void __launch_bounds__(256) crt_g_kernel(CrtMods mods, CrtK k,
     uint32_t a0[2], a1[2], a2[2];
     split21(sh[2 * lane][bb], a0[0], a1[0], a2[0]);
     split21(sh[2 * lane + 1][bb], a0[1], a1[1], a2[1]);
-    const long o = ((long)(b0 + bb) * k.KP + crt_x(k, j, c)) / 2;
+    const long o = NAT ? (((long)j * nr + b0 + bb) * ph + c) / 2
+                       : ((long)(b0 + bb) * k.KP + crt_x(k, j, c)) / 2;
     for (int m = 0; m < mods.nm; ++m) {
       const float x0 = residue(a0[0], a1[0], a2[0], mods, m), x1 = residue(a0[1], a1[1], a2[1], mods, m);
-      out[(long)m * plane + o] = pack16<false>(x0, x1);
-      if (nat && j < k.M)
-        nat[((((long)m * k.M + j) * nr + b0 + bb) * ph + c) / 2] = pack16<true>(x0, x1);
+      out[(long)m * (NAT ? (long)k.M * nr * ph / 2 : plane) + o] = pack16<NAT>(x0, x1);
     }
   }
 }
@@ -198,10 +216,11 @@ __device__ __forceinline__ void combine4(uint32_t w0, uint32_t w1, uint32_t c01,
   acc[3] = __dp2a_hi((int)c01, (int)hi, acc[3]);
 }
 
-// Exact integer from its (inverse-folded) residues, rounded to FP64 and scaled:
-// X = sum_m t_m (P / p_m) - round(sum_m t_m / p_m) P.
+// Exact integer from its (inverse-folded) residues, rounded to FP64 and scaled by
+// 2^scale: X = sum_m t_m (P / p_m) - round(sum_m t_m / p_m) P. *size: e with |X| < 2^e, or
+// kCrtNone.
 template <int W>
-__device__ __forceinline__ double crt_value(long long (&acc)[W], int scale) {
+__device__ __forceinline__ double crt_value(long long (&acc)[W], int scale, int *size) {
   uint32_t w[W];
   long long carry = 0;
 #pragma unroll
@@ -239,6 +258,7 @@ __device__ __forceinline__ double crt_value(long long (&acc)[W], int scale) {
       sticky |= w[i] != 0;
     }
   }
+  *size = kCrtNone;
   if (pos < 0) return 0.0;
   const int lz = __clz(a);
   uint64_t top = ((uint64_t)a << 32) | b;
@@ -249,8 +269,55 @@ __device__ __forceinline__ double crt_value(long long (&acc)[W], int scale) {
     sticky |= c != 0;
   }
   top |= sticky ? 1u : 0u;
+  *size = 32 * (pos + 1) - lz;
   const double v = scalbn(__ull2double_rn(top), 32 * (pos - 1) - lz + scale);
   return neg ? -v : v;
+}
+
+// Largest exponent of the integers of each result matrix, and the matrices left
+// to double arithmetic. What the integers hold of an entry is relative to the
+// largest products of its row and its column, so a result whose largest integer
+// is 2^guard below the largest a single product can be (operands whose large
+// entries never meet, or a sum that cancels) is computed again by the FP64 kernel
+// that follows, matrix by matrix.
+// A thread of a rebuild kernel goes through entries of ascending matrix i.
+struct CrtSize {
+  int i = -1, m = kCrtNone;
+  __device__ __forceinline__ void flush(int *size) {
+    if (m > kCrtNone) atomicMax(size + i, m);
+  }
+  __device__ __forceinline__ void note(int *size, int at, int e) {
+    if (at != i) {
+      flush(size);
+      i = at;
+      m = kCrtNone;
+    }
+    m = max(m, e);
+  }
+  // all threads of the block, at the end
+  __device__ __forceinline__ void finish(int *size) {
+    const int i0 = __reduce_max_sync(0xffffffffu, i);
+    if (i != i0) flush(size);
+    const int w = __reduce_max_sync(0xffffffffu, i == i0 ? m : kCrtNone);
+    if ((threadIdx.x & 31) == 0 && w > kCrtNone) atomicMax(size + i0, w);
+  }
+};
+// The last block to arrive marks the matrices i < M with some(i) (an operand product
+// that is not zero) and size[i] < least. head: the workspace's first integers.
+template <typename F>
+__device__ __forceinline__ void mark_small(int *head, const int *size, int M, int least, F some) {
+  __shared__ bool last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(head + kCrtTicket, 1) == (int)gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  for (int i = threadIdx.x; i < M; i += blockDim.x)
+    if (some(i) && *reinterpret_cast<const volatile int *>(size + i) < least) {
+      head[kCrtRows + i] = 1;
+      atomicCAS(head, 0, kCrtSome);
+    }
 }
 
 }  // namespace fedvr

@@ -2,9 +2,20 @@
 // (crt.cuh; Sec. 2.3, Eq. sigma2ndb): X_ab = sum_kl V_ak V_bl g_al gb_lk g_kb for
 // every mesh point, g = G[j], gb = G[M-1-j].
 //
-// V and the matrices g_j are rounded to integers of 57 to 59 bits relative to
-// their largest entries; X is then an integer below 2^(5 q) n^2, held by its
-// residues modulo 38 to 42 moduli. For each modulus, row (b, a) of P^(b) = g
+// Every operand is rounded to integers of 57 to 59 bits (q) after its rows and
+// columns are scaled by powers of two: V and gb so that each row and each column
+// has an entry within 2^-1 of one (their column scales are taken out of g again,
+// whose index is contracted with theirs), then g_al by rows and g_kb by columns. The
+// scales of a and b are applied to the result, those of k and l cancel. Mesh points
+// do not mix, so all scales are a mesh point's own. An exchange of uncoupled or
+// decaying parts keeps its small entries: He, n = 39, box 20: every entry of X within
+// 5e-17 of the sum of its terms' magnitudes (7e-16 in FP64 arithmetic; one exponent
+// per matrix left a quarter of them beyond 1e-14). In a box of 100 a tenth to a
+// half of the entries, those far below the largest of their row and column,
+// still have fewer bits than from FP64 arithmetic. A mesh point whose largest
+// integer is 2^10 below the largest product is left to the FP64 kernel.
+// X is an integer below 2^(5 q) n^2, held by its residues modulo 41 to 43
+// moduli. For each modulus, row (b, a) of P^(b) = g
 // diag(V_b) gb is one FP16 product of small integers: the A operand g_al V_bl is
 // formed and reduced in exact FP16 pair arithmetic, B = gb comes from its residue
 // plane, and P (|P| < 2^24, exact in FP32)
@@ -438,21 +449,100 @@ __global__ void __launch_bounds__(kThreads, 1) crt_sigma_kernel(const __grid_con
   if (warp == 0) tc::tmem_dealloc(tmem, 512);
 }
 
+// Largest exponents of the rows and, relative to them, of the columns of the
+// matrices G_j (blocks j < M) and V (block M): every row and column of
+// x 2^-(row + col) then has an entry in [1/2, 1) and none beyond. Empty ones get
+// kCrtFar / 5, which rounds what meets them to zero. A value that is not finite
+// raises *flag; some[j]: the matrix is not zero.
+constexpr int kEmpty = kCrtFar / 5;
+// out[c] (shared) = max over the rows a of f(x[a][c], a), for the whole block.
+template <typename F>
+__device__ __forceinline__ void column_max(int n, const double *x, int *out, F f) {
+  for (int c = threadIdx.x; c < n; c += blockDim.x) out[c] = kCrtNone;
+  __syncthreads();
+  const int da = blockDim.x / n, dc = blockDim.x % n;
+  int a = threadIdx.x / n, c = threadIdx.x % n;
+#pragma unroll 4
+  for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
+    const int v = f(x[e], a);
+    if (v > out[c]) atomicMax(out + c, v);
+    a += da;
+    c += dc;
+    if (c >= n) c -= n, ++a;
+  }
+  __syncthreads();
+}
+__global__ void __launch_bounds__(512)
+    crt_scale_kernel(int n, int M, const double *__restrict__ G, const double *__restrict__ V,
+                     int *__restrict__ row, int *__restrict__ col, int *__restrict__ some, int *flag) {
+  extern __shared__ int rs[];
+  int *cs = rs + n;
+  const int j = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
+  const double *x = j < M ? G + (long)j * n * n : V;
+  bool bad = false, any = false;
+  for (int a = tid >> 5; a < n; a += 16) {
+    int m = kCrtNone;
+    for (int c = lane; c < n; c += 32) {
+      const double v = x[(long)a * n + c];
+      m = max(m, exponent_of(v));
+      bad |= !isfinite(v);
+    }
+    m = __reduce_max_sync(0xffffffffu, m);
+    any |= m > kCrtNone;
+    if (lane == 0) rs[a] = row[(long)j * n + a] = m > kCrtNone ? m : kEmpty;
+  }
+  if (bad) *flag = 1;
+  any = __syncthreads_or(any);
+  if (tid == 0) some[j] = any;
+  column_max(n, x, cs, [&](double v, int a) { return exponent_of(v) - rs[a]; });
+  for (int c = tid; c < n; c += 512) col[(long)j * n + c] = cs[c] > kCrtNone / 2 ? cs[c] : kEmpty;
+}
+
+// Of mesh point j: ga_l = -(row scale of gb_l. and column scale of V_.l) and ra, the
+// largest exponents of the rows of g_al beside it; gk_k = -(column scale of gb_.k and of
+// V_.k) and cb, those of the columns of g_kb.
+__global__ void __launch_bounds__(512)
+    crt_meet_kernel(int n, int M, const double *__restrict__ G, const int *__restrict__ row,
+                    const int *__restrict__ col, int *__restrict__ ra, int *__restrict__ ga,
+                    int *__restrict__ cb, int *__restrict__ gk) {
+  extern __shared__ int rs[];
+  int *ul = rs, *uk = rs + n, *cs = uk + n;
+  const int j = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
+  const long o = (long)j * n, ob = (long)(M - 1 - j) * n;
+  const double *x = G + o * n;
+  for (int l = tid; l < n; l += 512) {
+    const int vc = col[(long)M * n + l];
+    ul[l] = row[ob + l] + vc;
+    uk[l] = col[ob + l] + vc;
+    ga[o + l] = -ul[l];
+    gk[o + l] = -uk[l];
+  }
+  __syncthreads();
+  for (int a = tid >> 5; a < n; a += 16) {
+    int m = kCrtNone;
+    for (int l = lane; l < n; l += 32) m = max(m, exponent_of(x[(long)a * n + l]) + ul[l]);
+    m = __reduce_max_sync(0xffffffffu, m);
+    if (lane == 0) ra[o + a] = max(m, kCrtFar);
+  }
+  column_max(n, x, cs, [&](double v, int k) { return exponent_of(v) + uk[k]; });
+  for (int b = tid; b < n; b += 512) cb[o + b] = max(cs[b], kCrtFar);
+}
+
 // Residues of a stack as plain 16-bit rows [m][k][nr][ph], four columns per thread.
 template <bool BF16>
 __global__ void __launch_bounds__(256) crt_rows_kernel(CrtMods mods, CrtK kk, int nr, int ph, int qb,
                                                        long plane, const double *__restrict__ A,
-                                                       const int *__restrict__ expo,
-                                                       uint2 *__restrict__ out) {
+                                                       CrtScale sc, uint2 *__restrict__ out) {
   const int k = blockIdx.y, n = kk.n, q4 = kk.nc / 4;
   const int t = blockIdx.x * 256 + threadIdx.x;
   if (t >= n * q4) return;
-  const int a = t / q4, c0 = (t % q4) * 4, e = expo[k];
+  const int a = t / q4, c0 = (t % q4) * 4;
   uint32_t a0[4], a1[4], a2[4];
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     long long x = 0;
-    if (c0 + q < n && e != kCrtZero) x = quantise(A[((long)k * n + a) * n + c0 + q], qb - e);
+    if (c0 + q < n)
+      x = quantise(A[((long)k * n + a) * n + c0 + q], qb - scale_at(sc, k, a, c0 + q));
     split21(x, a0[q], a1[q], a2[q]);
   }
   const long o = (((long)k * nr + a) * ph + c0) / 4;
@@ -464,17 +554,29 @@ __global__ void __launch_bounds__(256) crt_rows_kernel(CrtMods mods, CrtK kk, in
   }
 }
 
+// The marks of the last call.
+__global__ void crt_clear_kernel(int M, int *__restrict__ head, int *__restrict__ size) {
+  for (int j = threadIdx.x; j < M; j += blockDim.x) {
+    head[kCrtRows + j] = 0;
+    size[j] = kCrtNone;
+  }
+  if (threadIdx.x < 2) head[threadIdx.x] = 0;
+}
+
 // Sigma_ab = Sigma_ba = spin g_ab W_ab - X_ab, X from its residues.
 __global__ void __launch_bounds__(256)
     crt_sigma_rebuild_kernel(const __grid_constant__ CrtWords<10> t, int n, int M, int nc, int CT, int qb,
-                             double spin, const int8_t *__restrict__ R, const int *__restrict__ eg,
-                             const int *__restrict__ eV, const int *__restrict__ flag,
+                             double spin, const int8_t *__restrict__ R, const int *__restrict__ ra,
+                             const int *__restrict__ cb, const int *__restrict__ vr,
+                             const int *__restrict__ some, int *head, int *__restrict__ size,
                              const double *__restrict__ G, const double *__restrict__ W,
                              double *__restrict__ Sigma) {
-  if (*flag) return;
+  if (*reinterpret_cast<volatile int *>(head)) return;
   const long nn = (long)n * n, plane = (long)M * n * nc;
   const long total = (long)M * nn;
-  for (long x = (long)blockIdx.x * 256 + threadIdx.x; x < total; x += (long)gridDim.x * 256) {
+  const long x0 = total * blockIdx.x / gridDim.x, x1 = total * (blockIdx.x + 1) / gridDim.x;
+  CrtSize big;
+  for (long x = x0 + threadIdx.x; x < x1; x += 256) {
     const long row = x / n;
     const int b = (int)(x - row * n), j = (int)(row / n), a = (int)(row - (long)j * n);
     if (b > a) continue;
@@ -493,11 +595,16 @@ __global__ void __launch_bounds__(256)
     const int q = (int)rintf(f);
 #pragma unroll
     for (int i = 0; i < 10; ++i) acc[i] -= (long long)q * (long long)t.P[i];
-    const double X = crt_value<10>(acc, 2 * *eV + 2 * eg[j] + eg[M - 1 - j] - 5 * qb);
+    int e;
+    const double X = crt_value<10>(acc, vr[a] + vr[b] + ra[j * n + a] + cb[j * n + b] - 5 * qb, &e);
+    big.note(size, j, e);
     const double v = spin * G[x] * W[x] - X;
     Sigma[x] = v;
     Sigma[(long)j * nn + (long)b * n + a] = v;
   }
+  big.finish(size);
+  mark_small(head, size, M, 5 * qb - kCrtGuard,
+             [&](int j) { return some[j] && some[M - 1 - j] && some[M]; });
 }
 
 }  // namespace
@@ -541,13 +648,14 @@ bool crt_sigma_plan(int n, int M, CrtSigma *out) {
   // operand planes of a group of moduli within 6 GB
   const size_t per = 2 * (2 * M * mat + (size_t)n * c.k.KP + 2 * mat);
   c.group = (int)std::max<size_t>(1, std::min<size_t>(c.nm, (6ull << 30) / per));
-  size_t o = 256;
+  size_t o = (size_t)(kCrtRows + M) * 4;
+  o = (o + 255) / 256 * 256;
   auto take = [&](size_t bytes) {
     const size_t at = o;
     o += (bytes + 255) / 256 * 256;
     return at;
   };
-  c.o_exp = take((size_t)(M + 1) * 4);
+  c.o_exp = take((2 * (size_t)(M + 1) * n + 4 * (size_t)M * n + 2 * (size_t)(M + 1)) * 4);
   c.o_g = take((size_t)c.group * M * mat * 2);
   c.o_gt = take((size_t)c.group * M * mat * 2);
   c.o_B = take((size_t)c.group * n * c.k.KP * 2);
@@ -563,30 +671,37 @@ bool crt_sigma_plan(int n, int M, CrtSigma *out) {
 cudaError_t crt_sigma_apply(const CrtSigma &c, void *wsv, double spin, const double *V, const double *G,
                             const double *W, double *Sigma, int num_sms, cudaStream_t s) {
   uint8_t *ws = reinterpret_cast<uint8_t *>(wsv);
-  int *flag = reinterpret_cast<int *>(ws);
-  int *eg = reinterpret_cast<int *>(ws + c.o_exp), *eV = eg + c.k.M;
   const int n = c.k.n, M = c.k.M;
-  cudaError_t e = cudaMemsetAsync(flag, 0, sizeof(int), s);
+  int *head = reinterpret_cast<int *>(ws);
+  int *row = reinterpret_cast<int *>(ws + c.o_exp), *col = row + (long)(M + 1) * n;
+  int *ra = col + (long)(M + 1) * n, *ga = ra + (long)M * n, *cb = ga + (long)M * n, *gk = cb + (long)M * n;
+  int *some = gk + (long)M * n, *size = some + M + 1;
+  const int *vr = row + (long)M * n, *vc = col + (long)M * n;
+  crt_clear_kernel<<<1, 256, 0, s>>>(M, head, size);
+  crt_scale_kernel<<<M + 1, 512, 2 * n * sizeof(int), s>>>(n, M, G, V, row, col, some, head);
+  crt_meet_kernel<<<M, 512, 3 * n * sizeof(int), s>>>(n, M, G, row, col, ra, ga, cb, gk);
+  cudaError_t e =
+      cudaFuncSetAttribute(crt_sigma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c.smem);
   if (e != cudaSuccess) return e;
-  crt_exp_stack_kernel<<<M, 256, 0, s>>>((long)n * n, G, eg, flag);
-  crt_exp_stack_kernel<<<1, 256, 0, s>>>((long)n * n, V, eV, flag);
-  e = cudaFuncSetAttribute(crt_sigma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c.smem);
-  if (e != cudaSuccess) return e;
+  const CrtScale sg{nullptr, ra, ga, n, n}, sv{nullptr, vr, vc, 0, 0}, sb{nullptr, row, col, n, n},
+      se{nullptr, gk, cb, n, n};
   const long stack = (long)M * n * c.k.nc;
   const unsigned gx = (unsigned)((n * (c.k.nc / 4) + 255) / 256);
   const long mat = (long)c.nr * c.ph;
+  const dim3 gg(M + 3, (n + 31) / 32, (c.k.nc + 63) / 64);
   for (int m0 = 0; m0 < c.nm; m0 += c.group) {
     const int cnt = std::min(c.group, c.nm - m0);
     const CrtMods mods = crt_mods(c.nm, false, m0, cnt);
-    crt_rows_kernel<false><<<dim3(gx, M), 256, 0, s>>>(mods, c.k, c.nr, c.ph, c.q, M * mat, G, eg,
+    crt_rows_kernel<false><<<dim3(gx, M), 256, 0, s>>>(mods, c.k, c.nr, c.ph, c.q, M * mat, G, sg,
                                                        reinterpret_cast<uint2 *>(ws + c.o_g));
-    crt_rows_kernel<false><<<gx, 256, 0, s>>>(mods, c.k, c.nr, c.ph, c.q, mat, V, eV,
+    crt_rows_kernel<false><<<gx, 256, 0, s>>>(mods, c.k, c.nr, c.ph, c.q, mat, V, sv,
                                               reinterpret_cast<uint2 *>(ws + c.o_V));
     crt_rows_kernel<true><<<gx, 256, 0, s>>>(crt_mods(c.nm, true, m0, cnt), c.k, c.nr, c.ph, c.q, mat, V,
-                                             eV, reinterpret_cast<uint2 *>(ws + c.o_Vn));
-    crt_g_kernel<false><<<dim3(M + 3, (n + 31) / 32, (c.k.nc + 63) / 64), 256, 0, s>>>(
-        mods, c.k, c.q, G, eg, reinterpret_cast<uint32_t *>(ws + c.o_B),
-        reinterpret_cast<uint32_t *>(ws + c.o_gt), c.nr, c.ph);
+                                             sv, reinterpret_cast<uint2 *>(ws + c.o_Vn));
+    crt_g_kernel<false, false><<<gg, 256, 0, s>>>(mods, c.k, c.q, G, sb,
+                                                  reinterpret_cast<uint32_t *>(ws + c.o_B), 0, 0);
+    crt_g_kernel<false, true><<<gg, 256, 0, s>>>(mods, c.k, c.q, G, se,
+                                                 reinterpret_cast<uint32_t *>(ws + c.o_gt), c.nr, c.ph);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     SigmaArgs a{};
@@ -615,15 +730,15 @@ cudaError_t crt_sigma_apply(const CrtSigma &c, void *wsv, double spin, const dou
       a.p[m] = (float)kCrtMod[m0 + m];
       a.ip[m] = 1.0f / (float)kCrtMod[m0 + m];
     }
-    a.flag = flag;
+    a.flag = head;
     crt_sigma_kernel<<<(unsigned)std::min<long>(a.units, num_sms), kThreads, c.smem, s>>>(a);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
   const long total = (long)M * n * n;
   crt_sigma_rebuild_kernel<<<(unsigned)std::min<long>((total + 255) / 256, 152 * 16), 256, 0, s>>>(
-      crt_words<10>(c.nm), n, M, c.k.nc, c.CT, c.q, spin, reinterpret_cast<const int8_t *>(ws + c.o_R), eg,
-      eV, flag, G, W, Sigma);
+      crt_words<10>(c.nm), n, M, c.k.nc, c.CT, c.q, spin, reinterpret_cast<const int8_t *>(ws + c.o_R), ra,
+      cb, vr, some, head, size, G, W, Sigma);
   return cudaGetLastError();
 }
 

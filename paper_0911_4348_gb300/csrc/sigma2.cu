@@ -41,12 +41,14 @@ __global__ void __launch_bounds__(256) exchange_fp64_kernel(int n, int M, int ro
                                                             double *__restrict__ Sigma,
                                                             const int *__restrict__ gate) {
   extern __shared__ double xsm[];
-  if (gate && *gate == 0) return;
+  const int mode = gate ? *gate : 1;
+  if (mode == 0) return;
   double *Xs = xsm, *Ys = Xs + rows * kXL, *Vs = Ys + kXL * n, *Ps = Vs + rows * n;
   const int tiles = (n + rows - 1) / rows;
   for (long blk = blockIdx.x; blk < (long)tiles * n * M; blk += gridDim.x) {
   const int b = (int)(blk / tiles % n), j = (int)(blk / tiles / n), a0 = b + (int)(blk % tiles) * rows;
   if (a0 >= n) continue;  // past the last row of this column
+  if (mode == kCrtSome && !gate[kCrtRows + j]) continue;
   const int nr = min(rows, n - a0), nout = nr * n, tid = threadIdx.x;
   const long nn = (long)n * n;
   const double *g = G + (long)j * nn;

@@ -17,6 +17,7 @@
 // column pair (b, l) is a contiguous n x n matrix X_j^{bl}[a][k] and the action
 // of g_r (x) g_r on the row pair is the sandwich g_r X g_r^T. n <= 32.
 #include "common.cuh"
+#include "crt.cuh"
 
 namespace fedvr {
 namespace {
@@ -52,10 +53,12 @@ __global__ void tm_ladder_kernel(int n, int M, const ConvCoef *__restrict__ coef
                                  const double *__restrict__ G, const double *__restrict__ T,
                                  double *__restrict__ Y, const int *__restrict__ gate) {
   __shared__ double X[1024], gr[1024], tmp[1024];
-  if (gate && *gate == 0) return;
+  const int mode = gate ? *gate : 1;
+  if (mode == 0) return;
   const int n2 = n * n;
   for (long blk = blockIdx.x; blk < (long)M * n2; blk += gridDim.x) {
   const int i = (int)(blk / n2), bl = (int)(blk % n2);
+  if (mode == kCrtSome && !gate[kCrtRows + i]) continue;
   const int tid = threadIdx.x, a = tid / n, k = tid % n;
   double acc = 0.0, lo = 0.0, hi = 0.0;  // sums of rows kc and kc + 1
   bool ulo = false, uhi = false;         // whether they hold anything (the same for the block)

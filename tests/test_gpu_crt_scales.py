@@ -1,0 +1,155 @@
+"""FP64 contractions by residue arithmetic: inputs whose entries differ in size
+inside one matrix. Rows of the source, columns of g, single mesh points and the
+contracted index are scaled by powers of two down to 2^-60 (10^-18); the result has
+to be as accurate row by row and column by column as without the scales, which
+power-of-two factors do not change in double arithmetic. The exchange is also held
+entry by entry, on uncoupled blocks and on a Green's function that decays over 8 to 11
+orders of magnitude.
+
+Bounds. Relative to the products of its row's and column's scales an operand
+entry is rounded to 2^-57 (convolution) or 2^-58 (exchange); K products add up to
+sqrt(K) of such errors and K is below 1e5: 1e-13 as in the parity tests of the same
+kernels. Against the sum of the magnitudes of an entry's own terms, the exchange of a
+decaying g is held to 1e-13 too: the rounding of 2^-58 per factor leaves 2^10 for the
+distance between the largest term of an entry and its row's and column's scales."""
+import numpy as np
+import pytest
+
+from oracle import fedvr_oracle as O
+from paper_0911_4348_gb300 import workloads as W
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+TOL = 1e-13
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_0911_4348_gb300 import Context
+    c = Context()
+    yield c
+    c.close()
+
+
+def _dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).to("cuda")
+
+
+def _two(rng, n, span=60):
+    e = rng.integers(-span, 1, n)
+    e[rng.integers(n)] = 0
+    return np.ldexp(1.0, e)
+
+
+# (rows of the source, contracted index, columns of g) scaled or not
+@pytest.mark.parametrize("which", ["row", "column", "inner", "all"])
+@pytest.mark.parametrize("n,u,p,order", [(17, 2, 8, 2), (40, 2, 6, 2), (65, 1, 12, 4), (130, 1, 6, 2)])
+def test_convolution_of_scaled_rows_and_columns(ctx, n, u, p, order, which):
+    rng = W.system_rng(101, n)
+    M = 2 * u * p + 1
+    one = np.ones(n)
+    r = _two(rng, n) if which in ("row", "all") else one
+    t = _two(rng, n) if which in ("inner", "all") else one
+    s = _two(rng, n) if which in ("column", "all") else one
+    mag = 10.0 ** rng.uniform(-6, 1, size=(M, 1, 1))
+    A, G = mag * rng.uniform(-1, 1, (M, n, n)), rng.uniform(-1, 1, (M, n, n))
+    dHF = 0.1 * rng.uniform(-1, 1, (n, n))
+    left, right = r[:, None] / t[None, :], t[:, None] * s[None, :]
+    mesh = O.power_mesh(40.0, u, p)
+    want = O.conv1(dHF, A, G, mesh, 40.0, O.lag_table(mesh["tau"], 40.0),
+                   **({"quad": "cubic4"} if order == 4 else {}))
+    I1 = torch.empty((M, n, n), dtype=torch.float64, device="cuda")
+    ctx.set_quadrature(order)
+    ctx.conv_sigma_g(40.0, u, p, _dev(dHF * left), _dev(A * left), _dev(G * right), I1)
+    torch.cuda.synchronize()
+    ctx.set_quadrature(2)
+    got = I1.cpu().numpy() / r[:, None] / s[None, :]
+    assert np.max(np.abs(got - want)) < TOL * np.max(np.abs(want))
+    # every row and every column by itself, relative to the stack's largest entry of it
+    for ax in ((0, 2), (0, 1)):
+        assert np.all(np.max(np.abs(got - want), axis=ax) < 10 * TOL * np.max(np.abs(want), axis=ax))
+
+
+def test_convolution_of_empty_rows_and_columns(ctx):
+    n, u, p = 40, 2, 6
+    M = 2 * u * p + 1
+    rng = W.system_rng(102, n)
+    A, G, d = rng.uniform(-1, 1, (M, n, n)), rng.uniform(-1, 1, (M, n, n)), rng.uniform(-1, 1, (n, n))
+    for x in (A, d):
+        x[..., 3, :] = 0.0  # a row of the source
+        x[..., :, 5] = 0.0  # a contracted column of the source
+    G[:, 7, :] = 0.0        # a contracted row of g
+    G[:, :, 9] = 0.0        # a column of g
+    G[:, 5, :] *= 1e200     # meets the source's empty column only
+    mesh = O.power_mesh(40.0, u, p)
+    want = O.conv1(d, A, G, mesh, 40.0, O.lag_table(mesh["tau"], 40.0))
+    I1 = torch.empty((M, n, n), dtype=torch.float64, device="cuda")
+    ctx.conv_sigma_g(40.0, u, p, _dev(d), _dev(A), _dev(G), I1)
+    torch.cuda.synchronize()
+    got = I1.cpu().numpy()
+    assert np.max(np.abs(got - want)) < TOL * np.max(np.abs(want))
+    assert not got[:, 3, :].any() and not got[:, :, 9].any()
+
+
+def _exchange(ctx, V, G):
+    S = torch.empty(G.shape, dtype=torch.float64, device="cuda")
+    ctx.sigma2(_dev(V), _dev(G), S, 0.0)  # spin 0: the exchange alone
+    torch.cuda.synchronize()
+    return S.cpu().numpy()
+
+
+@pytest.mark.parametrize("n,M", [(33, 40), (65, 4), (130, 3), (257, 2)])
+def test_exchange_of_scaled_matrices(ctx, n, M):
+    # g_j -> D_j g_j D_j and V -> U V U: every mesh point with scales of its own
+    rng = W.system_rng(103, n)
+    G, V = W.random_symmetric_stack(rng, M, n), W.random_symmetric(rng, n)
+    u = np.ldexp(1.0, rng.integers(-15, 1, n))
+    D = np.stack([np.ldexp(1.0, rng.integers(-30, 1, n)) for _ in range(M)])
+    # the pair (j, M - 1 - j) shares k and l: opposite scales there, none left over
+    got = _exchange(ctx, V * u[:, None] * u[None, :],
+                    G * D[:, :, None] * D[:, None, :])
+    for j in sorted({0, M // 2, M - 1}):
+        g, gb = G[j] * D[j][:, None] * D[j][None, :], None
+        b = M - 1 - j
+        gb = G[b] * D[b][:, None] * D[b][None, :]
+        v = V * u[:, None] * u[None, :]
+        want = O.sigma2_tau(g, gb, v, 0.0)
+        f = u * D[j]
+        w, x = want / f[:, None] / f[None, :], got[j] / f[:, None] / f[None, :]
+        assert np.max(np.abs(x - w)) < TOL * np.max(np.abs(w)), j
+
+
+@pytest.mark.parametrize("scale", [1e-9, 1e-18])
+def test_exchange_of_uncoupled_blocks(ctx, scale):
+    n, M = 48, 9
+    rng = W.system_rng(104, n)
+    V = W.random_symmetric(rng, n)
+    G = np.zeros((M, n, n))
+    h = n // 2
+    G[:, :h, :h] = W.random_symmetric_stack(rng, M, h)
+    G[:, h:, h:] = scale * W.random_symmetric_stack(rng, M, n - h)
+    got = _exchange(ctx, V, G)
+    for j in range(M):
+        want = O.sigma2_tau(G[j], G[M - 1 - j], V, 0.0)
+        for s in (slice(0, h), slice(h, n)):
+            assert np.max(np.abs(got[j][s, s] - want[s, s])) < TOL * np.max(np.abs(want[s, s])), j
+
+
+@pytest.mark.parametrize("n_elem,order,half", [(10, 4, 10.0), (13, 5, 12.0)])
+def test_exchange_of_a_decaying_function_entry_by_entry(ctx, n_elem, order, half):
+    b = O.fedvr_basis(n_elem, order, -half, half, 0)
+    h = O.kinetic(b) + np.diag(O.potential(b["nodes"], [2.0], [0.0], 1.0))
+    V = O.interaction(b["nodes"], 1.0)
+    hf = O.hf_scf(h, V, 2.0, 1, 100.0, tol=1e-11)
+    mesh = O.power_mesh(100.0, 3, 8)
+    G = O.g0_mesh(hf["eps"], hf["C"], hf["mu"], mesh["tau"], 100.0)
+    G = 0.5 * (G + G.transpose(0, 2, 1))
+    M = G.shape[0]
+    assert np.min(np.abs(G[-1])) < 1e-8 * np.max(np.abs(G[-1]))
+    got = _exchange(ctx, V, G)
+    for j in range(M):
+        want = O.sigma2_tau(G[j], G[M - 1 - j], V, 0.0)
+        terms = -O.sigma2_tau(np.abs(G[j]), np.abs(G[M - 1 - j]), np.abs(V), 0.0)
+        assert np.all(np.abs(got[j] - want) <= TOL * np.abs(terms)), j
