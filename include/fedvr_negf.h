@@ -243,6 +243,20 @@ int fedvr_2b_read(fedvr_ctx *ctx, int out_on_device, double *G_out, double *Sigm
  * number of kernels that step launched. ms is a host array of 6 doubles. */
 int fedvr_stage_times(const fedvr_ctx *ctx, double *ms, int *launches);
 
+/* Workspace of the FP64 path's residue arithmetic (FEDVR_FP64). limit: most bytes
+ * that this context may hold for each of the convolution's and the exchange's,
+ * from the next prepare or stage-level call on; 0: none, every contraction in double
+ * arithmetic; -1: unchanged; below -1: the default again (16 GB, and no more than
+ * half of the device memory that is free when it is allocated). Buffers above a new
+ * limit are freed at once, as they are when another buffer of the context does not
+ * fit; a prepared run then goes on in double arithmetic. The result differs between the
+ * two within their rounding. state (may be NULL; 3 ints; synchronises): how the last
+ * FP64 first convolution (GW's and the T-matrix ladder's too) and the last exchange were
+ * computed -- 0 double arithmetic, 1 residues, 2 residues with some mesh points in
+ * double arithmetic, 3 all in double arithmetic after an input that was not
+ * finite -- and the passes over the moduli that the exchange took (0: none). */
+int fedvr_fp64_workspace(fedvr_ctx *ctx, long long limit, int *state);
+
 /* Graph replay of the iteration (the driver loop of Sec. 2.3 with its launch
  * overhead removed; the paper has no counterpart). With graphs enabled (the
  * default) the first regular fedvr_2b_step after fedvr_2b_prepare captures

@@ -207,6 +207,14 @@ class Context:
                                                C.byref(last)))
         return bool(last.value)
 
+    def fp64_workspace(self, limit=-1):
+        """Limit (bytes; 0: double arithmetic only, -1: leave, -2: the default) of
+        the FP64 path's residue workspaces; returns how the last convolution and
+        exchange were computed and the exchange's passes (``fedvr_fp64_workspace``)."""
+        state = np.zeros(3, dtype=np.int32)
+        self._check(self._lib.fedvr_fp64_workspace(self._h, int(limit), _iptr(state)))
+        return dict(conv=int(state[0]), exchange=int(state[1]), passes=int(state[2]))
+
     def conv1_splits(self, request=None) -> int:
         """Request the first convolution's split count (0 = measured choice,
         None = leave); returns the count of the prepared run."""

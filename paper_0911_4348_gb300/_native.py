@@ -34,6 +34,7 @@ SIGNATURES = {
     "fedvr_2b_step": (C.c_int, [_vp, C.c_double, _vp, C.c_int, _dp, _dp, _dp]),
     "fedvr_2b_read": (C.c_int, [_vp, C.c_int, _vp, _vp, _vp]),
     "fedvr_stage_times": (C.c_int, [_vp, _dp, _ip]),
+    "fedvr_fp64_workspace": (C.c_int, [_vp, C.c_longlong, _ip]),
     "fedvr_use_graphs": (C.c_int, [_vp, C.c_int, _ip]),
     "fedvr_conv1_splits": (C.c_int, [_vp, C.c_int, _ip]),
     "fedvr_set_quadrature": (C.c_int, [_vp, C.c_int]),

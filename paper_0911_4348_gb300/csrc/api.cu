@@ -9,6 +9,7 @@
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
 #include <chrono>
 #include <map>
 #include <mutex>
@@ -45,6 +46,10 @@ bool ensure(fedvr_ctx *ctx, DevBuf &buf, size_t bytes, const char *name) {
   buf.ptr = nullptr;
   buf.bytes = 0;
   cudaError_t e = cudaMalloc(&buf.ptr, bytes);
+  if (e != cudaSuccess && give_back(ctx)) {  // what only makes calls faster makes room
+    cudaGetLastError();
+    e = cudaMalloc(&buf.ptr, bytes);
+  }
   if (e != cudaSuccess) {
     buf.ptr = nullptr;
     cudaGetLastError();
@@ -57,8 +62,36 @@ bool ensure(fedvr_ctx *ctx, DevBuf &buf, size_t bytes, const char *name) {
   return true;
 }
 
-bool ensure_optional(fedvr_ctx *ctx, DevBuf &buf, size_t bytes) {
+bool give_back(fedvr_ctx *ctx) {
+  if (!ctx->w_crt.ptr && !ctx->w_crtx.ptr) return false;
+  drop_graph(ctx);  // captured with these addresses
+  DevBuf *bufs[2] = {&ctx->w_crt, &ctx->w_crtx};
+  for (int k = 0; k < 2; ++k)  // how the last calls were computed
+    if (bufs[k]->ptr &&
+        cudaMemcpyAsync(&ctx->kept_flag[k], bufs[k]->ptr, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream))
+      cudaGetLastError();
+  if (cudaStreamSynchronize(ctx->stream)) cudaGetLastError();
+  ctx->c1_plan.reset();
+  ctx->x_plan.reset();
+  release(ctx->w_crt);
+  release(ctx->w_crtx);
+  return true;
+}
+
+size_t optional_limit(const DevBuf &buf) {
+  size_t free_b = 0, total = 0;
+  if (cudaMemGetInfo(&free_b, &total) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  const size_t half = free_b / 2;
+  return std::max(buf.bytes, std::min(kOptionalMost, half));
+}
+
+bool ensure_optional(fedvr_ctx *ctx, DevBuf &buf, size_t bytes, long long limit) {
+  if (limit >= 0 && bytes > (size_t)limit) return false;
   if (buf.bytes >= bytes) return true;
+  if (limit < 0 && bytes > optional_limit(buf)) return false;
   void *p = nullptr;
   if (cudaMalloc(&p, bytes) != cudaSuccess) {
     cudaGetLastError();
@@ -149,17 +182,26 @@ int ensure_c1f(fedvr_ctx *ctx, int n, int M) {
 // First convolution of the FP64 path: by residues on the tensor cores
 // (crt_conv.cu) where its workspace can be had, with the FP64 kernel behind it
 // for what the residues leave to it; else the FP64 kernel alone. conv_f64_prepare
-// allocates and is called outside graph capture; conv_f64_source forms the
-// scales and residues of the source stack A (once for several applications, of
-// which G is the first: that one is called with fresh).
-int conv_f64_prepare(fedvr_ctx *ctx, int n, int M, int np, bool ext, CrtConv *plan) {
+// allocates and is called outside graph capture, after the call's other buffers;
+// conv_f64_source forms the scales and residues of the source stack A (once for
+// several applications, of which G is the first: that one is called with fresh).
+bool conv_f64_plan(fedvr_ctx *ctx, int n, int M, int np, bool ext, CrtConv *plan) {
   plan->bytes = 0;
   CrtConv c;
-  if (crt_conv_plan(n, M, np, ext, ctx->num_sms, &c) && ensure_optional(ctx, ctx->w_crt, c.bytes)) {
-    *plan = c;
-    return FEDVR_OK;
-  }
+  if (!crt_conv_plan(n, M, np, ext, ctx->num_sms, &c) || 
+      !ensure_optional(ctx, ctx->w_crt, c.bytes, ctx->opt_limit))
+    return false;
+  *plan = c;
+  return true;
+}
+int conv_f64_prepare(fedvr_ctx *ctx, int n, int M, int np, bool ext, CrtConv *plan) {
+  if (conv_f64_plan(ctx, n, M, np, ext, plan)) return FEDVR_OK;
   return ensure_c1f(ctx, n, M);
+}
+// The FP64 kernel's split scratch, or NULL where it is not there for this size (one split then).
+double *c1f_or_null(fedvr_ctx *ctx, int n, int M) {
+  const int sp = conv1_fp64_splits(n, M);
+  return ctx->w_c1f.bytes >= dsz((size_t)(sp > 1 ? sp - 1 : 1) * M * n * n) ? P<double>(ctx->w_c1f) : nullptr;
 }
 int conv_f64_source(fedvr_ctx *ctx, const CrtConv &c, const ConvCoef *coef, const double *dHF,
                     const double *A, const double *G, cudaStream_t s, int *launches) {
@@ -171,9 +213,11 @@ int conv_f64_source(fedvr_ctx *ctx, const CrtConv &c, const ConvCoef *coef, cons
 int conv_f64_apply(fedvr_ctx *ctx, const CrtConv &c, int n, int M, const ConvCoef *coef,
                    const double *dHF, const double *A, const double *G, double *I1, cudaStream_t s,
                    int *launches, bool fresh) {
+  ctx->conv_by_residues = c.bytes > 0;
   if (!c.bytes) {
-    FEDVR_CK(ctx, conv1_fp64(n, M, coef, dHF, A, G, I1, s, P<double>(ctx->w_c1f)));
-    *launches += conv1_fp64_splits(n, M) > 1 ? 2 : 1;
+    double *part = c1f_or_null(ctx, n, M);
+    FEDVR_CK(ctx, conv1_fp64(n, M, coef, dHF, A, G, I1, s, part));
+    *launches += part && conv1_fp64_splits(n, M) > 1 ? 2 : 1;
     return FEDVR_OK;
   }
   FEDVR_CK(ctx, crt_conv_apply(c, ctx->w_crt.ptr, G, coef, I1, ctx->num_sms, s, fresh));
@@ -189,9 +233,11 @@ int conv_f64(fedvr_ctx *ctx, const CrtConv &c, int n, int M, const ConvCoef *coe
     if (int r = conv_f64_source(ctx, c, coef, dHF, A, G, s, launches)) return r;
     return conv_f64_apply(ctx, c, n, M, coef, dHF, A, G, I1, s, launches, true);
   }
+  ctx->conv_by_residues = c.bytes > 0;
   if (!c.bytes) {
-    FEDVR_CK(ctx, conv1_fp64_q4(n, M, coef4, dHF, A, G, I1, s, P<double>(ctx->w_c1f)));
-    *launches += conv1_fp64_splits(n, M) > 1 ? 2 : 1;
+    double *part = c1f_or_null(ctx, n, M);
+    FEDVR_CK(ctx, conv1_fp64_q4(n, M, coef4, dHF, A, G, I1, s, part));
+    *launches += part && conv1_fp64_splits(n, M) > 1 ? 2 : 1;
     return FEDVR_OK;
   }
   FEDVR_CK(ctx, crt_conv_source4(c, ctx->w_crt.ptr, A, dHF, G, coef4, s));
@@ -202,15 +248,22 @@ int conv_f64(fedvr_ctx *ctx, const CrtConv &c, int n, int M, const ConvCoef *coe
 }
 
 // Second-Born self-energy of the FP64 path: the exchange by residues where its
-// workspace can be had (sigma_f64_prepare, outside capture).
-int sigma_f64_prepare(fedvr_ctx *ctx, int n, int M, CrtSigma *plan) {
+// workspace can be had (sigma_f64_prepare, outside capture, after the call's other
+// buffers): in one pass over the moduli, or in more passes where memory is short.
+void sigma_f64_prepare(fedvr_ctx *ctx, int n, int M, CrtSigma *plan) {
   plan->bytes = 0;
   CrtSigma c;
-  if (crt_sigma_plan(n, M, &c) && ensure_optional(ctx, ctx->w_crtx, c.bytes)) *plan = c;
-  return FEDVR_OK;
+  const long long own = ctx->opt_limit;
+  if (!crt_sigma_plan(n, M, own >= 0 ? (size_t)own : kOptionalMost, &c)) return;
+  if (own < 0 && c.bytes > ctx->w_crtx.bytes &&
+      !crt_sigma_plan(n, M, optional_limit(ctx->w_crtx), &c))
+    return;
+  if (!ensure_optional(ctx, ctx->w_crtx, c.bytes, own)) return;
+  *plan = c;
 }
 int sigma_f64(fedvr_ctx *ctx, const CrtSigma &c, int n, int M, double spin, const double *V,
               const double *G, double *Sigma, cudaStream_t s, int *launches) {
+  ctx->exchange_groups = c.bytes ? (c.nm + c.group - 1) / c.group : 0;
   FEDVR_CK(ctx, sigma2_fp64(n, M, spin, V, G, Sigma, P<double>(ctx->w_t1), P<double>(ctx->w_t2),
                             P<double>(ctx->w_t3), s, &c, ctx->w_crtx.ptr, ctx->num_sms));
   *launches += c.bytes ? 8 + 6 * ((c.nm + c.group - 1) / c.group) : 4;
@@ -283,8 +336,8 @@ int tm_solve(fedvr_ctx *ctx, int n, int M, const double *V, const double *G, dou
   // the ladder's convolution K * t by residues (pair space as matrices of n^2)
   // where its workspace can be had: K's residues once, Y holding K meanwhile
   CrtConv plan;
-  const bool crt = tm_crt(n, M) && crt_conv_plan(n * n, M, 2, false, ctx->num_sms, &plan) &&
-                   ensure_optional(ctx, ctx->w_crt, plan.bytes);
+  const bool crt = tm_crt(n, M) && conv_f64_plan(ctx, n * n, M, 2, false, &plan);
+  ctx->conv_by_residues = crt;
   FEDVR_CK(ctx, tm_source(n, M, V, G, src, s));
   if (!t_valid) FEDVR_CK(ctx, launch_copy(pstack, src, t, s));
   if (crt) {
@@ -321,6 +374,8 @@ int tm_workspace(fedvr_ctx *ctx, int n, int M) {
   ENSURE(ctx, m_y, dsz(pstack));
   ENSURE(ctx, g_coef, (size_t)M * M * sizeof(ConvCoef));
   ENSURE(ctx, g_res, 16);
+  CrtConv plan;  // the residues' workspace, if it can be had (tm_solve asks again)
+  if (tm_crt(n, M)) conv_f64_plan(ctx, n * n, M, 2, false, &plan);
   return FEDVR_OK;
 }
 
@@ -669,9 +724,7 @@ int phase_sigma_pre(fedvr_ctx *ctx, bool warm, cudaStream_t s, int *launches, in
     ctx->gw_last_inner = it;
     *launches += 2 + 2 * it;
   } else {
-    CrtSigma plan{};  // its workspace was allocated by fedvr_2b_prepare
-    if (ctx->x_crt && !crt_sigma_plan(n, M, &plan))
-      return fail(ctx, FEDVR_ERR_STATE, "residue workspace of another run");
+    const CrtSigma plan = ctx->x_plan ? *ctx->x_plan : CrtSigma{};
     if (int r = sigma_f64(ctx, plan, n, M, ctx->spin, V, G, S, s, launches)) return r;
   }
   return FEDVR_OK;
@@ -707,9 +760,7 @@ int phase_mid(fedvr_ctx *ctx, cudaStream_t s, int *launches) {
 // (3) FP64 first convolution (the split path launches its tensor-core kernel instead).
 int phase_conv1_fp64(fedvr_ctx *ctx, cudaStream_t s, int *launches) {
   const bool q4 = ctx->quad_order == 4;
-  CrtConv plan{};  // the workspace of either path was allocated by fedvr_2b_prepare
-  if (ctx->c1_crt && !crt_conv_plan(ctx->n, ctx->M, q4 ? 4 : 2, true, ctx->num_sms, &plan))
-    return fail(ctx, FEDVR_ERR_STATE, "residue workspace of another run");
+  const CrtConv plan = ctx->c1_plan ? *ctx->c1_plan : CrtConv{};
   return conv_f64(ctx, plan, ctx->n, ctx->M, P<ConvCoef>(ctx->w_coef),
                   q4 ? P<ConvCoef4>(ctx->w_q4coef) : nullptr, P<double>(ctx->w_dHF),
                   P<double>(ctx->w_S), P<double>(ctx->w_G), P<double>(ctx->w_I1), s, launches);
@@ -1197,16 +1248,6 @@ int fedvr_2b_prepare(fedvr_ctx *ctx, double beta, int u, int p, int precision) {
   ENSURE(ctx, w_dHF, dsz(nn));
   ENSURE(ctx, w_part, dsz(4 * (size_t)M + 3 * (size_t)n));  // launch_energy's partials
   ENSURE(ctx, w_red, dsz(8));
-  if (!is_split(precision)) {
-    CrtConv plan;
-    if (int r = conv_f64_prepare(ctx, n, M, ctx->quad_order == 4 ? 4 : 2, true, &plan)) return r;
-    ctx->c1_crt = plan.bytes > 0;
-    CrtSigma xplan{};
-    if (ctx->self_energy == 0) {
-      if (int r = sigma_f64_prepare(ctx, n, M, &xplan)) return r;
-    }
-    ctx->x_crt = xplan.bytes > 0;
-  }
   if (is_split(precision)) {
     float *ws, *S32;
     int *err;
@@ -1230,6 +1271,16 @@ int fedvr_2b_prepare(fedvr_ctx *ctx, double beta, int u, int p, int precision) {
     // the first outer step starts the inner iteration from its lowest order
     // (V Q V, or the ladder's V^ K V^)
     ctx->gw_w_valid = false;
+  }
+  ctx->c1_plan.reset();
+  ctx->x_plan.reset();
+  if (!is_split(precision)) {  // last: these make the run faster, the others make it possible
+    CrtConv plan;
+    if (int r = conv_f64_prepare(ctx, n, M, ctx->quad_order == 4 ? 4 : 2, true, &plan)) return r;
+    CrtSigma xplan{};
+    if (ctx->self_energy == 0) sigma_f64_prepare(ctx, n, M, &xplan);
+    if (plan.bytes) ctx->c1_plan = std::make_shared<CrtConv>(plan);
+    if (xplan.bytes) ctx->x_plan = std::make_shared<CrtSigma>(xplan);
   }
   double *tau = P<double>(ctx->w_tau), *w = P<double>(ctx->w_w);
   const double *eps = P<double>(ctx->b_eps), *C = P<double>(ctx->b_C);
@@ -1457,6 +1508,29 @@ int fedvr_set_quadrature(fedvr_ctx *ctx, int order) {
   ctx->quad_order = order;
   ctx->prepared = false;  // the tables of a prepared run belong to the old rule
   drop_graph(ctx);
+  return FEDVR_OK;
+}
+
+int fedvr_fp64_workspace(fedvr_ctx *ctx, long long limit, int *state) {
+  CHECK_CTX(ctx);
+  if (state) {
+    int head[2] = {ctx->kept_flag[0], ctx->kept_flag[1]};
+    cudaStream_t s = ctx->stream;
+    if (ctx->conv_by_residues && ctx->w_crt.ptr)
+      FEDVR_CK(ctx, cudaMemcpyAsync(head, ctx->w_crt.ptr, sizeof(int), cudaMemcpyDeviceToHost, s));
+    if (ctx->exchange_groups && ctx->w_crtx.ptr)
+      FEDVR_CK(ctx, cudaMemcpyAsync(head + 1, ctx->w_crtx.ptr, sizeof(int), cudaMemcpyDeviceToHost, s));
+    if (int r = sync(ctx)) return r;
+    const bool ran[2] = {ctx->conv_by_residues, ctx->exchange_groups > 0};
+    for (int k = 0; k < 2; ++k) state[k] = !ran[k] ? 0 : head[k] == 0 ? 1 : head[k] == kCrtSome ? 2 : 3;
+    state[2] = ctx->exchange_groups;
+  }
+  if (limit < -1) {
+    ctx->opt_limit = -1;
+  } else if (limit >= 0) {
+    ctx->opt_limit = limit;
+    if (ctx->w_crt.bytes > (size_t)limit || ctx->w_crtx.bytes > (size_t)limit) give_back(ctx);
+  }
   return FEDVR_OK;
 }
 
@@ -2063,7 +2137,7 @@ int fedvr_sigma2(fedvr_ctx *ctx, int n, int M, double spin, const double *V, con
   ENSURE(ctx, w_t3, dsz(stack));
   CrtSigma plan;
   int launches = 0;
-  if (int r = sigma_f64_prepare(ctx, n, M, &plan)) return r;
+  sigma_f64_prepare(ctx, n, M, &plan);
   return sigma_f64(ctx, plan, n, M, spin, V, G, Sigma, ctx->stream, &launches);
 }
 

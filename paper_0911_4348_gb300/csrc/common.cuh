@@ -7,12 +7,16 @@
 #include <stdint.h>
 #include <stdio.h>
 
+#include <memory>
 #include <string>
 #include <vector>
 
 #include "../../include/fedvr_negf.h"
 
 namespace fedvr {
+
+struct CrtConv;
+struct CrtSigma;
 
 // Device buffer that only grows; freed with the context.
 struct DevBuf {
@@ -108,10 +112,16 @@ struct fedvr_ctx {
   fedvr::DevBuf w_c1f;
   // residue workspace of the FP64 first convolution (crt_conv.cu)
   fedvr::DevBuf w_crt;
-  bool c1_crt = false;  // the prepared run's first convolution runs by residues
+  std::shared_ptr<fedvr::CrtConv> c1_plan;  // of the prepared run (empty: the FP64 kernel)
   // and of the FP64 exchange (crt_sigma.cu)
   fedvr::DevBuf w_crtx;
-  bool x_crt = false;
+  std::shared_ptr<fedvr::CrtSigma> x_plan;
+  // most bytes of one such workspace (-1: kOptionalMost and half of what is free), and
+  // what the last FP64 build used: residues in the convolution, passes of the exchange
+  long long opt_limit = -1;
+  bool conv_by_residues = false;
+  int exchange_groups = 0;
+  int kept_flag[2] = {0, 0};  // their flags, when the workspaces were given back
 };
 
 namespace fedvr {
@@ -121,9 +131,17 @@ int fail(fedvr_ctx *ctx, int code, const char *fmt, ...);
 // workspace (split-TF32 or FP64 per the prepared precision); synchronous.
 int sigma_of_current_g(fedvr_ctx *ctx);
 int cuda_fail(fedvr_ctx *ctx, cudaError_t e, const char *what, const char *file, int line);
-// The same for an optional workspace: false (no error recorded) if it cannot be had.
-bool ensure_optional(fedvr_ctx *ctx, DevBuf &buf, size_t bytes);
-// Ensure buf holds at least `bytes`; returns false (and records the error) on failure.
+// The same for an optional workspace (one that only makes a call faster): false, no
+// error recorded, if it cannot be had or is more than limit; without one (< 0) more
+// than optional_limit, half of the memory that is free and 16 GB, so that what
+// others allocate later still fits.
+constexpr size_t kOptionalMost = 16ull << 30;
+size_t optional_limit(const DevBuf &buf);
+bool ensure_optional(fedvr_ctx *ctx, DevBuf &buf, size_t bytes, long long limit = -1);
+// Frees the residue workspaces (a prepared run goes on with the FP64 kernels); false: none held.
+bool give_back(fedvr_ctx *ctx);
+// Ensure buf holds at least `bytes`, with give_back where they do not fit; returns
+// false (and records the error) on failure.
 bool ensure(fedvr_ctx *ctx, DevBuf &buf, size_t bytes, const char *name);
 void release(DevBuf &buf);
 // Destroy the context's captured iteration graph (if any).

@@ -130,7 +130,8 @@ struct CrtSigma {
   size_t o_exp, o_g, o_gt, o_B, o_V, o_Vn, o_R, bytes;
   size_t smem;
 };
-bool crt_sigma_plan(int n, int M, CrtSigma *out);
+// limit: most bytes of workspace; false also where one modulus at a time needs more.
+bool crt_sigma_plan(int n, int M, size_t limit, CrtSigma *out);
 // Sigma = spin g o W - X[g] with the exchange X by residues, W = V Q V given; the
 // first int of ws as for crt_conv_apply.
 cudaError_t crt_sigma_apply(const CrtSigma &c, void *ws, double spin, const double *V, const double *G,

@@ -614,7 +614,7 @@ __global__ void __launch_bounds__(256)
 // Measured (ms, FP64 / residues): n = 15, M = 129: 0.172 / 0.188; n = 24, M = 129:
 // 0.398 / 0.297; n = 39, M = 17: 0.250 / 0.274; n = 65, M = 5: 0.360 / 0.333;
 // n = 74, M = 9: 0.594 / 0.396; n = 119, M = 257: 53.5 / 9.6.
-bool crt_sigma_plan(int n, int M, CrtSigma *out) {
+bool crt_sigma_plan(int n, int M, size_t limit, CrtSigma *out) {
   if ((double)M * n * n * n * n < 4e7) return false;
   CrtSigma c{};
   c.k = crt_k(n, M);
@@ -645,25 +645,30 @@ bool crt_sigma_plan(int n, int M, CrtSigma *out) {
   if (!ok) return false;
   const size_t stack = (size_t)M * n * c.k.nc, mat = (size_t)c.nr * c.ph;
   if (stack >= (1ull << 31) || c.k.KP >= (1l << 31)) return false;
-  // operand planes of a group of moduli within 6 GB
+  // operand planes of a group of moduli within 6 GB, the groups of equal size; more
+  // groups where the workspace has to be smaller
   const size_t per = 2 * (2 * M * mat + (size_t)n * c.k.KP + 2 * mat);
-  c.group = (int)std::max<size_t>(1, std::min<size_t>(c.nm, (6ull << 30) / per));
-  size_t o = (size_t)(kCrtRows + M) * 4;
-  o = (o + 255) / 256 * 256;
-  auto take = [&](size_t bytes) {
-    const size_t at = o;
-    o += (bytes + 255) / 256 * 256;
-    return at;
-  };
-  c.o_exp = take((2 * (size_t)(M + 1) * n + 4 * (size_t)M * n + 2 * (size_t)(M + 1)) * 4);
-  c.o_g = take((size_t)c.group * M * mat * 2);
-  c.o_gt = take((size_t)c.group * M * mat * 2);
-  c.o_B = take((size_t)c.group * n * c.k.KP * 2);
-  c.o_V = take((size_t)c.group * mat * 2);
-  c.o_Vn = take((size_t)c.group * mat * 2);
-  c.o_R = take((size_t)c.CT * c.nm * stack);
-  c.bytes = o;
-  if (c.bytes > (16ull << 30)) return false;
+  int groups = (int)((c.nm * per + (6ull << 30) - 1) / (6ull << 30));
+  for (groups = std::min(std::max(groups, 1), c.nm);; ++groups) {
+    c.group = (c.nm + groups - 1) / groups;
+    size_t o = (size_t)(kCrtRows + M) * 4;
+    o = (o + 255) / 256 * 256;
+    auto take = [&](size_t bytes) {
+      const size_t at = o;
+      o += (bytes + 255) / 256 * 256;
+      return at;
+    };
+    c.o_exp = take((2 * (size_t)(M + 1) * n + 4 * (size_t)M * n + 2 * (size_t)(M + 1)) * 4);
+    c.o_g = take((size_t)c.group * M * mat * 2);
+    c.o_gt = take((size_t)c.group * M * mat * 2);
+    c.o_B = take((size_t)c.group * n * c.k.KP * 2);
+    c.o_V = take((size_t)c.group * mat * 2);
+    c.o_Vn = take((size_t)c.group * mat * 2);
+    c.o_R = take((size_t)c.CT * c.nm * stack);
+    c.bytes = o;
+    if (c.bytes <= limit) break;
+    if (c.group == 1) return false;
+  }
   *out = c;
   return true;
 }
