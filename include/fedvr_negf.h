@@ -540,7 +540,11 @@ int fedvr_conv_g0(fedvr_ctx *ctx, int n, double beta, int u, int p, const double
  * wait gives up at the limit, the kernel records the timeout in a device flag
  * and returns, and the call returns FEDVR_ERR_TIMEOUT and leaves the context
  * failed, as every timeout does (later calls: FEDVR_ERR_STATE). Nothing
- * faults or hangs. Synchronises the context's stream. */
+ * faults or hangs. Synchronises the context's stream. release = 2: as 0, but the
+ * timeout is recorded as the FP64 path's residue kernels record theirs, and the
+ * call returns FEDVR_OK without synchronising: those kernels' results are computed
+ * again in double arithmetic and the timeout is returned by the call that
+ * next synchronises, or by the first call after it was recorded. */
 int fedvr_selftest_wait(fedvr_ctx *ctx, int release, double limit_seconds);
 
 /* Real-time two-time Kadanoff-Baym propagation (Sec. 2, Eqs. kbe, skkbe and

@@ -341,8 +341,9 @@ class Context:
     def selftest_wait(self, release, limit_seconds=1e-3):
         """Run the bounded device-wait self-test (``fedvr_selftest_wait``):
         release=True must return normally; release=False raises FedvrError
-        with code -5 (timeout) and leaves the context failed."""
-        self._check(self._lib.fedvr_selftest_wait(self._h, 1 if release else 0, limit_seconds))
+        with code -5 (timeout) and leaves the context failed; release=2 records
+        the timeout as the residue kernels do and returns."""
+        self._check(self._lib.fedvr_selftest_wait(self._h, int(release), limit_seconds))
 
     def kbe_propagate(self, dt, n_steps, second_born=True, rho0=None, dv=None, want_rho=True,
                       precision=FP64):

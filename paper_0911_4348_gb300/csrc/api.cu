@@ -78,6 +78,26 @@ bool give_back(fedvr_ctx *ctx) {
   return true;
 }
 
+bool ensure_report(fedvr_ctx *ctx) {
+  if (ctx->report) return true;
+  void *p = nullptr;
+  if (cudaHostAlloc(&p, sizeof(int), cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  ctx->report = reinterpret_cast<int *>(p);
+  *ctx->report = 0;
+  return true;
+}
+
+bool take_report(fedvr_ctx *ctx) {
+  if (!ctx->report || !*reinterpret_cast<volatile int *>(ctx->report)) return false;
+  *ctx->report = 0;
+  ctx->failed = true;
+  fail(ctx, FEDVR_ERR_TIMEOUT, "a residue kernel's bounded wait gave up");
+  return true;
+}
+
 size_t optional_limit(const DevBuf &buf) {
   size_t free_b = 0, total = 0;
   if (cudaMemGetInfo(&free_b, &total) != cudaSuccess) {
@@ -131,6 +151,7 @@ using namespace fedvr;
     if (!(ctx)) return FEDVR_ERR_ARG;                                            \
     if ((ctx)->failed)                                                           \
       return FEDVR_ERR_STATE;                                                    \
+    if (take_report(ctx)) return FEDVR_ERR_TIMEOUT;                              \
   } while (0)
 
 namespace {
@@ -141,7 +162,7 @@ inline bool is_fin(double x) { return isfinite(x); }
 
 int sync(fedvr_ctx *ctx) {
   FEDVR_CK(ctx, cudaStreamSynchronize(ctx->stream));
-  return FEDVR_OK;
+  return take_report(ctx) ? FEDVR_ERR_TIMEOUT : FEDVR_OK;
 }
 
 int copy_out(fedvr_ctx *ctx, void *dst, const void *src, size_t bytes, bool on_device) {
@@ -188,9 +209,10 @@ int ensure_c1f(fedvr_ctx *ctx, int n, int M) {
 bool conv_f64_plan(fedvr_ctx *ctx, int n, int M, int np, bool ext, CrtConv *plan) {
   plan->bytes = 0;
   CrtConv c;
-  if (!crt_conv_plan(n, M, np, ext, ctx->num_sms, &c) || 
-      !ensure_optional(ctx, ctx->w_crt, c.bytes, ctx->opt_limit))
+  if (!crt_conv_plan(n, M, np, ext, ctx->num_sms, &c) ||
+      !ensure_optional(ctx, ctx->w_crt, c.bytes, ctx->opt_limit) || !ensure_report(ctx))
     return false;
+  c.report = ctx->report;
   *plan = c;
   return true;
 }
@@ -258,7 +280,8 @@ void sigma_f64_prepare(fedvr_ctx *ctx, int n, int M, CrtSigma *plan) {
   if (own < 0 && c.bytes > ctx->w_crtx.bytes &&
       !crt_sigma_plan(n, M, optional_limit(ctx->w_crtx), &c))
     return;
-  if (!ensure_optional(ctx, ctx->w_crtx, c.bytes, own)) return;
+  if (!ensure_optional(ctx, ctx->w_crtx, c.bytes, own) || !ensure_report(ctx)) return;
+  c.report = ctx->report;
   *plan = c;
 }
 int sigma_f64(fedvr_ctx *ctx, const CrtSigma &c, int n, int M, double spin, const double *V,
@@ -953,6 +976,7 @@ void fedvr_destroy(fedvr_ctx *ctx) {
   drop_graph(ctx);
   if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
   for (DevBuf *b : bufs) release(*b);
+  if (ctx->report) cudaFreeHost(ctx->report);
   for (int i = 0; i < 7; ++i)
     if (ctx->ev[i]) cudaEventDestroy(ctx->ev[i]);
   for (cudaEvent_t e : ctx->kbe_events) cudaEventDestroy(e);
@@ -2276,7 +2300,10 @@ int fedvr_selftest_wait(fedvr_ctx *ctx, int release, double limit_seconds) {
   int *flag = reinterpret_cast<int *>(P<double>(ctx->b_scal) + 10);
   cudaStream_t s = ctx->stream;
   FEDVR_CK(ctx, cudaMemsetAsync(flag, 0, sizeof(int), s));
-  FEDVR_CK(ctx, launch_wait_probe(release != 0, (unsigned long long)(limit_seconds * 1e9), flag, s));
+  if (release == 2 && !ensure_report(ctx)) return fail(ctx, FEDVR_ERR_CUDA, "no host memory");
+  FEDVR_CK(ctx, launch_wait_probe(release != 0 && release != 2, (unsigned long long)(limit_seconds * 1e9), flag,
+                                  release == 2 ? ctx->report : nullptr, s));
+  if (release == 2) return FEDVR_OK;
   int h_err = 0;
   FEDVR_CK(ctx, cudaMemcpyAsync(&h_err, flag, sizeof(int), cudaMemcpyDeviceToHost, s));
   if (int r = sync(ctx)) return r;

@@ -121,6 +121,8 @@ struct fedvr_ctx {
   long long opt_limit = -1;
   bool conv_by_residues = false;
   int exchange_groups = 0;
+  // host memory that a residue kernel's wait that gave up sets (report_timeout)
+  int *report = nullptr;
   int kept_flag[2] = {0, 0};  // their flags, when the workspaces were given back
 };
 
@@ -140,6 +142,10 @@ size_t optional_limit(const DevBuf &buf);
 bool ensure_optional(fedvr_ctx *ctx, DevBuf &buf, size_t bytes, long long limit = -1);
 // Frees the residue workspaces (a prepared run goes on with the FP64 kernels); false: none held.
 bool give_back(fedvr_ctx *ctx);
+// Allocates ctx->report; false if it cannot be had. take_report: whether a wait of the
+// residue kernels has given up (the context is failed then, with the message).
+bool ensure_report(fedvr_ctx *ctx);
+bool take_report(fedvr_ctx *ctx);
 // Ensure buf holds at least `bytes`, with give_back where they do not fit; returns
 // false (and records the error) on failure.
 bool ensure(fedvr_ctx *ctx, DevBuf &buf, size_t bytes, const char *name);
@@ -304,7 +310,8 @@ cudaError_t conv2_apply_f32(int n, int M, const float *K32, const double *C, con
 // selftest.cu: one warp waits (bounded by limit_ns, the tensor-core kernels'
 // wait helper) on an mbarrier that is released first (release) or never; a
 // wait that gives up sets *flag = 1.
-cudaError_t launch_wait_probe(bool release, unsigned long long limit_ns, int *flag,
+// With report (not NULL) it is recorded through report_timeout.
+cudaError_t launch_wait_probe(bool release, unsigned long long limit_ns, int *flag, int *report,
                               cudaStream_t s);
 
 // update.cu

@@ -97,6 +97,7 @@ struct CrtConv {
   int Mp;    // pitch of the weight table (zero entries from M on)
   int nm, CT, Np, RT, S, ncR;
   size_t o_exps, o_expg, o_E, o_er, o_size, o_sm, o_S, o_B, o_C, o_R, bytes;
+  int *report;  // host memory that a wait that gave up sets to 1 (the caller's)
 };
 // false: outside what the kernel takes (sizes, 32-bit offsets, workspace limit).
 bool crt_conv_plan(int n, int M, int np, bool ext, int num_sms, CrtConv *out);
@@ -129,6 +130,7 @@ struct CrtSigma {
   long T;                   // 128-row tiles per mesh point
   size_t o_exp, o_g, o_gt, o_B, o_V, o_Vn, o_R, bytes;
   size_t smem;
+  int *report;  // as CrtConv's
 };
 // limit: most bytes of workspace; false also where one modulus at a time needs more.
 bool crt_sigma_plan(int n, int M, size_t limit, CrtSigma *out);

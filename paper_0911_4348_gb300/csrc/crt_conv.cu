@@ -447,7 +447,7 @@ struct ConvArgs {
   const void *coef;     // [nm][M + 1][Mp] CrtEntry
   uint8_t *R;           // [S][nm][M n][ncR] residues of the result
   float p[kCrtMax], ip[kCrtMax];
-  int *flag;
+  int *flag, *report;
 };
 
 struct ConvItem {
@@ -799,7 +799,7 @@ __global__ void __launch_bounds__(kThreads, 1) crt_conv_kernel(const __grid_cons
   if (*abort_flag) {
     if (warp == kMmaWarp && (issued || lane == 0)) {
       if (issued) tc::mma_commit(drain);
-      atomicExch(p.flag, 2);  // the FP64 kernel that follows recomputes the result
+      tc::report_timeout(p.flag, 2, p.report);  // the FP64 kernel that follows recomputes the result
       if (issued) tc::mbar_wait(drain, 0, kWaitNs);
     }
     __syncthreads();
@@ -946,6 +946,7 @@ cudaError_t apply_t(const CrtConv &c, void *wsv, const double *G, const Coef *co
     a.ip[m] = 1.0f / (float)kCrtMod[m];
   }
   a.flag = w.head;
+  a.report = c.report;
   const size_t smem = 1024 + (size_t)a.nst * stage + 256;
   e = cudaFuncSetAttribute(crt_conv_kernel<NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;

@@ -55,7 +55,7 @@ struct SigmaArgs {
   const uint16_t *Vn;       // the same times the CRT inverse, bfloat16
   uint8_t *R;               // [CT][nm][M n][nc] residues of X (rows a, columns b <= a)
   float p[kCrtMax], ip[kCrtMax];
-  int *flag;
+  int *flag, *report;
 };
 
 // Unit: (modulus, column tile, mesh point, tile); a tile is 16 values of b x 8
@@ -440,7 +440,7 @@ __global__ void __launch_bounds__(kThreads, 1) crt_sigma_kernel(const __grid_con
   if (*abort_flag) {
     if (warp == kMmaWarp && (issued || lane == 0)) {
       if (issued) tc::mma_commit(drain);
-      atomicExch(p.flag, 2);  // the FP64 kernel that follows recomputes the result
+      tc::report_timeout(p.flag, 2, p.report);  // the FP64 kernel that follows recomputes the result
       if (issued) tc::mbar_wait(drain, 0, kWaitNs);
     }
     __syncthreads();
@@ -736,6 +736,7 @@ cudaError_t crt_sigma_apply(const CrtSigma &c, void *wsv, double spin, const dou
       a.ip[m] = 1.0f / (float)kCrtMod[m0 + m];
     }
     a.flag = head;
+    a.report = c.report;
     crt_sigma_kernel<<<(unsigned)std::min<long>(a.units, num_sms), kThreads, c.smem, s>>>(a);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;

@@ -12,7 +12,7 @@
 namespace fedvr {
 namespace {
 
-__global__ void wait_probe_kernel(int release, unsigned long long limit_ns, int *flag) {
+__global__ void wait_probe_kernel(int release, unsigned long long limit_ns, int *flag, int *report) {
   __shared__ uint64_t bar;
   const int lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
@@ -23,14 +23,17 @@ __global__ void wait_probe_kernel(int release, unsigned long long limit_ns, int 
   if (release && threadIdx.x == 0) tc::mbar_arrive(&bar);  // completes phase 0
   __syncwarp();
   // the same warp-collective bounded wait the tensor-core roles use
-  if (!tc::warp_wait(&bar, 0, limit_ns) && lane == 0) atomicExch(flag, 1);
+  if (!tc::warp_wait(&bar, 0, limit_ns) && lane == 0) {
+    if (report) tc::report_timeout(flag, 2, report);
+    else atomicExch(flag, 1);
+  }
 }
 
 }  // namespace
 
-cudaError_t launch_wait_probe(bool release, unsigned long long limit_ns, int *flag,
+cudaError_t launch_wait_probe(bool release, unsigned long long limit_ns, int *flag, int *report,
                               cudaStream_t s) {
-  wait_probe_kernel<<<1, 32, 0, s>>>(release ? 1 : 0, limit_ns, flag);
+  wait_probe_kernel<<<1, 32, 0, s>>>(release ? 1 : 0, limit_ns, flag, report);
   return cudaGetLastError();
 }
 

@@ -25,6 +25,15 @@ __device__ __forceinline__ uint64_t global_timer_ns() {
   return t;
 }
 
+// A wait that gave up in a kernel whose result another kernel computes again: `value`
+// in the flag that this one reads, and 1 in the host's memory, where the library finds
+// it at its next synchronisation or call.
+__device__ __forceinline__ void report_timeout(int *flag, int value, int *report) {
+  atomicExch(flag, value);
+  *reinterpret_cast<volatile int *>(report) = 1;
+  __threadfence_system();
+}
+
 // One thread of a converged warp. Roles that issue tcgen05 or TMA instructions
 // run under this instead of a lane test: their operands are uniform registers,
 // and only for an elected thread does the compiler know that one thread is active
