@@ -447,7 +447,7 @@ struct ConvArgs {
   const void *coef;     // [nm][M + 1][Mp] CrtEntry
   uint8_t *R;           // [S][nm][M n][ncR] residues of the result
   float p[kCrtMax], ip[kCrtMax];
-  int *flag, *report;
+  int *flag;
 };
 
 struct ConvItem {
@@ -799,7 +799,7 @@ __global__ void __launch_bounds__(kThreads, 1) crt_conv_kernel(const __grid_cons
   if (*abort_flag) {
     if (warp == kMmaWarp && (issued || lane == 0)) {
       if (issued) tc::mma_commit(drain);
-      tc::report_timeout(p.flag, 2, p.report);  // the FP64 kernel that follows recomputes the result
+      atomicExch(p.flag, 2);  // the FP64 kernel that follows recomputes the result
       if (issued) tc::mbar_wait(drain, 0, kWaitNs);
     }
     __syncthreads();
@@ -817,9 +817,12 @@ __global__ void __launch_bounds__(256) crt_rebuild_kernel(const __grid_constant_
                                                           const int *__restrict__ E,
                                                           const int *__restrict__ er,
                                                           const int *__restrict__ ec, int *head,
-                                                          int *__restrict__ size, int qb, bool tr,
-                                                          double *__restrict__ out) {
-  if (*reinterpret_cast<volatile int *>(head)) return;
+                                                          int *__restrict__ size, int *report, int qb,
+                                                          bool tr, double *__restrict__ out) {
+  if (const int f = *reinterpret_cast<volatile int *>(head)) {
+    if (f == 2 && blockIdx.x == 0 && threadIdx.x == 0) tc::report_timeout(report);
+    return;
+  }
   const long plane = rows * ncR;
   const long total = rows * n;
   const long x0 = total * blockIdx.x / gridDim.x, x1 = total * (blockIdx.x + 1) / gridDim.x;
@@ -946,7 +949,6 @@ cudaError_t apply_t(const CrtConv &c, void *wsv, const double *G, const Coef *co
     a.ip[m] = 1.0f / (float)kCrtMod[m];
   }
   a.flag = w.head;
-  a.report = c.report;
   const size_t smem = 1024 + (size_t)a.nst * stage + 256;
   e = cudaFuncSetAttribute(crt_conv_kernel<NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -957,7 +959,7 @@ cudaError_t apply_t(const CrtConv &c, void *wsv, const double *G, const Coef *co
   const long total = (long)M * n * n;
   crt_rebuild_kernel<7><<<(unsigned)std::min<long>((total + 255) / 256, 152 * 16), 256, 0, s>>>(
       crt_words<7>(c.nm), n, (long)M * n, c.ncR, c.S, reinterpret_cast<const int8_t *>(ws + c.o_R), w.E,
-      w.er, w.ec, w.head, w.size, c.q, tr, I1);
+      w.er, w.ec, w.head, w.size, c.report, c.q, tr, I1);
   return cudaGetLastError();
 }
 

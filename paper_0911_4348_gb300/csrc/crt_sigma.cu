@@ -55,7 +55,7 @@ struct SigmaArgs {
   const uint16_t *Vn;       // the same times the CRT inverse, bfloat16
   uint8_t *R;               // [CT][nm][M n][nc] residues of X (rows a, columns b <= a)
   float p[kCrtMax], ip[kCrtMax];
-  int *flag, *report;
+  int *flag;
 };
 
 // Unit: (modulus, column tile, mesh point, tile); a tile is 16 values of b x 8
@@ -440,7 +440,7 @@ __global__ void __launch_bounds__(kThreads, 1) crt_sigma_kernel(const __grid_con
   if (*abort_flag) {
     if (warp == kMmaWarp && (issued || lane == 0)) {
       if (issued) tc::mma_commit(drain);
-      tc::report_timeout(p.flag, 2, p.report);  // the FP64 kernel that follows recomputes the result
+      atomicExch(p.flag, 2);  // the FP64 kernel that follows recomputes the result
       if (issued) tc::mbar_wait(drain, 0, kWaitNs);
     }
     __syncthreads();
@@ -568,10 +568,13 @@ __global__ void __launch_bounds__(256)
     crt_sigma_rebuild_kernel(const __grid_constant__ CrtWords<10> t, int n, int M, int nc, int CT, int qb,
                              double spin, const int8_t *__restrict__ R, const int *__restrict__ ra,
                              const int *__restrict__ cb, const int *__restrict__ vr,
-                             const int *__restrict__ some, int *head, int *__restrict__ size,
+                             const int *__restrict__ some, int *head, int *__restrict__ size, int *report,
                              const double *__restrict__ G, const double *__restrict__ W,
                              double *__restrict__ Sigma) {
-  if (*reinterpret_cast<volatile int *>(head)) return;
+  if (const int f = *reinterpret_cast<volatile int *>(head)) {
+    if (f == 2 && blockIdx.x == 0 && threadIdx.x == 0) tc::report_timeout(report);
+    return;
+  }
   const long nn = (long)n * n, plane = (long)M * n * nc;
   const long total = (long)M * nn;
   const long x0 = total * blockIdx.x / gridDim.x, x1 = total * (blockIdx.x + 1) / gridDim.x;
@@ -736,7 +739,6 @@ cudaError_t crt_sigma_apply(const CrtSigma &c, void *wsv, double spin, const dou
       a.ip[m] = 1.0f / (float)kCrtMod[m0 + m];
     }
     a.flag = head;
-    a.report = c.report;
     crt_sigma_kernel<<<(unsigned)std::min<long>(a.units, num_sms), kThreads, c.smem, s>>>(a);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -744,7 +746,7 @@ cudaError_t crt_sigma_apply(const CrtSigma &c, void *wsv, double spin, const dou
   const long total = (long)M * n * n;
   crt_sigma_rebuild_kernel<<<(unsigned)std::min<long>((total + 255) / 256, 152 * 16), 256, 0, s>>>(
       crt_words<10>(c.nm), n, M, c.k.nc, c.CT, c.q, spin, reinterpret_cast<const int8_t *>(ws + c.o_R), ra,
-      cb, vr, some, head, size, G, W, Sigma);
+      cb, vr, some, head, size, c.report, G, W, Sigma);
   return cudaGetLastError();
 }
 

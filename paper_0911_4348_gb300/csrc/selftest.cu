@@ -24,7 +24,7 @@ __global__ void wait_probe_kernel(int release, unsigned long long limit_ns, int 
   __syncwarp();
   // the same warp-collective bounded wait the tensor-core roles use
   if (!tc::warp_wait(&bar, 0, limit_ns) && lane == 0) {
-    if (report) tc::report_timeout(flag, 2, report);
+    if (report) tc::report_timeout(report);
     else atomicExch(flag, 1);
   }
 }

@@ -25,11 +25,9 @@ __device__ __forceinline__ uint64_t global_timer_ns() {
   return t;
 }
 
-// A wait that gave up in a kernel whose result another kernel computes again: `value`
-// in the flag that this one reads, and 1 in the host's memory, where the library finds
-// it at its next synchronisation or call.
-__device__ __forceinline__ void report_timeout(int *flag, int value, int *report) {
-  atomicExch(flag, value);
+// A wait gave up in a kernel whose result is computed again by another: 1 into host
+// memory, where the library finds it at its next synchronisation or call.
+__device__ __forceinline__ void report_timeout(int *report) {
   *reinterpret_cast<volatile int *>(report) = 1;
   __threadfence_system();
 }
