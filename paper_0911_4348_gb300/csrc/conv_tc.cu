@@ -231,6 +231,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
         }
       }
+      tc::drain_loads(full, 2, cc);
     }
   } else if (warp == 21) {
     // ---- MMA issue: one accumulator block per JB mesh points ----
@@ -697,6 +698,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
         }
       }
+      tc::drain_loads(full, 2, cc);
     }
   } else if (warp == 21) {
     // ---- MMA issue (kind::f16, K = 16 per instruction) ----

@@ -665,10 +665,10 @@ __global__ void __launch_bounds__(kThreads, 1) crt_conv_kernel(const __grid_cons
     // ---- TMA: Np rows x 64 columns of this modulus' plane of g ----
     if (tc::elect_one()) {
       int s = 0;
-      uint32_t ph = 1;
+      uint32_t ph = 1, cc = 0;
       for (long w = blockIdx.x; w < p.items && !*abort_flag; w += gridDim.x) {
         const ConvItem it = conv_item(p, w);
-        for (int c = it.c_lo; c < it.c_hi; ++c) {
+        for (int c = it.c_lo; c < it.c_hi; ++c, ++cc) {
           if (!tc::mbar_wait(&empty[s], ph, kWaitNs)) {
             *abort_flag = 1;
             break;
@@ -682,6 +682,7 @@ __global__ void __launch_bounds__(kThreads, 1) crt_conv_kernel(const __grid_cons
           }
         }
       }
+      tc::drain_loads(full, (uint32_t)nst, cc);
     }
   } else if (warp == kMmaWarp) {
     // ---- MMA issue ----

@@ -254,8 +254,8 @@ __global__ void __launch_bounds__(kThreads, 1) crt_sigma_kernel(const __grid_con
       // ---- gb = G[M-1-j] of each (modulus, column tile, mesh point), all columns ----
       if (tc::elect_one()) {
         int bb = 0;
-        uint32_t bph = 1;
-        for (long w = w0; w < w1 && !*abort_flag; w += p.T - w % p.T) {
+        uint32_t bph = 1, loads = 0;
+        for (long w = w0; w < w1 && !*abort_flag; w += p.T - w % p.T, ++loads) {
           const Unit un = unit_at(p, w);
           if (!tc::mbar_wait(&bempty[bb], bph, kWaitNs)) {
             *abort_flag = 1;
@@ -272,6 +272,7 @@ __global__ void __launch_bounds__(kThreads, 1) crt_sigma_kernel(const __grid_con
             bph ^= 1;
           }
         }
+        tc::drain_loads(bfull, (uint32_t)p.nB, loads);
       }
     } else if (warp == kTmaP || warp == kTmaE) {
       // ---- operand rows of each tile: 8 rows a and 16 rows b ----
@@ -283,8 +284,8 @@ __global__ void __launch_bounds__(kThreads, 1) crt_sigma_kernel(const __grid_con
         const long mat = (long)p.nr * p.ph;
         Unit un = unit_at(p, w0);
         int sl = 0;
-        uint32_t ph = 1;
-        for (long w = w0; w < w1 && !*abort_flag; ++w) {
+        uint32_t ph = 1, loads = 0;
+        for (long w = w0; w < w1 && !*abort_flag; ++w, ++loads) {
           if (!tc::mbar_wait(&eb[sl], ph, kWaitNs)) {
             *abort_flag = 1;
             break;
@@ -300,6 +301,7 @@ __global__ void __launch_bounds__(kThreads, 1) crt_sigma_kernel(const __grid_con
             ph ^= 1;
           }
         }
+        tc::drain_loads(fb, (uint32_t)slots, loads);
       }
     } else if (warp == kMmaWarp) {
       if (tc::elect_one()) {

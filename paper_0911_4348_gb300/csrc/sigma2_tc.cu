@@ -293,6 +293,7 @@ __global__ void __launch_bounds__(XRoles<F16>::kThreads, 1)
           }
         }
       }
+      tc::drain_loads(full, 2, cc);
     }
   } else if (warp == R::kMma) {
     // ---- MMA issue: one accumulator per tile ----

@@ -135,6 +135,15 @@ __device__ __forceinline__ void bulk_load(void *smem_dst, const void *src, uint3
       : "memory");
 }
 
+// Waits until the last of `loads` copies (copy c completes phase c / nst of b[c % nst])
+// have landed, each at most 100 ms: at the end of a loading role, so that no copy is
+// in flight to the shared memory of a CTA that gave up. Without a timeout the
+// consumers wait for the same phases, with one they may never come.
+__device__ __forceinline__ void drain_loads(uint64_t *b, uint32_t nst, uint32_t loads) {
+  for (uint32_t c = loads > nst ? loads - nst : 0; c < loads; ++c)
+    mbar_wait(&b[c % nst], (c / nst) & 1, 100000000ull);
+}
+
 // Named barrier among `count` threads (a multiple of 32) of the CTA.
 __device__ __forceinline__ void named_bar(int id, int count) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
