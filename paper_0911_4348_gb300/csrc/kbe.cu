@@ -337,11 +337,16 @@ inline XchgKernel xchg_kernel(int n) {
   return k[xchg_plan(n).pairs - 1];
 }
 
-// x as a pair of floats (48 bits), and the product of two pairs rounded to FP32.
-// The FP64 pipe does neither the product nor its rounding fast.
+// x as a pair of floats (48 bits), and the product of two pairs rounded to FP32:
+// of zeros and values within 2^+-100 the FP32 value nearest to the product of the
+// doubles up to 2^-46 of it. The FP64 pipe does neither the product nor its rounding
+// fast. A value that is no such pair has a NaN for its second part: its products are
+// taken in FP64.
 __device__ __forceinline__ float2 two_floats(double x) {
   const float hi = (float)x;
-  return make_float2(hi, (float)(x - (double)hi));
+  const int f = (__double2hiint(x) >> 20) & 0x7ff;
+  const bool far = (f < 1023 - 100 || f >= 1023 + 100) && (__double_as_longlong(x) << 1) != 0;
+  return make_float2(hi, far ? __int_as_float(0x7fffffff) : (float)(x - (double)hi));
 }
 __device__ __forceinline__ float mul_pairs(float2 a, float2 b) {
   const float p = a.x * b.x;
@@ -383,16 +388,30 @@ __global__ void __launch_bounds__(256)
       A[(long)(n + k) * xld + n + l] = (float)y.x;
     }
   }
-  for (int x = threadIdx.x; x < nb * n; x += 256) vs[x] = two_floats(V[b0 * n + x]);
-  __syncthreads();
+  bool far = false;
+  for (int x = threadIdx.x; x < nb * n; x += 256) {
+    const float2 v = two_floats(V[b0 * n + x]);
+    vs[x] = v;
+    far |= v.y != v.y;
+  }
+  far = __syncthreads_or(far);
   int k = threadIdx.x / n, l = threadIdx.x % n;
   for (int x = threadIdx.x; x < n2; x += 256) {  // x = k n + l
     const float2 p = hx[x], q = hy[x];
     float *out = B + (long)k * xld + l;
-    for (int b = 0; b < nb; ++b, out += (long)n * xld) {
-      const float2 v = vs[b * n + l];
-      out[0] = mul_pairs(v, p);
-      out[n] = mul_pairs(v, q);
+    if (far || p.y != p.y || q.y != q.y) {
+      const double2 h = H[k * ld + l];
+      for (int b = 0; b < nb; ++b, out += (long)n * xld) {
+        const double v = V[(b0 + b) * n + l];
+        out[0] = (float)(-v * h.x);
+        out[n] = (float)(v * h.y);
+      }
+    } else {
+      for (int b = 0; b < nb; ++b, out += (long)n * xld) {
+        const float2 v = vs[b * n + l];
+        out[0] = mul_pairs(v, p);
+        out[n] = mul_pairs(v, q);
+      }
     }
     k += 256 / n;
     l += 256 % n;
