@@ -46,7 +46,7 @@ __global__ void __launch_bounds__(256, 2) mlp_gemm(int M, int N, int K, int kz, 
                                                    const float *__restrict__ bias,
                                                    float *__restrict__ Z, float *__restrict__ C,
                                                    int ldc) {
-  __shared__ float As[2][kGK][kGM + 4], Bs[2][kGK][kGN + 4];
+  __shared__ __align__(16) float As[2][kGK][kGM + 4], Bs[2][kGK][kGN + 4];  // read 16 bytes at a time
   const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
   const int m0 = blockIdx.y * kGM, n0 = blockIdx.x * kGN;
   const int kb = blockIdx.z * kz, ke = min(K, kb + kz);
