@@ -127,16 +127,6 @@ cudaError_t gemm(int M, int N, int K, const float *A, int lda, const Tb *B, int 
   return cudaGetLastError();
 }
 
-// Weight gradient W [M x N] = A^T D over the rows, and the bias gradient's column
-// sums of D, each in `slices` partial results.
-inline int wgrad_slices(int M, int N, int rows) {
-  const int tiles = ((N + kGN - 1) / kGN) * ((M + kGM - 1) / kGM);
-  int z = (608 + tiles - 1) / tiles;
-  z = z < kMlpSlices ? z : kMlpSlices;
-  const int most = (rows + 63) / 64;  // at least 64 rows per slice
-  return z < most ? z : most;
-}
-
 // part[z][c] = sum of rows z .. of D's column c; 32 columns x 8 row lanes per block.
 __global__ void __launch_bounds__(256) colsum_part_kernel(int rows, int cols, int rz,
                                                           const float *__restrict__ D,
@@ -166,19 +156,21 @@ __global__ void slice_sum_kernel(long count, int slices, long zs, const float *_
 }
 
 // Gradient of one layer: gW [in x out] = A^T D, gb = column sums of D, contiguous in
-// the parameter vector (W then b).
+// the parameter vector (W then b); in slices, or straight into g where there is one.
 cudaError_t layer_grad(int in, int out, int rows, const float *A, const float *D, float *g, float *part,
                        cudaStream_t s) {
-  const int z = wgrad_slices(in, out, rows);
+  const int z = mlp_wgrad_slices(in, out, rows);
   const int rz = ((rows + z - 1) / z + kGK - 1) / kGK * kGK;
   const int zu = (rows + rz - 1) / rz;  // slices that hold rows
   const long count = (long)in * out + out;
+  if (zu == 1) part = g;
   dim3 grid((out + kGN - 1) / kGN, (in + kGM - 1) / kGM, zu);
   mlp_gemm<true, false, float, EPI_STORE><<<grid, 256, 0, s>>>(in, out, rows, rz, count, A, in, D, out,
                                                                nullptr, nullptr, part, out);
   colsum_part_kernel<<<dim3((out + 31) / 32, zu), 256, 0, s>>>(rows, out, rz, D, part + (long)in * out,
                                                               count);
-  slice_sum_kernel<<<(unsigned)((count + 255) / 256), 256, 0, s>>>(count, zu, count, part, g);
+  if (zu > 1)
+    slice_sum_kernel<<<(unsigned)((count + 255) / 256), 256, 0, s>>>(count, zu, count, part, g);
   return cudaGetLastError();
 }
 
@@ -345,6 +337,25 @@ cudaError_t mlp_forward_t(const MlpNet &L, const Tw *W, const float *Wbias, int 
                                           Wbias + L.o_b3, nullptr, Y, L.dout, s);
 }
 
+int mlp_wgrad_slices(int in, int out, int rows) {
+  const int tiles = ((out + kGN - 1) / kGN) * ((in + kGM - 1) / kGM);
+  int z = (608 + tiles - 1) / tiles;
+  z = z < 16 ? z : 16;
+  const int most = (rows + 63) / 64;  // at least 64 rows per slice
+  return z < most ? z : most;
+}
+
+size_t mlp_slice_floats(const MlpNet &L, int rows) {
+  size_t most = 0;
+  const int in[3] = {L.din, L.H, L.H}, out[3] = {L.H, L.H, L.dout};
+  for (int k = 0; k < 3; ++k) {
+    const int z = mlp_wgrad_slices(in[k], out[k], rows);
+    const size_t f = z > 1 ? (size_t)z * (in[k] + 1) * out[k] : 0;
+    most = f > most ? f : most;
+  }
+  return most;
+}
+
 cudaError_t mlp_forward_f32(const MlpNet &L, const float *W, int rows, const float *X, float *act,
                             float *Y, cudaStream_t s) {
   return mlp_forward_t<float>(L, W, W, rows, X, act, Y, s);
@@ -358,7 +369,7 @@ cudaError_t mlp_forward_bf16(const MlpNet &L, const void *Wbf, const float *W, i
 
 // Loss and gradient of `rows` rows (forward included). grad has nparam floats;
 // dbuf holds rows x max(H, dout) x 2 floats; part >= 256 doubles (loss partials);
-// slices >= mlp_slice_floats floats.
+// slices >= mlp_slice_floats(L, rows) floats.
 cudaError_t mlp_loss_grad(const MlpNet &L, const float *W, int rows, const float *X,
                           const float *T, float *act, float *Y, float *dbuf, float *grad,
                           double *part, float *slices, cudaStream_t s) {

@@ -18,17 +18,13 @@ cudaError_t mlp_forward_f32(const MlpNet &L, const float *W, int rows, const flo
                             float *Y, cudaStream_t s);
 cudaError_t mlp_forward_bf16(const MlpNet &L, const void *Wbf, const float *W, int rows,
                              const float *X, float *act, float *Y, cudaStream_t s);
-// Slices of the mini-batch a weight gradient may be cut into, and the floats their
-// partial results take.
-constexpr int kMlpSlices = 16;
-inline size_t mlp_slice_floats(const MlpNet &L) {
-  const size_t l1 = (size_t)(L.din + 1) * L.H, l2 = (size_t)(L.H + 1) * L.H,
-               l3 = (size_t)(L.H + 1) * L.dout;
-  const size_t a = l1 > l2 ? l1 : l2;
-  return kMlpSlices * (a > l3 ? a : l3);
-}
+// Slices of the mini-batch that the weight gradient of an in x out layer is cut into, at
+// most (never fewer for more rows), and the floats that the partial results of a
+// network's layers take.
+int mlp_wgrad_slices(int in, int out, int rows);
+size_t mlp_slice_floats(const MlpNet &L, int rows);
 // dbuf: 2 * rows * max(H, dout) floats; part: 256 doubles of loss partials; slices:
-// mlp_slice_floats.
+// mlp_slice_floats(L, rows).
 cudaError_t mlp_loss_grad(const MlpNet &L, const float *W, int rows, const float *X,
                           const float *T, float *act, float *Y, float *dbuf, float *grad,
                           double *part, float *slices, cudaStream_t s);

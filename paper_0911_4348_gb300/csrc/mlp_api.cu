@@ -101,7 +101,6 @@ int ensure_rows(fedvr_mlp *m, int rows) {
   MENSURE(m, Y, (size_t)rows * L.dout * sizeof(float));
   MENSURE(m, dbuf, (size_t)2 * rows * wide * sizeof(float));
   MENSURE(m, part, 256 * sizeof(double));
-  MENSURE(m, slices, fedvr::mlp_slice_floats(m->L) * sizeof(float));
   return FEDVR_OK;
 }
 
@@ -227,6 +226,7 @@ int fedvr_mlp_loss_grad(fedvr_mlp *m, const float *X, const float *T, int rows, 
   if (!m || !X || !T || rows < 1 || rows > (1 << 20)) return FEDVR_ERR_ARG;
   if (m->failed) return FEDVR_ERR_STATE;
   if (int r = ensure_rows(m, rows)) return r;
+  MENSURE(m, slices, fedvr::mlp_slice_floats(m->L, rows) * sizeof(float));
   MCK(m, fedvr::mlp_loss_grad(m->L, P<float>(m->W), rows, X, T, P<float>(m->act), P<float>(m->Y),
                               P<float>(m->dbuf), P<float>(m->g), P<double>(m->part),
                               P<float>(m->slices), m->stream));
@@ -316,6 +316,7 @@ int fedvr_mlp_train(fedvr_mlp *m, int epochs, int batch, double lr, double *fina
   if (m->rows < 1) return mfail(m, FEDVR_ERR_STATE, "no training rows collected");
   const fedvr::MlpNet &L = m->L;
   if (int r = ensure_rows(m, batch)) return r;
+  MENSURE(m, slices, fedvr::mlp_slice_floats(L, batch) * sizeof(float));
   MENSURE(m, idx, (size_t)m->rows * sizeof(int));
   MENSURE(m, bX, (size_t)batch * L.din * sizeof(float));
   MENSURE(m, bT, (size_t)batch * L.dout * sizeof(float));
@@ -342,7 +343,7 @@ int fedvr_mlp_train(fedvr_mlp *m, int epochs, int batch, double lr, double *fina
       MCK(m, fedvr::mlp_loss_grad(L, P<float>(m->W), rows, P<float>(m->bX), P<float>(m->bT),
                                   P<float>(m->act), P<float>(m->Y), P<float>(m->dbuf),
                                   P<float>(m->g), P<double>(m->part),
-                              P<float>(m->slices), m->stream));
+                                  P<float>(m->slices), m->stream));
       MCK(m, fedvr::mlp_adam(L.nparam, (float)lr, ++m->adam_t, P<float>(m->g), P<float>(m->m),
                              P<float>(m->v), P<float>(m->W), m->stream));
       if (e == epochs - 1) {
