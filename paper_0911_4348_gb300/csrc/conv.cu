@@ -81,59 +81,59 @@ __global__ void __launch_bounds__(256) conv1_fp64_kernel(int n, int M, int rows,
   double *Xs = c1s, *Ys = c1s + rows * kC1K;
   const int tiles = (n + rows - 1) / rows;
   for (long blk = blockIdx.x; blk < (long)tiles * M * splits; blk += gridDim.x) {
-  const int a0 = (int)(blk % tiles) * rows, i = (int)(blk / tiles % M);
-  if (mode == kCrtSome && !gate[kCrtRows + i]) continue;
-  const int nr = min(rows, n - a0), nout = nr * n;
-  const long nn = (long)n * n;
-  const int tid = threadIdx.x;
-  double acc[kC1Q];
-  int xo[kC1Q], yo[kC1Q];
-  int nq = 0;
+    const int a0 = (int)(blk % tiles) * rows, i = (int)(blk / tiles % M);
+    if (mode == kCrtSome && !gate[kCrtRows + i]) continue;
+    const int nr = min(rows, n - a0), nout = nr * n;
+    const long nn = (long)n * n;
+    const int tid = threadIdx.x;
+    double acc[kC1Q];
+    int xo[kC1Q], yo[kC1Q];
+    int nq = 0;
 #pragma unroll
-  for (int q = 0; q < kC1Q; ++q) {
-    const int o = tid + 256 * q;
-    acc[q] = 0.0;
-    xo[q] = o < nout ? (o / n) * kC1K : 0;
-    yo[q] = o < nout ? o % n : 0;
-    nq += o < nout ? 1 : 0;
-  }
-  const int sp = (int)(blk / tiles / M);
-  const int j0 = (int)((long)M * sp / splits), j1 = (int)((long)M * (sp + 1) / splits);
-  for (int j = j0; j < j1; ++j) {
-    const CoefView cv = coef_view(coef[(long)i * M + j], M);
-    const double *g = G + (long)j * nn;
-    for (int c0 = 0; c0 < n; c0 += kC1K) {
-      const int nc = min(kC1K, n - c0);
-      for (int e = tid; e < nr * kC1K; e += 256) {
-        const int aa = e / kC1K, cc = e % kC1K;
-        double v = 0.0;
-        if (cc < nc) {
-          const long off = (long)(a0 + aa) * n + c0 + cc;
-          v = cv.c[0] * A[(long)cv.r[0] * nn + off] + cv.c[1] * A[(long)cv.r[1] * nn + off];
-          if (cv.np == 4)
-            v += cv.c[2] * A[(long)cv.r[2] * nn + off] + cv.c[3] * A[(long)cv.r[3] * nn + off];
-          if (cv.diag) v += dHF[off];
-        }
-        Xs[e] = v;
-      }
-      for (int e = tid; e < nc * n; e += 256) Ys[e] = g[(long)c0 * n + e];
-      __syncthreads();
-#pragma unroll 2
-      for (int cc = 0; cc < nc; ++cc) {
-#pragma unroll
-        for (int q = 0; q < kC1Q; ++q)
-          if (q < nq) acc[q] = fma(Xs[xo[q] + cc], Ys[cc * n + yo[q]], acc[q]);
-      }
-      __syncthreads();
+    for (int q = 0; q < kC1Q; ++q) {
+      const int o = tid + 256 * q;
+      acc[q] = 0.0;
+      xo[q] = o < nout ? (o / n) * kC1K : 0;
+      yo[q] = o < nout ? o % n : 0;
+      nq += o < nout ? 1 : 0;
     }
-  }
-  double *out = sp == 0 ? I1 : part + (long)(sp - 1) * M * nn;
+    const int sp = (int)(blk / tiles / M);
+    const int j0 = (int)((long)M * sp / splits), j1 = (int)((long)M * (sp + 1) / splits);
+    for (int j = j0; j < j1; ++j) {
+      const CoefView cv = coef_view(coef[(long)i * M + j], M);
+      const double *g = G + (long)j * nn;
+      for (int c0 = 0; c0 < n; c0 += kC1K) {
+        const int nc = min(kC1K, n - c0);
+        for (int e = tid; e < nr * kC1K; e += 256) {
+          const int aa = e / kC1K, cc = e % kC1K;
+          double v = 0.0;
+          if (cc < nc) {
+            const long off = (long)(a0 + aa) * n + c0 + cc;
+            v = cv.c[0] * A[(long)cv.r[0] * nn + off] + cv.c[1] * A[(long)cv.r[1] * nn + off];
+            if (cv.np == 4)
+              v += cv.c[2] * A[(long)cv.r[2] * nn + off] + cv.c[3] * A[(long)cv.r[3] * nn + off];
+            if (cv.diag) v += dHF[off];
+          }
+          Xs[e] = v;
+        }
+        for (int e = tid; e < nc * n; e += 256) Ys[e] = g[(long)c0 * n + e];
+        __syncthreads();
+#pragma unroll 2
+        for (int cc = 0; cc < nc; ++cc) {
 #pragma unroll
-  for (int q = 0; q < kC1Q; ++q) {
-    if (q >= nq) break;
-    const int o = tid + 256 * q;
-    out[(long)i * nn + (long)(a0 + o / n) * n + o % n] = acc[q];
-  }
+          for (int q = 0; q < kC1Q; ++q)
+            if (q < nq) acc[q] = fma(Xs[xo[q] + cc], Ys[cc * n + yo[q]], acc[q]);
+        }
+        __syncthreads();
+      }
+    }
+    double *out = sp == 0 ? I1 : part + (long)(sp - 1) * M * nn;
+#pragma unroll
+    for (int q = 0; q < kC1Q; ++q) {
+      if (q >= nq) break;
+      const int o = tid + 256 * q;
+      out[(long)i * nn + (long)(a0 + o / n) * n + o % n] = acc[q];
+    }
   }
 }
 

@@ -46,66 +46,67 @@ __global__ void __launch_bounds__(256) exchange_fp64_kernel(int n, int M, int ro
   double *Xs = xsm, *Ys = Xs + rows * kXL, *Vs = Ys + kXL * n, *Ps = Vs + rows * n;
   const int tiles = (n + rows - 1) / rows;
   for (long blk = blockIdx.x; blk < (long)tiles * n * M; blk += gridDim.x) {
-  const int b = (int)(blk / tiles % n), j = (int)(blk / tiles / n), a0 = b + (int)(blk % tiles) * rows;
-  if (a0 >= n) continue;  // past the last row of this column
-  if (mode == kCrtSome && !gate[kCrtRows + j]) continue;
-  const int nr = min(rows, n - a0), nout = nr * n, tid = threadIdx.x;
-  const long nn = (long)n * n;
-  const double *g = G + (long)j * nn;
-  const double *gb = G + (long)(M - 1 - j) * nn;
-  double acc[kXQ];
-  int xo[kXQ], yo[kXQ];
-  int nq = 0;
+    const int b = (int)(blk / tiles % n), j = (int)(blk / tiles / n);
+    const int a0 = b + (int)(blk % tiles) * rows;
+    if (a0 >= n) continue;  // past the last row of this column
+    if (mode == kCrtSome && !gate[kCrtRows + j]) continue;
+    const int nr = min(rows, n - a0), nout = nr * n, tid = threadIdx.x;
+    const long nn = (long)n * n;
+    const double *g = G + (long)j * nn;
+    const double *gb = G + (long)(M - 1 - j) * nn;
+    double acc[kXQ];
+    int xo[kXQ], yo[kXQ];
+    int nq = 0;
 #pragma unroll
-  for (int q = 0; q < kXQ; ++q) {
-    const int o = tid + 256 * q;
-    acc[q] = 0.0;
-    xo[q] = o < nout ? (o / n) * kXL : 0;
-    yo[q] = o < nout ? o % n : 0;
-    nq += o < nout ? 1 : 0;
-  }
-  for (int l0 = 0; l0 < n; l0 += kXL) {
-    const int nl = min(kXL, n - l0);
-    for (int e = tid; e < nr * kXL; e += 256) {
-      const int r = e / kXL, ll = e % kXL;
-      Xs[e] = ll < nl ? g[(long)(a0 + r) * n + l0 + ll] * V[(long)b * n + l0 + ll] : 0.0;
+    for (int q = 0; q < kXQ; ++q) {
+      const int o = tid + 256 * q;
+      acc[q] = 0.0;
+      xo[q] = o < nout ? (o / n) * kXL : 0;
+      yo[q] = o < nout ? o % n : 0;
+      nq += o < nout ? 1 : 0;
     }
-    for (int e = tid; e < nl * n; e += 256) Ys[e] = gb[(long)l0 * n + e];
-    __syncthreads();
+    for (int l0 = 0; l0 < n; l0 += kXL) {
+      const int nl = min(kXL, n - l0);
+      for (int e = tid; e < nr * kXL; e += 256) {
+        const int r = e / kXL, ll = e % kXL;
+        Xs[e] = ll < nl ? g[(long)(a0 + r) * n + l0 + ll] * V[(long)b * n + l0 + ll] : 0.0;
+      }
+      for (int e = tid; e < nl * n; e += 256) Ys[e] = gb[(long)l0 * n + e];
+      __syncthreads();
 #pragma unroll 2
-    for (int ll = 0; ll < nl; ++ll) {
+      for (int ll = 0; ll < nl; ++ll) {
 #pragma unroll
-      for (int q = 0; q < kXQ; ++q)
-        if (q < nq) acc[q] = fma(Xs[xo[q] + ll], Ys[ll * n + yo[q]], acc[q]);
+        for (int q = 0; q < kXQ; ++q)
+          if (q < nq) acc[q] = fma(Xs[xo[q] + ll], Ys[ll * n + yo[q]], acc[q]);
+      }
+      __syncthreads();
+    }
+#pragma unroll
+    for (int q = 0; q < kXQ; ++q) {
+      if (q >= nq) break;
+      const int o = tid + 256 * q, a = a0 + o / n, k = o % n;
+      Vs[o] = V[(long)a * n + k] * g[(long)k * n + b] * acc[q];
     }
     __syncthreads();
-  }
-#pragma unroll
-  for (int q = 0; q < kXQ; ++q) {
-    if (q >= nq) break;
-    const int o = tid + 256 * q, a = a0 + o / n, k = o % n;
-    Vs[o] = V[(long)a * n + k] * g[(long)k * n + b] * acc[q];
-  }
-  __syncthreads();
-  // row sums over k: segments of seg values by nseg threads per row, then the segments
-  const int nseg = min(n, 256 / nr), seg = (n + nseg - 1) / nseg;
-  if (tid < nr * nseg) {
-    const int r = tid / nseg, sgi = tid % nseg, k1 = min(n, (sgi + 1) * seg);
-    double p = 0.0;
-    for (int k = sgi * seg; k < k1; ++k) p += Vs[r * n + k];
-    Ps[tid] = p;
-  }
-  __syncthreads();
-  if (tid < nr) {
-    double x = 0.0;
-    for (int sgi = 0; sgi < nseg; ++sgi) x += Ps[tid * nseg + sgi];
-    const int a = a0 + tid;
-    const long ab = (long)a * n + b;
-    const double v = spin * g[ab] * W[(long)j * nn + ab] - x;
-    Sigma[(long)j * nn + ab] = v;
-    Sigma[(long)j * nn + (long)b * n + a] = v;
-  }
-  __syncthreads();  // Ps and the staged operands are rewritten by the next block
+    // row sums over k: segments of seg values by nseg threads per row, then the segments
+    const int nseg = min(n, 256 / nr), seg = (n + nseg - 1) / nseg;
+    if (tid < nr * nseg) {
+      const int r = tid / nseg, sgi = tid % nseg, k1 = min(n, (sgi + 1) * seg);
+      double p = 0.0;
+      for (int k = sgi * seg; k < k1; ++k) p += Vs[r * n + k];
+      Ps[tid] = p;
+    }
+    __syncthreads();
+    if (tid < nr) {
+      double x = 0.0;
+      for (int sgi = 0; sgi < nseg; ++sgi) x += Ps[tid * nseg + sgi];
+      const int a = a0 + tid;
+      const long ab = (long)a * n + b;
+      const double v = spin * g[ab] * W[(long)j * nn + ab] - x;
+      Sigma[(long)j * nn + ab] = v;
+      Sigma[(long)j * nn + (long)b * n + a] = v;
+    }
+    __syncthreads();  // Ps and the staged operands are rewritten by the next block
   }
 }
 

@@ -57,55 +57,55 @@ __global__ void tm_ladder_kernel(int n, int M, const ConvCoef *__restrict__ coef
   if (mode == 0) return;
   const int n2 = n * n;
   for (long blk = blockIdx.x; blk < (long)M * n2; blk += gridDim.x) {
-  const int i = (int)(blk / n2), bl = (int)(blk % n2);
-  if (mode == kCrtSome && !gate[kCrtRows + i]) continue;
-  const int tid = threadIdx.x, a = tid / n, k = tid % n;
-  double acc = 0.0, lo = 0.0, hi = 0.0;  // sums of rows kc and kc + 1
-  bool ulo = false, uhi = false;         // whether they hold anything (the same for the block)
-  int kc = -2;
-  // acc += g_r x g_r^T
-  auto sandwich = [&](int r, double x) {
-    __syncthreads();  // earlier readers of X, gr and tmp are done
-    X[tid] = x;
-    gr[tid] = G[(long)r * n2 + tid];
-    __syncthreads();
-    double s = 0.0;  // (X g_r^T)[a][k]
-    for (int q = 0; q < n; ++q) s = fma(X[a * n + q], gr[k * n + q], s);
-    tmp[tid] = s;
-    __syncthreads();
-    for (int q = 0; q < n; ++q) acc = fma(gr[a * n + q], tmp[q * n + k], acc);
-  };
-  double xn = T[(long)bl * n2 + tid];
-  for (int j = 0; j < M; ++j) {
-    const ConvCoef c = coef[(long)i * M + j];
-    const double x = xn;
-    if (j + 1 < M) xn = T[((long)(j + 1) * n2 + bl) * n2 + tid];
-    if (c.k != kc) {
-      if (uhi) sandwich(kc + 1, hi);
-      if (c.k == kc - 1) {  // row kc becomes the upper one
-        hi = lo;
-        uhi = ulo;
-      } else {
-        if (ulo) sandwich(kc, lo);
-        hi = 0.0;
-        uhi = false;
+    const int i = (int)(blk / n2), bl = (int)(blk % n2);
+    if (mode == kCrtSome && !gate[kCrtRows + i]) continue;
+    const int tid = threadIdx.x, a = tid / n, k = tid % n;
+    double acc = 0.0, lo = 0.0, hi = 0.0;  // sums of rows kc and kc + 1
+    bool ulo = false, uhi = false;         // whether they hold anything (the same for the block)
+    int kc = -2;
+    // acc += g_r x g_r^T
+    auto sandwich = [&](int r, double x) {
+      __syncthreads();  // earlier readers of X, gr and tmp are done
+      X[tid] = x;
+      gr[tid] = G[(long)r * n2 + tid];
+      __syncthreads();
+      double s = 0.0;  // (X g_r^T)[a][k]
+      for (int q = 0; q < n; ++q) s = fma(X[a * n + q], gr[k * n + q], s);
+      tmp[tid] = s;
+      __syncthreads();
+      for (int q = 0; q < n; ++q) acc = fma(gr[a * n + q], tmp[q * n + k], acc);
+    };
+    double xn = T[(long)bl * n2 + tid];
+    for (int j = 0; j < M; ++j) {
+      const ConvCoef c = coef[(long)i * M + j];
+      const double x = xn;
+      if (j + 1 < M) xn = T[((long)(j + 1) * n2 + bl) * n2 + tid];
+      if (c.k != kc) {
+        if (uhi) sandwich(kc + 1, hi);
+        if (c.k == kc - 1) {  // row kc becomes the upper one
+          hi = lo;
+          uhi = ulo;
+        } else {
+          if (ulo) sandwich(kc, lo);
+          hi = 0.0;
+          uhi = false;
+        }
+        lo = 0.0;
+        ulo = false;
+        kc = c.k;
       }
-      lo = 0.0;
-      ulo = false;
-      kc = c.k;
+      if (c.c1 != 0.0) {
+        lo = fma(c.c1, x, lo);
+        ulo = true;
+      }
+      if (c.c2 != 0.0) {
+        hi = fma(c.c2, x, hi);
+        uhi = true;
+      }
     }
-    if (c.c1 != 0.0) {
-      lo = fma(c.c1, x, lo);
-      ulo = true;
-    }
-    if (c.c2 != 0.0) {
-      hi = fma(c.c2, x, hi);
-      uhi = true;
-    }
-  }
-  if (uhi) sandwich(kc + 1, hi);
-  if (ulo) sandwich(kc, lo);
-  Y[((long)i * n2 + bl) * n2 + tid] = acc;
+    if (uhi) sandwich(kc + 1, hi);
+    if (ulo) sandwich(kc, lo);
+    Y[((long)i * n2 + bl) * n2 + tid] = acc;
   }
 }
 
