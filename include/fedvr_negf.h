@@ -247,7 +247,9 @@ int fedvr_stage_times(const fedvr_ctx *ctx, double *ms, int *launches);
  * that this context may hold for each of the convolution's and the exchange's,
  * from the next prepare or stage-level call on; 0: none, every contraction in double
  * arithmetic; -1: unchanged; below -1: the default again (16 GB, and no more than
- * half of the device memory that is free when it is allocated). Buffers above a new
+ * half of the device memory that is free when it is allocated). With a limit of its own
+ * a context uses the residues wherever they fit it, otherwise only at the sizes where
+ * they are the faster. Buffers above a new
  * limit are freed at once, as they are when another buffer of the context does not
  * fit; a prepared run then goes on in double arithmetic. The result differs between the
  * two within their rounding. state (may be NULL; 3 ints; synchronises): how the last

@@ -209,7 +209,7 @@ int ensure_c1f(fedvr_ctx *ctx, int n, int M) {
 bool conv_f64_plan(fedvr_ctx *ctx, int n, int M, int np, bool ext, CrtConv *plan) {
   plan->bytes = 0;
   CrtConv c;
-  if (!crt_conv_plan(n, M, np, ext, ctx->num_sms, &c) ||
+  if (!crt_conv_plan(n, M, np, ext, ctx->num_sms, ctx->opt_limit >= 0, &c) ||
       !ensure_optional(ctx, ctx->w_crt, c.bytes, ctx->opt_limit) || !ensure_report(ctx))
     return false;
   c.report = ctx->report;
@@ -276,9 +276,9 @@ void sigma_f64_prepare(fedvr_ctx *ctx, int n, int M, CrtSigma *plan) {
   plan->bytes = 0;
   CrtSigma c;
   const long long own = ctx->opt_limit;
-  if (!crt_sigma_plan(n, M, own >= 0 ? (size_t)own : kOptionalMost, &c)) return;
+  if (!crt_sigma_plan(n, M, own >= 0, own >= 0 ? (size_t)own : kOptionalMost, &c)) return;
   if (own < 0 && c.bytes > ctx->w_crtx.bytes &&
-      !crt_sigma_plan(n, M, optional_limit(ctx->w_crtx), &c))
+      !crt_sigma_plan(n, M, false, optional_limit(ctx->w_crtx), &c))
     return;
   if (!ensure_optional(ctx, ctx->w_crtx, c.bytes, own) || !ensure_report(ctx)) return;
   c.report = ctx->report;

@@ -100,7 +100,8 @@ struct CrtConv {
   int *report;  // host memory that a wait that gave up sets to 1 (the caller's)
 };
 // false: outside what the kernel takes (sizes, 32-bit offsets, workspace limit).
-bool crt_conv_plan(int n, int M, int np, bool ext, int num_sms, CrtConv *out);
+// any: also where the FP64 kernel is estimated to be the faster (from n = 12 on).
+bool crt_conv_plan(int n, int M, int np, bool ext, int num_sms, bool any, CrtConv *out);
 // ws: plan.bytes of device memory beginning with the flag and the marks (kCrtSome);
 // the caller's FP64 kernel follows and computes what they leave to it.
 // Source stack A (and, with ext, the diagonal operands from dHF and the end
@@ -133,7 +134,7 @@ struct CrtSigma {
   int *report;  // as CrtConv's
 };
 // limit: most bytes of workspace; false also where one modulus at a time needs more.
-bool crt_sigma_plan(int n, int M, size_t limit, CrtSigma *out);
+bool crt_sigma_plan(int n, int M, bool any, size_t limit, CrtSigma *out);
 // Sigma = spin g o W - X[g] with the exchange X by residues, W = V Q V given; the
 // first int of ws as for crt_conv_apply.
 cudaError_t crt_sigma_apply(const CrtSigma &c, void *ws, double spin, const double *V, const double *G,

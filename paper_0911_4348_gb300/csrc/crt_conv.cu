@@ -966,14 +966,16 @@ cudaError_t apply_t(const CrtConv &c, void *wsv, const double *G, const Coef *co
 
 }  // namespace
 
-// Where the residue path is taken: it costs eight launches (about 0.09 ms when
-// the host issues them one by one) against the FP64 kernel's one or two, so very
-// small problems stay with the FP64 kernel. Measured (ms, FP64 kernel / residues):
-// n = 21, M = 17: 0.079 / 0.098; n = 37, M = 13 (four rows): 0.178 / 0.203;
-// n = 15, M = 33: 0.113 / 0.095; n = 15, M = 129: 1.11 / 0.15; n = 130, M = 7:
-// 0.25 / 0.14; n = 119, M = 257: 190 / 9.0; n = 199, M = 513: 3574 / 104.
-bool crt_conv_plan(int n, int M, int np, bool ext, int num_sms, CrtConv *out) {
-  if (!((n >= 12 && M >= 24) || 2.0 * M * M * n * n * n >= 5e7)) return false;
+// Where the residue path is taken: its ten launches take about 90 us whatever the size
+// (four rows: 225), against the FP64 kernel's one or two, so very small problems stay with
+// the FP64 kernel. Measured (us, FP64 kernel / residues): n = 12, M = 25: 75 / 88; 13,
+// 33: 89 / 91; 16, 25: 91 / 88; 12, 41: 142 / 92; 15, 129: 1081 / 144; 37, 25: 180 / 109;
+// 130, 7: 242 / 142; four rows: n = 17, M = 25: 211 / 237; 16, 33: 222 / 226; 12, 41: 249
+// / 221; 37, 25: 302 / 255; two rows: n = 119, M = 257: 190 / 8.7 ms; n = 199, M = 513: 3574 /
+// 98 ms. With any, wherever it can run.
+bool crt_conv_plan(int n, int M, int np, bool ext, int num_sms, bool any, CrtConv *out) {
+  const bool small = n < 12 || M < 24 || n * M < (np == 4 ? 550 : 390);
+  if ((!any || n < 12) && small && 2.0 * M * M * n * n * n < 5e7) return false;
   CrtConv c{};
   c.k = crt_k(n, M);
   c.np = np;

@@ -614,13 +614,17 @@ __global__ void __launch_bounds__(256)
 
 }  // namespace
 
-// Where the residue path is taken: it costs eight launches more (about 0.05 ms
-// when the host issues them), so small builds stay with the FP64 exchange.
-// Measured (ms, FP64 / residues): n = 15, M = 129: 0.172 / 0.188; n = 24, M = 129:
-// 0.398 / 0.297; n = 39, M = 17: 0.250 / 0.274; n = 65, M = 5: 0.360 / 0.333;
-// n = 74, M = 9: 0.594 / 0.396; n = 119, M = 257: 53.5 / 9.6.
-bool crt_sigma_plan(int n, int M, size_t limit, CrtSigma *out) {
-  if ((double)M * n * n * n * n < 4e7) return false;
+// Where the residue path is taken: where it is the faster by an estimate in
+// microseconds. Residues: 110 for their 14 launches and the scales, and 1 per tile, CTA
+// and 64-wide column slice (the tiles of all moduli over 152 CTAs). FP64 kernel: M n^4
+// at 1e12 per second, less by 1 + (60 / n)^2 where rows of n columns fill its tiles
+// badly. Measured (us, FP64 / residues, the whole call): n = 10, M = 4097: 1631 / 2385;
+// 16, 700: 720 / 512; 20, 250: 424 / 381; 24, 129: 327 / 242; 33, 40: 203 / 272; 33,
+// 257: 1153 / 1178; 39, 30: 213 / 236; 39, 129: 827 / 646; 48, 8: 138 / 161; 48, 40: 460
+// / 332; 65, 5: 183 / 183; 74, 9: 420 / 250; 130, 2: 688 / 254; 119, 257: 53300 / 9660.
+// (The line was M n^4 = 4e7, which took n = 33 to 39 with few mesh points and n <= 12
+// to the slower side.) With any, wherever it can run.
+bool crt_sigma_plan(int n, int M, bool any, size_t limit, CrtSigma *out) {
   CrtSigma c{};
   c.k = crt_k(n, M);
   constexpr int kQ = 57, kQMax = 59;
@@ -631,6 +635,9 @@ bool crt_sigma_plan(int n, int M, size_t limit, CrtSigma *out) {
   c.NCB = c.k.full + ((c.k.NU & 2) ? 1 : 0) + ((c.k.NU & 1) ? 1 : 0);
   c.T = 0;
   for (int b0 = 0; b0 < n; b0 += 16) c.T += (n - b0 + 7) / 8;
+  const double tiles = (double)c.T * M * ((c.k.nc + 255) / 256) * c.nm / 152.0;
+  const double us_fp64 = 1e-6 * M * pow((double)n, 4.0) * (1.0 + 3600.0 / ((double)n * n));
+  if ((!any || n < 12) && us_fp64 < 110.0 + tiles * c.NCB) return false;
   // column tiles: gb of one tile (all columns l) has to fit shared memory beside
   // two stages of A and the staged rows
   c.nr = (n + 15) / 16 * 16;

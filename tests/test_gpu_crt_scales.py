@@ -29,6 +29,7 @@ def ctx():
         pytest.skip("no CUDA device")
     from paper_0911_4348_gb300 import Context
     c = Context()
+    c.fp64_workspace(8 << 30)  # a limit of its own: residues at every size here
     yield c
     c.close()
 
@@ -65,6 +66,7 @@ def test_convolution_of_scaled_rows_and_columns(ctx, n, u, p, order, which):
     ctx.conv_sigma_g(40.0, u, p, _dev(dHF * left), _dev(A * left), _dev(G * right), I1)
     torch.cuda.synchronize()
     ctx.set_quadrature(2)
+    assert ctx.fp64_workspace()["conv"] in (1, 2)
     got = I1.cpu().numpy() / r[:, None] / s[None, :]
     assert np.max(np.abs(got - want)) < TOL * np.max(np.abs(want))
     # every row and every column by itself, relative to the stack's largest entry of it
@@ -97,6 +99,7 @@ def _exchange(ctx, V, G):
     S = torch.empty(G.shape, dtype=torch.float64, device="cuda")
     ctx.sigma2(_dev(V), _dev(G), S, 0.0)  # spin 0: the exchange alone
     torch.cuda.synchronize()
+    assert ctx.fp64_workspace()["exchange"] in (1, 2)
     return S.cpu().numpy()
 
 

@@ -39,6 +39,7 @@ def _sigma(ctx, V, G):
 def test_exchange_in_several_passes(ctx, n, M):
     rng = W.system_rng(105, n)
     G, V = W.random_symmetric_stack(rng, M, n), W.random_symmetric(rng, n)
+    ctx.fp64_workspace(1 << 30)
     one = _sigma(ctx, V, G)
     st = ctx.fp64_workspace()
     assert st["exchange"] == 1 and st["passes"] == 1
@@ -58,8 +59,50 @@ def test_exchange_in_several_passes(ctx, n, M):
     else:
         pytest.fail("a limit of 64 KB cannot hold the planes of a modulus")
     assert {1, 2, 3} <= seen and max(seen) > 10  # one modulus' planes do not fit below that
-    ctx.fp64_workspace(-2)
+    ctx.fp64_workspace(1 << 30)
     assert np.array_equal(_sigma(ctx, V, G), one)
+
+
+# every remainder of the 64-wide column slices, one and two column tiles, one and two
+# buffers of gb, single and partial tile rows; by residues at every size
+@pytest.mark.parametrize("n,M", [(12, 40), (16, 40), (17, 33), (33, 9), (48, 5), (63, 4), (64, 4),
+                                 (65, 3), (79, 1), (97, 2), (112, 2), (130, 2), (255, 1), (272, 1)])
+def test_exchange_at_the_edges_of_its_tiles(ctx, n, M):
+    rng = W.system_rng(109, n)
+    G, V = W.random_symmetric_stack(rng, M, n), W.random_symmetric(rng, n)
+    ctx.fp64_workspace(8 << 30)
+    got = _sigma(ctx, V, G)
+    assert ctx.fp64_workspace()["exchange"] == 1
+    for j in sorted({0, M // 2, M - 1}):
+        want = O.sigma2_tau(G[j], G[M - 1 - j], V, 2.0)
+        assert np.max(np.abs(got[j] - want)) < TOL * np.max(np.abs(want)), j
+
+
+@pytest.mark.parametrize("n,u,p,order", [(12, 1, 3, 2), (12, 2, 6, 4), (16, 1, 4, 2), (33, 1, 3, 4),
+                                         (63, 1, 2, 2), (65, 1, 2, 2)])
+def test_small_convolutions_by_residues(ctx, n, u, p, order):
+    M = 2 * u * p + 1
+    rng = W.system_rng(110, n)
+    A, G, d = rng.uniform(-1, 1, (M, n, n)), rng.uniform(-1, 1, (M, n, n)), rng.uniform(-1, 1, (n, n))
+    mesh = O.power_mesh(40.0, u, p)
+    want = O.conv1(d, A, G, mesh, 40.0, O.lag_table(mesh["tau"], 40.0),
+                   **({"quad": "cubic4"} if order == 4 else {}))
+    I1 = torch.empty((M, n, n), dtype=torch.float64, device="cuda")
+    ctx.fp64_workspace(8 << 30)
+    ctx.set_quadrature(order)
+    ctx.conv_sigma_g(40.0, u, p, _dev(d), _dev(A), _dev(G), I1)
+    assert ctx.fp64_workspace()["conv"] == 1
+    assert np.max(np.abs(I1.cpu().numpy() - want)) < TOL * np.max(np.abs(want))
+
+
+# where the estimates of both sides cross: the call takes the side that measured faster
+@pytest.mark.parametrize("n,M,residues", [(10, 4097, 0), (16, 700, 1), (24, 129, 1), (33, 40, 0),
+                                          (39, 18, 0), (39, 129, 1), (74, 9, 1)])
+def test_exchange_takes_the_faster_side(ctx, n, M, residues):
+    G = torch.zeros((M, n, n), dtype=torch.float64, device="cuda")
+    G[:] = torch.eye(n, dtype=torch.float64, device="cuda")
+    ctx.sigma2(torch.ones((n, n), dtype=torch.float64, device="cuda"), G, torch.empty_like(G))
+    assert ctx.fp64_workspace()["exchange"] == residues
 
 
 def test_no_workspace_in_a_prepared_run(ctx):
@@ -148,7 +191,7 @@ def test_cancelling_mesh_points_in_double_arithmetic(ctx):
         ctx.conv_sigma_g(40.0, u, p, *dev, I1)
         return I1.cpu().numpy(), ctx.fp64_workspace()["conv"]
 
-    got, st = run(-2)
+    got, st = run(8 << 30)
     double, st0 = run(0)
     assert st == 2 and st0 == 0
     mesh = O.power_mesh(40.0, u, p)
@@ -174,6 +217,7 @@ def test_disjoint_blocks_of_the_exchange_in_double_arithmetic(ctx):
         G[j][a, a] = W.random_symmetric(rng, h)
         G[j][b, b] = 0.0
     G[0, 0, h] = G[0, h, 0] = 1e-3  # one entry that lets them meet
+    ctx.fp64_workspace(8 << 30)
     got = _sigma(ctx, V, G)
     st = ctx.fp64_workspace()
     assert st["exchange"] == 2
