@@ -2199,7 +2199,8 @@ int fedvr_conv_sigma_g(fedvr_ctx *ctx, int n, double beta, int u, int p, const d
     if (S > 1) ENSURE(ctx, w_c1p, dsz((size_t)(S - 1) * stack));
     if (ctx->c1_request == 0) {
       // no request: the split with the least time, a chunk of a tile taking about 1 us
-      // and a partial stack three passes over memory (n = 142, M = 1025: 1138 tiles are
+      // (0.7 at n = 142; the choice turns on whole waves of CTAs, the figure only weighs
+      // the partial stacks) and a partial stack three passes over memory (n = 142, M = 1025: 1138 tiles are
       // 8 waves of 152 CTAs with a last one half empty, 18.4 ms; two splits 17.05)
       const long RT = conv1_items(n, M, 1);
       const int KC = f16 ? (n + 63) / 64 : (n + 31) / 32, NB = conv1_blocks(n, M, f16);

@@ -29,7 +29,7 @@
 // Measured against 113-bit arithmetic on the HF Green's functions of He (n = 15
 // to 119) and on random stacks, the result is within 1e-16 (2-norm, relative; 2
 // to 6e-16 for the FP64 kernel): it is the exact sum of the rounded integers,
-// rounded to FP64 once. n = 119, M = 257: 190 -> 8.8 ms; n = 199, M = 513:
+// rounded to FP64 once. n = 119, M = 257: 190 -> 8.7 ms; n = 199, M = 513:
 // 3574 -> 98 ms. What bounds it (ncu, n = 119): the producers' instructions, some
 // 3,400 warp instructions per chunk of 256 rows x 64 columns against 512 cycles of
 // MMA (issue slots 53 %, tensor pipe 32 %).
@@ -471,8 +471,8 @@ __device__ __forceinline__ ConvItem conv_item(const ConvArgs &a, long w) {
 // Persistent kernel, one CTA per SM. Item: (modulus, split of the contraction,
 // column tile, 256-row tile of the stacked rows (i, a)); row tiles fastest, so
 // that the CTAs running at one time share one modulus' planes in L2. Warps 0-7
-// reduce and read the accumulators, 8-23 form the A operand, 24 loads g by TMA,
-// 25 issues the MMAs. A stage is 256 rows x 64 columns of A (two 128-row
+// reduce and read the accumulators, 8-15 form the A operand, 16 loads g by TMA,
+// 17 issues the MMAs. A stage is 256 rows x 64 columns of A (two 128-row
 // operands, one per accumulator) and Np rows x 64 columns of g, so each g tile
 // read from L2 feeds two MMAs. Every 16 chunks an accumulator is reduced modulo
 // p in place (TMEM -> registers -> TMEM), 8 chunks apart for the two, so one

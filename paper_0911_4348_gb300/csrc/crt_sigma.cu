@@ -26,7 +26,7 @@
 // Measured against 113-bit arithmetic (random stacks and the HF Green's functions
 // of He, n = 1 to 119), Sigma is as near as with the FP64 exchange: both are
 // within 1e-15 (2-norm, relative), set by the direct term's FP64 products.
-// n = 119, M = 257: 53.5 -> 9.6 ms; n = 199, M = 513: 754 -> 93 ms. What bounds it
+// n = 119, M = 257: 53.3 -> 9.7 ms; n = 199, M = 513: 754 -> 86 ms. What bounds it
 // (ncu, n = 119): FP32 and FP16 arithmetic of the operand formation and of the
 // epilogue (FMA pipe 60 %, issue slots 67 %, tensor pipe 17 %).
 #include <algorithm>

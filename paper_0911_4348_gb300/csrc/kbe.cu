@@ -51,7 +51,9 @@
 namespace fedvr {
 namespace {
 
-constexpr int kKbeMaxN = 80;  // exchange operands (2 n^2 + 1024 complex) fit one CTA's shared memory
+// The exchange's operands fit one CTA's shared memory: 2 n^2 complex values and a chunk of
+// pairs (xchg_plan), 2048 up to n = 72 and 1024 above.
+constexpr int kKbeMaxN = 80;
 
 __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
   return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
@@ -362,7 +364,8 @@ __device__ __forceinline__ float mul_pairs(float2 a, float2 b) {
 // V_bl gb_lk = -V_bl conj(H_kl). One block per kXopB values of b and entry, H in
 // shared memory as pairs of floats. Bound by writing Bp (2 n^3 floats per
 // entry): two FP64 products and conversions per value took 41 us on average
-// at n = 39, T = 81, now 22.
+// at n = 39, T = 81, now 22. Eight values of b share one reading of H; chosen
+// at n = 39 of the n <= 64 that take this path; no result depends on it.
 constexpr int kXopB = 8;
 size_t xop_smem(int n) { return ((size_t)2 * n * n + (size_t)kXopB * n) * sizeof(float2); }
 __global__ void __launch_bounds__(256)
@@ -424,7 +427,8 @@ __global__ void __launch_bounds__(256)
 // One block per kXsumB columns b and entry; V^T and the columns of g in shared
 // memory in FP32. Bound by reading P (2 n^3 floats per entry): with V and g
 // converted again by every thread 39 us on average at n = 39, T = 81, now
-// 18.
+// 18. Both constants were chosen at n = 39 of the n <= 64 that take this path; no result
+// depends on them.
 constexpr int kXsumB = 6, kXsumK = 10;
 size_t xsum_smem(int n) { return ((size_t)n * n + (size_t)2 * kXsumB * n) * sizeof(float); }
 __global__ void __launch_bounds__(256)

@@ -135,6 +135,9 @@ void dgemm_run(bool ta, bool tb, const GemmArgs &g, cudaStream_t s) {
 // tile area, a small tile's extra shared-memory traffic as a factor. 199^3: 20 us
 // in tiles of 8 (13.5 us at the FP64 peak), 119 us in 16 tiles of 64; the products
 // of a second-Born step at n = 15, M = 129: 198 us less together than in tiles of 64.
+// The factors are fitted to these two (one matrix, a stack of 129 small ones); where they
+// decide wrongly between two neighbours the costs differ by less than the factor, and
+// no result depends on the tile.
 cudaError_t dgemm_any(bool ta, bool tb, const GemmArgs &g, cudaStream_t s) {
   int dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);

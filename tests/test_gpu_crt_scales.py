@@ -156,3 +156,39 @@ def test_exchange_of_a_decaying_function_entry_by_entry(ctx, n_elem, order, half
         want = O.sigma2_tau(G[j], G[M - 1 - j], V, 0.0)
         terms = -O.sigma2_tau(np.abs(G[j]), np.abs(G[M - 1 - j]), np.abs(V), 0.0)
         assert np.all(np.abs(got[j] - want) <= TOL * np.abs(terms)), j
+
+
+def test_convolution_of_a_decaying_function(ctx):
+    # what is kept of an entry is relative to the largest products of its row and column
+    # over the mesh points, whatever the entry itself is: K = 2 M n roundings of 2^-57 each,
+    # a factor of 16 for the rounding of the scales to powers of two
+    b = O.fedvr_basis(13, 3, -25.0, 25.0, 0)
+    h = O.kinetic(b) + np.diag(O.potential(b["nodes"], [2.0], [0.0], 1.0))
+    V = O.interaction(b["nodes"], 1.0)
+    beta, u, p = 60.0, 3, 8
+    hf = O.hf_scf(h, V, 2.0, 1, beta, tol=1e-11)
+    mesh = O.power_mesh(beta, u, p)
+    lag = O.lag_table(mesh["tau"], beta)
+    G = O.g0_mesh(hf["eps"], hf["C"], hf["mu"], mesh["tau"], beta)
+    A = O.sigma2(G, V, 2.0)
+    M, n, _ = G.shape
+    d = 1e-3 * V * G[-1]
+    want = O.conv1(d, A, G, mesh, beta, lag)
+    assert np.min(np.abs(want[0])) < 1e-14 * np.max(np.abs(want[0]))
+    I1 = torch.empty((M, n, n), dtype=torch.float64, device="cuda")
+    ctx.conv_sigma_g(beta, u, p, _dev(d), _dev(A), _dev(G), I1)
+    assert ctx.fp64_workspace()["conv"] == 1
+    got = I1.cpu().numpy()
+    top = lambda X: np.max(np.abs(X), axis=(1, 2))
+    diag = (mesh["wm"] + mesh["wp"])[:, None, None] * np.maximum(np.abs(A[0]), np.abs(A[-1])) + np.abs(d)
+    src = np.concatenate([A, diag])
+    R = np.max(np.max(np.abs(src), axis=2) / top(src)[:, None], axis=0)
+    S = np.max(np.max(np.abs(G), axis=1) / top(G)[:, None], axis=0)
+    for i in range(M):
+        k = lag["k"][i]
+        E = np.max(mesh["w"] * np.maximum(top(A)[k], top(A)[np.minimum(k + 1, M - 1)]) * top(G))
+        E = max(E, top(src)[M + i] * top(G)[i])
+        bound = 16 * 2.0 ** -57 * np.sqrt(2.0 * M * n) * E * R[:, None] * S[None, :]
+        own = 1e-14 * np.abs(want[i])  # the double sums' own error
+        assert np.all(np.abs(got[i] - want[i]) <= bound + own), i
+        assert np.max(np.abs(got[i] - want[i])) < TOL * np.max(np.abs(want[i]))
