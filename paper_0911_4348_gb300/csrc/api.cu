@@ -244,7 +244,7 @@ int conv_f64_apply(fedvr_ctx *ctx, const CrtConv &c, int n, int M, const ConvCoe
   }
   FEDVR_CK(ctx, crt_conv_apply(c, ctx->w_crt.ptr, G, coef, I1, ctx->num_sms, s, fresh));
   FEDVR_CK(ctx, conv1_fp64(n, M, coef, dHF, A, G, I1, s, nullptr, P<int>(ctx->w_crt)));
-  *launches += fresh ? 5 : 7;
+  *launches += fresh ? 5 : 6;
   return FEDVR_OK;
 }
 // The whole first convolution (trapezoid or, with coef4, the fourth-order table).

@@ -284,26 +284,46 @@ __global__ void __launch_bounds__(1024)
   }
 }
 
-// s_b of another G with the same t_c: ec[b] = max over j, c of the exponent of
-// g_j[c][b] relative to its matrix, plus t_c.
+// f_j and s_b of another G with the same t_c: ec[b] = max over j, c of the exponent of
+// g_j[c][b] relative to its matrix, plus t_c. One CTA per matrix.
 template <bool TR>
-__global__ void __launch_bounds__(256)
-    crt_column_kernel(int n, int M, int chunk, const double *__restrict__ G, const int *__restrict__ eg,
-                      const int *__restrict__ et, int *__restrict__ ec) {
-  const long nn = (long)n * n, x = (long)blockIdx.x * 256 + threadIdx.x;
-  if (x >= nn) return;
-  const int k0 = blockIdx.y * chunk, k1 = min(M, k0 + chunk);
-  int m = kCrtNone;
-#pragma unroll 8
-  for (int k = k0; k < k1; ++k) {
-    const double v = G[(long)k * nn + x];
-    const int e = eg[k];
-    if (e != kCrtZero && v != 0.0) m = max(m, exponent_of(v) - e);
+__global__ void __launch_bounds__(512)
+    crt_column_kernel(int n, const double *__restrict__ G, const int *__restrict__ et,
+                      int *__restrict__ eg, int *__restrict__ ec, int *flag) {
+  extern __shared__ int cs_[];
+  __shared__ int top;
+  const long nn = (long)n * n;
+  const double *g = G + blockIdx.x * nn;
+  if (threadIdx.x == 0) top = kCrtNone;
+  for (int b = threadIdx.x; b < n; b += 512) cs_[b] = kCrtNone;
+  __syncthreads();
+  const int da = 512 / n, dc = 512 % n;
+  int a = threadIdx.x / n, c = threadIdx.x % n, m = kCrtNone;
+  bool bad = false;
+#pragma unroll 4
+  for (long x = threadIdx.x; x < nn; x += 512) {
+    const double v = g[x];
+    const int e = exponent_of(v), b = TR ? a : c;
+    bad |= !isfinite(v);
+    m = max(m, e);
+    if (e > kCrtNone) {
+      const int w = e + et[TR ? c : a];
+      if (w > cs_[b]) atomicMax(cs_ + b, w);
+    }
+    a += da;
+    c += dc;
+    if (c >= n) c -= n, ++a;
   }
-  if (m == kCrtNone) return;
-  const int c = (int)(TR ? x % n : x / n), b = (int)(TR ? x / n : x % n);
-  m += et[c];
-  if (m > *reinterpret_cast<volatile int *>(ec + b)) atomicMax(ec + b, m);
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0) atomicMax(&top, m);
+  if (bad) *flag = 1;
+  __syncthreads();
+  const int e = top;
+  if (threadIdx.x == 0) eg[blockIdx.x] = e > kCrtNone ? e : kCrtZero;
+  for (int b = threadIdx.x; b < n; b += 512) {
+    const int w = cs_[b] - e;
+    if (cs_[b] > kCrtNone && w > *reinterpret_cast<volatile int *>(ec + b)) atomicMax(ec + b, w);
+  }
 }
 
 // Residues of the source stack as bytes: planes [m][k][n nc] in the order of
@@ -904,15 +924,12 @@ cudaError_t apply_t(const CrtConv &c, void *wsv, const double *G, const Coef *co
   uint8_t *ws = reinterpret_cast<uint8_t *>(wsv);
   const ConvWs w = conv_ws(c, wsv);
   const int n = c.k.n, M = c.k.M;
-  const long nn = (long)n * n;
   if (!fresh) {
     cudaError_t e = cudaMemsetAsync(w.ec, 0x80, n * sizeof(int), s);
     if (e != cudaSuccess) return e;
-    crt_exp_stack_kernel<<<M, 256, 0, s>>>(nn, G, w.eg, w.head);
-    const int ch = entry_chunk(nn);
-    const dim3 ge((unsigned)((nn + 255) / 256), (unsigned)((M + ch - 1) / ch));
-    if (tr) crt_column_kernel<true><<<ge, 256, 0, s>>>(n, M, ch, G, w.eg, w.et, w.ec);
-    else crt_column_kernel<false><<<ge, 256, 0, s>>>(n, M, ch, G, w.eg, w.et, w.ec);
+    const size_t sm = n * sizeof(int);
+    if (tr) crt_column_kernel<true><<<M, 512, sm, s>>>(n, G, w.et, w.eg, w.ec, w.head);
+    else crt_column_kernel<false><<<M, 512, sm, s>>>(n, G, w.et, w.eg, w.ec, w.head);
   }
   const dim3 gg(M + 3, (n + 31) / 32, (c.k.nc + 63) / 64);
   const CrtScale sg{w.eg, w.nt, w.ec, 0, 0};
