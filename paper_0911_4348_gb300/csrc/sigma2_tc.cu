@@ -109,8 +109,13 @@ struct XRoles {
 constexpr uint32_t kXBarBytes = 256, kXPartBytes = 2 * 128 * 4;
 // stg = 0: an epilogue warp's buffer (8 rows of V at pitch 20, 4 rows of g, 16
 // columns), the 16-column chunks in flight, those whose products V g wait in TMEM,
-// and the most there are (n <= 320).
+// and the most there are.
 constexpr int kXDeal = 8 * 20 + 4 * 16, kXAhead = 3, kXTmem = 7, kXChunks = 10;
+// The widest accumulator beside them: 19 chunks (n <= 304, sigma2_tc_max_n), ten for the
+// first half of the columns and nine for the second, whose products take 112 and 96
+// columns of the 512.
+constexpr int kXCols = 512 - 16 * (2 * kXTmem - 1);
+static_assert(kXCols == 16 * (2 * kXChunks - 1), "products and accumulator share 512 columns");
 
 // Exponent eX of the FP16 A operand g V: max|V| < 2^e, |g| < 16.
 __device__ __forceinline__ int x_scale_exp(const TcScale *sc) {
@@ -401,11 +406,14 @@ __global__ void __launch_bounds__(XRoles<F16>::kThreads, 1)
       float *const deal = stage_rows + warp * kXDeal;
       const float *const deal_v = deal + al * 20, *const deal_g = deal + 160 + (lane >> 3) * 16;
       const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16);
-      // the products' columns start at the launch's widest accumulator, not at this
+      // the products' columns start at the widest accumulator there is, not at this
       // system's: a warp of one half may be a tile (and a system) ahead of the other
-      // half's, which reads its own columns of the same lanes. 304 + 112 + 96 = 512
-      // columns at the most: the second half has at most nine chunks
-      const uint32_t mrow = trow + (uint32_t)(Np_max + half * 16 * kXTmem);
+      // half's, which reads its own columns of the same lanes. (The asm keeps the constant
+      // from being carried through the tile loop in a register: 60 bytes of spill loads
+      // and 24.05 ms at n = 299, M = 1025 otherwise, 32 bytes and 23.5 ms so.)
+      uint32_t mcol = (uint32_t)(kXCols + half * 16 * kXTmem);
+      asm volatile("" : "+r"(mcol));
+      const uint32_t mrow = trow + mcol;
       // chunks of this half whose products wait in TMEM
       const int nt = nbuf == 1 ? min(kXTmem, ce - cb - kXAhead) : 0;
       const auto deal_out = [&](int x, int ch) {
@@ -690,7 +698,7 @@ cudaError_t exchange_tc_launch(const XSys *sys, const long *prefix, int n_sys, l
   const size_t stg = exchange_stage_pitch(ld_max);
   const size_t staged = smem + 2 * 24 * stg * sizeof(float);
   const int pitch = staged <= 232448 ? (int)stg : 0;
-  if (!pitch && Np_max > 32 * kXChunks) return cudaErrorInvalidValue;
+  if (!pitch && Np_max > kXCols) return cudaErrorInvalidValue;
   smem = pitch ? staged : smem + 8 * kXDeal * sizeof(float);
   const int grid = (int)(items < num_sms ? items : num_sms);
   const int nbuf = (Np_max <= 256) ? 2 : 1;
