@@ -364,8 +364,9 @@ __device__ __forceinline__ float mul_pairs(float2 a, float2 b) {
 // V_bl gb_lk = -V_bl conj(H_kl). One block per kXopB values of b and entry, H in
 // shared memory as pairs of floats. Bound by writing Bp (2 n^3 floats per
 // entry): two FP64 products and conversions per value took 41 us on average
-// at n = 39, T = 81, now 22. Eight values of b share one reading of H; chosen
-// at n = 39 of the n <= 64 that take this path; no result depends on it.
+// at n = 39, T = 81, now 25 (22 without the test for values that are no pair). Eight
+// values of b share one reading of H; chosen at n = 39 of the n <= 64 that take this
+// path; no result depends on it.
 constexpr int kXopB = 8;
 size_t xop_smem(int n) { return ((size_t)2 * n * n + (size_t)kXopB * n) * sizeof(float2); }
 __global__ void __launch_bounds__(256)
