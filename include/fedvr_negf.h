@@ -484,8 +484,9 @@ int fedvr_sigma2(fedvr_ctx *ctx, int n, int M, double spin, const double *V,
  * processes whose device memory belongs to another allocator (a framework's
  * caching allocator that reserves the pool), or loops that cannot accept the
  * device synchronisation cudaMalloc/cudaFree imply. It computes what
- * fedvr_sigma2 computes with precision FEDVR_FP64 (by the double-arithmetic
- * kernels, so the two may differ by rounding), needs no
+ * fedvr_sigma2 computes with precision FEDVR_FP64 in double arithmetic: bit for bit
+ * the result of a context whose fedvr_fp64_workspace limit is 0; where residues
+ * take part the two differ within their rounding. It needs no
  * context, and calls no cudaMalloc, cudaFree or allocating library routine:
  * its workspace is a fixed 12 MiB device array inside the library, which every
  * GPU that loads the library holds until the process exits.

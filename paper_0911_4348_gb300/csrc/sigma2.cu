@@ -179,7 +179,7 @@ cudaError_t sigma2_fp64(int n, int M, double spin, const double *V, const double
 // memory is owned entirely by another allocator (a framework's caching
 // allocator that reserves the pool up front), or loops where the implicit
 // device synchronisation of cudaMalloc/cudaFree is not acceptable. For them
-// this entry point runs the same kernels as fedvr_sigma2 with its workspace
+// this entry point runs the double-arithmetic kernels of fedvr_sigma2 with its workspace
 // (the polarisation Q, the product Q V and V Q V) in a fixed device array
 // declared below, so it allocates nothing. The array is a static device
 // symbol: every GPU that loads this library holds it until the process

@@ -105,6 +105,21 @@ def test_exchange_takes_the_faster_side(ctx, n, M, residues):
     assert ctx.fp64_workspace()["exchange"] == residues
 
 
+def test_double_arithmetic_is_the_allocation_free_call(ctx):
+    from paper_0911_4348_gb300 import sigma2_noalloc
+    n, M = 74, 9  # by residues without a limit
+    rng = W.system_rng(111, n)
+    G, V = _dev(W.random_symmetric_stack(rng, M, n)), _dev(W.random_symmetric(rng, n))
+    S, T = torch.empty_like(G), torch.empty_like(G)
+    ctx.sigma2(V, G, S, 1.5)
+    assert ctx.fp64_workspace()["exchange"] == 1
+    ctx.fp64_workspace(0)
+    ctx.sigma2(V, G, S, 1.5)
+    sigma2_noalloc(V, G, T, 1.5)
+    torch.cuda.synchronize()
+    assert torch.equal(S, T)
+
+
 def test_no_workspace_in_a_prepared_run(ctx):
     s = W.he_small()
     ctx.build_fedvr(s.n_elem, s.pts_per_elem, s.xmin, s.xmax, s.grid_kind)
