@@ -74,8 +74,13 @@ typedef enum {
                             below both (a function that decays away from its
                             diagonal) carry fewer correct bits than a sum in
                             double arithmetic. Small sizes, inputs that are not
-                            finite and results that cancel 2^10 below their
-                            products use double arithmetic throughout. */
+                            finite and mesh points whose result lies 2^10 below
+                            the largest products (sums that cancel, large
+                            entries that do not meet; 2^14 in the exchange) use
+                            double arithmetic throughout, so the largest entry
+                            of every mesh point's matrix is right whatever the
+                            inputs. fedvr_fp64_workspace asks for double
+                            arithmetic everywhere. */
   FEDVR_SPLIT_TF32 = 1,  /* Sigma^(2) (exchange and V Q V), I^(1) and, for
                             n_b >= 96, the I^(2) products on tensor cores:
                             hi+lo TF32 operands, FP32 accumulation, FP64

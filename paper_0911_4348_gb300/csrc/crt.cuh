@@ -34,12 +34,13 @@ constexpr int kCrtMod[kCrtMax] = {
 constexpr int kCrtQ = 56, kCrtQMax = 58;
 constexpr int kCrtQC = 54;
 // A result matrix whose largest integer has this many bits less than the largest
-// product could have is computed in double arithmetic instead. On the Green's
-// functions of He and H3+ (n = 11 to 118, M = 33 to 961) it has from 6 bits less to 7
-// more in the convolution and from 5 less to 1 more in the exchange; with 10 less
-// what the integers drop is still below 2^-44 of the largest entry for a single
-// product and about 2^-53 for the sums that occur.
-constexpr int kCrtGuard = 10;
+// product could have is computed in double arithmetic instead, and so is one whose
+// largest entry lies as far below the largest product of any row and column (kCrtGuardX in
+// the exchange). On the Green's functions of He and H3+ (n = 11 to 202, M = 33 to 961) both
+// are from 6 bits less to 7 more in the convolution; in the exchange the integer is
+// from 7 less to 1 more and the entry from 6 to 10 less, with rounding errors 2^-62 of
+// the largest product there (the sum's own terms average them out).
+constexpr int kCrtGuard = 10, kCrtGuardX = 14;
 constexpr int kCrtZero = -100000;  // exponent of an all-zero matrix
 constexpr int kCrtNone = -1000000; // exponent of a zero entry
 constexpr int kCrtFar = -20000;    // least exponent of a row or column that is used (an empty one)

@@ -19,8 +19,9 @@
 // What this keeps of an entry (a, b) is relative to the largest products of row a and
 // column b at any mesh point, not to the entry: entries far below both (a
 // Green's function that decays away from its diagonal) have fewer correct bits than
-// from the FP64 kernel. A result whose largest integer is 2^10 below the largest
-// product (mark_small) is left to the FP64 kernel.
+// from the FP64 kernel. A mesh point whose largest entry, or integer, is 2^10 below the
+// largest product (mark_small) is left to the FP64 kernel, so the largest entry of
+// every I1_i is right whatever the inputs.
 // The interpolation is done in the residues: for each modulus the A operand
 // sum_p c_p s_p of small integers is formed by the CUDA cores (dp2a on byte
 // pairs), reduced and written as FP16, the B operand is the residue plane of g,
@@ -215,9 +216,10 @@ inline int entry_chunk(long nn) { return nn < 4096 ? 8 : 32; }
 // Exponents r_a of the rows of the source, t_c of the contraction index and s_b of
 // the columns of G from the entries' (at most 0, or "none" far below): t_c moves
 // half the distance between what column c of the source and row c of G leave
-// unused, at most three times. Any t_c is right, since r_a and s_b are the largest of
-// what remains. One CTA.
-constexpr int kEquil = 3;
+// unused, until it rests or twelve times (where the rows of sparse matrices take up
+// the move, half of what is left remains each time). Any t_c is right, since r_a and s_b
+// are the largest of what remains. One CTA.
+constexpr int kEquil = 12;
 template <bool TR>
 __global__ void __launch_bounds__(1024)
     crt_equil_kernel(int n, const int *__restrict__ sm, const int *__restrict__ gm,
@@ -403,7 +405,7 @@ __global__ void __launch_bounds__(256) crt_coef_kernel(CrtMods mods, int M, int 
   if (threadIdx.x == 0) {  // the marks of the last apply
     if (i < M) {
       head[kCrtRows + i] = 0;
-      size[i] = kCrtNone;
+      size[2 * i] = size[2 * i + 1] = kCrtNone;
     } else {
       head[kCrtTicket] = 0;
       atomicCAS(head, kCrtSome, 0);
@@ -869,11 +871,23 @@ __global__ void __launch_bounds__(256) crt_rebuild_kernel(const __grid_constant_
     const int i = (int)(row / n), a = (int)(row - (long)i * n);
     const long o = tr ? (long)i * n * n + (long)col * n + a : x;
     int e;
-    out[o] = crt_value<W>(acc, E[i] + max(er[a], kCrtFar) + max(ec[col], kCrtFar) - kCrtQC - 2 * qb, &e);
-    big.note(size, i, e);
+    const double v =
+        crt_value<W>(acc, E[i] + max(er[a], kCrtFar) + max(ec[col], kCrtFar) - kCrtQC - 2 * qb, &e);
+    out[o] = v;
+    big.note(size, i, e, v);
   }
   big.finish(size);
-  mark_small(head, size, (int)(rows / n), kCrtQC + 2 * qb - kCrtGuard, [&](int i) { return E[i] != kCrtZero; });
+  if (!last_block(head)) return;
+  __shared__ int top[2];  // the largest scales of a row and of a column
+  if (threadIdx.x < 2) top[threadIdx.x] = kCrtFar;
+  __syncthreads();
+  for (int b = threadIdx.x; b < n; b += 256) {
+    atomicMax(top, er[b]);
+    atomicMax(top + 1, ec[b]);
+  }
+  __syncthreads();
+  mark_small(head, size, (int)(rows / n), kCrtQC + 2 * qb - kCrtGuard, [&](int i) { return E[i] != kCrtZero; },
+             [&](int i) { return E[i] + top[0] + top[1] - kCrtGuard; });
 }
 
 // The workspace's small arrays.
@@ -1033,7 +1047,7 @@ bool crt_conv_plan(int n, int M, int np, bool ext, int num_sms, bool any, CrtCon
   c.o_expg = take((size_t)M * 4);
   c.o_E = take((size_t)M * 4);
   c.o_er = take(4 * (size_t)n * 4);
-  c.o_size = take((size_t)M * 4);
+  c.o_size = take(2 * (size_t)M * 4);
   c.o_sm = take(2 * (size_t)n * n * 4);
   c.o_S = take((size_t)c.nm * c.KS * n * c.k.nc);
   c.o_B = take((size_t)c.nm * n * c.k.KP * 2);

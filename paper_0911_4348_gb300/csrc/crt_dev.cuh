@@ -274,50 +274,66 @@ __device__ __forceinline__ double crt_value(long long (&acc)[W], int scale, int 
   return neg ? -v : v;
 }
 
-// Largest exponent of the integers of each result matrix, and the matrices left
-// to double arithmetic. What the integers hold of an entry is relative to the
-// largest products of its row and its column, so a result whose largest integer
-// is 2^guard below the largest a single product can be (operands whose large
-// entries never meet, or a sum that cancels) is computed again by the FP64 kernel
-// that follows, matrix by matrix.
-// A thread of a rebuild kernel goes through entries of ascending matrix i.
+// What each result matrix reaches, and the matrices left to double arithmetic. What
+// the integers hold of an entry is relative to the largest products of its row and
+// its column. So a matrix whose largest integer is 2^kCrtGuard below the largest that a
+// single product can have, or whose largest entry is that far below the largest product
+// of any row and column (operands whose large entries never meet, or sums that
+// cancel), is computed again by the FP64 kernel that follows.
+// size[2 i]: largest exponent of its integers, size[2 i + 1]: of its entries. A thread of a
+// rebuild kernel goes through entries of ascending matrix i.
 struct CrtSize {
-  int i = -1, m = kCrtNone;
+  int i = -1, m = kCrtNone, r = kCrtNone;
   __device__ __forceinline__ void flush(int *size) {
-    if (m > kCrtNone) atomicMax(size + i, m);
+    if (m > kCrtNone) {
+      atomicMax(size + 2 * i, m);
+      atomicMax(size + 2 * i + 1, r);
+    }
   }
-  __device__ __forceinline__ void note(int *size, int at, int e) {
+  // an entry v of matrix at, its integer's exponent e
+  __device__ __forceinline__ void note(int *size, int at, int e, double v) {
     if (at != i) {
       flush(size);
       i = at;
-      m = kCrtNone;
+      m = r = kCrtNone;
     }
     m = max(m, e);
+    r = max(r, exponent_of(v));
   }
   // all threads of the block, at the end
   __device__ __forceinline__ void finish(int *size) {
     const int i0 = __reduce_max_sync(0xffffffffu, i);
     if (i != i0) flush(size);
     const int w = __reduce_max_sync(0xffffffffu, i == i0 ? m : kCrtNone);
-    if ((threadIdx.x & 31) == 0 && w > kCrtNone) atomicMax(size + i0, w);
+    const int v = __reduce_max_sync(0xffffffffu, i == i0 ? r : kCrtNone);
+    if ((threadIdx.x & 31) == 0 && w > kCrtNone) {
+      atomicMax(size + 2 * i0, w);
+      atomicMax(size + 2 * i0 + 1, v);
+    }
   }
 };
-// The last block to arrive marks the matrices i < M with some(i) (an operand product
-// that is not zero) and size[i] < least. head: the workspace's first integers.
-template <typename F>
-__device__ __forceinline__ void mark_small(int *head, const int *size, int M, int least, F some) {
+// True in the last block of the grid to arrive, after which all others' writes are seen.
+__device__ __forceinline__ bool last_block(int *head) {
   __shared__ bool last;
   __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) last = atomicAdd(head + kCrtTicket, 1) == (int)gridDim.x - 1;
   __syncthreads();
-  if (!last) return;
-  __threadfence();
-  for (int i = threadIdx.x; i < M; i += blockDim.x)
-    if (some(i) && *reinterpret_cast<const volatile int *>(size + i) < least) {
+  if (last) __threadfence();
+  return last;
+}
+// Marks the matrices i < M (all threads of the last block) with some(i), an operand
+// product that is not zero, whose largest integer has an exponent below least or whose
+// largest entry one below raw(i).
+template <typename F, typename R>
+__device__ __forceinline__ void mark_small(int *head, const int *size, int M, int least, F some, R raw) {
+  for (int i = threadIdx.x; i < M; i += blockDim.x) {
+    const volatile int *s = size + 2 * i;
+    if (some(i) && (s[0] < least || s[1] < raw(i))) {
       head[kCrtRows + i] = 1;
       atomicCAS(head, 0, kCrtSome);
     }
+  }
 }
 
 }  // namespace fedvr

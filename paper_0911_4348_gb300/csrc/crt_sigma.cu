@@ -13,7 +13,8 @@
 // per matrix left a quarter of them beyond 1e-14). In a box of 100 a tenth to a
 // half of the entries, those far below the largest of their row and column,
 // still have fewer bits than from FP64 arithmetic. A mesh point whose largest
-// integer is 2^10 below the largest product is left to the FP64 kernel.
+// integer is 2^10 below the largest product, or whose largest entry 2^14 below the
+// largest product of any row and column, is left to the FP64 kernel.
 // X is an integer below 2^(5 q) n^2, held by its residues modulo 41 to 43
 // moduli. For each modulus, row (b, a) of P^(b) = g
 // diag(V_b) gb is one FP16 product of small integers: the A operand g_al V_bl is
@@ -502,16 +503,18 @@ __global__ void __launch_bounds__(512)
 
 // Of mesh point j: ga_l = -(row scale of gb_l. and column scale of V_.l) and ra, the
 // largest exponents of the rows of g_al beside it; gk_k = -(column scale of gb_.k and of
-// V_.k) and cb, those of the columns of g_kb.
+// V_.k) and cb, those of the columns of g_kb; top, the largest scale of an entry of X.
 __global__ void __launch_bounds__(512)
     crt_meet_kernel(int n, int M, const double *__restrict__ G, const int *__restrict__ row,
                     const int *__restrict__ col, int *__restrict__ ra, int *__restrict__ ga,
-                    int *__restrict__ cb, int *__restrict__ gk) {
+                    int *__restrict__ cb, int *__restrict__ gk, int *__restrict__ top) {
   extern __shared__ int rs[];
+  __shared__ int best[2];
   int *ul = rs, *uk = rs + n, *cs = uk + n;
   const int j = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
   const long o = (long)j * n, ob = (long)(M - 1 - j) * n;
   const double *x = G + o * n;
+  if (tid < 2) best[tid] = 2 * kCrtFar;
   for (int l = tid; l < n; l += 512) {
     const int vc = col[(long)M * n + l];
     ul[l] = row[ob + l] + vc;
@@ -524,10 +527,18 @@ __global__ void __launch_bounds__(512)
     int m = kCrtNone;
     for (int l = lane; l < n; l += 32) m = max(m, exponent_of(x[(long)a * n + l]) + ul[l]);
     m = __reduce_max_sync(0xffffffffu, m);
-    if (lane == 0) ra[o + a] = max(m, kCrtFar);
+    if (lane == 0) {
+      ra[o + a] = max(m, kCrtFar);
+      atomicMax(best, max(m, kCrtFar) + row[(long)M * n + a]);
+    }
   }
   column_max(n, x, cs, [&](double v, int k) { return exponent_of(v) + uk[k]; });
-  for (int b = tid; b < n; b += 512) cb[o + b] = max(cs[b], kCrtFar);
+  for (int b = tid; b < n; b += 512) {
+    cb[o + b] = max(cs[b], kCrtFar);
+    atomicMax(best + 1, max(cs[b], kCrtFar) + row[(long)M * n + b]);
+  }
+  __syncthreads();
+  if (tid == 0) top[j] = best[0] + best[1];
 }
 
 // Residues of a stack as plain 16-bit rows [m][k][nr][ph], four columns per thread.
@@ -560,7 +571,7 @@ __global__ void __launch_bounds__(256) crt_rows_kernel(CrtMods mods, CrtK kk, in
 __global__ void crt_clear_kernel(int M, int *__restrict__ head, int *__restrict__ size) {
   for (int j = threadIdx.x; j < M; j += blockDim.x) {
     head[kCrtRows + j] = 0;
-    size[j] = kCrtNone;
+    size[2 * j] = size[2 * j + 1] = kCrtNone;
   }
   if (threadIdx.x < 2) head[threadIdx.x] = 0;
 }
@@ -570,7 +581,8 @@ __global__ void __launch_bounds__(256)
     crt_sigma_rebuild_kernel(const __grid_constant__ CrtWords<10> t, int n, int M, int nc, int CT, int qb,
                              double spin, const int8_t *__restrict__ R, const int *__restrict__ ra,
                              const int *__restrict__ cb, const int *__restrict__ vr,
-                             const int *__restrict__ some, int *head, int *__restrict__ size, int *report,
+                             const int *__restrict__ some, const int *__restrict__ top, int *head,
+                             int *__restrict__ size, int *report,
                              const double *__restrict__ G, const double *__restrict__ W,
                              double *__restrict__ Sigma) {
   if (const int f = *reinterpret_cast<volatile int *>(head)) {
@@ -602,14 +614,15 @@ __global__ void __launch_bounds__(256)
     for (int i = 0; i < 10; ++i) acc[i] -= (long long)q * (long long)t.P[i];
     int e;
     const double X = crt_value<10>(acc, vr[a] + vr[b] + ra[j * n + a] + cb[j * n + b] - 5 * qb, &e);
-    big.note(size, j, e);
+    big.note(size, j, e, X);
     const double v = spin * G[x] * W[x] - X;
     Sigma[x] = v;
     Sigma[(long)j * nn + (long)b * n + a] = v;
   }
   big.finish(size);
-  mark_small(head, size, M, 5 * qb - kCrtGuard,
-             [&](int j) { return some[j] && some[M - 1 - j] && some[M]; });
+  if (!last_block(head)) return;
+  mark_small(head, size, M, 5 * qb - kCrtGuard, [&](int j) { return some[j] && some[M - 1 - j] && some[M]; },
+             [&](int j) { return top[j] - kCrtGuardX; });
 }
 
 }  // namespace
@@ -670,7 +683,7 @@ bool crt_sigma_plan(int n, int M, bool any, size_t limit, CrtSigma *out) {
       o += (bytes + 255) / 256 * 256;
       return at;
     };
-    c.o_exp = take((2 * (size_t)(M + 1) * n + 4 * (size_t)M * n + 2 * (size_t)(M + 1)) * 4);
+    c.o_exp = take((2 * (size_t)(M + 1) * n + 4 * (size_t)M * n + 4 * (size_t)(M + 1)) * 4);
     c.o_g = take((size_t)c.group * M * mat * 2);
     c.o_gt = take((size_t)c.group * M * mat * 2);
     c.o_B = take((size_t)c.group * n * c.k.KP * 2);
@@ -692,11 +705,11 @@ cudaError_t crt_sigma_apply(const CrtSigma &c, void *wsv, double spin, const dou
   int *head = reinterpret_cast<int *>(ws);
   int *row = reinterpret_cast<int *>(ws + c.o_exp), *col = row + (long)(M + 1) * n;
   int *ra = col + (long)(M + 1) * n, *ga = ra + (long)M * n, *cb = ga + (long)M * n, *gk = cb + (long)M * n;
-  int *some = gk + (long)M * n, *size = some + M + 1;
+  int *some = gk + (long)M * n, *top = some + M + 1, *size = top + M;
   const int *vr = row + (long)M * n, *vc = col + (long)M * n;
   crt_clear_kernel<<<1, 256, 0, s>>>(M, head, size);
   crt_scale_kernel<<<M + 1, 512, 2 * n * sizeof(int), s>>>(n, M, G, V, row, col, some, head);
-  crt_meet_kernel<<<M, 512, 3 * n * sizeof(int), s>>>(n, M, G, row, col, ra, ga, cb, gk);
+  crt_meet_kernel<<<M, 512, 3 * n * sizeof(int), s>>>(n, M, G, row, col, ra, ga, cb, gk, top);
   cudaError_t e =
       cudaFuncSetAttribute(crt_sigma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c.smem);
   if (e != cudaSuccess) return e;
@@ -755,7 +768,7 @@ cudaError_t crt_sigma_apply(const CrtSigma &c, void *wsv, double spin, const dou
   const long total = (long)M * n * n;
   crt_sigma_rebuild_kernel<<<(unsigned)std::min<long>((total + 255) / 256, 152 * 16), 256, 0, s>>>(
       crt_words<10>(c.nm), n, M, c.k.nc, c.CT, c.q, spin, reinterpret_cast<const int8_t *>(ws + c.o_R), ra,
-      cb, vr, some, head, size, c.report, G, W, Sigma);
+      cb, vr, some, top, head, size, c.report, G, W, Sigma);
   return cudaGetLastError();
 }
 

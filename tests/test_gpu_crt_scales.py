@@ -158,6 +158,59 @@ def test_exchange_of_a_decaying_function_entry_by_entry(ctx, n_elem, order, half
         assert np.all(np.abs(got[j] - want) <= TOL * np.abs(terms)), j
 
 
+# Sparse and badly scaled in every index at once: no scales fit all products, so what the
+# integers cannot hold has to be left to double arithmetic. Mesh points may lie 2^10
+# below their largest products before that: 2^-47 sqrt(K) with K < 1e4 products, 1e-12.
+@pytest.mark.parametrize("seed", range(12))
+def test_sparse_and_badly_scaled_convolutions(ctx, seed):
+    rng = W.system_rng(112, seed)
+    n, u, p = int(rng.integers(12, 90)), int(rng.integers(1, 4)), int(rng.integers(2, 6))
+    order, M = int(rng.choice([2, 4])), 2 * u * p + 1
+    r, t, s = (np.ldexp(1.0, rng.integers(-200, 201, n)) for _ in range(3))
+    mesh = lambda: np.ldexp(1.0, rng.integers(-30, 31, M))[:, None, None]
+    A, G = rng.uniform(-1, 1, (M, n, n)) * mesh(), rng.uniform(-1, 1, (M, n, n)) * mesh()
+    A *= rng.random(A.shape) < 0.1
+    if seed % 2:
+        G *= rng.random(G.shape) < 0.1
+    A[rng.integers(M)] = 0.0
+    d = rng.uniform(-1, 1, (n, n))
+    left, right = r[:, None] / t[None, :], t[:, None] * s[None, :]
+    dev = [_dev(x) for x in (d * left, A * left, G * right)]
+    out, state = [], []
+    ctx.set_quadrature(order)
+    for limit in (0, 8 << 30):
+        ctx.fp64_workspace(limit)
+        I1 = torch.empty((M, n, n), dtype=torch.float64, device="cuda")
+        ctx.conv_sigma_g(40.0, u, p, *dev, I1)
+        out.append(I1.cpu().numpy())
+        state.append(ctx.fp64_workspace()["conv"])
+    ctx.set_quadrature(2)
+    assert state[0] == 0 and state[1] in (1, 2)
+    for i in range(M):
+        assert np.max(np.abs(out[1][i] - out[0][i])) <= 1e-12 * np.max(np.abs(out[0][i])), i
+
+
+@pytest.mark.parametrize("seed", range(12))
+def test_sparse_and_badly_scaled_exchange(ctx, seed):
+    rng = W.system_rng(113, seed)
+    n, M = int(rng.integers(12, 120)), int(rng.integers(1, 7))
+    G = W.random_symmetric_stack(rng, M, n)
+    keep = rng.random((n, n)) < 0.1
+    G = G * (keep | keep.T)
+    D = np.ldexp(1.0, rng.integers(-60, 61, (M, n)))
+    w = np.ldexp(1.0, rng.integers(-20, 21, n))
+    G = G * D[:, :, None] * D[:, None, :]
+    V = W.random_symmetric(rng, n) * w[:, None] * w[None, :]
+    ctx.fp64_workspace(0)
+    S = torch.empty(G.shape, dtype=torch.float64, device="cuda")
+    ctx.sigma2(_dev(V), _dev(G), S, 0.0)
+    want = S.cpu().numpy()
+    ctx.fp64_workspace(8 << 30)
+    got = _exchange(ctx, V, G)
+    for j in range(M):
+        assert np.max(np.abs(got[j] - want[j])) <= 1e-12 * np.max(np.abs(want[j])), j
+
+
 def test_convolution_of_a_decaying_function(ctx):
     # what is kept of an entry is relative to the largest products of its row and column
     # over the mesh points, whatever the entry itself is: K = 2 M n roundings of 2^-57 each,
