@@ -229,7 +229,7 @@ int conv_f64_source(fedvr_ctx *ctx, const CrtConv &c, const ConvCoef *coef, cons
                     const double *A, const double *G, cudaStream_t s, int *launches) {
   if (!c.bytes) return FEDVR_OK;
   FEDVR_CK(ctx, crt_conv_source(c, ctx->w_crt.ptr, A, dHF, G, coef, s));
-  *launches += 5;
+  *launches += 3;
   return FEDVR_OK;
 }
 int conv_f64_apply(fedvr_ctx *ctx, const CrtConv &c, int n, int M, const ConvCoef *coef,
@@ -265,7 +265,7 @@ int conv_f64(fedvr_ctx *ctx, const CrtConv &c, int n, int M, const ConvCoef *coe
   FEDVR_CK(ctx, crt_conv_source4(c, ctx->w_crt.ptr, A, dHF, G, coef4, s));
   FEDVR_CK(ctx, crt_conv_apply4(c, ctx->w_crt.ptr, G, coef4, I1, ctx->num_sms, s));
   FEDVR_CK(ctx, conv1_fp64_q4(n, M, coef4, dHF, A, G, I1, s, nullptr, P<int>(ctx->w_crt)));
-  *launches += 10;
+  *launches += 8;
   return FEDVR_OK;
 }
 

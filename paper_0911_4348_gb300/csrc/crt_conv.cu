@@ -155,63 +155,60 @@ __device__ __forceinline__ double2 diag_weights(const ConvCoef4 &c) {
   return make_double2(c.c[0], c.c[1]);
 }
 
-// Exponents of the source stack; matrices M .. 2 M - 1 (ext) are the diagonal
-// operands, formed on the fly, later ones never weighted.
+// Exponents e of the matrices (max |x| < 2^e; kCrtZero where there is nothing): es of the
+// source's KS (M .. 2 M - 1 with ext are the diagonal operands, formed on the fly, later
+// ones never weighted), then eg of G's M. And the largest exponent of each entry over the
+// mesh points, relative to its matrix: sm [n n] of the source, gm of G as stored. A value
+// that is not finite raises *flag. One CTA per matrix, which keeps its exponents in shared
+// memory (kept: nn 16-bit integers) where they fit, so that the diagonal operands, bound by
+// their FP64 arithmetic, are formed once. n = 119, M = 257: 119 us in three kernels, 83 in
+// this one; n = 15, M = 129: 16 and 6.
 template <typename Coef>
-__global__ void __launch_bounds__(256) crt_exp_kernel(long nn, int M, const double *__restrict__ A,
-                                                      const double *__restrict__ dHF,
-                                                      const Coef *__restrict__ coef, int *expo,
-                                                      int *flag) {
-  const int k = blockIdx.x;
-  if (k < M) {
-    const double *a = A + (long)k * nn;
-    matrix_exponent(nn, expo + k, flag, [&](long e) { return a[e]; });
-  } else if (k < 2 * M) {
-    const int i = k - M;
-    const double2 w = diag_weights(coef[(long)i * M + i]);
-    const double *a0 = A, *a1 = A + (long)(M - 1) * nn;
-    matrix_exponent(nn, expo + k, flag,
-                    [&](long e) { return diag_elem(w.x, w.y, a0[e], a1[e], dHF[e]); });
-  } else if (threadIdx.x == 0) {
-    expo[k] = kCrtZero;
+__global__ void __launch_bounds__(512)
+    crt_exp_kernel(long nn, int M, int KS, int Ks, bool kept, const double *__restrict__ A,
+                   const double *__restrict__ dHF, const Coef *__restrict__ coef,
+                   const double *__restrict__ G, int *__restrict__ es, int *__restrict__ eg,
+                   int *__restrict__ sm, int *__restrict__ gm, int *flag) {
+  extern __shared__ int16_t ke[];
+  __shared__ int top;
+  const int k = blockIdx.x, tid = threadIdx.x;
+  const bool src = k < KS;
+  int *e_out = src ? es + k : eg + (k - KS), *entry = src ? sm : gm;
+  if (src && k >= Ks) {
+    if (tid == 0) *e_out = kCrtZero;
+    return;
   }
-}
-
-// Largest exponent of each entry over the mesh points, relative to the matrices'
-// own: sm [n n] of the source stack (its ext diagonal operands too), gm [n n] of G as
-// stored. `chunk` matrices per block row, the source's first.
-template <typename Coef>
-__global__ void __launch_bounds__(256)
-    crt_entry_kernel(long nn, int M, int Ks, int chunk, const double *__restrict__ A,
-                     const double *__restrict__ dHF, const Coef *__restrict__ coef,
-                     const int *__restrict__ es, const double *__restrict__ G,
-                     const int *__restrict__ eg, int *__restrict__ sm, int *__restrict__ gm) {
-  const long x = (long)blockIdx.x * 256 + threadIdx.x;
-  if (x >= nn) return;
-  const int sc = (Ks + chunk - 1) / chunk;
-  const bool src = (int)blockIdx.y < sc;
-  const int k0 = (src ? blockIdx.y : blockIdx.y - sc) * chunk, k1 = min(src ? Ks : M, k0 + chunk);
-  const double *X = src ? A : G;
-  const int *ex = src ? es : eg;
+  double2 w = make_double2(0.0, 0.0);
+  const bool diag = src && k >= M;
+  if (diag) w = diag_weights(coef[(long)(k - M) * M + (k - M)]);
+  const double *X = src ? A + (diag ? 0 : (long)k * nn) : G + (long)(k - KS) * nn;
+  const double *X1 = A + (long)(M - 1) * nn;
+  auto value = [&](long x) { return diag ? diag_elem(w.x, w.y, X[x], X1[x], dHF[x]) : X[x]; };
+  if (tid == 0) top = kCrtNone;
+  __syncthreads();
   int m = kCrtNone;
-  auto note = [&](double v, int e) {
-    if (e != kCrtZero && v != 0.0) m = max(m, exponent_of(v) - e);
-  };
-#pragma unroll 8
-  for (int k = k0; k < min(k1, M); ++k) note(X[(long)k * nn + x], ex[k]);
-  if (k1 > M) {
-    const double s0 = A[x], s1 = A[(long)(M - 1) * nn + x], h = dHF[x];
-#pragma unroll 8
-    for (int k = max(k0, M); k < k1; ++k) {
-      const double2 w = diag_weights(coef[(long)(k - M) * M + (k - M)]);
-      note(diag_elem(w.x, w.y, s0, s1, h), ex[k]);
-    }
+  bool bad = false;
+#pragma unroll 4
+  for (long x = tid; x < nn; x += 512) {
+    const int e = exponent_of(value(x));
+    bad |= e == 1025;  // the exponent of infinities and NaN
+    m = max(m, e);
+    if (kept) ke[x] = (int16_t)max(e, -32768);
   }
-  if (m > kCrtNone) atomicMax((src ? sm : gm) + x, m);
+  if (bad) *flag = 1;
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((tid & 31) == 0) atomicMax(&top, m);
+  __syncthreads();
+  const int e0 = top;
+  if (tid == 0) *e_out = e0 > kCrtNone ? e0 : kCrtZero;
+  if (e0 == kCrtNone) return;
+#pragma unroll 4
+  for (long x = tid; x < nn; x += 512) {
+    const int e = kept ? ke[x] : max(exponent_of(value(x)), -32768);
+    if (e == -32768) continue;
+    if (e - e0 > *reinterpret_cast<volatile int *>(entry + x)) atomicMax(entry + x, e - e0);
+  }
 }
-// Matrices per block row of the passes over the mesh points: many blocks, but few
-// enough atomics.
-inline int entry_chunk(long nn) { return nn < 4096 ? 8 : 32; }
 
 // Exponents r_a of the rows of the source, t_c of the contraction index and s_b of
 // the columns of G from the entries' (at most 0, or "none" far below): t_c moves
@@ -916,11 +913,12 @@ cudaError_t source_t(const CrtConv &c, void *wsv, const double *A, const double 
   cudaError_t e = cudaMemsetAsync(w.head, 0, 2 * sizeof(int), s);
   if (e == cudaSuccess) e = cudaMemsetAsync(w.sm, 0x80, 2 * nn * sizeof(int), s);  // far below kCrtNone
   if (e != cudaSuccess) return e;
-  crt_exp_kernel<Coef><<<c.KS, 256, 0, s>>>(nn, M, A, dHF, coef, w.es, w.head);
-  crt_exp_stack_kernel<<<M, 256, 0, s>>>(nn, G, w.eg, w.head);
-  const int ch = entry_chunk(nn);
-  const dim3 ge((unsigned)((nn + 255) / 256), (unsigned)((Ks + ch - 1) / ch + (M + ch - 1) / ch));
-  crt_entry_kernel<Coef><<<ge, 256, 0, s>>>(nn, M, Ks, ch, A, dHF, coef, w.es, G, w.eg, w.sm, w.gm);
+  const size_t ks = nn * sizeof(int16_t);
+  const bool kept = ks <= 112 * 1024;  // two CTAs per SM
+  e = cudaFuncSetAttribute(crt_exp_kernel<Coef>, cudaFuncAttributeMaxDynamicSharedMemorySize, 112 * 1024);
+  if (e != cudaSuccess) return e;
+  crt_exp_kernel<Coef><<<c.KS + M, 512, kept ? ks : 0, s>>>(nn, M, c.KS, Ks, kept, A, dHF, coef, G, w.es,
+                                                            w.eg, w.sm, w.gm, w.head);
   const size_t sm = 5 * (size_t)n * sizeof(int);
   if (tr) crt_equil_kernel<true><<<1, 1024, sm, s>>>(n, w.sm, w.gm, w.er, w.et, w.ec, w.nt);
   else crt_equil_kernel<false><<<1, 1024, sm, s>>>(n, w.sm, w.gm, w.er, w.et, w.ec, w.nt);

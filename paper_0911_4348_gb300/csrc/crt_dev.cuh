@@ -98,39 +98,6 @@ __device__ __forceinline__ long crt_x(const CrtK &k, int j, int c) {
   return x + (long)j * 16 + r;
 }
 
-// Exponent e of each matrix of a stack (max |x| < 2^e), one CTA per matrix; a
-// value that is not finite raises *flag. elem(k, x): entry x of matrix k.
-template <typename F>
-__device__ __forceinline__ void matrix_exponent(long nn, int *expo, int *flag, F elem) {
-  unsigned long long m = 0;
-  for (long e = threadIdx.x; e < nn; e += 256) {
-    const unsigned long long b =
-        (unsigned long long)__double_as_longlong(elem(e)) & 0x7fffffffffffffffull;
-    m = b > m ? b : m;
-  }
-  __shared__ unsigned long long sh[8];
-  for (int o = 16; o > 0; o >>= 1) {
-    const unsigned long long y = __shfl_xor_sync(0xffffffffu, m, o);
-    m = y > m ? y : m;
-  }
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = m;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < 8; ++w) m = sh[w] > m ? sh[w] : m;
-    if (m >= 0x7ff0000000000000ull) {
-      *flag = 1;
-      *expo = kCrtZero;
-    } else {
-      *expo = m ? ilogb(__longlong_as_double((long long)m)) + 1 : kCrtZero;
-    }
-  }
-}
-static __global__ void __launch_bounds__(256) crt_exp_stack_kernel(long nn, const double *__restrict__ A,
-                                                                   int *expo, int *flag) {
-  const double *a = A + (long)blockIdx.x * nn;
-  matrix_exponent(nn, expo + blockIdx.x, flag, [&](long e) { return a[e]; });
-}
-
 // Residue bytes of four columns c0 .. c0 + 3 of row a of matrix k into planes
 // [m][k][n nc] in the order of src_off.
 __device__ __forceinline__ void put_source(const CrtMods &mods, const CrtK &kk, long plane, int k, int a,
